@@ -79,7 +79,8 @@ static void validate_gates(int n, const sv_gate *gates, int64_t n_gates) {
 // the kernel copies them into shared memory.
 struct BlockProg {
     size_t off;
-    int nseg, ngate;
+    int nseg, gate_bytes;  // SIMT: bytes of the gate area
+    bool fixed = false;    // SIMT complex128: fixed-point gate area
     int r = 0;         // tensor-core register-group width of the sweep
     GatherLayout lay;  // gathered sections only
     int op_index = -1;
@@ -189,7 +190,7 @@ static void build_programs_tc(const sv_plan *plan, const sv_gate *gates, int r_p
             align(256);
             bp.off = host.size();
             bp.nseg = (int)(p1 - p0);
-            bp.ngate = 0;
+            bp.gate_bytes = 0;
             for (size_t k = p0; k < p1; ++k) {
                 const HostSeg &s = segs[k];
                 DevSeg d;
@@ -290,17 +291,25 @@ static void build_programs(const sv_plan *plan, const sv_gate *gates, int seg_bi
             }
             if (dgates.size() > 32767) fail(SV_ERR_UNSUPPORTED, "too many gates in one blocking section");
             d.g1 = (int16_t)dgates.size();
+            if constexpr (sizeof(T) == 8)
+                if (std::all_of(dgates.begin() + d.g0, dgates.end(), exact_gate)) d.flags |= kSegRaw;
             dsegs.push_back(d);
         }
         align(256);
         bp.off = host.size();
         bp.nseg = (int)dsegs.size();
-        bp.ngate = (int)dgates.size();
         const unsigned char *p = reinterpret_cast<const unsigned char *>(dsegs.data());
         host.insert(host.end(), p, p + dsegs.size() * sizeof(DevSeg));
         align(16);
-        p = reinterpret_cast<const unsigned char *>(dgates.data());
-        host.insert(host.end(), p, p + dgates.size() * sizeof(DevGate<T>));
+        // complex128: fixed-point gates where every gate is unitary (their area is never the larger)
+        std::vector<unsigned char> area;
+        if constexpr (sizeof(T) == 8) bp.fixed = encode_fx(dgates, area);
+        if (!bp.fixed) {
+            p = reinterpret_cast<const unsigned char *>(dgates.data());
+            area.assign(p, p + dgates.size() * sizeof(DevGate<T>));
+        }
+        bp.gate_bytes = (int)area.size();
+        host.insert(host.end(), area.begin(), area.end());
         align(16);
         progs.push_back(bp);
     }
@@ -313,7 +322,7 @@ void build_simt_programs(const sv_plan *plan, const sv_gate *gates, int dtype, S
     if (dtype == SV_C64) build_programs<float>(plan, gates, out.seg_bits, out.host, progs);
     else build_programs<double>(plan, gates, out.seg_bits, out.host, progs);
     out.progs.clear();
-    for (const BlockProg &bp : progs) out.progs.push_back(SimtPrograms::Prog{bp.off, bp.nseg, bp.ngate, bp.op_index});
+    for (const BlockProg &bp : progs) out.progs.push_back(SimtPrograms::Prog{bp.off, bp.nseg, bp.gate_bytes, bp.fixed, bp.op_index});
 }
 
 static void upload_program(sv_state *h, const std::vector<unsigned char> &host) {
@@ -658,11 +667,11 @@ sv_status sv_apply_circuit(sv_handle h, const sv_gate *gates, int64_t n_gates, s
                         launch_block_tc(h->amp, h->n, plan->c, bp.gathered ? &bp.lay : nullptr, base + bp.off, bp.nseg,
                                         h->dev_err, bp.r, h->stream, wait_ns);
                     else if (!bp.gathered)
-                        launch_block(h->dtype, h->amp, h->n, plan->c, base + bp.off, bp.nseg, bp.ngate, h->dev_err,
-                                     seg_bits, h->stream, wait_ns);
+                        launch_block(h->dtype, h->amp, h->n, plan->c, base + bp.off, bp.nseg, bp.gate_bytes, bp.fixed,
+                                     h->dev_err, seg_bits, h->stream, wait_ns);
                     else
-                        launch_block_gather(h->dtype, h->amp, h->n, bp.lay, base + bp.off, bp.nseg, bp.ngate,
-                                            h->dev_err, seg_bits, h->stream, wait_ns);
+                        launch_block_gather(h->dtype, h->amp, h->n, bp.lay, base + bp.off, bp.nseg, bp.gate_bytes,
+                                            bp.fixed, h->dev_err, seg_bits, h->stream, wait_ns);
                     mark_end(h);
                     ++st.sweeps_block;
                     ++st.kernel_launches;
@@ -717,8 +726,8 @@ sv_status sv_apply_plan_ops(sv_handle h, const sv_gate *gates, int64_t n_gates, 
             while (bi < progs.size() && progs[bi].op_index < oi) ++bi;
             if (bi == progs.size() || progs[bi].op_index != oi) fail(SV_ERR_PLAN, "no program for a blocking section");
             const BlockProg &bp = progs[bi];
-            launch_block(h->dtype, h->amp, h->n, plan->c, base + bp.off, bp.nseg, bp.ngate, h->dev_err, seg_bits,
-                         h->stream, wait_ns);
+            launch_block(h->dtype, h->amp, h->n, plan->c, base + bp.off, bp.nseg, bp.gate_bytes, bp.fixed, h->dev_err,
+                         seg_bits, h->stream, wait_ns);
         } else {
             // pairs inside the piece; the others move data between pieces and are the caller's
             std::vector<std::pair<int32_t, int32_t>> local;

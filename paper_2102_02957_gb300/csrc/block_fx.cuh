@@ -1,0 +1,396 @@
+// Register-group engine of complex128 sections on the integer pipe (arithmetic: fixed64.cuh).
+//
+// Same shape as run_segment: a thread loads the 16 amplitudes spanned by the group's 4 chunk bits,
+// applies every gate of the group, stores them back.  In between the components are block
+// fixed-point integers with one exponent per thread, converted once each way per group -- or, in a
+// group that only exchanges amplitudes and flips signs (kSegRaw), the doubles' own words.
+//
+// Bound by the multiply-add pipe (57 % busy on random-layer sections, where run_segment kept the
+// FP64 pipe full) and by the dependent chains that two warps per scheduler leave exposed: 168
+// registers a thread allow no more, and 3 x 128 threads of 128 registers spill (217 ms against 166
+// for the first line below).  Measured against FP64 register groups, n qubits, 12-bit chunks:
+//   27, 8 random layers (12 sections, 44 groups)       417 -> 169 ms
+//   28, QFT with diagonals outside the chunk           393 -> 239 ms
+//   25, quantum volume of 10 layers, gathered chunks   108 -> 38.6 ms
+//
+// The section's gate area is a table of 16-byte headers {op, payload offset, outside bits, code},
+// then the payloads (encode_fx writes them):
+//   OP_DENSE1 / OP_DENSE2  4 / 16 entries {re h, re l, im h, im l}     OP_REAL1  4 x {h, l}
+//   OP_DIAG1 / OP_DIAG2    2 / 4 entries   OP_DIAGX  2 or 4 OP_DIAG1   OP_PERM2  4 ints
+#pragma once
+#include "block_core.cuh"
+#include "fixed64.cuh"
+
+namespace sv {
+namespace {
+
+// Real and imaginary component of every amplitude of the thread's group.
+template <int NA>
+struct FxGroup {
+    fx::Real re[NA], im[NA];
+};
+
+struct FxEntry {
+    int rh, rl, ih, il;
+};
+__device__ __forceinline__ FxEntry lds_entry(uint32_t a) {
+    FxEntry e;
+    ldc_i4(a, e.rh, e.rl, e.ih, e.il);
+    return e;
+}
+
+// (yr, yi) accumulators += entry * (xr + i xi)
+__device__ __forceinline__ void fx_cmac(fx::Acc &yr, fx::Acc &yi, const FxEntry &m, const fx::Real &xr, const fx::Real &xi) {
+    fx::mac(yr, xr, m.rh, m.rl);
+    fx::mac(yr, xi, -m.ih, -m.il);
+    fx::mac(yi, xi, m.rh, m.rl);
+    fx::mac(yi, xr, m.ih, m.il);
+}
+
+template <int NA, int A>
+__device__ __forceinline__ void fx_dense1(FxGroup<NA> &v, uint32_t ma) {
+    const FxEntry m0 = lds_entry(ma), m1 = lds_entry(ma + 16), m2 = lds_entry(ma + 32), m3 = lds_entry(ma + 48);
+#pragma unroll
+    for (int x = 0; x < NA; ++x) {
+        if (x & (1 << A)) continue;
+        const int y = x | (1 << A);
+        fx::Acc pr, pi, qr, qi;
+        fx_cmac(pr, pi, m0, v.re[x], v.im[x]);
+        fx_cmac(pr, pi, m1, v.re[y], v.im[y]);
+        fx_cmac(qr, qi, m2, v.re[x], v.im[x]);
+        fx_cmac(qr, qi, m3, v.re[y], v.im[y]);
+        v.re[x] = fx::fin(pr); v.im[x] = fx::fin(pi);
+        v.re[y] = fx::fin(qr); v.im[y] = fx::fin(qi);
+    }
+}
+
+// Real matrix (RY, H): half the products.
+template <int NA, int A>
+__device__ __forceinline__ void fx_real1(FxGroup<NA> &v, uint32_t ma) {
+    const FxEntry r0 = lds_entry(ma), r1 = lds_entry(ma + 16);  // rows {m0 h, m0 l, m1 h, m1 l}
+#pragma unroll
+    for (int x = 0; x < NA; ++x) {
+        if (x & (1 << A)) continue;
+        const int y = x | (1 << A);
+#pragma unroll
+        for (int part = 0; part < 2; ++part) {
+            fx::Real &a = part ? v.im[x] : v.re[x], &b = part ? v.im[y] : v.re[y];
+            fx::Acc p, q;
+            fx::mac(p, a, r0.rh, r0.rl);
+            fx::mac(p, b, r0.ih, r0.il);
+            fx::mac(q, a, r1.rh, r1.rl);
+            fx::mac(q, b, r1.ih, r1.il);
+            a = fx::fin(p);
+            b = fx::fin(q);
+        }
+    }
+}
+
+template <int NA, int A, int B>
+__device__ __forceinline__ void fx_dense2(FxGroup<NA> &v, uint32_t ma) {
+#pragma unroll
+    for (int x = 0; x < NA; ++x) {
+        if (x & ((1 << A) | (1 << B))) continue;
+        const int id[4] = {x, x | (1 << A), x | (1 << B), x | (1 << A) | (1 << B)};
+        fx::Real xr[4], xi[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) { xr[k] = v.re[id[k]]; xi[k] = v.im[id[k]]; }
+#pragma unroll
+        for (int rr = 0; rr < 4; ++rr) {
+            fx::Acc yr, yi, ii{0, 0};  // ii: the products of imaginary parts, subtracted
+#pragma unroll
+            for (int cc = 0; cc < 4; ++cc) {
+                const FxEntry m = lds_entry(ma + 16 * (4 * rr + cc));
+                fx::mac(yr, xr[cc], m.rh, m.rl);
+                fx::mac(ii, xi[cc], m.ih, m.il);
+                fx::mac(yi, xi[cc], m.rh, m.rl);
+                fx::mac(yi, xr[cc], m.ih, m.il);
+            }
+            yr.hi -= ii.hi;
+            yr.mid -= ii.mid;
+            v.re[id[rr]] = fx::fin(yr);
+            v.im[id[rr]] = fx::fin(yi);
+        }
+    }
+}
+
+// Diagonal entry l on the amplitudes whose gate bits read l; entries of exactly 1 and -1 take no
+// products (uniform over the warp).
+template <int NA, int A, int B, int NL>
+__device__ __forceinline__ void fx_diag(FxGroup<NA> &v, uint32_t ma, bool raw) {
+#pragma unroll
+    for (int l = 0; l < NL; ++l) {
+        const FxEntry d = lds_entry(ma + 16 * l);
+        const bool real = d.rl == 0 && d.ih == 0 && d.il == 0;
+        if (real && d.rh == fx::kOne) continue;
+        if (real && d.rh == -fx::kOne) {
+#pragma unroll
+            for (int x = 0; x < NA; ++x)
+                if ((((x >> A) & 1) | (NL == 4 ? ((x >> B) & 1) << 1 : 0)) == l) {
+                    v.re[x] = raw ? fx::flip_sign(v.re[x]) : fx::negate(v.re[x]);
+                    v.im[x] = raw ? fx::flip_sign(v.im[x]) : fx::negate(v.im[x]);
+                }
+            continue;
+        }
+#pragma unroll
+        for (int x = 0; x < NA; ++x)
+            if ((((x >> A) & 1) | (NL == 4 ? ((x >> B) & 1) << 1 : 0)) == l) {
+                fx::Acc yr, yi;
+                fx_cmac(yr, yi, d, v.re[x], v.im[x]);
+                v.re[x] = fx::fin(yr);
+                v.im[x] = fx::fin(yi);
+            }
+    }
+}
+
+template <int NA, int A>
+__device__ __forceinline__ void fx_x1(FxGroup<NA> &v) {
+#pragma unroll
+    for (int x = 0; x < NA; ++x) {
+        if (x & (1 << A)) continue;
+        const int y = x | (1 << A);
+        fx::Real t = v.re[x]; v.re[x] = v.re[y]; v.re[y] = t;
+        t = v.im[x]; v.im[x] = v.im[y]; v.im[y] = t;
+    }
+}
+
+template <int NA, int A, int B, int U, int V>
+__device__ __forceinline__ void fx_xchg2(FxGroup<NA> &v) {
+#pragma unroll
+    for (int x = 0; x < NA; ++x) {
+        if (x & ((1 << A) | (1 << B))) continue;
+        const int id[4] = {x, x | (1 << A), x | (1 << B), x | (1 << A) | (1 << B)};
+        fx::Real t = v.re[id[U]]; v.re[id[U]] = v.re[id[V]]; v.re[id[V]] = t;
+        t = v.im[id[U]]; v.im[id[U]] = v.im[id[V]]; v.im[id[V]] = t;
+    }
+}
+
+template <int NA, int A, int B>
+__device__ __forceinline__ void fx_perm2(FxGroup<NA> &v, uint32_t ma) {
+    int p[4];
+    ldc_i4(ma, p[0], p[1], p[2], p[3]);
+#pragma unroll
+    for (int x = 0; x < NA; ++x) {
+        if (x & ((1 << A) | (1 << B))) continue;
+        const int id[4] = {x, x | (1 << A), x | (1 << B), x | (1 << A) | (1 << B)};
+        fx::Real xr[4], xi[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) { xr[k] = v.re[id[k]]; xi[k] = v.im[id[k]]; }
+#pragma unroll
+        for (int rr = 0; rr < 4; ++rr) {
+            const int s = p[rr];
+            v.re[id[rr]] = s == 0 ? xr[0] : s == 1 ? xr[1] : s == 2 ? xr[2] : xr[3];
+            v.im[id[rr]] = s == 0 ? xi[0] : s == 1 ? xi[1] : s == 2 ? xi[2] : xi[3];
+        }
+    }
+}
+
+template <int NA, int A>
+__device__ __forceinline__ void fx_one(int op, FxGroup<NA> &v, uint32_t m, bool raw) {
+    if (op == OP_DENSE1) fx_dense1<NA, A>(v, m);
+    else if (op == OP_REAL1) fx_real1<NA, A>(v, m);
+    else if (op == OP_X1) fx_x1<NA, A>(v);
+    else fx_diag<NA, A, 0, 2>(v, m, raw);
+}
+
+template <int NA, int A, int B>
+__device__ __forceinline__ void fx_two(int op, FxGroup<NA> &v, uint32_t m, bool raw) {
+    if (op == OP_DENSE2) fx_dense2<NA, A, B>(v, m);
+    else if (op == OP_DIAG2) fx_diag<NA, A, B, 4>(v, m, raw);
+    else if (op == OP_CXA) fx_xchg2<NA, A, B, 1, 3>(v);
+    else if (op == OP_CXB) fx_xchg2<NA, A, B, 2, 3>(v);
+    else if (op == OP_SWAP2) fx_xchg2<NA, A, B, 1, 2>(v);
+    else fx_perm2<NA, A, B>(v, m);
+}
+
+__device__ __forceinline__ void fx_apply(int op, int code, uint32_t m, FxGroup<16> &v, bool raw) {
+    if (op == OP_DENSE1 || op == OP_REAL1 || op == OP_DIAG1 || op == OP_X1) {
+        switch (code) {
+            case 0: fx_one<16, 0>(op, v, m, raw); break;
+            case 1: fx_one<16, 1>(op, v, m, raw); break;
+            case 2: fx_one<16, 2>(op, v, m, raw); break;
+            default: fx_one<16, 3>(op, v, m, raw); break;
+        }
+    } else {
+        switch (code) {
+            case 0 * 8 + 1: fx_two<16, 0, 1>(op, v, m, raw); break;
+            case 0 * 8 + 2: fx_two<16, 0, 2>(op, v, m, raw); break;
+            case 0 * 8 + 3: fx_two<16, 0, 3>(op, v, m, raw); break;
+            case 1 * 8 + 2: fx_two<16, 1, 2>(op, v, m, raw); break;
+            case 1 * 8 + 3: fx_two<16, 1, 3>(op, v, m, raw); break;
+            default: fx_two<16, 2, 3>(op, v, m, raw); break;
+        }
+    }
+}
+
+// Payload of a gate of group [g0, g1) once its outside bits are read off the chunk's origin.
+struct FxGate {
+    int op, code;
+    uint32_t m;
+};
+__device__ __forceinline__ FxGate fx_gate(uint32_t gates, int gi, int64_t origin) {
+    int op, off, rb, code;
+    ldc_i4(gates + 16u * (uint32_t)gi, op, off, rb, code);
+    uint32_t m = gates + (uint32_t)off;
+    if (op == OP_DIAGX) {
+        const int e0 = rb & 0xFF, e1 = (rb >> 8) & 0xFF;
+        int v = (int)((origin >> e0) & 1);
+        if (e1 != 0xFF) v |= (int)((origin >> e1) & 1) << 1;
+        m += (uint32_t)(32 * v);
+        op = OP_DIAG1;
+    }
+    return FxGate{op, code, m};
+}
+
+__device__ __forceinline__ double fx_entry_value(uint32_t a) {
+    const int h = lds_s32(a), l = lds_s32(a + 4);
+    return ((double)h * 4294967296.0 + (double)l) * 0x1p-61;
+}
+
+// The group in FP64, for components outside the fixed-point range (infinities, NaN, magnitudes
+// near the ends of the exponent range).  Not a hot path: one copy of the code, amplitudes in
+// local memory.
+__device__ __noinline__ void fx_group_fp64(double *re, double *im, uint32_t gates, int g0, int g1, int64_t origin) {
+    for (int gi = g0; gi < g1; ++gi) {
+        const FxGate g = fx_gate(gates, gi, origin);
+        const bool one = g.op == OP_DENSE1 || g.op == OP_REAL1 || g.op == OP_DIAG1 || g.op == OP_X1;
+        const int dim = one ? 2 : 4;
+        const int ba = one ? 1 << g.code : 1 << (g.code >> 3), bb = one ? 0 : 1 << (g.code & 7);
+        for (int x = 0; x < 16; ++x) {
+            if (x & (ba | bb)) continue;
+            double xr[4], xi[4], yr[4], yi[4];
+            for (int k = 0; k < dim; ++k) {
+                const int i = x | ((k & 1) ? ba : 0) | ((k & 2) ? bb : 0);
+                xr[k] = re[i];
+                xi[k] = im[i];
+            }
+            for (int r = 0; r < dim; ++r) {
+                int from = -1;  // exchanges move the amplitude of row `from`
+                if (g.op == OP_X1) from = r ^ 1;
+                else if (g.op == OP_CXA) from = r == 1 ? 3 : r == 3 ? 1 : r;
+                else if (g.op == OP_CXB) from = r == 2 ? 3 : r == 3 ? 2 : r;
+                else if (g.op == OP_SWAP2) from = r == 1 ? 2 : r == 2 ? 1 : r;
+                else if (g.op == OP_PERM2) from = lds_s32(g.m + 4 * r);
+                if (from >= 0) {
+                    yr[r] = xr[from];
+                    yi[r] = xi[from];
+                    continue;
+                }
+                if (g.op == OP_DIAG1 || g.op == OP_DIAG2) {
+                    const double dr = fx_entry_value(g.m + 16 * r), di = fx_entry_value(g.m + 16 * r + 8);
+                    const bool unit = dr == 1.0 && di == 0.0;
+                    yr[r] = unit ? xr[r] : dr * xr[r] - di * xi[r];
+                    yi[r] = unit ? xi[r] : dr * xi[r] + di * xr[r];
+                    continue;
+                }
+                double sr = 0, si = 0;
+                for (int c = 0; c < dim; ++c) {
+                    const uint32_t e = g.m + (g.op == OP_REAL1 ? 8 : 16) * (dim * r + c);
+                    const double mr = fx_entry_value(e), mi = g.op == OP_REAL1 ? 0.0 : fx_entry_value(e + 8);
+                    cmul_acc(sr, si, mr, mi, xr[c], xi[c]);
+                }
+                yr[r] = sr;
+                yi[r] = si;
+            }
+            for (int k = 0; k < dim; ++k) {
+                const int i = x | ((k & 1) ? ba : 0) | ((k & 2) ? bb : 0);
+                re[i] = yr[k];
+                im[i] = yi[k];
+            }
+        }
+    }
+}
+
+// One register group of 4 bits over the chunk in shared memory (see run_segment for the addressing).
+template <int NC>
+__device__ __forceinline__ void run_segment_fx(uint32_t buf, uint32_t seg, uint32_t gates, int ctid, const int *swz,
+                                               int c, int64_t origin) {
+    constexpr int R = 4, NA = 1 << R;
+    int po[R], pf[R];
+#pragma unroll
+    for (int j = 0; j < R; ++j) {
+        const int p = lds_s8(seg + j);
+        po[j] = 1 << p;
+        pf[j] = po[j] ^ swz[p];
+    }
+    const int lane = ctid & 31;
+    int lbase = 0, lfb = 0;
+#pragma unroll
+    for (int j = 0; j < 5; ++j) {
+        const int p = lds_s8(seg + 8 + j);
+        if ((lane >> j) & 1) { lbase |= 1 << p; lfb ^= swz[p]; }
+    }
+    const int nrest = lds_s8(seg + 13), flags = lds_s8(seg + 14);
+    const int g0 = lds_s16(seg + 32), g1 = lds_s16(seg + 34);
+    const int G = 1 << (c - R);
+    uint32_t ld_step[R], st_step[R];
+#pragma unroll
+    for (int j = 0; j < R; ++j) {
+        ld_step[j] = (uint32_t)((flags & 1) ? po[j] : pf[j]) << 4;
+        st_step[j] = (uint32_t)((flags & 2) ? po[j] : pf[j]) << 4;
+    }
+    for (int gb = ctid; (gb & ~31) < G; gb += NC) {  // whole warps: the range test votes
+        int bs = lbase, fb = lfb;
+        for (int j = 0; j < nrest; ++j)
+            if ((gb >> (5 + j)) & 1) {
+                const int p = lds_s8(seg + 16 + j);
+                bs |= 1 << p;
+                fb ^= swz[p];
+            }
+        const bool live = gb < G;
+        const uint32_t ld0 = (uint32_t)((flags & 1) ? bs : bs ^ fb) << 4, st0 = (uint32_t)((flags & 2) ? bs : bs ^ fb) << 4;
+        double dr[NA], di[NA];
+        int top = 0, any = 0;
+        uint32_t off = ld0;
+#pragma unroll
+        for (int b = 0; b < NA; ++b) {
+            if (b) off ^= ld_step[low_bit(b)];
+            const int g = b ^ (b >> 1);
+            dr[g] = di[g] = 0.0;
+            if (live) SM<double>::ld(buf + off, dr[g], di[g]);
+        }
+#pragma unroll
+        for (int b = 0; b < NA; ++b) {
+            fx::scan(dr[b], top, any);
+            fx::scan(di[b], top, any);
+        }
+        const bool raw = (flags & kSegRaw) != 0;
+        if (!raw && __any_sync(0xFFFFFFFFu, fx::special(top, any))) {
+            double lr[NA], li[NA];
+#pragma unroll
+            for (int b = 0; b < NA; ++b) { lr[b] = dr[b]; li[b] = di[b]; }
+            fx_group_fp64(lr, li, gates, g0, g1, origin);
+#pragma unroll
+            for (int b = 0; b < NA; ++b) { dr[b] = lr[b]; di[b] = li[b]; }
+        } else {
+            const int E = fx::exponent(top);
+            FxGroup<NA> v;
+#pragma unroll
+            for (int b = 0; b < NA; ++b) {
+                v.re[b] = raw ? fx::from_bits(dr[b]) : fx::from_double(dr[b], E);
+                v.im[b] = raw ? fx::from_bits(di[b]) : fx::from_double(di[b], E);
+            }
+            for (int gi = g0; gi < g1; ++gi) {
+                const FxGate g = fx_gate(gates, gi, origin);
+                fx_apply(g.op, g.code, g.m, v, raw);
+            }
+#pragma unroll
+            for (int b = 0; b < NA; ++b) {
+                dr[b] = raw ? fx::to_bits(v.re[b]) : fx::to_double(v.re[b], E);
+                di[b] = raw ? fx::to_bits(v.im[b]) : fx::to_double(v.im[b], E);
+            }
+        }
+        if (live) {
+            off = st0;
+#pragma unroll
+            for (int b = 0; b < NA; ++b) {
+                if (b) off ^= st_step[low_bit(b)];
+                const int g = b ^ (b >> 1);
+                SM<double>::st(buf + off, dr[g], di[g]);
+            }
+        }
+    }
+}
+
+}  // namespace
+}  // namespace sv

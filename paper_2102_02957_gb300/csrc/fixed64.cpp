@@ -1,0 +1,117 @@
+// Host side of the block fixed-point path (fixed64.cuh): which gates it takes and their payloads.
+#include <cmath>
+#include <cstring>
+
+#include "sv_internal.h"
+
+namespace sv {
+namespace {
+
+// Gate entry as two signed 32-bit factors: m * 2^61 = h * 2^32 + l, |l| < 2^31.
+void split(double m, int32_t &h, int32_t &l) {
+    int64_t M = std::llrint(std::ldexp(m, 61));
+    if ((int32_t)(uint32_t)(uint64_t)M == INT32_MIN) ++M;  // keep -l representable
+    l = (int32_t)(uint32_t)(uint64_t)M;
+    h = (int32_t)((M - l) / (int64_t(1) << 32));
+}
+
+}  // namespace
+
+bool fx_unitary(const double *m, int dim) {
+    for (int i = 0; i < dim; ++i)
+        for (int j = 0; j < dim; ++j) {
+            double re = i == j ? -1.0 : 0.0, im = 0.0;
+            for (int r = 0; r < dim; ++r) {
+                const double *a = m + 2 * (r * dim + i), *b = m + 2 * (r * dim + j);
+                re += a[0] * b[0] + a[1] * b[1];
+                im += a[0] * b[1] - a[1] * b[0];
+            }
+            if (!(std::fabs(re) + std::fabs(im) <= 1e-9)) return false;  // NaN entries too
+        }
+    return true;
+}
+
+void fx_pack(const double *m, int count, int32_t *entries) {
+    for (int k = 0; k < 2 * count; ++k) split(m[k], entries[2 * k], entries[2 * k + 1]);
+}
+
+bool exact_gate(const DevGate<double> &g) {
+    int entries = 0;
+    switch (g.op) {
+        case OP_X1: case OP_CXA: case OP_CXB: case OP_SWAP2: case OP_PERM2: return true;
+        case OP_DIAG1: entries = 2; break;
+        case OP_DIAG2: entries = 4; break;
+        case OP_DIAGX: entries = ((g.b >> 8) & 0xFF) == 0xFF ? 4 : 8; break;
+        default: return false;
+    }
+    for (int l = 0; l < entries; ++l)
+        if (std::fabs(g.m[2 * l]) != 1.0 || g.m[2 * l + 1] != 0.0) return false;
+    return true;
+}
+
+bool encode_fx(const std::vector<DevGate<double>> &gates, std::vector<unsigned char> &out) {
+    std::vector<unsigned char> body;
+    std::vector<int32_t> head;
+    const size_t table = gates.size() * 16;
+    auto put = [&](const void *p, size_t bytes) {
+        const unsigned char *b = static_cast<const unsigned char *>(p);
+        body.insert(body.end(), b, b + bytes);
+    };
+    auto put_entries = [&](const double *m, int count) {
+        int32_t e[64];
+        fx_pack(m, count, e);
+        put(e, (size_t)count * 16);
+    };
+    auto put_diag = [&](const double *d, int count) {
+        for (int l = 0; l < count; ++l)
+            if (!(std::fabs(d[2 * l] * d[2 * l] + d[2 * l + 1] * d[2 * l + 1] - 1.0) <= 1e-9)) return false;
+        put_entries(d, count);
+        return true;
+    };
+    for (const DevGate<double> &g : gates) {
+        int32_t op = g.op;
+        const size_t off = table + body.size();
+        switch (g.op) {
+            case OP_DENSE1:
+                if (!fx_unitary(g.m, 2)) return false;
+                if (g.m[1] == 0.0 && g.m[3] == 0.0 && g.m[5] == 0.0 && g.m[7] == 0.0) {
+                    op = OP_REAL1;
+                    const double re[4] = {g.m[0], g.m[2], g.m[4], g.m[6]};
+                    put_entries(re, 2);
+                } else {
+                    put_entries(g.m, 4);
+                }
+                break;
+            case OP_DENSE2:
+                if (!fx_unitary(g.m, 4)) return false;
+                put_entries(g.m, 16);
+                break;
+            case OP_DIAG1:
+                if (!put_diag(g.m, 2)) return false;
+                break;
+            case OP_DIAG2:
+                if (!put_diag(g.m, 4)) return false;
+                break;
+            case OP_DIAGX: {
+                // variants that the gate has: 2 for one outside qubit, 4 for two
+                const int nv = ((g.b >> 8) & 0xFF) == 0xFF ? 2 : 4;
+                if (!put_diag(g.m, 2 * nv)) return false;
+                break;
+            }
+            case OP_PERM2: {
+                int32_t p[4];
+                for (int r = 0; r < 4; ++r) p[r] = (int32_t)g.m[r];
+                put(p, sizeof(p));
+                break;
+            }
+            default: break;  // register exchanges: no payload
+        }
+        head.insert(head.end(), {op, (int32_t)off, g.b, g.code});
+    }
+    const unsigned char *h = reinterpret_cast<const unsigned char *>(head.data());
+    out.assign(h, h + table);
+    out.insert(out.end(), body.begin(), body.end());
+    return true;
+}
+
+}  // namespace sv

@@ -39,6 +39,7 @@
 #include <mutex>
 
 #include "block_core.cuh"
+#include "block_fx.cuh"
 #include "ptx.cuh"
 #include "sv_internal.h"
 
@@ -178,9 +179,9 @@ constexpr int CG2 = 2;  // consumer groups per CTA (default)
 
 // G consumer groups per CTA; tensor-core groups keep NB tile buffers each
 // (G * NB * TcGeom<R>::COLS <= 512 TMEM columns).
-template <typename T, int R, int NC, int KU, bool TC, int G, int NB>
+template <typename T, int R, int NC, int KU, bool TC, int G, int NB, bool FX>
 __device__ __forceinline__ void block_body(typename V2<T>::type *__restrict__ state, int c, int64_t nchunks, int nbuf,
-                                           const unsigned char *__restrict__ prog, int nseg, int ngate, int *err,
+                                           const unsigned char *__restrict__ prog, int nseg, int gate_bytes, int *err,
                                            const CUtensorMap &tmap, const GatherArgs &ga_in, uint64_t wait_ns) {
     using T2 = typename V2<T>::type;
     __shared__ GatherArgs ga;  // gathered chunks (rank > 0); rank 0 = contiguous chunk j
@@ -193,10 +194,10 @@ __device__ __forceinline__ void block_body(typename V2<T>::type *__restrict__ st
     // groups' B operands (tensor cores), 16-byte aligned
     const int seg_bytes = (int)((nseg * sizeof(DevSeg) + 15) & ~size_t(15));
     constexpr int kBBytes = TcGeom<(R < 3 ? 3 : R)>::B_BYTES;  // B operand of one tensor-core group
-    const int prog_bytes = seg_bytes + (TC ? nseg * kBBytes : ngate * (int)sizeof(DevGate<T>));
+    const int prog_bytes = seg_bytes + (TC ? nseg * kBBytes : gate_bytes);
     unsigned char *sprog = smem + (size_t)nbuf * chunk_bytes;
     const DevSeg *segs = reinterpret_cast<const DevSeg *>(sprog);
-    const DevGate<T> *gates = reinterpret_cast<const DevGate<T> *>(sprog + seg_bytes);
+    const unsigned char *gates = sprog + seg_bytes;
     uint64_t *full = reinterpret_cast<uint64_t *>(sprog + ((prog_bytes + 15) & ~15));
     uint64_t *empty = full + nbuf;
     uint64_t *done = empty + nbuf;
@@ -284,6 +285,8 @@ __device__ __forceinline__ void block_body(typename V2<T>::type *__restrict__ st
                                                       ptx::smem_addr(sprog + seg_bytes) + (uint32_t)(si * kBBytes), ctid,
                                                       swz, c, tmem_base + (uint32_t)(cg * NB * TcGeom<R>::COLS), bar_id,
                                                       &mma_bar[2 * cg], mma_phase, abort_flag, &s_wait_ns);
+            } else if constexpr (FX) {
+                run_segment_fx<NC>(ptx::smem_addr(buf), seg_addr, ptx::smem_addr(gates), ctid, swz, c, origin);
             } else {
                 run_segment<T, R, NC, KU>(ptx::smem_addr(buf), seg_addr, ptx::smem_addr(gates), ctid, swz, c, origin);
             }
@@ -317,12 +320,12 @@ __device__ __forceinline__ void block_body(typename V2<T>::type *__restrict__ st
 }
 
 // SIMT sections: launch bounds let the compiler fit two 256-thread consumer groups.
-template <typename T, int R, int NC, int KU, bool TC, int G = CG2, int NB = 2>
+template <typename T, int R, int NC, int KU, bool TC, int G = CG2, int NB = 2, bool FX = false>
 __global__ void __launch_bounds__(G * NC + kSvcThreads, 1)
     k_block(typename V2<T>::type *__restrict__ state, int c, int64_t nchunks, int nbuf,
-            const unsigned char *__restrict__ prog, int nseg, int ngate, int *err,
+            const unsigned char *__restrict__ prog, int nseg, int gate_bytes, int *err,
             const __grid_constant__ CUtensorMap tmap, const GatherArgs ga_in, uint64_t wait_ns) {
-    block_body<T, R, NC, KU, TC, G, NB>(state, c, nchunks, nbuf, prog, nseg, ngate, err, tmap, ga_in, wait_ns);
+    block_body<T, R, NC, KU, TC, G, NB, FX>(state, c, nchunks, nbuf, prog, nseg, gate_bytes, err, tmap, ga_in, wait_ns);
 }
 
 // Tensor-core sections: one CTA per SM (it takes all of the SM's tensor memory).  The register
@@ -339,13 +342,16 @@ static_assert(tc_max_regs(576) == 96 && tc_max_regs(320) == 168, "register budge
 template <typename T, int R, int NC, int KU, bool TC, int G, int NB>
 __global__ void __maxnreg__(tc_max_regs(G * NC + kSvcThreads))
     k_block_tc(typename V2<T>::type *__restrict__ state, int c, int64_t nchunks, int nbuf,
-               const unsigned char *__restrict__ prog, int nseg, int ngate, int *err,
+               const unsigned char *__restrict__ prog, int nseg, int gate_bytes, int *err,
                const __grid_constant__ CUtensorMap tmap, const GatherArgs ga_in, uint64_t wait_ns) {
-    block_body<T, R, NC, KU, TC, G, NB>(state, c, nchunks, nbuf, prog, nseg, ngate, err, tmap, ga_in, wait_ns);
+    block_body<T, R, NC, KU, TC, G, NB, false>(state, c, nchunks, nbuf, prog, nseg, gate_bytes, err, tmap, ga_in,
+                                               wait_ns);
 }
 
-template <typename T, int R, int NC, int KU, bool TC = false, int G = CG2, int NB = 2>
-void launch_typed(void *state, int n, int ce, const void *prog, int nseg, int ngate, int *err, cudaStream_t st,
+constexpr size_t kMaxBlockSmem = 227 * 1024 - 1024;  // minus the static swizzle table (1 KiB aligned)
+
+template <typename T, int R, int NC, int KU, bool TC = false, int G = CG2, int NB = 2, bool FX = false>
+void launch_typed(void *state, int n, int ce, const void *prog, int nseg, int gate_bytes, int *err, cudaStream_t st,
                   const CUtensorMap &tmap, const GatherArgs &ga, uint64_t wait_ns) {
     if (ce - R - 5 > kMaxRest) fail(SV_ERR_UNSUPPORTED, "chunk too wide for the register-group layout");
     using T2 = typename V2<T>::type;
@@ -353,14 +359,14 @@ void launch_typed(void *state, int n, int ce, const void *prog, int nseg, int ng
     const int64_t nchunks = int64_t(1) << (n - ce);
     const size_t seg_bytes = (nseg * sizeof(DevSeg) + 15) & ~size_t(15);
     const size_t prog_bytes =
-        (seg_bytes + (TC ? (size_t)nseg * TcGeom<(R < 3 ? 3 : R)>::B_BYTES : ngate * sizeof(DevGate<T>)) + 15) &
+        (seg_bytes + (TC ? (size_t)nseg * TcGeom<(R < 3 ? 3 : R)>::B_BYTES : (size_t)gate_bytes) + 15) &
         ~size_t(15);
     if (TC && G * NB * TcGeom<(R < 3 ? 3 : R)>::COLS > 512) fail(SV_ERR_UNSUPPORTED, "tile buffers exceed tensor memory");
     int nbuf = TC ? G + 2 : 3;  // tensor cores: every consumer group holds a chunk, plus prefetch
     // program + mbarriers (full, empty, done per buffer; two per consumer group), abort flag,
     // TMEM address
     const size_t extra = prog_bytes + (size_t)(3 * nbuf + 2 * G) * 8 + 16;
-    const size_t max_smem = 227 * 1024 - 1024;  // minus the static swizzle table (1 KiB aligned)
+    const size_t max_smem = kMaxBlockSmem;
     while (nbuf > 1 && nbuf * chunk_bytes + extra > max_smem) --nbuf;
     size_t smem = nbuf * chunk_bytes + extra;
     if (smem > max_smem) fail(SV_ERR_UNSUPPORTED, "chunk and section program do not fit in shared memory");
@@ -380,11 +386,11 @@ void launch_typed(void *state, int n, int ce, const void *prog, int nseg, int ng
     if constexpr (TC) {
         auto kern = k_block_tc<T, R, NC, KU, TC, G, NB>;
         kern<<<grid_of(kern), G * NC + kSvcThreads, smem, st>>>((T2 *)state, ce, nchunks, nbuf, (const unsigned char *)prog, nseg,
-                                                     ngate, err, tmap, ga, wait_ns);
+                                                     gate_bytes, err, tmap, ga, wait_ns);
     } else {
-        auto kern = k_block<T, R, NC, KU, TC, G, NB>;
+        auto kern = k_block<T, R, NC, KU, TC, G, NB, FX>;
         kern<<<grid_of(kern), G * NC + kSvcThreads, smem, st>>>((T2 *)state, ce, nchunks, nbuf, (const unsigned char *)prog, nseg,
-                                                     ngate, err, tmap, ga, wait_ns);
+                                                     gate_bytes, err, tmap, ga, wait_ns);
     }
     check_cuda(cudaGetLastError(), "block kernel launch");
 }
@@ -432,43 +438,34 @@ CUtensorMap make_gather_map(void *state, const GatherLayout &lay, int elem_bytes
 
 }  // namespace
 
-size_t devgate_bytes(int dtype) { return dtype == SV_C64 ? sizeof(DevGate<float>) : sizeof(DevGate<double>); }
-
-// Threads per consumer group: 2^4-amplitude groups need ~96 registers (2 x 256 threads fit the
-// register file), 2^5-amplitude and complex128 groups ~170 (2 x 128 threads).
 // Threads per consumer group: complex64 with 2^4-amplitude register groups runs 2 x 256
 // consumers (17 warps, <= 96 registers a thread); 2^5-amplitude groups and complex128 run
 // 2 x 128 (9 warps, <= 168 registers).  Each thread holds one register group at a time.
-int block_threads(int ce, int seg_bits, int dtype) {
-    (void)ce;
-    return (dtype == SV_C64 && seg_bits == 4) ? 256 : 128;
-}
-
-static void dispatch(int dtype, int r, int nc, void *state, int n, int ce, const void *prog, int nseg, int ngates,
+static void dispatch(int dtype, int r, void *state, int n, int ce, const void *prog, int nseg, int gate_bytes, bool fixed,
                      int *err, cudaStream_t st, const CUtensorMap &m, const GatherArgs &ga, uint64_t wait_ns) {
-    (void)nc;
     if (dtype == SV_C64) {
-        if (r == 4) launch_typed<float, 4, 256, 1>(state, n, ce, prog, nseg, ngates, err, st, m, ga, wait_ns);
-        else launch_typed<float, 5, 128, 1>(state, n, ce, prog, nseg, ngates, err, st, m, ga, wait_ns);
+        if (r == 4) launch_typed<float, 4, 256, 1>(state, n, ce, prog, nseg, gate_bytes, err, st, m, ga, wait_ns);
+        else launch_typed<float, 5, 128, 1>(state, n, ce, prog, nseg, gate_bytes, err, st, m, ga, wait_ns);
+    } else if (fixed) {
+        launch_typed<double, 4, 128, 1, false, CG2, 2, true>(state, n, ce, prog, nseg, gate_bytes, err, st, m, ga, wait_ns);
     } else {
-        launch_typed<double, 4, 128, 1>(state, n, ce, prog, nseg, ngates, err, st, m, ga, wait_ns);
+        launch_typed<double, 4, 128, 1>(state, n, ce, prog, nseg, gate_bytes, err, st, m, ga, wait_ns);
     }
 }
 
-void launch_block(int dtype, void *state, int n, int c, const void *dev_prog, int nseg, int ngates, int *dev_err,
-                  int seg_bits, cudaStream_t st, uint64_t wait_ns) {
+void launch_block(int dtype, void *state, int n, int c, const void *dev_prog, int nseg, int gate_bytes, bool fixed,
+                  int *dev_err, int seg_bits, cudaStream_t st, uint64_t wait_ns) {
     const int ce = c < n ? c : n;
     if (ce < 4) fail(SV_ERR_UNSUPPORTED, "blocked path needs a chunk of at least 4 bits");
     const int r = seg_bits < ce ? seg_bits : ce;  // the register groups were built with this width
     GatherArgs ga{};  // rank 0: contiguous chunk j
     CUtensorMap none;
     std::memset(&none, 0, sizeof(none));
-    dispatch(dtype, r, block_threads(ce, r, dtype), state, n, ce, dev_prog, nseg, ngates, dev_err, st, none, ga,
-             wait_ns);
+    dispatch(dtype, r, state, n, ce, dev_prog, nseg, gate_bytes, fixed, dev_err, st, none, ga, wait_ns);
 }
 
 void launch_block_gather(int dtype, void *state, int n, const GatherLayout &lay, const void *dev_prog, int nseg,
-                         int ngates, int *dev_err, int seg_bits, cudaStream_t st, uint64_t wait_ns) {
+                         int gate_bytes, bool fixed, int *dev_err, int seg_bits, cudaStream_t st, uint64_t wait_ns) {
     const int ce = lay.ce;
     if (ce < 4) fail(SV_ERR_UNSUPPORTED, "blocked path needs a chunk of at least 4 bits");
     if (reinterpret_cast<uintptr_t>(state) % 16) fail(SV_ERR_ARG, "state buffer not 16-byte aligned");
@@ -478,8 +475,7 @@ void launch_block_gather(int dtype, void *state, int n, const GatherLayout &lay,
         fail(SV_ERR_UNSUPPORTED, "gathered chunk boxes smaller than 128 bytes (pin more low bits)");
     const CUtensorMap m = make_gather_map(state, lay, elem);
     const int r = seg_bits < ce ? seg_bits : ce;
-    dispatch(dtype, r, block_threads(ce, r, dtype), state, n, ce, dev_prog, nseg, ngates, dev_err, st, m, lay.args,
-             wait_ns);
+    dispatch(dtype, r, state, n, ce, dev_prog, nseg, gate_bytes, fixed, dev_err, st, m, lay.args, wait_ns);
 }
 
 }  // namespace sv

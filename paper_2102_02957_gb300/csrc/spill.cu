@@ -187,7 +187,8 @@ void run_pass(const Pass &p, const sv_plan &plan, int dtype, unsigned char *host
                 for (const auto &q : sp.progs)
                     if (q.op_index == op) pr = &q;
                 if (!pr) fail(SV_ERR_PLAN, "no program for a blocking section");
-                launch_block(dtype, buf, nsub, plan.c, prog + pr->off, pr->nseg, pr->ngate, dev_err, sp.seg_bits, st[k],
+                launch_block(dtype, buf, nsub, plan.c, prog + pr->off, pr->nseg, pr->gate_bytes, pr->fixed != 0, dev_err,
+                             sp.seg_bits, st[k],
                              wait_ns);
             } else if (!pairs[i].empty()) {
                 launch_permute(dtype, buf, nsub, pairs[i], st[k]);

@@ -105,6 +105,7 @@ enum : int32_t {
     OP_CXB = 6,    // exchange 2 <-> 3: control = b, target = a
     OP_SWAP2 = 7,  // exchange 1 <-> 2
     OP_X1 = 8,     // 1-qubit bit flip
+    OP_REAL1 = 10, // dense 1-qubit gate with real entries (fixed-point programs only)
     OP_DIAGX = 9   // diagonal gate with qubits outside the chunk: b = e0 | e1 << 8 (state bits,
                    // 0xFF = none); variant v = bit e0 + 2 bit e1 of the chunk's origin selects
                    // m[4v..4v+3], a diagonal (d0, d1) on register bit a (a phase: d0 = d1, a = 0)
@@ -116,12 +117,14 @@ struct DevSeg {
     int8_t pos[8];    // group bits (ascending); r of them used
     int8_t lane[5];
     int8_t nrest;
-    int8_t flags;     // 1: read the natural (unswizzled) layout, 2: write the natural layout
+    int8_t flags;     // 1: read the natural (unswizzled) layout, 2: write the natural layout, kSegRaw
     int8_t r;
     int8_t rest[16];
     int16_t g0, g1;   // gate range [g0, g1) in the section's gate array
 };
 static_assert(sizeof(DevSeg) == 36, "DevSeg layout");
+
+constexpr int kSegRaw = 4;  // fixed-point programs: every gate of the group is exact_gate()
 
 template <typename T>
 struct DevGate {
@@ -150,6 +153,17 @@ int plan_segment_count(const sv_plan &plan);
 
 template <typename T>
 void encode_gate(const sv_gate &g, const BlockGate &bg, const HostSeg &seg, DevGate<T> &out);
+
+// Block fixed-point programs of complex128 sections (fixed64.cuh, block_fx.cuh).
+// Whether the dim x dim matrix is unitary to 1e-9, as the fixed-point ranges need.
+bool fx_unitary(const double *m, int dim);
+// Fixed-point factors of `count` complex entries (4 ints each).
+void fx_pack(const double *m, int count, int32_t *entries);
+// Whether a gate only exchanges amplitudes or multiplies them by 1 or -1.
+bool exact_gate(const DevGate<double> &g);
+// The gate area of a section's program: header table and payloads.  false (out untouched) when a
+// gate is not unitary.
+bool encode_fx(const std::vector<DevGate<double>> &gates, std::vector<unsigned char> &out);
 
 // Gathered chunk: the state is viewed as a tensor of rank <= 5 whose dimension d covers the
 // index bits [s[d], s[d+1]); each dimension starts with a run of chunk bits (its box, at most
@@ -243,7 +257,7 @@ void launch_init_basis(int dtype, void *state, int n, uint64_t basis, cudaStream
 struct SimtPrograms {
     struct Prog {
         size_t off;
-        int nseg, ngate, op_index;
+        int nseg, gate_bytes, fixed, op_index;
     };
     std::vector<unsigned char> host;
     std::vector<Prog> progs;
@@ -259,17 +273,19 @@ void launch_permute(int dtype, void *state, int n, const std::vector<std::pair<i
 
 // Bounded device waits: wait_ns (kDefaultWaitNs unless the plan sets wait_limit_ms).
 constexpr uint64_t kDefaultWaitNs = 4000000000ull;
-void launch_block(int dtype, void *state, int n, int c, const void *dev_prog, int nseg, int ngates, int *dev_err,
-                  int seg_bits, cudaStream_t st, uint64_t wait_ns = kDefaultWaitNs);
+// SIMT sections: the program is nseg register groups and a gate area of gate_bytes bytes, gate
+// records (DevGate) or, `fixed` (complex128), a fixed-point area (encode_fx).
+void launch_block(int dtype, void *state, int n, int c, const void *dev_prog, int nseg, int gate_bytes, bool fixed,
+                  int *dev_err, int seg_bits, cudaStream_t st, uint64_t wait_ns = kDefaultWaitNs);
 // Blocking section over a gathered chunk (bits in `mask`), fetched and written back with
 // tensor copies.
 void launch_block_gather(int dtype, void *state, int n, const GatherLayout &lay, const void *dev_prog, int nseg,
-                         int ngates, int *dev_err, int seg_bits, cudaStream_t st, uint64_t wait_ns = kDefaultWaitNs);
+                         int gate_bytes, bool fixed, int *dev_err, int seg_bits, cudaStream_t st,
+                         uint64_t wait_ns = kDefaultWaitNs);
 // Tensor-core blocking section (complex64, register groups of seg_bits = 3, 4 or 5 bits, B
 // operands in the program, tc_b_bytes(seg_bits) each); `lay` null for a contiguous chunk of c bits.
 void launch_block_tc(void *state, int n, int c, const GatherLayout *lay, const void *dev_prog, int nseg, int *dev_err,
                      int seg_bits, cudaStream_t st, uint64_t wait_ns = kDefaultWaitNs);
-size_t devgate_bytes(int dtype);
 
 // readouts
 void launch_probs(int dtype, const void *state, int n, double *out, int64_t first, int64_t count,

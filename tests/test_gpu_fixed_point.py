@@ -1,0 +1,95 @@
+"""complex128 gates in block fixed point (csrc/fixed64.cuh): ranges, exact cases and the FP64 paths
+beside it, per-gate and blocked, against the oracle."""
+import numpy as np
+import pytest
+
+import circuitgen as cg
+from oracle import sim
+
+pytestmark = pytest.mark.gpu
+
+# (n, plan options); None: the per-gate path
+PATHS = [(7, None), (11, None), (6, dict(chunk_bits=4)), (9, dict(chunk_bits=6)), (14, dict(chunk_bits=12)),
+         (13, dict(chunk_bits=10, gather_pinned=4)), (13, dict(chunk_bits=8, diag_outside=1))]
+
+
+@pytest.fixture(scope="module")
+def sv():
+    import paper_2102_02957_gb300 as m
+    return m
+
+
+def mixed(n, seed):
+    return cg.random_layers(n, 2, seed) + cg.quantum_volume(n, 1, seed) + cg.hea(n, 1, seed, 0) + cg.qft(n, with_swaps=False)
+
+
+def run(sv, n, desc, opts, start):
+    gates = sv.make_gates(desc)
+    st = sv.StateVector(n, "c128")
+    st.set_state(start)
+    st.apply(gates, sv.Plan(n, gates, **opts) if opts is not None else None)
+    return st.get_state()
+
+
+def bound(desc, start):
+    """A gate's output component is a sum of at most 8 products of factors of modulus <= 1: FP64 is
+    off by at most 8 * 2^-53 * 2 max|x| per gate; gates keep 2-norms, so the sum over gates of the
+    2-norm bounds every component.  Both sides round: twice that."""
+    return 2 * len(desc) * 16 * 2.0 ** -53 * np.linalg.norm(start)
+
+
+@pytest.mark.parametrize("n,opts", PATHS)
+@pytest.mark.parametrize("scale,spread", [(1.0, 0), (1.0, 40), (2.0 ** -900, 0), (2.0 ** -990, 0), (2.0 ** 1010, 0)])
+def test_scaled_states(sv, n, opts, scale, spread):
+    rng = np.random.default_rng(n)
+    start = rng.standard_normal(1 << n) + 1j * rng.standard_normal(1 << n)
+    start = start / np.linalg.norm(start) * 10.0 ** -rng.uniform(0, spread, 1 << n) if spread else start / np.linalg.norm(start)
+    desc = mixed(n, 3)
+    want = sim.apply(start.astype(np.complex128).copy(), n, desc)  # scales by powers of two are exact
+    got = run(sv, n, desc, opts, start * scale) / scale
+    floor = 2.0 ** -1074 / scale * 64 * len(desc) if scale < 2.0 ** -950 else 0.0  # subnormal steps
+    assert np.abs(got - want).max() <= bound(desc, start) + floor
+
+
+@pytest.mark.parametrize("n,opts", PATHS)
+def test_exchanges_and_signs_are_exact(sv, n, opts):
+    rng = np.random.default_rng(7)
+    start = rng.standard_normal(1 << n) + 1j * rng.standard_normal(1 << n)
+    desc = [("x", (q,), ()) for q in range(0, n, 2)]
+    for q in range(n - 1):
+        desc += [("cx", (q, q + 1), ()), ("cx", (q + 1, q), ()), ("cz", (q, q + 1), ()), ("z", (q,), ())]
+    perm = np.eye(4)[[2, 0, 3, 1]]
+    desc.append(("unitary", (0, n - 1), (perm.astype(np.complex128),)))
+    want = sim.apply(start.copy(), n, desc)
+    assert np.array_equal(run(sv, n, desc, opts, start), want)
+    zero = np.zeros(1 << n, dtype=np.complex128)
+    assert np.array_equal(run(sv, n, mixed(n, 5), opts, zero), zero)
+
+
+@pytest.mark.parametrize("n,opts", PATHS[:5])
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+def test_non_finite_amplitudes_stay_in_their_groups(sv, n, opts, bad):
+    rng = np.random.default_rng(1)
+    start = rng.standard_normal(1 << n) + 1j * rng.standard_normal(1 << n)
+    desc = [("u3", (1,), (0.7, 1.1, 2.3)), ("unitary", (0, 2), (cg.haar_unitary(rng),))]
+    want = sim.apply(start.copy(), n, desc)
+    hit = 5
+    start[hit] = complex(bad, 0.25)
+    got = run(sv, n, desc, opts, start)
+    reached = (np.arange(1 << n) | 7) == (hit | 7)
+    assert not np.isfinite(got[reached]).any()
+    assert np.abs(got[~reached] - want[~reached]).max() <= bound(desc, start[~reached])
+
+
+@pytest.mark.parametrize("n,opts", PATHS[:6])
+def test_non_unitary_gates_stay_fp64(sv, n, opts):
+    rng = np.random.default_rng(2)
+    start = rng.standard_normal(1 << n) + 1j * rng.standard_normal(1 << n)
+    big = 40.0 * (rng.standard_normal((4, 4)) + 1j * rng.standard_normal((4, 4)))
+    one = 1e-3 * (rng.standard_normal((2, 2)) + 1j * rng.standard_normal((2, 2)))
+    desc = [("unitary", (n - 1, 0), (big,)), ("unitary", (1,), (one,)), ("u3", (0,), (0.3, 0.2, 0.1))]
+    want = sim.apply(start.copy(), n, desc)
+    got = run(sv, n, desc, opts, start)
+    # norms grow by at most ||big|| ||one||; 8 products of 2^-53 each per gate, on both sides
+    scale = np.linalg.norm(big, 2) * np.linalg.norm(one, 2) * np.linalg.norm(start)
+    assert np.abs(got - want).max() <= 2 * 3 * 16 * 2.0 ** -53 * scale
