@@ -248,8 +248,6 @@ void launch_mlp_reduce(const float *part, int nblk, const double *lpart, double 
 // ------------------------------------------------------------------ kernels (launchers)
 struct Mat1 { float m[8]; };
 struct Mat2 { float m[32]; };
-struct Mat1d { double m[8]; };
-struct Mat2d { double m[32]; };
 
 void launch_gate(int dtype, void *state, int n, const sv_gate &g, cudaStream_t st);
 void launch_init_basis(int dtype, void *state, int n, uint64_t basis, cudaStream_t st);
