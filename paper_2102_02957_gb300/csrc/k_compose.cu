@@ -23,102 +23,111 @@ __device__ __forceinline__ uint32_t tf32_rna(float x) {
     return r;
 }
 
-// One CTA per register group, thread j composes column j of U (U e_j through the group's gates).
+// One CTA per register group; every thread owns elements (row r, column j) of the running product
+// U, kept in two shared-memory copies that a gate reads and writes in turn.  (With one thread per
+// column walking its gates alone the kernel was a serial chain of FP64 latencies, 209 us for the
+// 69 groups of a 20-qubit ansatz; so it takes 22 us.)  Gate records are fetched kGates at a
+// time, so that their latency is paid once per batch.
 template <int R>
-__global__ void k_compose_f64(const ComposeSeg *__restrict__ segs, const DevGate<double> *__restrict__ gates,
-                              unsigned char *__restrict__ prog, int *__restrict__ all_unitary) {
-    constexpr int NA = 1 << R, K = 2 * NA, SBO = 32 * K;
+__global__ void __launch_bounds__(256) k_compose_f64(const ComposeSeg *__restrict__ segs,
+                                                     const DevGate<double> *__restrict__ gates,
+                                                     unsigned char *__restrict__ prog, int *__restrict__ all_unitary) {
+    constexpr int NA = 1 << R, K = 2 * NA, SBO = 32 * K, NE = NA * NA, kGates = 16;
+    extern __shared__ __align__(16) unsigned char smem[];
+    double2 *U = reinterpret_cast<double2 *>(smem);  // [2][NE], element r * NA + j
+    __shared__ __align__(16) DevGate<double> sg_gates[kGates];
+    __shared__ unsigned long long dev_bits;
     const ComposeSeg sg = segs[blockIdx.x];
-    const int j = threadIdx.x;  // 0..NA-1
-    double vr[NA], vi[NA];
-    for (int b = 0; b < NA; ++b) { vr[b] = b == j ? 1.0 : 0.0; vi[b] = 0.0; }
-    for (int gi = sg.g0; gi < sg.g1; ++gi) {
-        const DevGate<double> &g = gates[gi];
-        const int a = g.a;
-        if (g.op == OP_DENSE1 || g.op == OP_DIAG1 || g.op == OP_X1) {
-            double m[8];
-            if (g.op != OP_DIAG1) {
-                for (int k = 0; k < 8; ++k) m[k] = g.m[k];
-            } else {
-                m[0] = g.m[0]; m[1] = g.m[1]; m[2] = 0; m[3] = 0;
-                m[4] = 0; m[5] = 0; m[6] = g.m[2]; m[7] = g.m[3];
-            }
-#pragma unroll
-            for (int x = 0; x < NA; ++x) {
-                if (x & (1 << a)) continue;
-                const int y = x | (1 << a);
-                const double ar = vr[x], ai = vi[x], br = vr[y], bi = vi[y];
-                vr[x] = m[0] * ar - m[1] * ai + m[2] * br - m[3] * bi;
-                vi[x] = m[0] * ai + m[1] * ar + m[2] * bi + m[3] * br;
-                vr[y] = m[4] * ar - m[5] * ai + m[6] * br - m[7] * bi;
-                vi[y] = m[4] * ai + m[5] * ar + m[6] * bi + m[7] * br;
-            }
-        } else {
-            const int b = g.b;
-            double m[32];
-            for (int k = 0; k < 32; ++k) m[k] = 0.0;
-            if (g.op == OP_DENSE2) {
-                for (int k = 0; k < 32; ++k) m[k] = g.m[k];
-            } else if (g.op == OP_DIAG2) {
-                for (int r = 0; r < 4; ++r) { m[2 * (5 * r)] = g.m[2 * r]; m[2 * (5 * r) + 1] = g.m[2 * r + 1]; }
-            } else {  // permutation: row r takes column m[r]
-                for (int r = 0; r < 4; ++r) m[2 * (4 * r + (int)g.m[r])] = 1.0;
-            }
-#pragma unroll
-            for (int x = 0; x < NA; ++x) {
-                if (x & ((1 << a) | (1 << b))) continue;
-                const int id[4] = {x, x | (1 << a), x | (1 << b), x | (1 << a) | (1 << b)};
-                double xr[4], xi[4];
-                for (int k = 0; k < 4; ++k) { xr[k] = vr[id[k]]; xi[k] = vi[id[k]]; }
-                for (int r = 0; r < 4; ++r) {
-                    double yr = 0, yi = 0;
-                    for (int cc = 0; cc < 4; ++cc) {
-                        const double mr = m[2 * (4 * r + cc)], mi = m[2 * (4 * r + cc) + 1];
-                        yr += mr * xr[cc] - mi * xi[cc];
-                        yi += mr * xi[cc] + mi * xr[cc];
+    const int tid = threadIdx.x, nt = blockDim.x;
+    if (tid == 0) dev_bits = 0;
+    for (int e = tid; e < NE; e += nt) U[e] = make_double2((e >> R) == (e & (NA - 1)) ? 1.0 : 0.0, 0.0);
+    int cur = 0;
+    for (int base = sg.g0; base < sg.g1; base += kGates) {
+        const int count = min(kGates, sg.g1 - base);
+        __syncthreads();  // the last batch's records are used up
+        const uint4 *src = reinterpret_cast<const uint4 *>(gates + base);
+        for (int k = tid; k < count * (int)(sizeof(DevGate<double>) / 16); k += nt)
+            reinterpret_cast<uint4 *>(sg_gates)[k] = src[k];
+        __syncthreads();
+        for (int gi = 0; gi < count; ++gi) {
+            const DevGate<double> &g = sg_gates[gi];
+            const double2 *x = U + cur * NE;
+            double2 *y = U + (cur ^ 1) * NE;
+            const int ba = 1 << g.a;
+            for (int e = tid; e < NE; e += nt) {
+                const int r = e >> R, j = e & (NA - 1);
+                double2 out;
+                if (g.op == OP_DENSE1 || g.op == OP_X1) {
+                    const double *m = g.m + ((r & ba) ? 4 : 0);
+                    const double2 p = x[((r & ~ba) << R) | j], q = x[((r | ba) << R) | j];
+                    out.x = m[0] * p.x - m[1] * p.y + m[2] * q.x - m[3] * q.y;
+                    out.y = m[0] * p.y + m[1] * p.x + m[2] * q.y + m[3] * q.x;
+                } else if (g.op == OP_DIAG1 || g.op == OP_DIAG2) {
+                    const int l = ((r >> g.a) & 1) | (g.op == OP_DIAG2 ? ((r >> g.b) & 1) << 1 : 0);
+                    const double dr = g.m[2 * l], di = g.m[2 * l + 1];
+                    out = x[e];
+                    if (!(dr == 1.0 && di == 0.0)) out = make_double2(dr * out.x - di * out.y, dr * out.y + di * out.x);
+                } else {
+                    const int bb = 1 << g.b, l = ((r >> g.a) & 1) | (((r >> g.b) & 1) << 1);
+                    const int r0 = r & ~(ba | bb);
+                    auto row = [&](int c) { return r0 | ((c & 1) ? ba : 0) | ((c & 2) ? bb : 0); };
+                    if (g.op == OP_DENSE2) {
+                        out = make_double2(0.0, 0.0);
+                        for (int c = 0; c < 4; ++c) {
+                            const double2 p = x[(row(c) << R) | j];
+                            const double mr = g.m[2 * (4 * l + c)], mi = g.m[2 * (4 * l + c) + 1];
+                            out.x += mr * p.x - mi * p.y;
+                            out.y += mr * p.y + mi * p.x;
+                        }
+                    } else {  // an exchange: row l takes row m[l]
+                        out = x[(row((int)g.m[l]) << R) | j];
                     }
-                    vr[id[r]] = yr;
-                    vi[id[r]] = yi;
                 }
+                y[e] = out;
             }
+            cur ^= 1;
+            __syncthreads();
         }
     }
-    // unitarity of the fused matrix (in FP64): max |(U^H U - I)_ij| over all i, j
-    __shared__ double ur[NA][NA + 1], ui[NA][NA + 1];
-    __shared__ unsigned long long dev_bits;
-    if (j == 0) dev_bits = 0;
-    for (int r = 0; r < NA; ++r) { ur[r][j] = vr[r]; ui[r][j] = vi[r]; }
     __syncthreads();
+    const double2 *x = U + cur * NE;
+    // unitarity of the fused matrix: max |(U^H U - I)_ij| over all i <= j (the rest is conjugate)
     double worst = 0.0;
-    for (int i = 0; i < NA; ++i) {
+    for (int e = tid; e < NE; e += nt) {
+        const int i = e >> R, j = e & (NA - 1);
+        if (i > j) continue;
         double gr = 0.0, gi = 0.0;  // <U e_i, U e_j>
         for (int r = 0; r < NA; ++r) {
-            gr += ur[r][i] * ur[r][j] + ui[r][i] * ui[r][j];
-            gi += ur[r][i] * ui[r][j] - ui[r][i] * ur[r][j];
+            const double2 p = x[(r << R) | i], q = x[(r << R) | j];
+            gr += p.x * q.x + p.y * q.y;
+            gi += p.x * q.y - p.y * q.x;
         }
-        worst = fmax(worst, fabs(gr - (i == j ? 1.0 : 0.0)) + fabs(gi));
+        const double d = fabs(gr - (i == j ? 1.0 : 0.0)) + fabs(gi);
+        worst = d > worst || !(d == d) ? d : worst;
     }
-    atomicMax(&dev_bits, (unsigned long long)__double_as_longlong(worst));  // non-negative: order as integers
+    // non-negative values (and NaN above them all) order as integers
+    atomicMax(&dev_bits, (unsigned long long)__double_as_longlong(worst) & 0x7FFFFFFFFFFFFFFFull);
     __syncthreads();
     const bool unitary = __longlong_as_double((long long)dev_bits) <= 1e-10;
-    if (j == 0 && !unitary && all_unitary) atomicAnd(all_unitary, 0);
-    if (j == 0 && sg.flag_off != kNoFlag) *reinterpret_cast<int *>(prog + sg.flag_off) = unitary ? 1 : 0;
-    // column j of U is (vr, vi); write B entries with input index c = j
+    if (tid == 0 && !unitary && all_unitary) atomicAnd(all_unitary, 0);
+    if (tid == 0 && sg.flag_off != kNoFlag) *reinterpret_cast<int *>(prog + sg.flag_off) = unitary ? 1 : 0;
     unsigned char *bhi = prog + sg.b_off, *blo = bhi + 4 * K * K;
     auto b_offset = [](int k, int n) {
         return (uint32_t)((n >> 3) * SBO + (k >> 2) * 128 + (n & 7) * 16 + (k & 3) * 4);
     };
-    for (int r = 0; r < NA; ++r) {
-        const double u_re = vr[r], u_im = vi[r];
+    for (int e = tid; e < NE; e += nt) {
+        const int r = e >> R, j = e & (NA - 1);
+        const double u_re = x[e].x, u_im = x[e].y;
         const double val[4] = {u_re, -u_im, u_im, u_re};  // (k, n) = (2j, 2r), (2j+1, 2r), (2j, 2r+1), (2j+1, 2r+1)
         const int kk[4] = {2 * j, 2 * j + 1, 2 * j, 2 * j + 1};
         const int nn[4] = {2 * r, 2 * r, 2 * r + 1, 2 * r + 1};
-        for (int e = 0; e < 4; ++e) {
-            const float f = (float)val[e];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float f = (float)val[q];
             const uint32_t hi = tf32_rna(f);
-            const uint32_t lo = tf32_rna((float)(val[e] - (double)__uint_as_float(hi)));
-            *reinterpret_cast<uint32_t *>(bhi + b_offset(kk[e], nn[e])) = hi;
-            *reinterpret_cast<uint32_t *>(blo + b_offset(kk[e], nn[e])) = lo;
+            const uint32_t lo = tf32_rna((float)(val[q] - (double)__uint_as_float(hi)));
+            *reinterpret_cast<uint32_t *>(bhi + b_offset(kk[q], nn[q])) = hi;
+            *reinterpret_cast<uint32_t *>(blo + b_offset(kk[q], nn[q])) = lo;
         }
     }
 }
@@ -131,9 +140,10 @@ void launch_compose(const void *dev_segs, int nseg, const void *dev_gates, void 
     const ComposeSeg *sg = (const ComposeSeg *)dev_segs;
     const DevGate<double> *g = (const DevGate<double> *)dev_gates;
     unsigned char *p = (unsigned char *)dev_prog;
-    if (r == 3) k_compose_f64<3><<<nseg, 8, 0, st>>>(sg, g, p, all_unitary);
-    else if (r == 4) k_compose_f64<4><<<nseg, 16, 0, st>>>(sg, g, p, all_unitary);
-    else if (r == 5) k_compose_f64<5><<<nseg, 32, 0, st>>>(sg, g, p, all_unitary);
+    const size_t smem = (size_t)32 << (2 * r);  // two copies of the 2^r x 2^r product (at most 32 KiB)
+    if (r == 3) k_compose_f64<3><<<nseg, 64, smem, st>>>(sg, g, p, all_unitary);
+    else if (r == 4) k_compose_f64<4><<<nseg, 256, smem, st>>>(sg, g, p, all_unitary);
+    else if (r == 5) k_compose_f64<5><<<nseg, 256, smem, st>>>(sg, g, p, all_unitary);
     else fail(SV_ERR_UNSUPPORTED, "fused groups have 3, 4 or 5 bits");
     check_cuda(cudaGetLastError(), "compose kernel launch");
 }
