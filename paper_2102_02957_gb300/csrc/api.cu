@@ -52,16 +52,79 @@ static void ensure_scratch(sv_state *h, size_t bytes) {
     h->scratch_bytes = bytes;
 }
 
-void check_dev_error(sv_state *h) {
-    int e = 0;
-    check_cuda(cudaMemcpyAsync(&e, h->dev_err, sizeof(int), cudaMemcpyDeviceToHost, h->stream), "read error word");
-    check_cuda(cudaStreamSynchronize(h->stream), "cudaStreamSynchronize");
+static void raise_dev_error(sv_state *h, int e) {
     if (e != DEV_OK) {
         int zero = 0;
         cudaMemcpy(h->dev_err, &zero, sizeof(int), cudaMemcpyHostToDevice);
         if (e == DEV_ERR_TIMEOUT) fail(SV_ERR_TIMEOUT, "a bounded device wait expired");
         fail(SV_ERR_CUDA, "device error word set");
     }
+}
+
+void check_dev_error(sv_state *h) {
+    int e = 0;
+    check_cuda(cudaMemcpyAsync(&e, h->dev_err, sizeof(int), cudaMemcpyDeviceToHost, h->stream), "read error word");
+    check_cuda(cudaStreamSynchronize(h->stream), "cudaStreamSynchronize");
+    raise_dev_error(h, e);
+}
+
+// Result words of readouts in pinned host memory, which a readout's last kernel writes directly: one
+// stream synchronisation brings value and error word, without copies.  One 32 KiB block for the
+// process, handed out one slot per handle and given back with it; handles beyond kSlots use
+// device memory and a copy.
+namespace {
+struct SlotPool {
+    static constexpr int kSlots = 512, kBytes = 64;
+    std::mutex mu;
+    unsigned char *base = nullptr;
+    bool tried = false;
+    std::vector<int> free;
+
+    Readout *take() {
+        std::lock_guard<std::mutex> lk(mu);
+        if (!tried) {
+            tried = true;
+            void *p = nullptr;
+            if (cudaHostAlloc(&p, (size_t)kSlots * kBytes, cudaHostAllocPortable | cudaHostAllocMapped) == cudaSuccess) {
+                base = static_cast<unsigned char *>(p);
+                for (int k = kSlots - 1; k >= 0; --k) free.push_back(k);
+            } else {
+                cudaGetLastError();
+            }
+        }
+        if (free.empty()) return nullptr;
+        const int k = free.back();
+        free.pop_back();
+        return reinterpret_cast<Readout *>(base + (size_t)k * kBytes);
+    }
+    void give(Readout *r) {
+        std::lock_guard<std::mutex> lk(mu);
+        free.push_back((int)((reinterpret_cast<unsigned char *>(r) - base) / kBytes));
+    }
+};
+SlotPool &slots() {
+    static SlotPool *pool = new SlotPool();  // outlives every handle
+    return *pool;
+}
+}  // namespace
+
+static Readout *readout_words(sv_state *h) {
+    if (!h->slot) h->slot = slots().take();
+    return h->slot ? h->slot : reinterpret_cast<Readout *>(reinterpret_cast<unsigned char *>(h->dev_err) + 16);
+}
+
+// Wait for the readout whose last kernel wrote readout_words(h).
+static double finish_readout(sv_state *h) {
+    Readout r;
+    if (h->slot) {
+        check_cuda(cudaStreamSynchronize(h->stream), "cudaStreamSynchronize");
+        r = *h->slot;
+    } else {
+        check_cuda(cudaMemcpyAsync(&r, readout_words(h), sizeof(r), cudaMemcpyDeviceToHost, h->stream), "read result");
+        check_cuda(cudaStreamSynchronize(h->stream), "cudaStreamSynchronize");
+    }
+    raise_dev_error(h, r.err);
+    return r.value;
 }
 
 static void validate_gates(int n, const sv_gate *gates, int64_t n_gates) {
@@ -410,7 +473,7 @@ sv_status sv_create(int32_t n, int32_t dtype, void *dev_buf, size_t bytes, void 
         check_cuda(cudaMalloc(&h->amp, need), "cudaMalloc(state)");
         h->owns_amp = true;
     }
-    check_cuda(cudaMalloc(&h->dev_err, sizeof(int)), "cudaMalloc(error word)");
+    check_cuda(cudaMalloc(&h->dev_err, 16 + sizeof(Readout)), "cudaMalloc(error word)");
     check_cuda(cudaMemsetAsync(h->dev_err, 0, sizeof(int), h->stream), "cudaMemsetAsync");
     *out = h.release();
     SV_API_END
@@ -421,6 +484,7 @@ sv_status sv_destroy(sv_handle h) {
     if (!h) return SV_OK;
     cudaStreamSynchronize(h->stream);
     if (h->owns_amp && h->amp) cudaFree(h->amp);
+    if (h->slot) slots().give(h->slot);
     if (h->dev_err) cudaFree(h->dev_err);
     if (h->scratch) cudaFree(h->scratch);
     if (h->prog) cudaFree(h->prog);
@@ -829,13 +893,8 @@ sv_status sv_norm2(sv_handle h, double *out) {
     const int nb = reduce_blocks(h->n);
     ensure_scratch(h, (size_t)nb * sizeof(double));
     launch_partial_norm(h->dtype, h->amp, h->n, h->scratch, nb, h->stream);
-    std::vector<double> part((size_t)nb);
-    check_cuda(cudaMemcpyAsync(part.data(), h->scratch, nb * sizeof(double), cudaMemcpyDeviceToHost, h->stream),
-               "cudaMemcpyAsync(partials)");
-    check_dev_error(h);
-    double s = 0;
-    for (double v : part) s += v;
-    *out = s;
+    launch_finish(h->scratch, nb, h->dev_err, readout_words(h), h->stream);
+    *out = finish_readout(h);
     SV_API_END
 }
 
@@ -844,17 +903,13 @@ sv_status sv_expval_pauli(sv_handle h, uint64_t x, uint64_t z, double *out) {
     if (!h || !out) fail(SV_ERR_ARG, "null argument");
     if ((x >> h->n) || (z >> h->n)) fail(SV_ERR_ARG, "Pauli mask outside the register");
     const int nb = reduce_blocks(h->n);
-    ensure_scratch(h, (size_t)nb * 2 * sizeof(double));
+    ensure_scratch(h, (size_t)nb * sizeof(double));
     launch_partial_expval(h->dtype, h->amp, h->n, x, z, h->scratch, nb, h->stream);
-    std::vector<double> part((size_t)nb * 2);
-    check_cuda(cudaMemcpyAsync(part.data(), h->scratch, nb * 2 * sizeof(double), cudaMemcpyDeviceToHost, h->stream),
-               "cudaMemcpyAsync(partials)");
-    check_dev_error(h);
-    double sr = 0, si = 0;
-    for (int b = 0; b < nb; ++b) {
-        sr += part[2 * b];
-        si += part[2 * b + 1];
-    }
+    launch_finish(h->scratch, nb, h->dev_err, readout_words(h), h->stream);
+    // the sum is real where x and z overlap in an even number of qubits, imaginary otherwise
+    const double v = finish_readout(h);
+    const bool odd = __builtin_popcountll(x & z) & 1;
+    double sr = odd ? 0.0 : v, si = odd ? v : 0.0;
     // multiply by i^{popc(x & z)}
     switch (__builtin_popcountll(x & z) & 3) {
         case 1: { double t = sr; sr = -si; si = t; break; }
@@ -874,47 +929,16 @@ sv_status sv_sample(sv_handle h, int64_t shots, uint64_t seed, uint64_t *out) {
     if (shots == 0) return SV_OK;
     const int sb = std::min(h->n, 10);
     const int64_t nb = int64_t(1) << (h->n - sb);
-    // scratch: range sums, then per-shot (prefix, range, target) and results
-    const size_t need = (size_t)nb * sizeof(double) + (size_t)shots * (sizeof(double) * 2 + sizeof(int64_t) + sizeof(uint64_t)) + 1024;
-    ensure_scratch(h, need);
-    double *sums = h->scratch;
-    launch_block_sums(h->dtype, h->amp, h->n, sb, sums, h->stream);
-    std::vector<double> incl((size_t)nb);
-    check_cuda(cudaMemcpyAsync(incl.data(), sums, nb * sizeof(double), cudaMemcpyDeviceToHost, h->stream),
-               "cudaMemcpyAsync(range sums)");
-    check_dev_error(h);
-    double acc = 0;
-    for (int64_t b = 0; b < nb; ++b) {
-        acc += incl[(size_t)b];
-        incl[(size_t)b] = acc;
-    }
-    const double total = acc;
+    // scratch: range sums, their blocks' totals, the shots
+    const int64_t nt = sample_totals(h->n, sb);
+    ensure_scratch(h, (size_t)(nb + nt) * sizeof(double) + (size_t)shots * sizeof(uint64_t));
+    double *sums = h->scratch, *totals = sums + nb;
+    uint64_t *d_out = reinterpret_cast<uint64_t *>(totals + nt);
+    launch_sample(h->dtype, h->amp, h->n, sb, sums, totals, seed, shots, d_out, h->dev_err, readout_words(h), h->stream);
+    const double total = finish_readout(h);
     if (!(total > 0)) fail(SV_ERR_ARG, "state has zero norm");
-    std::vector<double> prefix((size_t)shots), target((size_t)shots);
-    std::vector<int64_t> blk((size_t)shots);
-    for (int64_t s = 0; s < shots; ++s) {
-        const double t = splitmix_uniform(seed, (uint64_t)s) * total;
-        // smallest range whose inclusive prefix exceeds t
-        int64_t lo = 0, hi = nb - 1;
-        while (lo < hi) {
-            const int64_t mid = lo + (hi - lo) / 2;
-            if (incl[(size_t)mid] > t) hi = mid; else lo = mid + 1;
-        }
-        blk[(size_t)s] = lo;
-        prefix[(size_t)s] = lo > 0 ? incl[(size_t)lo - 1] : 0.0;
-        target[(size_t)s] = t;
-    }
-    unsigned char *p = reinterpret_cast<unsigned char *>(h->scratch) + (((size_t)nb * sizeof(double) + 255) / 256) * 256;
-    double *d_prefix = reinterpret_cast<double *>(p);
-    double *d_target = d_prefix + shots;
-    int64_t *d_blk = reinterpret_cast<int64_t *>(d_target + shots);
-    uint64_t *d_out = reinterpret_cast<uint64_t *>(d_blk + shots);
-    check_cuda(cudaMemcpyAsync(d_prefix, prefix.data(), shots * sizeof(double), cudaMemcpyHostToDevice, h->stream), "H2D");
-    check_cuda(cudaMemcpyAsync(d_target, target.data(), shots * sizeof(double), cudaMemcpyHostToDevice, h->stream), "H2D");
-    check_cuda(cudaMemcpyAsync(d_blk, blk.data(), shots * sizeof(int64_t), cudaMemcpyHostToDevice, h->stream), "H2D");
-    launch_sample_within(h->dtype, h->amp, h->n, sb, d_prefix, d_blk, d_target, shots, d_out, h->stream);
     check_cuda(cudaMemcpyAsync(out, d_out, shots * sizeof(uint64_t), cudaMemcpyDeviceToHost, h->stream), "D2H");
-    check_dev_error(h);
+    check_cuda(cudaStreamSynchronize(h->stream), "cudaStreamSynchronize");
     SV_API_END
 }
 

@@ -296,11 +296,18 @@ void launch_renorm(int dtype, void *state, int n, const double *partials, int nb
                    cudaStream_t st);
 void launch_partial_expval(int dtype, const void *state, int n, uint64_t x, uint64_t z,
                            double *partials, int nblocks, cudaStream_t st);
-void launch_block_sums(int dtype, const void *state, int n, int sum_bits, double *sums, cudaStream_t st);
-void launch_sample_within(int dtype, const void *state, int n, int sum_bits, const double *prefix,
-                          const int64_t *shot_block, const double *shot_target, int64_t shots,
-                          uint64_t *out, cudaStream_t st);
-double splitmix_uniform(uint64_t seed, uint64_t s);
+// Result words of a readout: a value and the handle's device error word.
+struct Readout {
+    double value;
+    int err;
+};
+// out->value = sum of the partials.
+void launch_finish(const double *partials, int nblocks, const int *err, Readout *out, cudaStream_t st);
+// Inverse-CDF sampling over ranges of 2^sb amplitudes: sums holds 2^(n-sb) doubles, totals
+// sample_totals(n, sb); total->value receives the squared norm.
+int64_t sample_totals(int n, int sb);
+void launch_sample(int dtype, const void *state, int n, int sb, double *sums, double *totals, uint64_t seed, int64_t shots,
+                   uint64_t *out, const int *err, Readout *total, cudaStream_t st);
 
 int num_sms();
 
@@ -319,7 +326,8 @@ struct sv_state {
     void *amp = nullptr;      // device amplitudes
     bool owns_amp = false;
     cudaStream_t stream = nullptr;
-    int *dev_err = nullptr;   // device error word
+    int *dev_err = nullptr;   // device error word, then (16 bytes on) a Readout
+    sv::Readout *slot = nullptr;  // pinned result words (api.cu's pool)
     double *scratch = nullptr;  // device scratch for reductions
     size_t scratch_bytes = 0;
     void *prog = nullptr;     // device block programs
