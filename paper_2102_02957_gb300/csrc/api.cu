@@ -143,7 +143,8 @@ static void validate_gates(int n, const sv_gate *gates, int64_t n_gates) {
 struct BlockProg {
     size_t off;
     int nseg, gate_bytes;  // SIMT: bytes of the gate area
-    bool fixed = false;    // SIMT complex128: fixed-point gate area
+    bool fixed = false;    // complex128: fixed-point gate area
+    bool oz = false;       // complex128: tensor-core sweep (block_oz.cuh)
     int r = 0;         // tensor-core register-group width of the sweep
     GatherLayout lay;  // gathered sections only
     int op_index = -1;
@@ -307,13 +308,22 @@ static void build_programs_tc(const sv_plan *plan, const sv_gate *gates, int r_p
     host.insert(host.end(), p, p + sizeof(one));
 }
 
+// Section programs with SIMT register groups, and (complex128, `oz` non-null) tensor-core sweeps:
+// sections of unitary gates that do more than exchange amplitudes and flip signs, none of them outside
+// its chunk, on chunks that hold a 128-row tile.  There a group costs about as much whatever its
+// gates are, less than one dense gate costs on the integer pipe (block_fx.cuh).  A section with
+// more groups than fit beside the chunks takes several sweeps.  *oz receives the groups to compose.
 template <typename T>
 static void build_programs(const sv_plan *plan, const sv_gate *gates, int seg_bits, std::vector<unsigned char> &host,
-                           std::vector<BlockProg> &progs) {
+                           std::vector<BlockProg> &progs, std::vector<OzCompose> *oz = nullptr) {
     host.clear();
     progs.clear();
     auto align = [&](size_t a) {
         while (host.size() % a) host.push_back(0);
+    };
+    auto put = [&](const void *data, size_t bytes) {
+        const unsigned char *p = static_cast<const unsigned char *>(data);
+        host.insert(host.end(), p, p + bytes);
     };
     for (const PlanOp &op0 : plan->ops) {
         if (op0.kind != 2 && op0.kind != 4) continue;
@@ -358,19 +368,59 @@ static void build_programs(const sv_plan *plan, const sv_gate *gates, int seg_bi
                 if (std::all_of(dgates.begin() + d.g0, dgates.end(), exact_gate)) d.flags |= kSegRaw;
             dsegs.push_back(d);
         }
-        align(256);
-        bp.off = host.size();
-        bp.nseg = (int)dsegs.size();
-        const unsigned char *p = reinterpret_cast<const unsigned char *>(dsegs.data());
-        host.insert(host.end(), p, p + dsegs.size() * sizeof(DevSeg));
-        align(16);
         // complex128: fixed-point gates where every gate is unitary (their area is never the larger)
         std::vector<unsigned char> area;
         if constexpr (sizeof(T) == 8) bp.fixed = encode_fx(dgates, area);
+        if constexpr (sizeof(T) == 8) {
+            int per = 0;  // groups per sweep
+            if (oz && bp.fixed && std::any_of(dsegs.begin(), dsegs.end(), [](const DevSeg &d) { return !(d.flags & kSegRaw); }) &&
+                std::none_of(dgates.begin(), dgates.end(), [](const DevGate<T> &g) { return g.op == OP_DIAGX; }))
+                per = oz_max_segs(width, area.size());
+            if (per > 0) {
+                const int nseg = (int)dsegs.size(), sweeps = (nseg + per - 1) / per;
+                for (int w = 0; w < sweeps; ++w) {
+                    const int s0 = (int)((int64_t)nseg * w / sweeps), s1 = (int)((int64_t)nseg * (w + 1) / sweeps);
+                    const int g0 = dsegs[(size_t)s0].g0, g1 = dsegs[(size_t)s1 - 1].g1;
+                    encode_fx(std::vector<DevGate<T>>(dgates.begin() + g0, dgates.begin() + g1), area);
+                    align(256);
+                    bp.oz = true;
+                    bp.off = host.size();
+                    bp.nseg = s1 - s0;
+                    bp.gate_bytes = (int)area.size();
+                    for (int k = s0; k < s1; ++k) {
+                        DevSeg d = dsegs[(size_t)k];
+                        d.flags = (int8_t)((k == s0 ? 1 : 0) | (k + 1 == s1 ? 2 : 0));
+                        d.g0 = (int16_t)(d.g0 - g0);
+                        d.g1 = (int16_t)(d.g1 - g0);
+                        put(&d, sizeof(d));
+                    }
+                    align(16);
+                    for (int k = s0; k < s1; ++k) {
+                        const OzSeg a = oz_addresses(segs[(size_t)k], width, k == s0, k + 1 == s1);
+                        put(&a, sizeof(a));
+                    }
+                    const size_t gates_off = host.size();
+                    host.insert(host.end(), area.begin(), area.end());
+                    align(16);
+                    const size_t b_off = host.size();
+                    host.resize(b_off + (size_t)bp.nseg * kOzBBytes, 0);
+                    for (int k = s0; k < s1; ++k)
+                        oz->push_back(OzCompose{(uint32_t)gates_off, (uint32_t)(b_off + (size_t)(k - s0) * kOzBBytes),
+                                                dsegs[(size_t)k].g0 - g0, dsegs[(size_t)k].g1 - g0});
+                    progs.push_back(bp);
+                }
+                continue;
+            }
+        }
         if (!bp.fixed) {
-            p = reinterpret_cast<const unsigned char *>(dgates.data());
+            const unsigned char *p = reinterpret_cast<const unsigned char *>(dgates.data());
             area.assign(p, p + dgates.size() * sizeof(DevGate<T>));
         }
+        align(256);
+        bp.off = host.size();
+        bp.nseg = (int)dsegs.size();
+        put(dsegs.data(), dsegs.size() * sizeof(DevSeg));
+        align(16);
         bp.gate_bytes = (int)area.size();
         host.insert(host.end(), area.begin(), area.end());
         align(16);
@@ -706,9 +756,18 @@ sv_status sv_apply_circuit(sv_handle h, const sv_gate *gates, int64_t n_gates, s
             launch_partial_norm(h->dtype, h->amp, h->n, h->scratch, nb_norm, h->stream);
             ++st.kernel_launches;
         }
-        if (tc) build_programs_tc(plan, gates, tc_bits, host, progs, cs_off, ncs, g_off, flag_off);
-        else if (h->dtype == SV_C64) build_programs<float>(plan, gates, seg_bits, host, progs);
-        else build_programs<double>(plan, gates, seg_bits, host, progs);
+        std::vector<OzCompose> oz;  // complex128 groups to fuse
+        size_t oz_off = 0;
+        if (tc) {
+            build_programs_tc(plan, gates, tc_bits, host, progs, cs_off, ncs, g_off, flag_off);
+        } else if (h->dtype == SV_C64) {
+            build_programs<float>(plan, gates, seg_bits, host, progs);
+        } else {
+            build_programs<double>(plan, gates, seg_bits, host, progs, &oz);
+            oz_off = host.size();
+            const unsigned char *p = reinterpret_cast<const unsigned char *>(oz.data());
+            host.insert(host.end(), p, p + oz.size() * sizeof(OzCompose));
+        }
         upload_program(h, host);
         const unsigned char *base = static_cast<const unsigned char *>(h->prog);
         int *unitary_flag = tc ? reinterpret_cast<int *>(static_cast<unsigned char *>(h->prog) + flag_off) : nullptr;
@@ -718,6 +777,10 @@ sv_status sv_apply_circuit(sv_handle h, const sv_gate *gates, int64_t n_gates, s
                     launch_compose(base + cs_off[w], ncs[w], base + g_off, h->prog, unitary_flag, w + 3, h->stream);
                     ++st.kernel_launches;
                 }
+        }
+        if (!oz.empty()) {
+            launch_compose_oz(base + oz_off, (int)oz.size(), h->prog, h->stream);
+            ++st.kernel_launches;
         }
         const uint64_t wait_ns = plan->wait_limit_ms > 0 ? (uint64_t)plan->wait_limit_ms * 1000000ull : kDefaultWaitNs;
         size_t bi = 0;
@@ -730,6 +793,9 @@ sv_status sv_apply_circuit(sv_handle h, const sv_gate *gates, int64_t n_gates, s
                     if (tc)
                         launch_block_tc(h->amp, h->n, plan->c, bp.gathered ? &bp.lay : nullptr, base + bp.off, bp.nseg,
                                         h->dev_err, bp.r, h->stream, wait_ns);
+                    else if (bp.oz)
+                        launch_block_oz(h->amp, h->n, plan->c, bp.gathered ? &bp.lay : nullptr, base + bp.off, bp.nseg,
+                                        bp.gate_bytes, h->dev_err, h->stream, wait_ns);
                     else if (!bp.gathered)
                         launch_block(h->dtype, h->amp, h->n, plan->c, base + bp.off, bp.nseg, bp.gate_bytes, bp.fixed,
                                      h->dev_err, seg_bits, h->stream, wait_ns);

@@ -114,4 +114,30 @@ bool encode_fx(const std::vector<DevGate<double>> &gates, std::vector<unsigned c
     return true;
 }
 
+OzSeg oz_addresses(const HostSeg &seg, int width, bool natural_ld, bool natural_st) {
+    OzSeg out{};
+    auto slot = [&](int index, bool natural) {
+        int s = index;
+        for (int k = 3; !natural && k < width; ++k)
+            if ((index >> k) & 1) s ^= kSwz128[k];
+        return (uint32_t)s * 16u;
+    };
+    for (int side = 0; side < 2; ++side) {
+        uint32_t *t = side ? out.st : out.ld;
+        const bool natural = side ? natural_st : natural_ld;
+        auto fill = [&](int at, int count, const int32_t *bits) {
+            for (int v = 0; v < count; ++v) {
+                int index = 0;
+                for (int k = 0; (v >> k) != 0; ++k)
+                    if ((v >> k) & 1) index |= 1 << bits[k];
+                t[at + v] = slot(index, natural);
+            }
+        };
+        fill(0, 32, seg.lane);
+        fill(32, std::min(16, 1 << seg.nrest), seg.rest);
+        fill(48, 16, seg.pos);
+    }
+    return out;
+}
+
 }  // namespace sv

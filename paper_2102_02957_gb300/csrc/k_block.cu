@@ -40,6 +40,7 @@
 
 #include "block_core.cuh"
 #include "block_fx.cuh"
+#include "block_oz.cuh"
 #include "ptx.cuh"
 #include "sv_internal.h"
 
@@ -175,15 +176,24 @@ __device__ __forceinline__ void store_chunks(T2 *state, int c, int64_t count, in
     ptx::bulk_wait<0>();
 }
 
+// Register-group engines of a section kernel besides the SIMT one (run_segment).
+enum : int { ENG_NONE = 0, ENG_FX = 1, ENG_OZ = 2 };
+
 constexpr int CG2 = 2;  // consumer groups per CTA (default)
 
 // G consumer groups per CTA; tensor-core groups keep NB tile buffers each
 // (G * NB * TcGeom<R>::COLS <= 512 TMEM columns).
-template <typename T, int R, int NC, int KU, bool TC, int G, int NB, bool FX>
+// Service threads of a section kernel: producer and store warp, and for complex128 tensor-core
+// sections a warp per half row that issues its MMAs; mbarriers per consumer group beside the ring's.
+constexpr int svc_threads(int eng) { return eng == ENG_OZ ? 128 : kSvcThreads; }
+constexpr int mma_bars(int eng) { return eng == ENG_OZ ? 4 : 2; }
+
+template <typename T, int R, int NC, int KU, bool TC, int G, int NB, int ENG>
 __device__ __forceinline__ void block_body(typename V2<T>::type *__restrict__ state, int c, int64_t nchunks, int nbuf,
                                            const unsigned char *__restrict__ prog, int nseg, int gate_bytes, int *err,
                                            const CUtensorMap &tmap, const GatherArgs &ga_in, uint64_t wait_ns) {
     using T2 = typename V2<T>::type;
+    constexpr int kSvc = svc_threads(ENG), kBars = mma_bars(ENG);
     __shared__ GatherArgs ga;  // gathered chunks (rank > 0); rank 0 = contiguous chunk j
     if (threadIdx.x == 0) ga = ga_in;
     extern __shared__ __align__(1024) unsigned char smem[];
@@ -194,17 +204,21 @@ __device__ __forceinline__ void block_body(typename V2<T>::type *__restrict__ st
     // groups' B operands (tensor cores), 16-byte aligned
     const int seg_bytes = (int)((nseg * sizeof(DevSeg) + 15) & ~size_t(15));
     constexpr int kBBytes = TcGeom<(R < 3 ? 3 : R)>::B_BYTES;  // B operand of one tensor-core group
-    const int prog_bytes = seg_bytes + (TC ? nseg * kBBytes : gate_bytes);
+    const int tab_bytes = ENG == ENG_OZ ? nseg * (int)sizeof(OzSeg) : 0;
+    const int gate_pad = (gate_bytes + 15) & ~15;  // complex128 tensor-core programs: gate area, then B operands
+    const int prog_bytes =
+        seg_bytes + tab_bytes + (ENG == ENG_OZ ? gate_pad + nseg * kOzBBytes : TC ? nseg * kBBytes : gate_bytes);
     unsigned char *sprog = smem + (size_t)nbuf * chunk_bytes;
     const DevSeg *segs = reinterpret_cast<const DevSeg *>(sprog);
-    const unsigned char *gates = sprog + seg_bytes;
+    const unsigned char *gates = sprog + seg_bytes + tab_bytes;
     uint64_t *full = reinterpret_cast<uint64_t *>(sprog + ((prog_bytes + 15) & ~15));
     uint64_t *empty = full + nbuf;
     uint64_t *done = empty + nbuf;
-    uint64_t *mma_bar = done + nbuf;  // two per consumer group (tensor-core path)
-    volatile int *abort_flag = reinterpret_cast<volatile int *>(mma_bar + 2 * G);
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(mma_bar + 2 * G) + 1;
+    uint64_t *mma_bar = done + nbuf;  // kBars per consumer group (tensor-core paths): MMAs done, tile ready
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(mma_bar + kBars * G);
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(mma_bar + kBars * G) + 1;
     __shared__ int swz[24];
+    [[maybe_unused]] __shared__ OzShared oz[ENG == ENG_OZ ? G : 1];
     // the wait bound lives in shared memory: waits are rare, a register for it in every thread is not
     __shared__ uint64_t s_wait_ns;
     constexpr uint32_t kTmemCols = 512;  // G consumer groups x NB tile buffers x TcGeom<R>::COLS
@@ -219,11 +233,11 @@ __device__ __forceinline__ void block_body(typename V2<T>::type *__restrict__ st
             ptx::mbar_init(&empty[s], 1);
             ptx::mbar_init(&done[s], 1);
         }
-        for (int g = 0; g < 2 * G; ++g) ptx::mbar_init(&mma_bar[g], 1);
+        for (int g = 0; g < kBars * G; ++g) ptx::mbar_init(&mma_bar[g], (g % kBars) < 2 ? 1 : NC / 32);
         *abort_flag = 0;
         ptx::fence_mbar_init();
     }
-    constexpr int kTmemWarp = kSvcThreads / 32;  // the first consumer warp allocates tensor memory
+    constexpr int kTmemWarp = kSvc / 32;  // the first consumer warp allocates tensor memory
     if (TC && (threadIdx.x >> 5) == kTmemWarp) ptx::tmem_alloc(ptx::smem_addr(tmem_slot), kTmemCols);
     if (TC) {
         ptx::fence_proxy_async_smem();  // B operands written by generic stores, read by the tensor cores
@@ -235,12 +249,21 @@ __device__ __forceinline__ void block_body(typename V2<T>::type *__restrict__ st
 
     const int64_t count = blockIdx.x < nchunks ? (nchunks - 1 - blockIdx.x) / gridDim.x + 1 : 0;
 
-    if (threadIdx.x < kSvcThreads) {
+    if (threadIdx.x < kSvc) {
         // ------------------------------------------------- producer (warp 0), store (warp 1)
         if (threadIdx.x < 32)
             produce_chunks<T2>(state, c, count, nbuf, bufs, full, empty, abort_flag, err, ga, &tmap, wait_ns);
-        else
+        else if (threadIdx.x < 64)
             store_chunks<T2>(state, c, count, nbuf, bufs, done, empty, abort_flag, err, ga, &tmap, wait_ns);
+        if constexpr (ENG == ENG_OZ) {
+            static_assert(ENG != ENG_OZ || G == 1, "one consumer group");
+            if (threadIdx.x >= 64) {
+                oz_issue((int)(threadIdx.x >> 5) - 2, ptx::smem_addr(gates) + (uint32_t)gate_pad, nseg, c, count, tmem_base,
+                         mma_bar, abort_flag, err, &s_wait_ns, &oz[0]);
+                ptx::tc_fence_before();
+                ptx::named_bar_sync(1 + G, G * NC + 64);  // before tensor memory is freed
+            }
+        }
         return;
     }
 
@@ -249,8 +272,8 @@ __device__ __forceinline__ void block_body(typename V2<T>::type *__restrict__ st
     // overlap another group's arithmetic; each group synchronises on its own named barrier.
     // (Two groups sharing a chunk, each with half of its tiles, was measured slower: the shared
     // barriers between register groups cost more than the deeper prefetch gained.)
-    const int cg = (threadIdx.x - kSvcThreads) / NC;
-    const int ctid = (threadIdx.x - kSvcThreads) % NC;
+    const int cg = (threadIdx.x - kSvc) / NC;
+    const int ctid = (threadIdx.x - kSvc) % NC;
     const int bar_id = 1 + cg;
     uint32_t mma_phase[2] = {0, 0};
     // A parity wait cannot tell this chunk's load (use u = it / nbuf of slot s) from the slot's
@@ -271,23 +294,35 @@ __device__ __forceinline__ void block_body(typename V2<T>::type *__restrict__ st
             atomicCAS(err, DEV_OK, DEV_ERR_TIMEOUT);
             *abort_flag = 1;
         }
+        if constexpr (ENG == ENG_OZ) {  // the last chunk's values are read: cleared before the barrier
+            if (ctid < kOzMaxSegs) oz[cg].high[ctid] = 0;
+            if (ctid == 0) oz[cg].top = oz[cg].any = oz[cg].skip = 0;
+        }
         // every thread of the group leaves together (the flag is read before the barrier)
         if (ptx::named_bar_or(bar_id, NC, bad || *abort_flag)) break;
         T2 *buf = bufs + (size_t)s * chunk_amps;
         // state index of the chunk's first amplitude (its bits outside the chunk are the chunk's)
         const int64_t origin = ga.rank > 0 ? gather_origin(ga, j, 0) : j << c;
         bool failed = false;
-        for (int si = 0; si < nseg; ++si) {
+        if constexpr (ENG == ENG_OZ) {
+            const uint32_t gates_s = ptx::smem_addr(gates);
+            failed = !run_chunk_oz<NC>(ptx::smem_addr(buf), ptx::smem_addr(segs), gates_s - (uint32_t)tab_bytes, gates_s, gates_s + (uint32_t)gate_pad, nseg,
+                                       ctid, swz, c, origin, tmem_base, bar_id, &mma_bar[kBars * cg],
+                                       mma_phase, abort_flag, &s_wait_ns, &oz[cg]);
+            ptx::fence_proxy_async_smem();
+            if (ptx::named_bar_or(bar_id, NC, failed)) failed = true;
+        }
+        for (int si = 0; ENG != ENG_OZ && si < nseg; ++si) {
             const uint32_t seg_addr = ptx::smem_addr(segs) + (uint32_t)(si * sizeof(DevSeg));
             [[maybe_unused]] bool ok = true;
-            if constexpr (TC) {
+            if constexpr (TC && ENG == ENG_NONE) {
                 ok = run_segment_tc<R, NC, false, NB>(ptx::smem_addr(buf), seg_addr,
                                                       ptx::smem_addr(sprog + seg_bytes) + (uint32_t)(si * kBBytes), ctid,
                                                       swz, c, tmem_base + (uint32_t)(cg * NB * TcGeom<R>::COLS), bar_id,
                                                       &mma_bar[2 * cg], mma_phase, abort_flag, &s_wait_ns);
-            } else if constexpr (FX) {
+            } else if constexpr (ENG == ENG_FX) {
                 run_segment_fx<NC>(ptx::smem_addr(buf), seg_addr, ptx::smem_addr(gates), ctid, swz, c, origin);
-            } else {
+            } else if constexpr (ENG == ENG_NONE) {
                 run_segment<T, R, NC, KU>(ptx::smem_addr(buf), seg_addr, ptx::smem_addr(gates), ctid, swz, c, origin);
             }
             if (si == nseg - 1) ptx::fence_proxy_async_smem();  // the store copies read the chunk
@@ -311,7 +346,7 @@ __device__ __forceinline__ void block_body(typename V2<T>::type *__restrict__ st
     if constexpr (TC) {
         // every consumer is done with tensor memory before the allocating warp frees it
         ptx::tc_fence_before();
-        ptx::named_bar_sync(1 + G, G * NC);
+        ptx::named_bar_sync(1 + G, G * NC + (ENG == ENG_OZ ? 64 : 0));
         if ((threadIdx.x >> 5) == kTmemWarp) {
             ptx::tc_fence_after();
             ptx::tmem_dealloc(tmem_base, kTmemCols);
@@ -320,12 +355,12 @@ __device__ __forceinline__ void block_body(typename V2<T>::type *__restrict__ st
 }
 
 // SIMT sections: launch bounds let the compiler fit two 256-thread consumer groups.
-template <typename T, int R, int NC, int KU, bool TC, int G = CG2, int NB = 2, bool FX = false>
+template <typename T, int R, int NC, int KU, bool TC, int G = CG2, int NB = 2, int ENG = ENG_NONE>
 __global__ void __launch_bounds__(G * NC + kSvcThreads, 1)
     k_block(typename V2<T>::type *__restrict__ state, int c, int64_t nchunks, int nbuf,
             const unsigned char *__restrict__ prog, int nseg, int gate_bytes, int *err,
             const __grid_constant__ CUtensorMap tmap, const GatherArgs ga_in, uint64_t wait_ns) {
-    block_body<T, R, NC, KU, TC, G, NB, FX>(state, c, nchunks, nbuf, prog, nseg, gate_bytes, err, tmap, ga_in, wait_ns);
+    block_body<T, R, NC, KU, TC, G, NB, ENG>(state, c, nchunks, nbuf, prog, nseg, gate_bytes, err, tmap, ga_in, wait_ns);
 }
 
 // Tensor-core sections: one CTA per SM (it takes all of the SM's tensor memory).  The register
@@ -339,18 +374,18 @@ constexpr int tc_max_regs(int threads) {
 }
 static_assert(tc_max_regs(576) == 96 && tc_max_regs(320) == 168, "register budget per thread");
 
-template <typename T, int R, int NC, int KU, bool TC, int G, int NB>
-__global__ void __maxnreg__(tc_max_regs(G * NC + kSvcThreads))
+template <typename T, int R, int NC, int KU, bool TC, int G, int NB, int ENG>
+__global__ void __maxnreg__(tc_max_regs(G * NC + svc_threads(ENG)))
     k_block_tc(typename V2<T>::type *__restrict__ state, int c, int64_t nchunks, int nbuf,
                const unsigned char *__restrict__ prog, int nseg, int gate_bytes, int *err,
                const __grid_constant__ CUtensorMap tmap, const GatherArgs ga_in, uint64_t wait_ns) {
-    block_body<T, R, NC, KU, TC, G, NB, false>(state, c, nchunks, nbuf, prog, nseg, gate_bytes, err, tmap, ga_in,
+    block_body<T, R, NC, KU, TC, G, NB, ENG>(state, c, nchunks, nbuf, prog, nseg, gate_bytes, err, tmap, ga_in,
                                                wait_ns);
 }
 
 constexpr size_t kMaxBlockSmem = 227 * 1024 - 1024;  // minus the static swizzle table (1 KiB aligned)
 
-template <typename T, int R, int NC, int KU, bool TC = false, int G = CG2, int NB = 2, bool FX = false>
+template <typename T, int R, int NC, int KU, bool TC = false, int G = CG2, int NB = 2, int ENG = ENG_NONE>
 void launch_typed(void *state, int n, int ce, const void *prog, int nseg, int gate_bytes, int *err, cudaStream_t st,
                   const CUtensorMap &tmap, const GatherArgs &ga, uint64_t wait_ns) {
     if (ce - R - 5 > kMaxRest) fail(SV_ERR_UNSUPPORTED, "chunk too wide for the register-group layout");
@@ -359,13 +394,17 @@ void launch_typed(void *state, int n, int ce, const void *prog, int nseg, int ga
     const int64_t nchunks = int64_t(1) << (n - ce);
     const size_t seg_bytes = (nseg * sizeof(DevSeg) + 15) & ~size_t(15);
     const size_t prog_bytes =
-        (seg_bytes + (TC ? (size_t)nseg * TcGeom<(R < 3 ? 3 : R)>::B_BYTES : (size_t)gate_bytes) + 15) &
+        (seg_bytes +
+         (ENG == ENG_OZ ? (((size_t)gate_bytes + 15) & ~size_t(15)) + (size_t)nseg * (kOzBBytes + sizeof(OzSeg))
+          : TC          ? (size_t)nseg * TcGeom<(R < 3 ? 3 : R)>::B_BYTES
+                        : (size_t)gate_bytes) +
+         15) &
         ~size_t(15);
-    if (TC && G * NB * TcGeom<(R < 3 ? 3 : R)>::COLS > 512) fail(SV_ERR_UNSUPPORTED, "tile buffers exceed tensor memory");
-    int nbuf = TC ? G + 2 : 3;  // tensor cores: every consumer group holds a chunk, plus prefetch
+    if (TC && ENG == ENG_NONE && G * NB * TcGeom<(R < 3 ? 3 : R)>::COLS > 512) fail(SV_ERR_UNSUPPORTED, "tile buffers exceed tensor memory");
+    int nbuf = TC && ENG == ENG_NONE ? G + 2 : 3;  // tensor cores: every consumer group holds a chunk, plus prefetch
     // program + mbarriers (full, empty, done per buffer; two per consumer group), abort flag,
     // TMEM address
-    const size_t extra = prog_bytes + (size_t)(3 * nbuf + 2 * G) * 8 + 16;
+    const size_t extra = prog_bytes + (size_t)(3 * nbuf + mma_bars(ENG) * G) * 8 + 16;
     const size_t max_smem = kMaxBlockSmem;
     while (nbuf > 1 && nbuf * chunk_bytes + extra > max_smem) --nbuf;
     size_t smem = nbuf * chunk_bytes + extra;
@@ -377,19 +416,19 @@ void launch_typed(void *state, int n, int ce, const void *prog, int nseg, int ga
         check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
                    "cudaFuncSetAttribute(block)");
         int per_sm = 0;
-        check_cuda(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, G * NC + kSvcThreads, smem),
+        check_cuda(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, G * NC + svc_threads(ENG), smem),
                    "occupancy(block)");
         if (per_sm < 1) per_sm = 1;
         if (TC) per_sm = 1;  // each CTA allocates all 512 tensor-memory columns of its SM
         return (unsigned)std::min<int64_t>(nchunks, (int64_t)num_sms() * per_sm);
     };
     if constexpr (TC) {
-        auto kern = k_block_tc<T, R, NC, KU, TC, G, NB>;
-        kern<<<grid_of(kern), G * NC + kSvcThreads, smem, st>>>((T2 *)state, ce, nchunks, nbuf, (const unsigned char *)prog, nseg,
+        auto kern = k_block_tc<T, R, NC, KU, TC, G, NB, ENG>;
+        kern<<<grid_of(kern), G * NC + svc_threads(ENG), smem, st>>>((T2 *)state, ce, nchunks, nbuf, (const unsigned char *)prog, nseg,
                                                      gate_bytes, err, tmap, ga, wait_ns);
     } else {
-        auto kern = k_block<T, R, NC, KU, TC, G, NB, FX>;
-        kern<<<grid_of(kern), G * NC + kSvcThreads, smem, st>>>((T2 *)state, ce, nchunks, nbuf, (const unsigned char *)prog, nseg,
+        auto kern = k_block<T, R, NC, KU, TC, G, NB, ENG>;
+        kern<<<grid_of(kern), G * NC + svc_threads(ENG), smem, st>>>((T2 *)state, ce, nchunks, nbuf, (const unsigned char *)prog, nseg,
                                                      gate_bytes, err, tmap, ga, wait_ns);
     }
     check_cuda(cudaGetLastError(), "block kernel launch");
@@ -447,7 +486,7 @@ static void dispatch(int dtype, int r, void *state, int n, int ce, const void *p
         if (r == 4) launch_typed<float, 4, 256, 1>(state, n, ce, prog, nseg, gate_bytes, err, st, m, ga, wait_ns);
         else launch_typed<float, 5, 128, 1>(state, n, ce, prog, nseg, gate_bytes, err, st, m, ga, wait_ns);
     } else if (fixed) {
-        launch_typed<double, 4, 128, 1, false, CG2, 2, true>(state, n, ce, prog, nseg, gate_bytes, err, st, m, ga, wait_ns);
+        launch_typed<double, 4, 128, 1, false, CG2, 2, ENG_FX>(state, n, ce, prog, nseg, gate_bytes, err, st, m, ga, wait_ns);
     } else {
         launch_typed<double, 4, 128, 1>(state, n, ce, prog, nseg, gate_bytes, err, st, m, ga, wait_ns);
     }
@@ -507,6 +546,36 @@ void launch_block_tc(void *state, int n, int c, const GatherLayout *lay, const v
         launch_typed<float, 4, 128, 1, true, 4, 1>(state, n, ce, dev_prog, nseg, 0, dev_err, st, m, ga, wait_ns);
     else
         launch_typed<float, 4, 128, 1, true, 2, 2>(state, n, ce, dev_prog, nseg, 0, dev_err, st, m, ga, wait_ns);
+}
+
+// Shared memory beside the chunk buffers: barriers and flags (launch_typed's `extra`), the groups'
+// static words.
+int oz_max_segs(int ce, size_t gate_bytes) {
+    if (ce < 11 || ce > 13) return 0;
+    const size_t chunk = size_t(16) << ce;
+    // two chunk buffers (one computed on, one in transfer) where that leaves room for two groups
+    for (int bufs = 2; bufs >= 1; --bufs) {
+        const size_t fixed = bufs * chunk + kOzMaxSegs * sizeof(DevSeg) + ((gate_bytes + 15) & ~size_t(15)) + 1024;
+        const size_t room = fixed < kMaxBlockSmem ? (kMaxBlockSmem - fixed) / (kOzBBytes + sizeof(OzSeg)) : 0;
+        if (room >= 2 || (bufs == 1 && room >= 1)) return (int)std::min<size_t>(room, kOzMaxSegs);
+    }
+    return 0;
+}
+
+void launch_block_oz(void *state, int n, int c, const GatherLayout *lay, const void *dev_prog, int nseg, int gate_bytes,
+                     int *dev_err, cudaStream_t st, uint64_t wait_ns) {
+    const int ce = lay ? lay->ce : (c < n ? c : n);
+    if (ce < 11 || nseg < 1 || nseg > kOzMaxSegs) fail(SV_ERR_UNSUPPORTED, "complex128 tensor-core sections need chunks of at least 2^11 amplitudes");
+    GatherArgs ga{};
+    CUtensorMap m;
+    std::memset(&m, 0, sizeof(m));
+    if (lay) {
+        if ((size_t)lay->args.box_amps * 16 < 128)
+            fail(SV_ERR_UNSUPPORTED, "gathered chunk boxes smaller than 128 bytes (pin more low bits)");
+        m = make_gather_map(state, *lay, 16);
+        ga = lay->args;
+    }
+    launch_typed<double, 4, 512, 1, true, 1, 1, ENG_OZ>(state, n, ce, dev_prog, nseg, gate_bytes, dev_err, st, m, ga, wait_ns);
 }
 
 }  // namespace sv

@@ -12,6 +12,9 @@
 // B_lo follows B_hi directly, so that the pair reads as one K x 2K operand [B_hi | B_lo].
 // The high part is B rounded to TF32 (round to nearest), the low part the remainder, also
 // rounded to nearest TF32 (the tensor cores would otherwise truncate it, a one-sided error).
+#include <cuda_fp16.h>
+
+#include "fixed64.cuh"
 #include "sv_internal.h"
 
 namespace sv {
@@ -132,7 +135,92 @@ __global__ void __launch_bounds__(256) k_compose_f64(const ComposeSeg *__restric
     }
 }
 
+// Fused unitary of a complex128 group (block_oz.cuh), in block fixed point with the fixed scale 2^59
+// (all entries of unitaries are at most 1), from the section's own gate area; then
+// M = round(U 2^54) in balanced base-256 digits as FP16 B operands.  One CTA per group, one thread
+// per element (row r, column j); element products read and write two shared copies in turn.
+__global__ void __launch_bounds__(256) k_compose_fx(const OzCompose *__restrict__ groups, unsigned char *__restrict__ prog) {
+    constexpr int NA = 16;
+    __shared__ fx::Real Ur[2][NA * NA], Ui[2][NA * NA];
+    const OzCompose sg = groups[blockIdx.x];
+    const unsigned char *gates = prog + sg.gates_off;
+    const int e = threadIdx.x, r = e >> 4, j = e & 15;
+    int cur = 0;
+    Ur[0][e] = r == j ? fx::pack(1ll << 59) : fx::Real{0, 0};
+    Ui[0][e] = fx::Real{0, 0};
+    __syncthreads();
+    for (int gi = sg.g0; gi < sg.g1; ++gi) {
+        const int4 hd = reinterpret_cast<const int4 *>(gates)[gi];  // op, payload offset, -, code
+        const int op = hd.x, code = hd.w;
+        const int4 *pay = reinterpret_cast<const int4 *>(gates + hd.y);
+        const bool one = op == OP_DENSE1 || op == OP_REAL1 || op == OP_DIAG1 || op == OP_X1;
+        const int ba = one ? 1 << code : 1 << (code >> 3), bb = one ? 0 : 1 << (code & 7);
+        const int l = ((r & ba) ? 1 : 0) | ((r & bb) ? 2 : 0), r0 = r & ~(ba | bb);
+        auto at = [&](int c) { return ((r0 | ((c & 1) ? ba : 0) | ((c & 2) ? bb : 0)) << 4) | j; };
+        fx::Acc yr, yi;
+        auto term = [&](int c, int4 m) {
+            const fx::Real xr = Ur[cur][at(c)], xi = Ui[cur][at(c)];
+            fx::mac(yr, xr, m.x, m.y);
+            fx::mac(yr, xi, -m.z, -m.w);
+            fx::mac(yi, xi, m.x, m.y);
+            fx::mac(yi, xr, m.z, m.w);
+        };
+        int from = -1;
+        if (op == OP_DENSE1) {
+            for (int c = 0; c < 2; ++c) term(c, pay[2 * l + c]);
+        } else if (op == OP_REAL1) {
+            const int4 row = pay[l];
+            term(0, make_int4(row.x, row.y, 0, 0));
+            term(1, make_int4(row.z, row.w, 0, 0));
+        } else if (op == OP_DENSE2) {
+            for (int c = 0; c < 4; ++c) term(c, pay[4 * l + c]);
+        } else if (op == OP_DIAG1 || op == OP_DIAG2) {
+            term(l, pay[l]);
+        } else if (op == OP_X1) {
+            from = l ^ 1;
+        } else if (op == OP_CXA) {
+            from = (l & 1) ? l ^ 2 : l;
+        } else if (op == OP_CXB) {
+            from = (l & 2) ? l ^ 1 : l;
+        } else if (op == OP_SWAP2) {
+            from = ((l & 1) << 1) | (l >> 1);
+        } else {
+            from = reinterpret_cast<const int *>(pay)[l];
+        }
+        const int nx = cur ^ 1;
+        Ur[nx][e] = from >= 0 ? Ur[cur][at(from)] : fx::fin(yr);
+        Ui[nx][e] = from >= 0 ? Ui[cur][at(from)] : fx::fin(yi);
+        cur = nx;
+        __syncthreads();
+    }
+    // entries (k, n) = (2j, 2r), (2j + 1, 2r), (2j, 2r + 1), (2j + 1, 2r + 1) = re, -im, im, re
+    constexpr long long kBias = 0x0080808080808080ll;
+    const long long re = (fx::value(Ur[cur][e]) + 16) >> 5, im = (fx::value(Ui[cur][e]) + 16) >> 5;
+    unsigned char *b = prog + sg.b_off + (r >> 3) * (kOzBBytes / 2);
+#pragma unroll
+    for (int part = 0; part < 2; ++part) {
+        const int n = 2 * (r & 7) + part;  // output real within its half row
+        const unsigned long long lo = (unsigned long long)((part ? im : re) + kBias), hi = (unsigned long long)((part ? re : -im) + kBias);
+#pragma unroll
+        for (int d = 0; d < 8; ++d) {
+            const int row = 16 * d + n;  // N row of digit block d
+            __half2 v = __floats2half2_rn(0.f, 0.f);
+            if (d < 7) {
+                const int s = 8 * (6 - d);
+                v = __floats2half2_rn((float)((int)((lo >> s) & 255) - 128), (float)((int)((hi >> s) & 255) - 128));
+            }
+            *reinterpret_cast<__half2 *>(b + (row >> 3) * 512 + (j >> 2) * 128 + (row & 7) * 16 + (j & 3) * 4) = v;
+        }
+    }
+}
+
 }  // namespace
+
+void launch_compose_oz(const void *dev_groups, int ngroups, void *dev_prog, cudaStream_t st) {
+    if (ngroups <= 0) return;
+    k_compose_fx<<<ngroups, 256, 0, st>>>((const OzCompose *)dev_groups, (unsigned char *)dev_prog);
+    check_cuda(cudaGetLastError(), "compose kernel launch");
+}
 
 void launch_compose(const void *dev_segs, int nseg, const void *dev_gates, void *dev_prog, int *all_unitary, int r,
                     cudaStream_t st) {

@@ -161,6 +161,24 @@ bool fx_unitary(const double *m, int dim);
 void fx_pack(const double *m, int count, int32_t *entries);
 // Whether a gate only exchanges amplitudes or multiplies them by 1 or -1.
 bool exact_gate(const DevGate<double> &g);
+// Tensor-core programs of complex128 sections (block_oz.cuh): after the gate area, per register
+// group the B operand of its unitary in base-256 digits, two halves of 16 output reals, each 8 digit
+// blocks side by side (the last zero), K-major FP16.
+constexpr int kOzBBytes = 16384;
+// Addresses of a register group's rows in the chunk, loading and storing side: byte offsets of the 32
+// lanes, of the 16 row blocks (quarter | tile << 2) and of the 16 amplitudes, to be combined by
+// exclusive or (both the natural and the swizzled layout are linear).  Programs hold one per group
+// between the groups' DevSegs and the gate area.
+struct OzSeg {
+    uint32_t ld[64], st[64];
+};
+OzSeg oz_addresses(const HostSeg &seg, int width, bool natural_ld, bool natural_st);
+// One group to compose: gates [g0, g1) of the gate area at gates_off of the program, B at b_off.
+struct OzCompose {
+    uint32_t gates_off, b_off;
+    int32_t g0, g1;
+};
+void launch_compose_oz(const void *dev_groups, int ngroups, void *dev_prog, cudaStream_t st);
 // The gate area of a section's program: header table and payloads.  false (out untouched) when a
 // gate is not unitary.
 bool encode_fx(const std::vector<DevGate<double>> &gates, std::vector<unsigned char> &out);
@@ -280,6 +298,12 @@ void launch_block(int dtype, void *state, int n, int c, const void *dev_prog, in
 void launch_block_gather(int dtype, void *state, int n, const GatherLayout &lay, const void *dev_prog, int nseg,
                          int gate_bytes, bool fixed, int *dev_err, int seg_bits, cudaStream_t st,
                          uint64_t wait_ns = kDefaultWaitNs);
+// Register groups (at most) that one tensor-core sweep of a complex128 chunk of ce bits takes beside
+// gate_bytes of gate area; 0: the chunk cannot run there.
+int oz_max_segs(int ce, size_t gate_bytes);
+// Tensor-core blocking section of a complex128 state; `lay` null for a contiguous chunk of c bits.
+void launch_block_oz(void *state, int n, int c, const GatherLayout *lay, const void *dev_prog, int nseg, int gate_bytes,
+                     int *dev_err, cudaStream_t st, uint64_t wait_ns = kDefaultWaitNs);
 // Tensor-core blocking section (complex64, register groups of seg_bits = 3, 4 or 5 bits, B
 // operands in the program, tc_b_bytes(seg_bits) each); `lay` null for a contiguous chunk of c bits.
 void launch_block_tc(void *state, int n, int c, const GatherLayout *lay, const void *dev_prog, int nseg, int *dev_err,
