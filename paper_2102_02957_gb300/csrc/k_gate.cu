@@ -22,6 +22,15 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kUnroll = 2;
 
+// Gates of a circuit are launched with programmatic dependence (launch_after): a gate's blocks may be
+// placed while the last gate's are finishing, and wait here, before their first access to the state,
+// until it has completed and its writes are visible.  (480 gates on 16 qubits,
+// complex128: 1.97 ms without, 1.07 so.)
+__device__ __forceinline__ void after_last_gate() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 __device__ __forceinline__ int64_t insert0(int64_t x, int p) {
     const int64_t low = x & ((int64_t(1) << p) - 1);
     return ((x >> p) << (p + 1)) | low;
@@ -63,6 +72,7 @@ __device__ __forceinline__ void apply2(const T *m, T (&xr)[4], T (&xi)[4]) {
 
 // ---- complex64, 1 qubit, k == 0: each unit is one pair.
 __global__ void __launch_bounds__(kThreads) k_gate1_c64_lo(float4 *a, int64_t units, Mat1 M) {
+    after_last_gate();
     const int64_t g0 = (int64_t)blockIdx.x * kThreads * kUnroll + threadIdx.x;
     float4 A[kUnroll];
 #pragma unroll
@@ -79,6 +89,7 @@ __global__ void __launch_bounds__(kThreads) k_gate1_c64_lo(float4 *a, int64_t un
 // ---- complex64, 2 qubits, one of them is qubit 0: 2 units per group.  `zero_is_q0` says
 // whether the gate's q[0] (low local bit) is qubit 0.
 __global__ void __launch_bounds__(kThreads) k_gate2_c64_lo(float4 *a, int64_t groups, int po, int zero_is_q0, Mat2 M) {
+    after_last_gate();
     const int64_t g0 = (int64_t)blockIdx.x * kThreads * kUnroll + threadIdx.x;
     float4 U0[kUnroll], U1[kUnroll];
     int64_t base[kUnroll];
@@ -144,6 +155,7 @@ __device__ __forceinline__ uint4 quarter_turns(uint4 u, int turn) {
 
 template <int NA>
 __global__ void __launch_bounds__(kThreads) k_gate_move(uint4 *a, const __grid_constant__ GateArgs<NA, Moves> P) {
+    after_last_gate();
     const int64_t g0 = (int64_t)blockIdx.x * kThreads * kUnroll + threadIdx.x;
     uint4 U[kUnroll][NA];
     int64_t base[kUnroll];
@@ -185,6 +197,7 @@ __device__ __forceinline__ void apply_n(const float *m, float (&xr)[NA], float (
 
 template <int NA>
 __global__ void __launch_bounds__(kThreads) k_gate_c64(float4 *a, const __grid_constant__ GateArgs<NA, MatC64<NA>> P) {
+    after_last_gate();
     const int64_t g0 = (int64_t)blockIdx.x * kThreads * kUnroll + threadIdx.x;
     float4 U[kUnroll][NA];
     int64_t base[kUnroll];
@@ -277,6 +290,7 @@ __device__ __forceinline__ void apply_fx(const MatC128<NA> &M, double2 (&U)[NA])
 // over more CTAs.
 template <int NA, bool FX, int UN>
 __global__ void __launch_bounds__(kThreads) k_gate_c128(double2 *a, const __grid_constant__ GateArgs<NA, MatC128<NA>> P) {
+    after_last_gate();
     const int64_t g0 = (int64_t)blockIdx.x * kThreads * UN + threadIdx.x;
     double2 U[UN][NA];
     int64_t base[UN];
@@ -301,6 +315,7 @@ __global__ void __launch_bounds__(kThreads) k_gate_c128(double2 *a, const __grid
 
 // complex64 with n == 1: the whole state is one unit.
 __global__ void k_gate1_c64_single(float4 *a, Mat1 M) {
+    after_last_gate();
     float4 A = a[0];
     apply1(M.m, A.x, A.y, A.z, A.w);
     a[0] = A;
@@ -308,6 +323,20 @@ __global__ void k_gate1_c64_single(float4 *a, Mat1 M) {
 
 template <typename T>
 __global__ void k_set_one(T *a, uint64_t idx) { a[idx] = T{1, 0}; }
+
+template <typename... P, typename... A>
+void launch_after(void (*kernel)(P...), unsigned grid, unsigned block, cudaStream_t st, A... args) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    check_cuda(cudaLaunchKernelEx(&cfg, kernel, P(args)...), "per-gate kernel launch");
+}
 
 inline unsigned grid_for(int64_t groups, int unroll = kUnroll) {
     return (unsigned)((groups + (int64_t)kThreads * unroll - 1) / ((int64_t)kThreads * unroll));
@@ -381,14 +410,14 @@ void launch_move(void *state, const Touched &t, int units_log2, int nq, const in
         P.m.from[j] = t.from[j];
         P.m.turn[j] = t.turn[j];
     }
-    k_gate_move<NA><<<grid_for(P.groups), kThreads, 0, st>>>((uint4 *)state, P);
+    launch_after(k_gate_move<NA>, grid_for(P.groups), kThreads, st, (uint4 *)state, P);
 }
 
 template <int NA>
 void launch_c64(void *state, const Touched &t, int units_log2, int nq, const int *q, cudaStream_t st) {
     auto P = sweep_args<NA, MatC64<NA>>(t, units_log2, nq, q);
     for (int i = 0; i < 2 * NA * NA; ++i) P.m.m[i] = (float)t.m[i];
-    k_gate_c64<NA><<<grid_for(P.groups), kThreads, 0, st>>>((float4 *)state, P);
+    launch_after(k_gate_c64<NA>, grid_for(P.groups), kThreads, st, (float4 *)state, P);
 }
 
 template <int NA>
@@ -399,10 +428,10 @@ void launch_c128(void *state, const Touched &t, int n, int nq, const int *q, cud
     const bool small = P.groups <= (int64_t)num_sms() * kThreads * kUnroll;  // at most one CTA per SM
     if (fx_unitary(t.m, NA)) {
         fx_pack(t.m, NA * NA, P.m.e);
-        if (small) k_gate_c128<NA, true, 1><<<grid_for(P.groups, 1), kThreads, 0, st>>>(a, P);
-        else k_gate_c128<NA, true, kUnroll><<<grid_for(P.groups), kThreads, 0, st>>>(a, P);
+        if (small) launch_after(k_gate_c128<NA, true, 1>, grid_for(P.groups, 1), kThreads, st, a, P);
+        else launch_after(k_gate_c128<NA, true, kUnroll>, grid_for(P.groups), kThreads, st, a, P);
     } else {
-        k_gate_c128<NA, false, 1><<<grid_for(P.groups, 1), kThreads, 0, st>>>(a, P);
+        launch_after(k_gate_c128<NA, false, 1>, grid_for(P.groups, 1), kThreads, st, a, P);
     }
 }
 
@@ -415,19 +444,18 @@ void launch_gate(int dtype, void *state, int n, const sv_gate &g, cudaStream_t s
             Mat1 M;
             for (int i = 0; i < 8; ++i) M.m[i] = (float)g.m[i];
             if (n == 1) {
-                k_gate1_c64_single<<<1, 1, 0, st>>>(a, M);
+                launch_after(k_gate1_c64_single, 1, 1, st, a, M);
             } else {
                 const int64_t units = int64_t(1) << (n - 1);
-                k_gate1_c64_lo<<<grid_for(units), kThreads, 0, st>>>(a, units, M);
+                launch_after(k_gate1_c64_lo, grid_for(units), kThreads, st, a, units, M);
             }
         } else {
             Mat2 M;
             for (int i = 0; i < 32; ++i) M.m[i] = (float)g.m[i];
             const int other = g.q[0] == 0 ? g.q[1] : g.q[0];
             const int64_t groups = int64_t(1) << (n - 2);
-            k_gate2_c64_lo<<<grid_for(groups), kThreads, 0, st>>>(a, groups, other - 1, g.q[0] == 0 ? 1 : 0, M);
+            launch_after(k_gate2_c64_lo, grid_for(groups), kThreads, st, a, groups, other - 1, g.q[0] == 0 ? 1 : 0, M);
         }
-        check_cuda(cudaGetLastError(), "per-gate kernel launch");
         return;
     }
     const Touched t = touched_states(g);
@@ -448,7 +476,6 @@ void launch_gate(int dtype, void *state, int n, const sv_gate &g, cudaStream_t s
         else if (t.n == 2) launch_c128<2>(state, t, n, g.nq, q, st);
         else launch_c128<4>(state, t, n, g.nq, q, st);
     }
-    check_cuda(cudaGetLastError(), "per-gate kernel launch");
 }
 
 void launch_init_basis(int dtype, void *state, int n, uint64_t basis, cudaStream_t st) {
