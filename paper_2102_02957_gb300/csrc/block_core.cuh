@@ -425,7 +425,8 @@ __device__ __forceinline__ void tmem_ld_n(uint32_t taddr, uint32_t *o) {
 // with FP32 accumulation; the row's result is D[:, 0:K] + D[:, K:2K] = A_hi B_hi + A_lo B_hi +
 // A_hi B_lo (3xTF32).  Stacking B_hi and B_lo along N makes 2K/8 MMAs per tile instead of 3K/8:
 // an MMA of N <= 128 costs its issuing thread about the same time whatever N is.
-// NB (1 or 2) tiles are in flight per group; `mbar[k]` signals buffer k's MMAs' completion.
+// NB (1 or 2) tiles are in flight per group; `mbar[k]` signals buffer k's MMAs' completion.  With one
+// buffer the group takes tiles t0, t0 + ts, ... of the chunk (several groups may share it).
 //
 // RENORM: callers that cannot restore the state's norm once per circuit set RENORM: for a group
 // whose fused matrix is unitary (the int after the B operand is nonzero) each output row is
@@ -433,7 +434,7 @@ __device__ __forceinline__ void tmem_ld_n(uint32_t taddr, uint32_t *o) {
 template <int R, int NC, bool RENORM = false, int NB = 2>
 __device__ __forceinline__ bool run_segment_tc(uint32_t buf, uint32_t seg, uint32_t bhi, int ctid, const int *swz,
                                                int c, uint32_t tcol, int bar_id, uint64_t *mbar, uint32_t (&phase)[2],
-                                               volatile int *abort_flag, const uint64_t *wait_ns) {
+                                               volatile int *abort_flag, const uint64_t *wait_ns, int t0 = 0, int ts = 1) {
     using G = TcGeom<R>;
     constexpr int NA = G::NA, K = G::K;
     constexpr int CH = 8;  // amplitudes per TMEM access batch (16 columns): fewer live registers
@@ -601,7 +602,7 @@ __device__ __forceinline__ bool run_segment_tc(uint32_t buf, uint32_t seg, uint3
         }
         finish((T - 1) & 1, pb, ps, pn);
     } else {  // one tile buffer: tiles one after another
-        for (int t = 0; t < T; ++t) {
+        for (int t = t0; t < T; t += ts) {
             if (!stage(t, 0, pb, ps, pn)) return false;
             finish(0, pb, ps, pn);
         }

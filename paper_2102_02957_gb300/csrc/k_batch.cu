@@ -18,8 +18,6 @@
 namespace sv {
 namespace {
 
-// Threads per CTA: 256 for SIMT-only batches, 128 (one 128-row tensor-core tile) when sections
-// run on the tensor cores.
 constexpr int RB = 4;     // register-group width
 
 __device__ __forceinline__ int ld_acquire(const int *p) {
@@ -65,17 +63,19 @@ __device__ __forceinline__ void copy_prog(unsigned char *dst, const unsigned cha
 
 // A CTA holds POOLS independent workers ("pools") of NT threads; each drains the queue on its
 // own with its own chunk and program buffers and its own named barrier.  SIMT batches: one pool
-// of 256 threads, two CTAs per SM.  Tensor-core batches: pools of 128 threads (one 128-row tile
-// each) in one CTA per SM sharing its 512 tensor-memory columns: two pools of two tile buffers
-// for chunks of up to 13 bits, or three of one buffer for chunks of up to 12 bits (more
-// independent tile chains in flight; the smaller chunk buffers make room for the third).
+// of 256 threads, two CTAs per SM.  Tensor-core batches: one CTA per SM whose pools share its 512
+// tensor-memory columns, a 128-row tile buffer for every 128 threads: three pools of 128 for chunks of
+// up to 12 bits (more independent tile chains in flight; the smaller chunk buffers make room for the
+// third), else two pools of 256, whose two halves take alternate tiles of their chunk.  (Pools
+// of 128 with two buffers each left the SM 8 warps: 80 noisy trajectories of 12 to 22 qubits and 16
+// ansatz sets took 20.5 ms, now 18.3.)
 template <int NT, int POOLS>
 __device__ __forceinline__ void pool_sync(int p) {
     if constexpr (POOLS == 1) __syncthreads();
     else ptx::named_bar_sync(1 + p, NT);
 }
 
-template <int NT, int POOLS, int NB>
+template <int NT, int POOLS>
 __global__ void __launch_bounds__(NT * POOLS, POOLS >= 2 ? 1 : 2) k_batch(const BatchOp *__restrict__ ops, int nops,
                                                       const unsigned char *__restrict__ progs, float2 *const *amps,
                                                       int *ops_done, int *chunks_done, unsigned long long *next,
@@ -118,8 +118,10 @@ __global__ void __launch_bounds__(NT * POOLS, POOLS >= 2 ? 1 : 2) k_batch(const 
     }
     __syncthreads();
     if constexpr (TC) ptx::tc_fence_after();
-    static_assert(!TC || POOLS * NB * TcGeom<4>::COLS <= 512, "tile buffers exceed tensor memory");
-    const uint32_t tmem_pool = TC ? s_tmem + (uint32_t)(p * NB * TcGeom<4>::COLS) : 0u;
+    constexpr int kSubs = NT / 128;  // tensor-core groups per pool, each with a tile buffer
+    static_assert(!TC || POOLS * kSubs * TcGeom<4>::COLS <= 512, "tile buffers exceed tensor memory");
+    const int sub = ctid >> 7;
+    const uint32_t tmem_sub = TC ? s_tmem + (uint32_t)((p * kSubs + sub) * TcGeom<4>::COLS) : 0u;
     uint32_t mma_phase[2] = {0, 0};
     BatchOp &op = s_bop[p];
     while (true) {
@@ -191,23 +193,25 @@ __global__ void __launch_bounds__(NT * POOLS, POOLS >= 2 ? 1 : 2) k_batch(const 
             const uint32_t seg_s = ptx::smem_addr(sprog) + 16u;
             const uint32_t body_s = seg_s + (uint32_t)((hd.x * sizeof(DevSeg) + 15) & ~size_t(15));
             for (int si = 0; si < hd.x; ++si) {
+                bool failed = false;
                 if (op.tc) {
                     // fused group on the tensor cores, unbiased per row (the batch has no
-                    // per-circuit norm restoration); the return value is uniform over the pool
-                    if constexpr (TC) {
-                        if (!run_segment_tc<4, NT, true, NB>(chunk_s, seg_s + (uint32_t)(si * sizeof(DevSeg)),
-                                                      body_s + (uint32_t)(si * kBatchTcGroupBytes), ctid, c_swz64, ce,
-                                                      tmem_pool, 1 + p, s_mma[p], mma_phase, &s_tc_abort[p],
-                                                      &s_wait_ns)) {
-                            tc_failed = true;
-                            break;
-                        }
-                    }
+                    // per-circuit norm restoration)
+                    if constexpr (TC)
+                        failed = !run_segment_tc<4, 128, true, 1>(
+                            chunk_s, seg_s + (uint32_t)(si * sizeof(DevSeg)), body_s + (uint32_t)(si * kBatchTcGroupBytes),
+                            ctid & 127, c_swz64, ce, tmem_sub, 1 + POOLS + p * kSubs + sub, &s_mma[p][sub], mma_phase,
+                            &s_tc_abort[p], &s_wait_ns, sub, kSubs);
                 } else {
                     run_segment<float, RB, NT, 1>(chunk_s, seg_s + (uint32_t)(si * sizeof(DevSeg)), body_s, ctid,
                                                   c_swz64, ce, obase);
                 }
-                pool_sync<NT, POOLS>(p);
+                if constexpr (TC) {  // the pool's halves leave together
+                    tc_failed = ptx::named_bar_or(1 + p, NT, failed);
+                    if (tc_failed) break;
+                } else {
+                    pool_sync<NT, POOLS>(p);
+                }
             }
             poff += (uint32_t)hd.z;
         }
@@ -248,10 +252,10 @@ void launch_batch(const void *dev_ops, int nops, const void *dev_progs, void *co
                   int *dev_chunks_done, unsigned long long *dev_next, int64_t total, int from_zero, int use_tc,
                   int *dev_err, cudaStream_t st, uint64_t wait_ns, int stall_state) {
     const int prog_cap = use_tc == 2 ? kBatchMaxProgBytesTc3 : use_tc ? kBatchMaxProgBytesTc : kBatchMaxProgBytes;
-    const int pools = use_tc == 2 ? 3 : use_tc ? 2 : 1, nt = use_tc ? 128 : 256;
+    const int pools = use_tc == 2 ? 3 : use_tc ? 2 : 1, nt = use_tc == 2 ? 128 : 256;
     const int cap_bits = use_tc == 2 ? kBatchTc3ChunkBits : kBatchMaxChunkBits;
     const size_t smem = (size_t)pools * ((size_t(1) << cap_bits) * sizeof(float2) + (size_t)prog_cap);
-    auto kern = use_tc == 2 ? k_batch<128, 3, 1> : use_tc ? k_batch<128, 2, 2> : k_batch<256, 1, 1>;
+    auto kern = use_tc == 2 ? k_batch<128, 3> : use_tc ? k_batch<256, 2> : k_batch<256, 1>;
     check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
                "cudaFuncSetAttribute(batch)");
     int per_sm = 0;
