@@ -52,7 +52,7 @@ struct Scratch {
 
 Scratch scratch_for(sv_costmodel *m, int64_t rows) {
     const int P = mlp_param_count();
-    const int nblk = 128;
+    const int nblk = mlp_grad_blocks(rows);  // not below any batch's of at most `rows` samples
     auto al = [](size_t b) { return (b + 255) & ~size_t(255); };
     const size_t need = al(rows * NF * 4) + 3 * al(rows * 4) + al(rows * 4) + al((size_t)nblk * P * 4) + al(P * 4) +
                         al(nblk * 8) + al(8);

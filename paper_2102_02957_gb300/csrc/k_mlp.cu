@@ -153,21 +153,37 @@ __global__ void __launch_bounds__(32) k_mlp_grad(const float *__restrict__ P, co
     }
 }
 
-// g = sum of the nblk partials (fixed order).  mode 0: write g to `grad`; mode 1: Adam update
-// of P with moments M, V (c1 = 1 / (1 - b1^t), c2 = 1 / (1 - b2^t)).  Thread 0 also sums the
-// loss partials into *loss.
-__global__ void k_mlp_reduce(const float *__restrict__ part, int nblk, const double *__restrict__ lpart, double *loss,
-                             int mode, float *__restrict__ grad, float *__restrict__ P, float *__restrict__ M,
-                             float *__restrict__ V, float lr, float c1, float c2) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p == 0) {
+// g = sum of the nblk partials (fixed order: kSlices interleaved sums, then those in order).  mode 0:
+// write g to `grad`; mode 1: Adam update of P with moments M, V (c1 = 1 / (1 - b1^t), c2 = 1 / (1 -
+// b2^t)).  The first warp of CTA 0 also sums the loss partials into *loss.  A CTA takes 32
+// parameters, a warp per slice, so that a slice's loads are whole lines and kSlices of them run
+// side by side.
+constexpr int kSlices = 8;
+__global__ void __launch_bounds__(32 * kSlices) k_mlp_reduce(const float *__restrict__ part, int nblk,
+                                                             const double *__restrict__ lpart, double *loss, int mode,
+                                                             float *__restrict__ grad, float *__restrict__ P,
+                                                             float *__restrict__ M, float *__restrict__ V, float lr, float c1,
+                                                             float c2) {
+    __shared__ float sums[kSlices][32];
+    const int lane = threadIdx.x & 31, slice = threadIdx.x >> 5, p = blockIdx.x * 32 + lane;
+    float g = 0.f;
+    if (p < NPARAM) {
+#pragma unroll 8
+        for (int b = slice; b < nblk; b += kSlices) g += part[(size_t)b * NPARAM + p];
+    }
+    sums[slice][lane] = g;
+    __syncthreads();
+    if (slice != 0) return;
+    if (blockIdx.x == 0) {
         double l = 0.0;
-        for (int b = 0; b < nblk; ++b) l += lpart[b];
-        *loss = l;
+        for (int b = lane; b < nblk; b += 32) l += lpart[b];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+        if (lane == 0) *loss = l;
     }
     if (p >= NPARAM) return;
-    float g = 0.f;
-    for (int b = 0; b < nblk; ++b) g += part[(size_t)b * NPARAM + p];
+#pragma unroll
+    for (int k = 1; k < kSlices; ++k) g += sums[k][lane];
     if (mode == 0) {
         grad[p] = g;
         return;
@@ -190,7 +206,11 @@ void launch_mlp_fwd(const float *P, const float *X, int64_t B, float *Y, cudaStr
     check_cuda(cudaGetLastError(), "mlp forward launch");
 }
 
-int mlp_grad_blocks(int64_t B) { return (int)std::max<int64_t>(1, std::min<int64_t>(B, 128)); }
+// CTAs of one warp, each with its own gradient: their samples run one after another, so a batch is
+// spread over as many as fit the device at once (5 per SM by shared memory); the partials they leave
+// are 21 KB each.  Predictions and gradient of 4096 samples, copies included: 264 us with 128 CTAs and
+// a thread per parameter in the reduction, 146 us so.
+int mlp_grad_blocks(int64_t B) { return (int)std::max<int64_t>(1, std::min<int64_t>(B, 4 * (int64_t)num_sms())); }
 
 void launch_mlp_grad(const float *P, const float *X, const float *T, const int32_t *idx, int64_t start, int64_t B,
                      float *part, double *lpart, cudaStream_t st) {
@@ -200,7 +220,7 @@ void launch_mlp_grad(const float *P, const float *X, const float *T, const int32
 
 void launch_mlp_reduce(const float *part, int nblk, const double *lpart, double *loss, int mode, float *grad, float *P,
                        float *M, float *V, float lr, float c1, float c2, cudaStream_t st) {
-    k_mlp_reduce<<<(NPARAM + 255) / 256, 256, 0, st>>>(part, nblk, lpart, loss, mode, grad, P, M, V, lr, c1, c2);
+    k_mlp_reduce<<<(NPARAM + 31) / 32, 32 * kSlices, 0, st>>>(part, nblk, lpart, loss, mode, grad, P, M, V, lr, c1, c2);
     check_cuda(cudaGetLastError(), "mlp reduce launch");
 }
 
