@@ -364,13 +364,25 @@ static void build_programs(const sv_plan *plan, const sv_gate *gates, int seg_bi
             }
             if (dgates.size() > 32767) fail(SV_ERR_UNSUPPORTED, "too many gates in one blocking section");
             d.g1 = (int16_t)dgates.size();
+            if constexpr (sizeof(T) == 8) gather_outside_diagonals(dgates, (size_t)d.g0);
             if constexpr (sizeof(T) == 8)
                 if (std::all_of(dgates.begin() + d.g0, dgates.end(), exact_gate)) d.flags |= kSegRaw;
             dsegs.push_back(d);
         }
-        // complex128: fixed-point gates where every gate is unitary (their area is never the larger)
+        // complex128: fixed-point gates where every gate is unitary (their area is never the larger);
+        // merged diagonals take some more room, and give way where a consumer group would lose its chunk
         std::vector<unsigned char> area;
-        if constexpr (sizeof(T) == 8) bp.fixed = encode_fx(dgates, area);
+        if constexpr (sizeof(T) == 8) {
+            std::vector<int> starts;
+            for (const DevSeg &d : dsegs) starts.push_back(d.g0);
+            bp.fixed = encode_fx(dgates, starts, false, area);
+            std::vector<unsigned char> merged;
+            if (bp.fixed && std::any_of(dgates.begin(), dgates.end(), [](const DevGate<T> &g) { return g.op == OP_DIAGX; }) &&
+                encode_fx(dgates, starts, true, merged) &&
+                fx_buffers(width, (int)dsegs.size(), merged.size()) >=
+                    std::min(kFxGroups, fx_buffers(width, (int)dsegs.size(), area.size())))
+                area.swap(merged);
+        }
         if constexpr (sizeof(T) == 8) {
             int per = 0;  // groups per sweep
             if (oz && bp.fixed && std::any_of(dsegs.begin(), dsegs.end(), [](const DevSeg &d) { return !(d.flags & kSegRaw); }) &&
@@ -381,7 +393,7 @@ static void build_programs(const sv_plan *plan, const sv_gate *gates, int seg_bi
                 for (int w = 0; w < sweeps; ++w) {
                     const int s0 = (int)((int64_t)nseg * w / sweeps), s1 = (int)((int64_t)nseg * (w + 1) / sweeps);
                     const int g0 = dsegs[(size_t)s0].g0, g1 = dsegs[(size_t)s1 - 1].g1;
-                    encode_fx(std::vector<DevGate<T>>(dgates.begin() + g0, dgates.begin() + g1), area);
+                    encode_fx(std::vector<DevGate<T>>(dgates.begin() + g0, dgates.begin() + g1), {}, false, area);
                     align(256);
                     bp.oz = true;
                     bp.off = host.size();

@@ -10,13 +10,15 @@
 // registers a thread allow no more, and 3 x 128 threads of 128 registers spill (217 ms against 166
 // for the first line below).  Measured against FP64 register groups, n qubits, 12-bit chunks:
 //   27, 8 random layers (12 sections, 44 groups)       417 -> 169 ms
-//   28, QFT with diagonals outside the chunk           393 -> 239 ms
+//   28, QFT with diagonals outside the chunk           393 -> 239 ms, with merged runs 160 ms
 //   25, quantum volume of 10 layers, gathered chunks   108 -> 38.6 ms
 //
 // The section's gate area is a table of 16-byte headers {op, payload offset, outside bits, code},
 // then the payloads (encode_fx writes them):
 //   OP_DENSE1 / OP_DENSE2  4 / 16 entries {re h, re l, im h, im l}     OP_REAL1  4 x {h, l}
 //   OP_DIAG1 / OP_DIAG2    2 / 4 entries   OP_DIAGX  2 or 4 OP_DIAG1   OP_PERM2  4 ints
+//   OP_DIAGRUN  the run's gates and 16 entries per consumer group, filled per chunk (fx_merge): a
+//   QFT section has up to 16 controlled phases from outside the chunk on each of its qubits
 #pragma once
 #include "block_core.cuh"
 #include "fixed64.cuh"
@@ -203,8 +205,12 @@ __device__ __forceinline__ void fx_two(int op, FxGroup<NA> &v, uint32_t m, bool 
     else fx_perm2<NA, A, B>(v, m);
 }
 
+__device__ __forceinline__ void fx_diag16(FxGroup<16> &v, uint32_t ma);
+
 __device__ __forceinline__ void fx_apply(int op, int code, uint32_t m, FxGroup<16> &v, bool raw) {
-    if (op == OP_DENSE1 || op == OP_REAL1 || op == OP_DIAG1 || op == OP_X1) {
+    if (op == OP_DIAGRUN) {
+        fx_diag16(v, m);
+    } else if (op == OP_DENSE1 || op == OP_REAL1 || op == OP_DIAG1 || op == OP_X1) {
         switch (code) {
             case 0: fx_one<16, 0>(op, v, m, raw); break;
             case 1: fx_one<16, 1>(op, v, m, raw); break;
@@ -223,23 +229,77 @@ __device__ __forceinline__ void fx_apply(int op, int code, uint32_t m, FxGroup<1
     }
 }
 
+// Diagonal of all 16 amplitudes (a merged run).
+__device__ __forceinline__ void fx_diag16(FxGroup<16> &v, uint32_t ma) {
+#pragma unroll
+    for (int x = 0; x < 16; ++x) {
+        FxEntry d;  // rewritten for every chunk: not a pure load like the program's
+        asm volatile("ld.shared.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(d.rh), "=r"(d.rl), "=r"(d.ih), "=r"(d.il) : "r"(ma + 16u * x));
+        if (d.rh == fx::kOne && d.rl == 0 && d.ih == 0 && d.il == 0) continue;
+        fx::Acc yr, yi;
+        fx_cmac(yr, yi, d, v.re[x], v.im[x]);
+        v.re[x] = fx::fin(yr);
+        v.im[x] = fx::fin(yi);
+    }
+}
+
 // Payload of a gate of group [g0, g1) once its outside bits are read off the chunk's origin.
 struct FxGate {
     int op, code;
     uint32_t m;
+    int more;  // further headers that belong to it
 };
-__device__ __forceinline__ FxGate fx_gate(uint32_t gates, int gi, int64_t origin) {
+__device__ __forceinline__ uint32_t fx_variant(int outside, int64_t origin) {
+    const int e0 = outside & 0xFF, e1 = (outside >> 8) & 0xFF;
+    int v = (int)((origin >> e0) & 1);
+    if (e1 != 0xFF) v |= (int)((origin >> e1) & 1) << 1;
+    return (uint32_t)(32 * v);
+}
+__device__ __forceinline__ FxGate fx_gate(uint32_t gates, int gi, int64_t origin, int cg) {
     int op, off, rb, code;
     ldc_i4(gates + 16u * (uint32_t)gi, op, off, rb, code);
     uint32_t m = gates + (uint32_t)off;
+    int more = 0;
     if (op == OP_DIAGX) {
-        const int e0 = rb & 0xFF, e1 = (rb >> 8) & 0xFF;
-        int v = (int)((origin >> e0) & 1);
-        if (e1 != 0xFF) v |= (int)((origin >> e1) & 1) << 1;
-        m += (uint32_t)(32 * v);
+        m += fx_variant(rb, origin);
         op = OP_DIAG1;
+    } else if (op == OP_DIAGRUN) {
+        more = rb - 1;
+        m += (uint32_t)(16 + 16 * rb + 256 * cg);
     }
-    return FxGate{op, code, m};
+    return FxGate{op, code, m, more};
+}
+
+// Entries of the merged runs of gates [g0, g1) for this chunk: thread x < 16 of a warp multiplies
+// entry x over the run's gates, a warp per run in turn (products in the scale 2^59 of fixed64.cuh).
+__device__ __forceinline__ void fx_merge(uint32_t gates, int g0, int g1, int64_t origin, int cg, int ctid, int nwarps) {
+    const int lane = ctid & 31;
+    int turn = 0;
+    for (int gi = g0; gi < g1; ++gi) {
+        int op, off, count, code;
+        ldc_i4(gates + 16u * (uint32_t)gi, op, off, count, code);
+        if (op != OP_DIAGRUN) continue;
+        if (turn++ % nwarps == (ctid >> 5) && lane < 16) {
+            const uint32_t list = gates + (uint32_t)off + 16;
+            fx::Real pr = fx::pack(1ll << 59), pi{0, 0};
+            for (int k = 0; k < count; ++k) {
+                int goff, outside, bit, unused;
+                ldc_i4(list + 16u * (uint32_t)k, goff, outside, bit, unused);
+                const FxEntry d = lds_entry(gates + (uint32_t)goff + fx_variant(outside, origin) + 16u * (uint32_t)((lane >> bit) & 1));
+                fx::Acc yr, yi;
+                fx_cmac(yr, yi, d, pr, pi);
+                pr = fx::fin(yr);
+                pi = fx::fin(yi);
+            }
+            fx::Real er = fx::pack(fx::value(pr) * 4), ei = fx::pack(fx::value(pi) * 4);  // entries' scale 2^61
+            er.l += er.l == (int)0x80000000;  // keep -l representable
+            ei.l += ei.l == (int)0x80000000;
+            asm volatile("st.shared.v4.s32 [%0], {%1, %2, %3, %4};" ::"r"(list + (uint32_t)(16 * count + 256 * cg + 16 * lane)),
+                         "r"(er.h), "r"(er.l), "r"(ei.h), "r"(ei.l)
+                         : "memory");
+        }
+        gi += count - 1;
+    }
 }
 
 __device__ __forceinline__ double fx_entry_value(uint32_t a) {
@@ -250,9 +310,20 @@ __device__ __forceinline__ double fx_entry_value(uint32_t a) {
 // The group in FP64, for components outside the fixed-point range (infinities, NaN, magnitudes
 // near the ends of the exponent range).  Not a hot path: one copy of the code, amplitudes in
 // local memory.
-__device__ __noinline__ void fx_group_fp64(double *re, double *im, uint32_t gates, int g0, int g1, int64_t origin) {
+__device__ __noinline__ void fx_group_fp64(double *re, double *im, uint32_t gates, int g0, int g1, int64_t origin, int cg) {
     for (int gi = g0; gi < g1; ++gi) {
-        const FxGate g = fx_gate(gates, gi, origin);
+        const FxGate g = fx_gate(gates, gi, origin, cg);
+        if (g.op == OP_DIAGRUN) {
+            gi += g.more;
+            for (int x = 0; x < 16; ++x) {
+                const double dr = fx_entry_value(g.m + 16 * x), di = fx_entry_value(g.m + 16 * x + 8);
+                if (dr == 1.0 && di == 0.0) continue;
+                const double a = re[x], b = im[x];
+                re[x] = dr * a - di * b;
+                im[x] = dr * b + di * a;
+            }
+            continue;
+        }
         const bool one = g.op == OP_DENSE1 || g.op == OP_REAL1 || g.op == OP_DIAG1 || g.op == OP_X1;
         const int dim = one ? 2 : 4;
         const int ba = one ? 1 << g.code : 1 << (g.code >> 3), bb = one ? 0 : 1 << (g.code & 7);
@@ -304,7 +375,7 @@ __device__ __noinline__ void fx_group_fp64(double *re, double *im, uint32_t gate
 // One register group of 4 bits over the chunk in shared memory (see run_segment for the addressing).
 template <int NC>
 __device__ __forceinline__ void run_segment_fx(uint32_t buf, uint32_t seg, uint32_t gates, int ctid, const int *swz,
-                                               int c, int64_t origin) {
+                                               int c, int64_t origin, int cg, int bar_id) {
     constexpr int R = 4, NA = 1 << R;
     int po[R], pf[R];
 #pragma unroll
@@ -323,6 +394,12 @@ __device__ __forceinline__ void run_segment_fx(uint32_t buf, uint32_t seg, uint3
     const int nrest = lds_s8(seg + 13), flags = lds_s8(seg + 14);
     const int g0 = lds_s16(seg + 32), g1 = lds_s16(seg + 34);
     const int G = 1 << (c - R);
+    bool merged = false;  // uniform: whether the group has merged runs
+    for (int gi = g0; gi < g1; ++gi) merged = merged || lds_s32(gates + 16u * (uint32_t)gi) == OP_DIAGRUN;
+    if (merged) {
+        fx_merge(gates, g0, g1, origin, cg, ctid, NC / 32);
+        ptx::named_bar_sync(bar_id, NC);
+    }
     uint32_t ld_step[R], st_step[R];
 #pragma unroll
     for (int j = 0; j < R; ++j) {
@@ -359,7 +436,7 @@ __device__ __forceinline__ void run_segment_fx(uint32_t buf, uint32_t seg, uint3
             double lr[NA], li[NA];
 #pragma unroll
             for (int b = 0; b < NA; ++b) { lr[b] = dr[b]; li[b] = di[b]; }
-            fx_group_fp64(lr, li, gates, g0, g1, origin);
+            fx_group_fp64(lr, li, gates, g0, g1, origin, cg);
 #pragma unroll
             for (int b = 0; b < NA; ++b) { dr[b] = lr[b]; di[b] = li[b]; }
         } else {
@@ -371,8 +448,9 @@ __device__ __forceinline__ void run_segment_fx(uint32_t buf, uint32_t seg, uint3
                 v.im[b] = raw ? fx::from_bits(di[b]) : fx::from_double(di[b], E);
             }
             for (int gi = g0; gi < g1; ++gi) {
-                const FxGate g = fx_gate(gates, gi, origin);
+                const FxGate g = fx_gate(gates, gi, origin, cg);
                 fx_apply(g.op, g.code, g.m, v, raw);
+                gi += g.more;
             }
 #pragma unroll
             for (int b = 0; b < NA; ++b) {

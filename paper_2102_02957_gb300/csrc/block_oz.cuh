@@ -177,7 +177,7 @@ __device__ __noinline__ void oz_chunk_fp64(uint32_t buf, uint32_t segs, uint32_t
                     if (pass == 0) SM<double>::ld(buf + 16u * (uint32_t)slot, re[x], im[x]);
                     else SM<double>::st(buf + 16u * (uint32_t)slot, re[x], im[x]);
                 }
-                if (pass == 0) fx_group_fp64(re, im, gates, g0, g1, origin);
+                if (pass == 0) fx_group_fp64(re, im, gates, g0, g1, origin, 0);
             }
         }
         ptx::named_bar_sync(bar_id, NC);

@@ -1,4 +1,5 @@
 // Host side of the block fixed-point path (fixed64.cuh): which gates it takes and their payloads.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 
@@ -49,7 +50,33 @@ bool exact_gate(const DevGate<double> &g) {
     return true;
 }
 
-bool encode_fx(const std::vector<DevGate<double>> &gates, std::vector<unsigned char> &out) {
+void gather_outside_diagonals(std::vector<DevGate<double>> &gates, size_t first) {
+    std::vector<DevGate<double>> out, pending;
+    for (size_t i = first; i < gates.size(); ++i) {
+        const DevGate<double> &g = gates[i];
+        if (g.op == OP_DIAGX) {
+            pending.push_back(g);
+            continue;
+        }
+        if (g.op != OP_DIAG1 && g.op != OP_DIAG2) {
+            const bool one = g.op == OP_DENSE1 || g.op == OP_X1;
+            std::vector<DevGate<double>> keep;
+            for (const DevGate<double> &d : pending) {
+                bool phase = true;  // equal entries in every variant
+                for (int v = 0; v < 4; ++v) phase = phase && d.m[4 * v] == d.m[4 * v + 2] && d.m[4 * v + 1] == d.m[4 * v + 3];
+                if (!phase && (d.a == g.a || (!one && d.a == g.b))) out.push_back(d);
+                else keep.push_back(d);
+            }
+            pending.swap(keep);
+        }
+        out.push_back(g);
+    }
+    out.insert(out.end(), pending.begin(), pending.end());
+    std::copy(out.begin(), out.end(), gates.begin() + (ptrdiff_t)first);
+}
+
+bool encode_fx(const std::vector<DevGate<double>> &gates, const std::vector<int> &group_starts, bool merge,
+               std::vector<unsigned char> &out) {
     std::vector<unsigned char> body;
     std::vector<int32_t> head;
     const size_t table = gates.size() * 16;
@@ -107,6 +134,29 @@ bool encode_fx(const std::vector<DevGate<double>> &gates, std::vector<unsigned c
             default: break;  // register exchanges: no payload
         }
         head.insert(head.end(), {op, (int32_t)off, g.b, g.code});
+    }
+    // merged runs: {count, 0, 0, 0}, {payload offset, outside bits, code, 0} per gate, then each
+    // consumer group's 16 entries; the run's first header points here
+    for (size_t i = 0; merge && i < gates.size();) {
+        size_t j = i;
+        while (j < gates.size() && gates[j].op == OP_DIAGX &&
+               (j == i || std::find(group_starts.begin(), group_starts.end(), (int)j) == group_starts.end()))
+            ++j;
+        // runs of signs alone stay apart: groups that only exchange and flip signs work on doubles' words
+        if (j - i >= 2 && !std::all_of(gates.begin() + (ptrdiff_t)i, gates.begin() + (ptrdiff_t)j, exact_gate)) {
+            const size_t off = table + body.size();
+            const int32_t count[4] = {(int32_t)(j - i), 0, 0, 0};
+            put(count, sizeof(count));
+            for (size_t k = i; k < j; ++k) {
+                const int32_t row[4] = {head[4 * k + 1], head[4 * k + 2], head[4 * k + 3], 0};
+                put(row, sizeof(row));
+            }
+            body.resize(body.size() + (size_t)kFxGroups * 256, 0);
+            head[4 * i] = OP_DIAGRUN;
+            head[4 * i + 1] = (int32_t)off;
+            head[4 * i + 2] = (int32_t)(j - i);
+        }
+        i = std::max(j, i + 1);
     }
     const unsigned char *h = reinterpret_cast<const unsigned char *>(head.data());
     out.assign(h, h + table);

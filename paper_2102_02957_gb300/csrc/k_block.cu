@@ -179,6 +179,7 @@ __device__ __forceinline__ void store_chunks(T2 *state, int c, int64_t count, in
 // Register-group engines of a section kernel besides the SIMT one (run_segment).
 enum : int { ENG_NONE = 0, ENG_FX = 1, ENG_OZ = 2 };
 
+static_assert(kFxGroups == 2, "scratch for merged diagonals");
 constexpr int CG2 = 2;  // consumer groups per CTA (default)
 
 // G consumer groups per CTA; tensor-core groups keep NB tile buffers each
@@ -321,7 +322,7 @@ __device__ __forceinline__ void block_body(typename V2<T>::type *__restrict__ st
                                                       swz, c, tmem_base + (uint32_t)(cg * NB * TcGeom<R>::COLS), bar_id,
                                                       &mma_bar[2 * cg], mma_phase, abort_flag, &s_wait_ns);
             } else if constexpr (ENG == ENG_FX) {
-                run_segment_fx<NC>(ptx::smem_addr(buf), seg_addr, ptx::smem_addr(gates), ctid, swz, c, origin);
+                run_segment_fx<NC>(ptx::smem_addr(buf), seg_addr, ptx::smem_addr(gates), ctid, swz, c, origin, cg, bar_id);
             } else if constexpr (ENG == ENG_NONE) {
                 run_segment<T, R, NC, KU>(ptx::smem_addr(buf), seg_addr, ptx::smem_addr(gates), ctid, swz, c, origin);
             }
@@ -546,6 +547,13 @@ void launch_block_tc(void *state, int n, int c, const GatherLayout *lay, const v
         launch_typed<float, 4, 128, 1, true, 4, 1>(state, n, ce, dev_prog, nseg, 0, dev_err, st, m, ga, wait_ns);
     else
         launch_typed<float, 4, 128, 1, true, 2, 2>(state, n, ce, dev_prog, nseg, 0, dev_err, st, m, ga, wait_ns);
+}
+
+int fx_buffers(int ce, int nseg, size_t gate_bytes) {
+    const size_t chunk = size_t(16) << ce, fixed = nseg * sizeof(DevSeg) + gate_bytes + 256;
+    int n = 3;
+    while (n > 0 && n * chunk + fixed > kMaxBlockSmem) --n;
+    return n;
 }
 
 // Shared memory beside the chunk buffers: barriers and flags (launch_typed's `extra`), the groups'

@@ -106,6 +106,7 @@ enum : int32_t {
     OP_SWAP2 = 7,  // exchange 1 <-> 2
     OP_X1 = 8,     // 1-qubit bit flip
     OP_REAL1 = 10, // dense 1-qubit gate with real entries (fixed-point programs only)
+    OP_DIAGRUN = 11, // the next `b` gates, all OP_DIAGX, as one 16-entry diagonal per chunk (likewise)
     OP_DIAGX = 9   // diagonal gate with qubits outside the chunk: b = e0 | e1 << 8 (state bits,
                    // 0xFF = none); variant v = bit e0 + 2 bit e1 of the chunk's origin selects
                    // m[4v..4v+3], a diagonal (d0, d1) on register bit a (a phase: d0 = d1, a = 0)
@@ -179,9 +180,16 @@ struct OzCompose {
     int32_t g0, g1;
 };
 void launch_compose_oz(const void *dev_groups, int ngroups, void *dev_prog, cudaStream_t st);
+// Moves the OP_DIAGX gates of a register group's list as far back as they commute (a diagonal on a
+// register bit passes every gate that is diagonal or acts on other bits, a phase every gate), so
+// that they meet in few runs.
+void gather_outside_diagonals(std::vector<DevGate<double>> &gates, size_t first);
 // The gate area of a section's program: header table and payloads.  false (out untouched) when a
-// gate is not unitary.
-bool encode_fx(const std::vector<DevGate<double>> &gates, std::vector<unsigned char> &out);
+// gate is not unitary.  Runs of OP_DIAGX gates within a group (group_starts: each group's first gate)
+// are merged where `merge` is set.
+bool encode_fx(const std::vector<DevGate<double>> &gates, const std::vector<int> &group_starts, bool merge,
+               std::vector<unsigned char> &out);
+constexpr int kFxGroups = 2;  // consumer groups of the integer-pipe kernel, each with its own merged diagonals
 
 // Gathered chunk: the state is viewed as a tensor of rank <= 5 whose dimension d covers the
 // index bits [s[d], s[d+1]); each dimension starts with a run of chunk bits (its box, at most
@@ -298,6 +306,8 @@ void launch_block(int dtype, void *state, int n, int c, const void *dev_prog, in
 void launch_block_gather(int dtype, void *state, int n, const GatherLayout &lay, const void *dev_prog, int nseg,
                          int gate_bytes, bool fixed, int *dev_err, int seg_bits, cudaStream_t st,
                          uint64_t wait_ns = kDefaultWaitNs);
+// Chunk buffers that an integer-pipe section of 2^ce amplitudes gets beside its program.
+int fx_buffers(int ce, int nseg, size_t gate_bytes);
 // Register groups (at most) that one tensor-core sweep of a complex128 chunk of ce bits takes beside
 // gate_bytes of gate area; 0: the chunk cannot run there.
 int oz_max_segs(int ce, size_t gate_bytes);

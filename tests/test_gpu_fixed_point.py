@@ -93,3 +93,31 @@ def test_non_unitary_gates_stay_fp64(sv, n, opts):
     # norms grow by at most ||big|| ||one||; 8 products of 2^-53 each per gate, on both sides
     scale = np.linalg.norm(big, 2) * np.linalg.norm(one, 2) * np.linalg.norm(start)
     assert np.abs(got - want).max() <= 2 * 3 * 16 * 2.0 ** -53 * scale
+
+
+@pytest.mark.parametrize("n,opts", [(13, dict(chunk_bits=6, diag_outside=1)), (15, dict(chunk_bits=10, diag_outside=1)),
+                                    (16, dict(chunk_bits=12, diag_outside=1)), (15, dict(chunk_bits=9, gather_pinned=4, diag_outside=1)),
+                                    (14, dict(chunk_bits=5, diag_outside=1))])
+@pytest.mark.parametrize("kind", ["qft", "between_dense", "signs"])
+def test_merged_outside_diagonals(sv, n, opts, kind):
+    """Runs of diagonals from outside the chunk become one per chunk; they may pass diagonal gates and
+    gates on other bits, not dense gates or exchanges on theirs."""
+    rng = np.random.default_rng(n)
+    if kind == "qft":
+        desc = cg.qft(n)
+    elif kind == "signs":
+        desc = [("cz", (int(a), int(b)), ()) for a, b in (rng.choice(n, 2, replace=False) for _ in range(60))]
+    else:
+        desc = []
+        for _ in range(40):
+            a, b = (int(v) for v in rng.choice(n, 2, replace=False))
+            desc += [("cp", (a, b), (float(rng.uniform(0, 6)),)), ("rz", (a,), (float(rng.uniform(0, 6)),)),
+                     ("cp", (b, n - 1 - b if n - 1 - b != b else (b + 1) % n), (0.4,))]
+            desc.append([("u3", (a,), (0.3, 0.2, 0.1)), ("cx", (b, a), ()), ("x", (b,), ()), ("ry", (b,), (0.7,))][int(rng.integers(4))])
+    start = rng.standard_normal(1 << n) + 1j * rng.standard_normal(1 << n)
+    want = sim.apply(start.copy(), n, desc)
+    got = run(sv, n, desc, opts, start)
+    if kind == "signs":
+        assert np.array_equal(got, want)
+    else:
+        assert np.abs(got - want).max() <= bound(desc, start)
