@@ -218,7 +218,10 @@ sv_status sv_shard_unpack(sv_handle h, int32_t bit, int32_t value, const void *d
  * amplitudes (layout as sv_dtype; pinned memory lets the copies run at the link's rate).  The
  * plan runs in passes, each streaming the state through the device work buffer once: consecutive
  * sections and chunk_swap / reordering rounds share a pass when their sub-states fit half the
- * buffer (two are in flight, so copies overlap kernels).  dev_work: a DEVICE buffer of work_bytes
+ * buffer (two are in flight, so copies overlap kernels).  Where that takes fewer passes, the same
+ * circuit runs as sections of as many qubits as fit, gathered from host memory in place, instead
+ * of the plan's own schedule (circuits without SWAP relabels, plans that restore the layout; the
+ * result is the same up to rounding).  dev_work: a DEVICE buffer of work_bytes
  * (the caller's), or NULL to let the library allocate work_bytes for the call; it must hold two
  * sub-states of 2^(c+2) amplitudes unless it holds the whole state twice.  Sections run on SIMT
  * register groups.  Synchronous: returns when the state in host memory is final.  passes (may be

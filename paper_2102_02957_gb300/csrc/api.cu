@@ -444,10 +444,27 @@ static void build_programs(const sv_plan *plan, const sv_gate *gates, int seg_bi
 void build_simt_programs(const sv_plan *plan, const sv_gate *gates, int dtype, SimtPrograms &out) {
     out.seg_bits = (dtype == SV_C64 && plan->seg_bits == 5) ? 5 : 4;
     std::vector<BlockProg> progs;
+    std::vector<OzCompose> oz;
     if (dtype == SV_C64) build_programs<float>(plan, gates, out.seg_bits, out.host, progs);
-    else build_programs<double>(plan, gates, out.seg_bits, out.host, progs);
+    else build_programs<double>(plan, gates, out.seg_bits, out.host, progs, &oz);
+    out.oz_off = out.host.size();
+    out.noz = (int)oz.size();
+    const unsigned char *p = reinterpret_cast<const unsigned char *>(oz.data());
+    out.host.insert(out.host.end(), p, p + oz.size() * sizeof(OzCompose));
     out.progs.clear();
-    for (const BlockProg &bp : progs) out.progs.push_back(SimtPrograms::Prog{bp.off, bp.nseg, bp.gate_bytes, bp.fixed, bp.op_index});
+    for (const BlockProg &bp : progs)
+        out.progs.push_back(
+            SimtPrograms::Prog{bp.off, bp.nseg, bp.gate_bytes, bp.op_index, bp.fixed, bp.oz, bp.gathered, bp.lay});
+}
+
+void launch_section(int dtype, void *state, int n, int c, const unsigned char *base, const SimtPrograms::Prog &p,
+                    int seg_bits, int *dev_err, cudaStream_t st, uint64_t wait_ns) {
+    if (p.oz)
+        launch_block_oz(state, n, c, p.gathered ? &p.lay : nullptr, base + p.off, p.nseg, p.gate_bytes, dev_err, st, wait_ns);
+    else if (p.gathered)
+        launch_block_gather(dtype, state, n, p.lay, base + p.off, p.nseg, p.gate_bytes, p.fixed, dev_err, seg_bits, st, wait_ns);
+    else
+        launch_block(dtype, state, n, c, base + p.off, p.nseg, p.gate_bytes, p.fixed, dev_err, seg_bits, st, wait_ns);
 }
 
 static void upload_program(sv_state *h, const std::vector<unsigned char> &host) {
@@ -748,8 +765,6 @@ sv_status sv_apply_circuit(sv_handle h, const sv_gate *gates, int64_t n_gates, s
         }
         std::vector<unsigned char> host;
         std::vector<BlockProg> progs;
-        // SIMT register groups: 4 bits, or 5 for complex64
-        const int seg_bits = (h->dtype == SV_C64 && plan->seg_bits == 5) ? 5 : 4;
         // tensor cores: complex64 with chunks of at least 128 rows of the plan's r-bit groups
         const int tc_bits = plan->seg_bits;
         const bool tc = plan->use_tc && h->dtype == SV_C64 && std::min(plan->c, plan->n) - plan->reserve >= tc_bits + 7;
@@ -768,19 +783,10 @@ sv_status sv_apply_circuit(sv_handle h, const sv_gate *gates, int64_t n_gates, s
             launch_partial_norm(h->dtype, h->amp, h->n, h->scratch, nb_norm, h->stream);
             ++st.kernel_launches;
         }
-        std::vector<OzCompose> oz;  // complex128 groups to fuse
-        size_t oz_off = 0;
-        if (tc) {
-            build_programs_tc(plan, gates, tc_bits, host, progs, cs_off, ncs, g_off, flag_off);
-        } else if (h->dtype == SV_C64) {
-            build_programs<float>(plan, gates, seg_bits, host, progs);
-        } else {
-            build_programs<double>(plan, gates, seg_bits, host, progs, &oz);
-            oz_off = host.size();
-            const unsigned char *p = reinterpret_cast<const unsigned char *>(oz.data());
-            host.insert(host.end(), p, p + oz.size() * sizeof(OzCompose));
-        }
-        upload_program(h, host);
+        SimtPrograms sp;
+        if (tc) build_programs_tc(plan, gates, tc_bits, host, progs, cs_off, ncs, g_off, flag_off);
+        else build_simt_programs(plan, gates, h->dtype, sp);
+        upload_program(h, tc ? host : sp.host);
         const unsigned char *base = static_cast<const unsigned char *>(h->prog);
         int *unitary_flag = tc ? reinterpret_cast<int *>(static_cast<unsigned char *>(h->prog) + flag_off) : nullptr;
         if (tc) {  // fuse every register group into its B operand, in FP64 on the GPU
@@ -790,8 +796,8 @@ sv_status sv_apply_circuit(sv_handle h, const sv_gate *gates, int64_t n_gates, s
                     ++st.kernel_launches;
                 }
         }
-        if (!oz.empty()) {
-            launch_compose_oz(base + oz_off, (int)oz.size(), h->prog, h->stream);
+        if (sp.noz) {
+            launch_compose_oz(base + sp.oz_off, sp.noz, h->prog, h->stream);
             ++st.kernel_launches;
         }
         const uint64_t wait_ns = plan->wait_limit_ms > 0 ? (uint64_t)plan->wait_limit_ms * 1000000ull : kDefaultWaitNs;
@@ -799,25 +805,25 @@ sv_status sv_apply_circuit(sv_handle h, const sv_gate *gates, int64_t n_gates, s
         for (size_t oi = 0; oi < plan->ops.size(); ++oi) {
             const PlanOp &op = plan->ops[oi];
             if (op.kind == 2 || op.kind == 4) {
-                for (; bi < progs.size() && progs[bi].op_index == (int)oi; ++bi) {
-                    const BlockProg &bp = progs[bi];
+                auto sweep = [&](auto launch) {
                     mark_begin(h, 1, (int)oi);
-                    if (tc)
-                        launch_block_tc(h->amp, h->n, plan->c, bp.gathered ? &bp.lay : nullptr, base + bp.off, bp.nseg,
-                                        h->dev_err, bp.r, h->stream, wait_ns);
-                    else if (bp.oz)
-                        launch_block_oz(h->amp, h->n, plan->c, bp.gathered ? &bp.lay : nullptr, base + bp.off, bp.nseg,
-                                        bp.gate_bytes, h->dev_err, h->stream, wait_ns);
-                    else if (!bp.gathered)
-                        launch_block(h->dtype, h->amp, h->n, plan->c, base + bp.off, bp.nseg, bp.gate_bytes, bp.fixed,
-                                     h->dev_err, seg_bits, h->stream, wait_ns);
-                    else
-                        launch_block_gather(h->dtype, h->amp, h->n, bp.lay, base + bp.off, bp.nseg, bp.gate_bytes,
-                                            bp.fixed, h->dev_err, seg_bits, h->stream, wait_ns);
+                    launch();
                     mark_end(h);
                     ++st.sweeps_block;
                     ++st.kernel_launches;
+                };
+                for (; tc && bi < progs.size() && progs[bi].op_index == (int)oi; ++bi) {
+                    const BlockProg &bp = progs[bi];
+                    sweep([&] {
+                        launch_block_tc(h->amp, h->n, plan->c, bp.gathered ? &bp.lay : nullptr, base + bp.off, bp.nseg,
+                                        h->dev_err, bp.r, h->stream, wait_ns);
+                    });
                 }
+                for (; !tc && bi < sp.progs.size() && sp.progs[bi].op_index == (int)oi; ++bi)
+                    sweep([&] {
+                        launch_section(h->dtype, h->amp, h->n, plan->c, base, sp.progs[bi], sp.seg_bits, h->dev_err,
+                                       h->stream, wait_ns);
+                    });
                 continue;
             } else {
                 mark_begin(h, 2, (int)oi);
@@ -853,23 +859,20 @@ sv_status sv_apply_plan_ops(sv_handle h, const sv_gate *gates, int64_t n_gates, 
         const GateKey k{gates[i].nq, gates[i].q[0], gates[i].nq == 2 ? gates[i].q[1] : -1, gates[i].flags};
         if (!(k == plan->keys[(size_t)i])) fail(SV_ERR_PLAN, "gate " + std::to_string(i) + " differs from the planned list");
     }
-    std::vector<unsigned char> host;
-    std::vector<BlockProg> progs;
-    const int seg_bits = (h->dtype == SV_C64 && plan->seg_bits == 5) ? 5 : 4;
-    if (h->dtype == SV_C64) build_programs<float>(plan, gates, seg_bits, host, progs);
-    else build_programs<double>(plan, gates, seg_bits, host, progs);
-    upload_program(h, host);
+    SimtPrograms sp;
+    build_simt_programs(plan, gates, h->dtype, sp);
+    upload_program(h, sp.host);
     const unsigned char *base = static_cast<const unsigned char *>(h->prog);
+    if (sp.noz) launch_compose_oz(base + sp.oz_off, sp.noz, h->prog, h->stream);
     const uint64_t wait_ns = plan->wait_limit_ms > 0 ? (uint64_t)plan->wait_limit_ms * 1000000ull : kDefaultWaitNs;
     size_t bi = 0;  // programs are in op order
     for (int32_t oi = op_begin; oi < op_end; ++oi) {
         const PlanOp &op = plan->ops[(size_t)oi];
         if (op.kind == 2) {
-            while (bi < progs.size() && progs[bi].op_index < oi) ++bi;
-            if (bi == progs.size() || progs[bi].op_index != oi) fail(SV_ERR_PLAN, "no program for a blocking section");
-            const BlockProg &bp = progs[bi];
-            launch_block(h->dtype, h->amp, h->n, plan->c, base + bp.off, bp.nseg, bp.gate_bytes, bp.fixed, h->dev_err,
-                         seg_bits, h->stream, wait_ns);
+            while (bi < sp.progs.size() && sp.progs[bi].op_index < oi) ++bi;
+            if (bi == sp.progs.size() || sp.progs[bi].op_index != oi) fail(SV_ERR_PLAN, "no program for a blocking section");
+            for (; bi < sp.progs.size() && sp.progs[bi].op_index == oi; ++bi)
+                launch_section(h->dtype, h->amp, h->n, plan->c, base, sp.progs[bi], sp.seg_bits, h->dev_err, h->stream, wait_ns);
         } else {
             // pairs inside the piece; the others move data between pieces and are the caller's
             std::vector<std::pair<int32_t, int32_t>> local;

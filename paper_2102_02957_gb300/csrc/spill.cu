@@ -14,8 +14,13 @@
 // half the buffer: two sub-states are in flight, on two streams, so one's copies overlap the
 // other's kernels); m is then the largest value with m + |{pair bits >= m}| <= M.  A round whose
 // pairs alone do not fit is split into several items (its transpositions commute).
+//
+// Most of a chunk_swap's traffic over the link is the price of contiguous chunks.  Where it takes fewer
+// passes, the circuit runs instead as sections of M qubits gathered from host memory in place
+// (gathered_passes), each a pass with a plan of its own inside.
 #include <algorithm>
 #include <cstring>
+#include <functional>
 #include <vector>
 
 #include "sv_internal.h"
@@ -126,30 +131,31 @@ std::vector<Pass> make_passes(const sv_plan &plan, int M) {
     return passes;
 }
 
-// Run one pass: for every value of the state bits >= m outside H, gather the sub-state's 2^|H|
-// slabs, run the pass's items on it, write it back.  Sub-states alternate between the two halves
-// of the work buffer and the two streams.
-void run_pass(const Pass &p, const sv_plan &plan, int dtype, unsigned char *host, unsigned char *host_dev,
-              unsigned char *work, size_t half_bytes, const unsigned char *prog, const SimtPrograms &sp, int *dev_err,
-              cudaStream_t *st, uint64_t wait_ns) {
-    const int n = plan.n, m = p.m, nh = (int)p.high.size(), nsub = m + nh;
-    const size_t elem = dtype == SV_C64 ? 8 : 16;
+// A pass as it runs: slabs of 2^m amplitudes, H, and the work on one sub-state of m + |H| qubits.
+struct PassRun {
+    int m = 0;
+    std::vector<int> high;
+    std::function<void(void *buf, int nsub, cudaStream_t st)> work;
+};
+
+int local_bit(const std::vector<int> &high, int m, int b) {
+    return b < m ? b : m + (int)(std::find(high.begin(), high.end(), b) - high.begin());
+}
+
+// For every value of the state bits >= m outside H, gather the sub-state's 2^|H| slabs, run the
+// pass's work on it, write it back.  Sub-states alternate between the two halves of the work
+// buffer and the two streams.
+void run_pass(const PassRun &p, int n, size_t elem, unsigned char *host, unsigned char *host_dev, unsigned char *work,
+              size_t half_bytes, cudaStream_t *st) {
+    const int m = p.m, nh = (int)p.high.size(), nsub = m + nh;
     const size_t slab_bytes = (size_t(1) << m) * elem;
     if ((size_t(1) << nsub) * elem > half_bytes) fail(SV_ERR_ARG, "host-resident pass does not fit the work buffer");
     std::vector<int> outer;  // state bits >= m not in H: they number the sub-states
     for (int b = m; b < n; ++b)
         if (std::find(p.high.begin(), p.high.end(), b) == p.high.end()) outer.push_back(b);
-    // the items' pairs in sub-state bit numbers
-    auto local_bit = [&](int b) {
-        if (b < m) return b;
-        return m + (int)(std::find(p.high.begin(), p.high.end(), b) - p.high.begin());
-    };
-    std::vector<std::vector<std::pair<int32_t, int32_t>>> pairs(p.items.size());
-    for (size_t i = 0; i < p.items.size(); ++i)
-        for (const auto &pq : p.items[i].pairs) pairs[i].emplace_back(local_bit(pq.first), local_bit(pq.second));
     const int64_t nsubs = int64_t(1) << outer.size();
-    // small slabs (passes that carry many high swap bits) move by kernel when the host memory is
-    // mapped into the device's address space
+    // small slabs (passes that carry many high bits) move by kernel when the host memory is mapped
+    // into the device's address space
     const bool by_kernel = host_dev && slab_bytes < kKernelSlabBytes;
     SlabArgs sa{};
     sa.m = m;
@@ -180,20 +186,7 @@ void run_pass(const Pass &p, const sv_plan &plan, int dtype, unsigned char *host
                                            st[k]),
                            "cudaMemcpyAsync(host slab in)");
         }
-        for (size_t i = 0; i < p.items.size(); ++i) {
-            const int op = p.items[i].op;
-            if (plan.ops[(size_t)op].kind == 2) {
-                const SimtPrograms::Prog *pr = nullptr;
-                for (const auto &q : sp.progs)
-                    if (q.op_index == op) pr = &q;
-                if (!pr) fail(SV_ERR_PLAN, "no program for a blocking section");
-                launch_block(dtype, buf, nsub, plan.c, prog + pr->off, pr->nseg, pr->gate_bytes, pr->fixed != 0, dev_err,
-                             sp.seg_bits, st[k],
-                             wait_ns);
-            } else if (!pairs[i].empty()) {
-                launch_permute(dtype, buf, nsub, pairs[i], st[k]);
-            }
-        }
+        p.work(buf, nsub, st[k]);
         if (by_kernel) {
             k_slab_copy<false><<<grid, 256, 0, st[k]>>>(reinterpret_cast<uint4 *>(buf), reinterpret_cast<uint4 *>(host_dev), sa);
             check_cuda(cudaGetLastError(), "slab scatter launch");
@@ -204,6 +197,69 @@ void run_pass(const Pass &p, const sv_plan &plan, int dtype, unsigned char *host
                            "cudaMemcpyAsync(host slab out)");
         }
     }
+}
+
+// Gathered passes: the same circuit as sections of M qubits gathered from host memory, so that no
+// chunk_swap crosses the link; each section is one pass whose gates run on its sub-state under a
+// plan of their own (gathered chunks of c bits where they fit).  For circuits without SWAP
+// relabels whose output is in the natural layout.
+struct GatheredPass {
+    int m = 0;
+    std::vector<int> high;
+    std::vector<sv_gate> gates;  // on sub-state bits
+    std::unique_ptr<sv_plan> plan;
+    SimtPrograms sp;
+    size_t off = 0;  // of its programs in the upload
+};
+
+// The sections of the circuit on M-bit chunks with the low bits pinned: the widest slabs among those
+// with the fewest sections.  Slabs under 1 MiB are worth it only where a kernel can copy them.
+std::unique_ptr<sv_plan> outer_plan(int n, const sv_gate *gates, int64_t n_gates, int M, size_t elem, bool mapped) {
+    const int wide = elem == 8 ? 17 : 16;  // 1 MiB
+    std::unique_ptr<sv_plan> best;
+    for (int pinned : {wide + 2, wide, 14, 12, 10}) {
+        if (pinned > M - 4 || (pinned < wide && !mapped)) continue;
+        for (int look = 0; look < (n_gates <= 4000 ? 2 : 1); ++look) {
+            sv_options o;
+            sv_options_default(&o);
+            o.chunk_bits = M;
+            o.gather_pinned = pinned;
+            o.lookahead = look;
+            std::unique_ptr<sv_plan> p(plan_blocking(n, gates, n_gates, o));
+            if (!best || p->ops.size() < best->ops.size()) best = std::move(p);
+        }
+    }
+    return best;
+}
+
+std::vector<GatheredPass> gathered_passes(const sv_plan &outer, const sv_gate *gates, int c, int seg_bits, int dtype) {
+    std::vector<GatheredPass> out;
+    for (const PlanOp &op : outer.ops) {
+        if (op.gates.empty()) continue;
+        GatheredPass g;
+        const uint64_t mask = op.kind == 4 ? op.mask : (uint64_t(1) << std::min(outer.c, outer.n)) - 1;
+        while (g.m < outer.n && ((mask >> g.m) & 1)) ++g.m;
+        for (int b = g.m; b < outer.n; ++b)
+            if ((mask >> b) & 1) g.high.push_back(b);
+        for (const BlockGate &bg : op.gates) {
+            sv_gate s = gates[bg.gi];
+            for (int j = 0; j < s.nq; ++j) s.q[j] = local_bit(g.high, g.m, bg.phys[j]);
+            g.gates.push_back(s);
+        }
+        const int nsub = g.m + (int)g.high.size();
+        sv_options o;
+        sv_options_default(&o);
+        o.chunk_bits = std::min(c, nsub);
+        o.seg_bits = seg_bits;
+        if (o.chunk_bits >= 9 && o.chunk_bits < nsub) {
+            o.gather_pinned = 4;
+            o.lookahead = g.gates.size() <= 4000;
+        }
+        g.plan.reset(plan_blocking(nsub, g.gates.data(), (int64_t)g.gates.size(), o));
+        build_simt_programs(g.plan.get(), g.gates.data(), dtype, g.sp);
+        out.push_back(std::move(g));
+    }
+    return out;
 }
 
 }  // namespace
@@ -241,24 +297,6 @@ extern "C" sv_status sv_apply_circuit_host(int32_t n, int32_t dtype, void *host_
             check_cuda(cudaMalloc(&owned, 2 * half_bytes), "cudaMalloc(work buffer)");
             dev_work = owned;
         }
-        SimtPrograms sp;
-        build_simt_programs(plan, gates, dtype, sp);
-        check_cuda(cudaMalloc(&progbuf, std::max<size_t>(sp.host.size(), 256)), "cudaMalloc(programs)");
-        check_cuda(cudaMalloc(&dev_err, sizeof(int)), "cudaMalloc(error word)");
-        const cudaStream_t caller = (cudaStream_t)cuda_stream;
-        check_cuda(cudaMemsetAsync(dev_err, 0, sizeof(int), caller), "cudaMemsetAsync");
-        if (!sp.host.empty())
-            check_cuda(cudaMemcpyAsync(progbuf, sp.host.data(), sp.host.size(), cudaMemcpyHostToDevice, caller),
-                       "upload programs");
-        for (auto &s : st) check_cuda(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking), "cudaStreamCreate");
-        check_cuda(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming), "cudaEventCreate");
-        auto join = [&](cudaStream_t from, cudaStream_t to) {
-            check_cuda(cudaEventRecord(ev, from), "cudaEventRecord");
-            check_cuda(cudaStreamWaitEvent(to, ev, 0), "cudaStreamWaitEvent");
-        };
-        join(caller, st[0]);
-        join(caller, st[1]);
-        const uint64_t wait_ns = plan->wait_limit_ms > 0 ? (uint64_t)plan->wait_limit_ms * 1000000ull : kDefaultWaitNs;
         // the device's address of the host state, if the GPU can address it directly (pinned and
         // mapped host memory); else every slab goes through a copy
         unsigned char *host_dev = nullptr;
@@ -269,10 +307,88 @@ extern "C" sv_status sv_apply_circuit_host(int32_t n, int32_t dtype, void *host_
                 host_dev = static_cast<unsigned char *>(at.devicePointer);
             cudaGetLastError();  // an unregistered pointer leaves an error state; clear it
         }
-        const std::vector<Pass> passes = make_passes(*plan, M);
-        for (const Pass &p : passes) {
-            run_pass(p, *plan, dtype, static_cast<unsigned char *>(host_amps), host_dev, static_cast<unsigned char *>(dev_work),
-                     half_bytes, static_cast<const unsigned char *>(progbuf), sp, dev_err, st, wait_ns);
+        // the plan's own passes, or gathered ones where they take fewer trips over the link (26 qubits,
+        // 4 random layers, an eighth of the state on the device: 2 instead of 14, 47 to 55 -> 17 ms)
+        std::vector<Pass> passes = make_passes(*plan, M);
+        std::vector<GatheredPass> gathered;
+        bool natural = plan->restore && M < n && reinterpret_cast<uintptr_t>(dev_work) % 16 == 0;
+        for (int64_t i = 0; i < n_gates; ++i) natural = natural && !(gates[i].flags & SV_GATE_SWAP);
+        if (natural && passes.size() > 1) {
+            const std::unique_ptr<sv_plan> outer = outer_plan(n, gates, n_gates, M, elem, host_dev != nullptr);
+            if (outer && outer->ops.size() < passes.size()) gathered = gathered_passes(*outer, gates, c, plan->seg_bits, dtype);
+        }
+        SimtPrograms sp;
+        std::vector<unsigned char> programs;
+        if (gathered.empty()) {
+            build_simt_programs(plan, gates, dtype, sp);
+            programs = sp.host;
+        }
+        for (GatheredPass &g : gathered) {
+            programs.resize((programs.size() + 255) / 256 * 256);
+            g.off = programs.size();
+            programs.insert(programs.end(), g.sp.host.begin(), g.sp.host.end());
+        }
+        check_cuda(cudaMalloc(&progbuf, std::max<size_t>(programs.size(), 256)), "cudaMalloc(programs)");
+        check_cuda(cudaMalloc(&dev_err, sizeof(int)), "cudaMalloc(error word)");
+        const cudaStream_t caller = (cudaStream_t)cuda_stream;
+        check_cuda(cudaMemsetAsync(dev_err, 0, sizeof(int), caller), "cudaMemsetAsync");
+        unsigned char *const prog = static_cast<unsigned char *>(progbuf);
+        if (!programs.empty())
+            check_cuda(cudaMemcpyAsync(prog, programs.data(), programs.size(), cudaMemcpyHostToDevice, caller),
+                       "upload programs");
+        launch_compose_oz(prog + sp.oz_off, sp.noz, prog, caller);
+        for (const GatheredPass &g : gathered) launch_compose_oz(prog + g.off + g.sp.oz_off, g.sp.noz, prog + g.off, caller);
+        for (auto &s : st) check_cuda(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking), "cudaStreamCreate");
+        check_cuda(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming), "cudaEventCreate");
+        auto join = [&](cudaStream_t from, cudaStream_t to) {
+            check_cuda(cudaEventRecord(ev, from), "cudaEventRecord");
+            check_cuda(cudaStreamWaitEvent(to, ev, 0), "cudaStreamWaitEvent");
+        };
+        join(caller, st[0]);
+        join(caller, st[1]);
+        const uint64_t wait_ns = plan->wait_limit_ms > 0 ? (uint64_t)plan->wait_limit_ms * 1000000ull : kDefaultWaitNs;
+        std::vector<PassRun> runs;
+        if (gathered.empty()) {
+            for (const Pass &p : passes) {
+                // the items' pairs in sub-state bit numbers
+                std::vector<std::vector<std::pair<int32_t, int32_t>>> pairs(p.items.size());
+                for (size_t i = 0; i < p.items.size(); ++i)
+                    for (const auto &pq : p.items[i].pairs)
+                        pairs[i].emplace_back(local_bit(p.high, p.m, pq.first), local_bit(p.high, p.m, pq.second));
+                runs.push_back(PassRun{p.m, p.high, [&, pairs](void *buf, int nsub, cudaStream_t s) {
+                                           for (size_t i = 0; i < p.items.size(); ++i) {
+                                               const int op = p.items[i].op;
+                                               if (plan->ops[(size_t)op].kind != 2) {
+                                                   if (!pairs[i].empty()) launch_permute(dtype, buf, nsub, pairs[i], s);
+                                                   continue;
+                                               }
+                                               bool found = false;
+                                               for (const auto &q : sp.progs)
+                                                   if (q.op_index == op) {
+                                                       found = true;
+                                                       launch_section(dtype, buf, nsub, plan->c, prog, q, sp.seg_bits, dev_err,
+                                                                      s, wait_ns);
+                                                   }
+                                               if (!found) fail(SV_ERR_PLAN, "no program for a blocking section");
+                                           }
+                                       }});
+            }
+        } else {
+            for (const GatheredPass &g : gathered)
+                runs.push_back(PassRun{g.m, g.high, [&](void *buf, int nsub, cudaStream_t s) {
+                                           size_t k = 0;
+                                           for (size_t op = 0; op < g.plan->ops.size(); ++op) {
+                                               if (g.plan->ops[op].kind == 1 || g.plan->ops[op].kind == 3)
+                                                   launch_permute(dtype, buf, nsub, g.plan->ops[op].pairs, s);
+                                               for (; k < g.sp.progs.size() && g.sp.progs[k].op_index == (int)op; ++k)
+                                                   launch_section(dtype, buf, nsub, g.plan->c, prog + g.off, g.sp.progs[k],
+                                                                  g.sp.seg_bits, dev_err, s, wait_ns);
+                                           }
+                                       }});
+        }
+        for (const PassRun &r : runs) {
+            run_pass(r, n, elem, static_cast<unsigned char *>(host_amps), host_dev, static_cast<unsigned char *>(dev_work),
+                     half_bytes, st);
             // the next pass reads what either stream wrote back
             join(st[0], st[1]);
             join(st[1], st[0]);
@@ -284,7 +400,7 @@ extern "C" sv_status sv_apply_circuit_host(int32_t n, int32_t dtype, void *host_
         check_cuda(cudaStreamSynchronize(caller), "cudaStreamSynchronize");
         if (e == DEV_ERR_TIMEOUT) fail(SV_ERR_TIMEOUT, "a bounded device wait expired");
         if (e != DEV_OK) fail(SV_ERR_CUDA, "device error word set");
-        if (passes_out) *passes_out = (int32_t)passes.size();
+        if (passes_out) *passes_out = (int32_t)runs.size();
     } catch (const sv::Error &err) {
         sv::set_error(err.msg);
         status = err.code;

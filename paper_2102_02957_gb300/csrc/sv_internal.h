@@ -277,17 +277,25 @@ struct Mat2 { float m[32]; };
 
 void launch_gate(int dtype, void *state, int n, const sv_gate &g, cudaStream_t st);
 void launch_init_basis(int dtype, void *state, int n, uint64_t basis, cudaStream_t st);
-// SIMT section programs of a contiguous-chunk plan, laid out as one device upload (api.cu).
+// Section programs of a plan with SIMT register groups (complex128: tensor-core sweeps where they
+// apply), laid out as one device upload (api.cu).
 struct SimtPrograms {
     struct Prog {
         size_t off;
-        int nseg, gate_bytes, fixed, op_index;
+        int nseg, gate_bytes, op_index;
+        bool fixed, oz, gathered;
+        GatherLayout lay;  // gathered chunks
     };
     std::vector<unsigned char> host;
     std::vector<Prog> progs;
+    size_t oz_off = 0;  // groups to compose once uploaded (launch_compose_oz)
+    int noz = 0;
     int seg_bits = 4;
 };
 void build_simt_programs(const sv_plan *plan, const sv_gate *gates, int dtype, SimtPrograms &out);
+// Launch one section of 2^n amplitudes (chunks of c bits) from its program at base + p.off.
+void launch_section(int dtype, void *state, int n, int c, const unsigned char *base, const SimtPrograms::Prog &p,
+                    int seg_bits, int *dev_err, cudaStream_t st, uint64_t wait_ns);
 // Amplitudes with bit `bit` == value, in index order, to / from a buffer of 2^(n-1) (k_shard.cu).
 void launch_shard_half(bool pack, int dtype, void *state, int n, int bit, int value, void *buf, cudaStream_t st);
 

@@ -97,3 +97,26 @@ def test_non_finite_chunk_runs_in_fp64(sv, bad):
     reached = (np.arange(1 << n) | 7) == 7  # the three dense qubits' coset (bit 4 of index 5 is 0)
     assert not np.isfinite(got[reached]).any()
     assert np.abs(got[~reached] - want[~reached]).max() <= bound(desc, start[~reached])
+
+
+@pytest.mark.parametrize("dtype", ["c64", "c128"])
+@pytest.mark.parametrize("n,c,share,pinned_host", [(18, 9, 4, True), (20, 10, 8, True), (21, 12, 4, False), (19, 6, 8, True), (20, 11, 16, True)])
+def test_host_resident_gathered_passes(sv, dtype, n, c, share, pinned_host):
+    """The gathered passes of host-resident states: both types, mapped and pageable host memory, chunk
+    widths on either side of the gathered inner plan's."""
+    import torch
+    desc = cg.random_layers(n, 3, 2) + cg.quantum_volume(n, 1, 3)
+    rng = np.random.default_rng(n)
+    start = rng.standard_normal(1 << n) + 1j * rng.standard_normal(1 << n)
+    start /= np.linalg.norm(start)
+    want = sim.apply(start.copy(), n, desc)
+    gates = sv.make_gates(desc)
+    plan = sv.Plan(n, gates, chunk_bits=c)
+    ct = np.complex64 if dtype == "c64" else np.complex128
+    host = torch.from_numpy(start.astype(ct))
+    host = host.pin_memory() if pinned_host else host
+    passes = sv.apply_host(n, host, gates, plan, (1 << n) // share * host.element_size(), dtype=dtype)
+    info = plan.info()
+    assert 1 <= passes < info.n_blocks + info.n_swap_rounds + info.n_unpermute_rounds
+    tol = 1e-5 if dtype == "c64" else 1e-12
+    assert np.abs(host.numpy() - want).max() <= tol
