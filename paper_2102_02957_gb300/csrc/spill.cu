@@ -308,7 +308,7 @@ extern "C" sv_status sv_apply_circuit_host(int32_t n, int32_t dtype, void *host_
             cudaGetLastError();  // an unregistered pointer leaves an error state; clear it
         }
         // the plan's own passes, or gathered ones where they take fewer trips over the link (26 qubits,
-        // 4 random layers, an eighth of the state on the device: 2 instead of 14, 47 to 55 -> 17 ms)
+        // 4 random layers, an eighth of the state on the device: 2 passes instead of 9, 47 to 55 -> 17 ms)
         std::vector<Pass> passes = make_passes(*plan, M);
         std::vector<GatheredPass> gathered;
         bool natural = plan->restore && M < n && reinterpret_cast<uintptr_t>(dev_work) % 16 == 0;

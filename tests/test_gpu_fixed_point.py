@@ -121,3 +121,29 @@ def test_merged_outside_diagonals(sv, n, opts, kind):
         assert np.array_equal(got, want)
     else:
         assert np.abs(got - want).max() <= bound(desc, start)
+
+
+@pytest.mark.parametrize("n,opts", [(6, dict(chunk_bits=4)), (9, dict(chunk_bits=5)), (14, dict(chunk_bits=13)), (14, dict(chunk_bits=12, seg_bits=5)),
+                                    (13, dict(chunk_bits=9, gather_pinned=4)), (13, dict(chunk_bits=8, diag_outside=1))])
+@pytest.mark.parametrize("kind", ["pairs", "everything"])
+def test_fused_complex64_gates(sv, n, opts, kind):
+    """Fused records of complex64 sections: every kind of gate before and after every other, same and
+    different pairs in both orders, non-unitary matrices among them."""
+    rng = np.random.default_rng(n + len(kind))
+    desc = []
+    for _ in range(60):
+        a, b = (int(v) for v in rng.choice(n if kind == "everything" else 4, 2, replace=False))
+        desc.append([("u3", (a,), (0.3, 0.2, 0.1)), ("x", (a,), ()), ("rz", (a,), (0.4,)), ("cx", (a, b), ()), ("cz", (a, b), ()),
+                     ("cp", (a, b), (0.5,)), ("unitary", (a, b), (cg.haar_unitary(rng),)), ("h", (b,), ()),
+                     ("unitary", (a, b), (np.eye(4, dtype=np.complex128)[[1, 2, 3, 0]],)),
+                     ("unitary", (a,), (np.array([[0.9, 0.1j], [0.2, 1.1]]),))][int(rng.integers(10))])
+    start = rng.standard_normal(1 << n) + 1j * rng.standard_normal(1 << n)
+    start = (start / np.linalg.norm(start)).astype(np.complex64)
+    want = sim.apply(start.astype(np.complex128), n, desc)
+    gates = sv.make_gates(desc)
+    st = sv.StateVector(n, "c64")
+    st.set_state(start)
+    st.apply(gates, sv.Plan(n, gates, **opts))
+    # per gate 8 products of 2^-24 each, on norms that the non-unitary gates change by at most 1.2
+    grown = 1.2 ** sum(1 for k, q, p in desc if k == "unitary" and len(q) == 1)
+    assert np.abs(st.get_state() - want).max() <= len(desc) * 16 * 2.0 ** -24 * grown
