@@ -17,7 +17,7 @@
 // then the payloads (encode_fx writes them):
 //   OP_DENSE1 / OP_DENSE2  4 / 16 entries {re h, re l, im h, im l}     OP_REAL1  4 x {h, l}
 //   OP_DIAG1 / OP_DIAG2    2 / 4 entries   OP_DIAGX  2 or 4 OP_DIAG1   OP_PERM2  4 ints
-//   OP_DIAGRUN  the run's gates and 16 entries per consumer group, filled per chunk (fx_merge): a
+//   OP_DIAGRUN  the run's gates and kFxRunBytes of tables, filled per chunk (fx_merge): a
 //   QFT section has up to 16 controlled phases from outside the chunk on each of its qubits
 #pragma once
 #include "block_core.cuh"
@@ -265,40 +265,81 @@ __device__ __forceinline__ FxGate fx_gate(uint32_t gates, int gi, int64_t origin
         op = OP_DIAG1;
     } else if (op == OP_DIAGRUN) {
         more = rb - 1;
-        m += (uint32_t)(16 + 16 * rb + 256 * cg);
+        m += (uint32_t)(16 + 16 * rb + kFxRunBytes / kFxGroups * cg);
     }
     return FxGate{op, code, m, more};
 }
 
-// Entries of the merged runs of gates [g0, g1) for this chunk: thread x < 16 of a warp multiplies
-// entry x over the run's gates, a warp per run in turn (products in the scale 2^59 of fixed64.cuh).
-__device__ __forceinline__ void fx_merge(uint32_t gates, int g0, int g1, int64_t origin, int cg, int ctid, int nwarps) {
-    const int lane = ctid & 31;
-    int turn = 0;
-    for (int gi = g0; gi < g1; ++gi) {
-        int op, off, count, code;
-        ldc_i4(gates + 16u * (uint32_t)gi, op, off, count, code);
-        if (op != OP_DIAGRUN) continue;
-        if (turn++ % nwarps == (ctid >> 5) && lane < 16) {
+// Product of two values of the scale 2^59 of fixed64.cuh, both at most 1 in modulus.
+__device__ __forceinline__ void fx_product(fx::Real &ar, fx::Real &ai, const fx::Real &br, const fx::Real &bi) {
+    // b in the entries' scale 2^61, its low part negatable
+    fx::Real er = fx::pack(fx::value(br) * 4), ei = fx::pack(fx::value(bi) * 4);
+    er.l += er.l == (int)0x80000000;
+    ei.l += ei.l == (int)0x80000000;
+    fx::Acc yr, yi;
+    fx_cmac(yr, yi, FxEntry{er.h, er.l, ei.h, ei.l}, ar, ai);
+    ar = fx::fin(yr);
+    ai = fx::fin(yi);
+}
+
+// Tables of the merged runs of gates [g0, g1) for this chunk (NC threads, ends in a barrier).  The run
+// is cut into a part per half warp: lane x of a half multiplies entry x over every eighth gate,
+// the halves join by shuffle, and a half warp multiplies the warps' parts.  (One half warp alone took
+// a chain of up to 64 products per group, longer than the group's own work.)
+template <int NC>
+__device__ __forceinline__ void fx_merge(uint32_t gates, int g0, int g1, int64_t origin, int cg, int ctid, int bar_id) {
+    constexpr int W = NC / 32;
+    const int lane = ctid & 31, warp = ctid >> 5, x = lane & 15;
+    auto store = [](uint32_t a, const fx::Real &r, const fx::Real &i) {
+        asm volatile("st.shared.v4.s32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(r.h), "r"(r.l), "r"(i.h), "r"(i.l) : "memory");
+    };
+    for (int pass = 0; pass < 2; ++pass) {
+        for (int gi = g0; gi < g1; ++gi) {
+            int op, off, count, code;
+            ldc_i4(gates + 16u * (uint32_t)gi, op, off, count, code);
+            if (op != OP_DIAGRUN) continue;
+            gi += count - 1;
             const uint32_t list = gates + (uint32_t)off + 16;
+            const uint32_t table = list + (uint32_t)(16 * count + kFxRunBytes / kFxGroups * cg), parts = table + 256;
             fx::Real pr = fx::pack(1ll << 59), pi{0, 0};
-            for (int k = 0; k < count; ++k) {
-                int goff, outside, bit, unused;
-                ldc_i4(list + 16u * (uint32_t)k, goff, outside, bit, unused);
-                const FxEntry d = lds_entry(gates + (uint32_t)goff + fx_variant(outside, origin) + 16u * (uint32_t)((lane >> bit) & 1));
-                fx::Acc yr, yi;
-                fx_cmac(yr, yi, d, pr, pi);
-                pr = fx::fin(yr);
-                pi = fx::fin(yi);
+            if (pass == 0) {
+                for (int k = 2 * warp; k < count; k += 2 * W) {  // whole warps: the vote
+                    const int mine = k + (lane >> 4);
+                    FxEntry d{fx::kOne, 0, 0, 0};
+                    if (mine < count) {
+                        int goff, outside, bit, unused;
+                        ldc_i4(list + 16u * (uint32_t)mine, goff, outside, bit, unused);
+                        d = lds_entry(gates + (uint32_t)goff + fx_variant(outside, origin) + 16u * (uint32_t)((x >> bit) & 1));
+                    }
+                    // an outside qubit that reads 0 leaves a controlled phase out
+                    if (!__any_sync(0xFFFFFFFFu, d.rh != fx::kOne || d.rl || d.ih || d.il)) continue;
+                    fx::Acc yr, yi;
+                    fx_cmac(yr, yi, d, pr, pi);
+                    pr = fx::fin(yr);
+                    pi = fx::fin(yi);
+                }
+                fx::Real qr, qi;
+                qr.h = __shfl_xor_sync(0xFFFFFFFFu, pr.h, 16);
+                qr.l = __shfl_xor_sync(0xFFFFFFFFu, pr.l, 16);
+                qi.h = __shfl_xor_sync(0xFFFFFFFFu, pi.h, 16);
+                qi.l = __shfl_xor_sync(0xFFFFFFFFu, pi.l, 16);
+                fx_product(pr, pi, qr, qi);
+                if (lane < 16) store(parts + 256u * (uint32_t)warp + 16u * (uint32_t)x, pr, pi);
+            } else if (warp == 0) {
+                for (int w = 0; w < W; ++w) {
+                    fx::Real qr, qi;
+                    asm volatile("ld.shared.v4.s32 {%0, %1, %2, %3}, [%4];"
+                                 : "=r"(qr.h), "=r"(qr.l), "=r"(qi.h), "=r"(qi.l)
+                                 : "r"(parts + 256u * (uint32_t)w + 16u * (uint32_t)x));
+                    fx_product(pr, pi, qr, qi);
+                }
+                fx::Real er = fx::pack(fx::value(pr) * 4), ei = fx::pack(fx::value(pi) * 4);
+                er.l += er.l == (int)0x80000000;
+                ei.l += ei.l == (int)0x80000000;
+                if (lane < 16) store(table + 16u * (uint32_t)x, er, ei);
             }
-            fx::Real er = fx::pack(fx::value(pr) * 4), ei = fx::pack(fx::value(pi) * 4);  // entries' scale 2^61
-            er.l += er.l == (int)0x80000000;  // keep -l representable
-            ei.l += ei.l == (int)0x80000000;
-            asm volatile("st.shared.v4.s32 [%0], {%1, %2, %3, %4};" ::"r"(list + (uint32_t)(16 * count + 256 * cg + 16 * lane)),
-                         "r"(er.h), "r"(er.l), "r"(ei.h), "r"(ei.l)
-                         : "memory");
         }
-        gi += count - 1;
+        ptx::named_bar_sync(bar_id, NC);
     }
 }
 
@@ -396,10 +437,7 @@ __device__ __forceinline__ void run_segment_fx(uint32_t buf, uint32_t seg, uint3
     const int G = 1 << (c - R);
     bool merged = false;  // uniform: whether the group has merged runs
     for (int gi = g0; gi < g1; ++gi) merged = merged || lds_s32(gates + 16u * (uint32_t)gi) == OP_DIAGRUN;
-    if (merged) {
-        fx_merge(gates, g0, g1, origin, cg, ctid, NC / 32);
-        ptx::named_bar_sync(bar_id, NC);
-    }
+    if (merged) fx_merge<NC>(gates, g0, g1, origin, cg, ctid, bar_id);
     uint32_t ld_step[R], st_step[R];
 #pragma unroll
     for (int j = 0; j < R; ++j) {

@@ -2,8 +2,8 @@
 // digits (the splitting scheme of Ozaki, Ogita, Oishi and Rump 2012).
 //
 // A section's chunk becomes block fixed point with one exponent: X = x 2^-e, |X| < 2^55, int64 in
-// place of every double.  A register group is one 2^4 x 2^4 unitary U, M = round(U 2^54), composed
-// by k_compose_fx to 2^-59.  X and M are written in balanced base-256 digits, seven each (digit 0
+// place of every double.  A register group is one 2^4 x 2^4 unitary U, M = round(U 2^(54 + s)), s = 0, 1
+// or 2 as its largest entry allows, composed by k_compose_fx to 2^-59.  X and M are written in balanced base-256 digits, seven each (digit 0
 // the most significant), which FP16 holds exactly; as in the complex64 path a row is the group's 16
 // amplitudes as K = 32 reals, a tile is 128 rows, and
 //     D_d = sum_{i + j = d} A_i B_j,   d = 0..7,   |D_d| <= 7 * 32 * 2^14 < 2^22,
@@ -11,7 +11,7 @@
 // B's blocks j = 0..6 and one of zeros lie side by side along N, so digit i is one MMA of
 // N = 16 (8 - i) per K step for 16 output reals (a half row), its D columns shifted by 16 i:
 // 14 MMAs per half, 1120 cycles per tile at the FP16 rate.  The thread that drains a row sums
-//     V = sum_d D_d 2^{8 (6 - d) - 2} = X U 2^4
+//     V = sum_d D_d 2^{8 (6 - d) - 4} = X U 2^(2 + s)
 // in int64 and stores it to the chunk; the largest V of the chunk sets the shift back to 55 bits
 // that the next group's staging applies, with rounding.  Only a section's first group reads
 // doubles and only its last writes them.
@@ -28,7 +28,7 @@
 // conversions of a group there 1.5.
 //
 // Precision: a unit of X is 2^-54 to 2^-55 of the chunk's largest component; each group rounds once to it,
-// and U is within 2^-55, where FP64 rounds four to eight times per gate.  Chunks with a non-finite
+// and U is within 2^-(55 + s), where FP64 rounds four to eight times per gate.  Chunks with a non-finite
 // component or one whose largest is outside 2^-923 .. 2^1017 run their gates in FP64
 // (fx_group_fp64).
 #pragma once
@@ -47,7 +47,7 @@ struct OzShared {
     unsigned high[kOzMaxSegs];   // largest magnitude's high word after each group
 };
 
-enum : int { OZ_LD = 0, OZ_ST = 256 };  // byte offsets of OzSeg's tables
+enum : int { OZ_LD = 0, OZ_ST = 256, OZ_SCALE = 512 };  // byte offsets of OzSeg's tables
 
 __device__ __forceinline__ uint32_t lds_u32(uint32_t a) {
     uint32_t v;
@@ -122,7 +122,7 @@ __device__ __forceinline__ void fma2(uint32_t x, uint32_t y, float m, uint32_t c
         : "r"(x), "r"(y), "r"(__float_as_uint(m)), "r"(cx), "r"(cy));
 }
 
-// V = sum_d D_d 2^{8 (6 - d) - 2} of an amplitude's two components, D_d exact FP32 integers below
+// V = sum_d D_d 2^{8 (6 - d) - 4} of an amplitude's two components, D_d exact FP32 integers below
 // 2^22 in magnitude.  Adding 1.5 * 2^23 leaves u = D + 2^22 in the low 23 bits of b; for a pair of
 // diagonals P = (b_k << 8) + b_{k+1} = 256 D_k + D_{k+1} + kOff without wrapping (the shift drops
 // the exponent bits), so all offsets are one constant of the 64-bit sum.  D_6 + D_7 / 256 is summed in
@@ -132,18 +132,18 @@ __device__ __forceinline__ void oz_sum(const uint32_t (&dr)[8], const uint32_t (
     constexpr uint32_t kMagicBits = 0x4B400000u;
     constexpr unsigned long long kOff = 0x4B000000ull + 257ull * (1ull << 22);
     constexpr unsigned long long kConst =
-        0ull - (kOff * ((1ull << 38) + (1ull << 22) + (1ull << 6)) + (unsigned long long)kMagicBits);
+        0ull - (kOff * ((1ull << 36) + (1ull << 20) + (1ull << 4)) + (unsigned long long)kMagicBits);
     uint32_t br[6], bi[6], fr, fi, lr, li;
 #pragma unroll
     for (int k = 0; k < 6; ++k) add2(dr[k], di[k], kMagic, br[k], bi[k]);
     fma2(dr[7], di[7], 1.0f / 256, dr[6], di[6], fr, fi);
-    fma2(fr, fi, 0.25f, kMagicBits, kMagicBits, lr, li);
+    fma2(fr, fi, 0.0625f, kMagicBits, kMagicBits, lr, li);
     auto total = [&](const uint32_t (&b)[6], uint32_t low) {
         unsigned long long t = kConst + low;
-        t += (unsigned long long)((b[4] << 8) + b[5]) * 64u;
-        t += (unsigned long long)((b[2] << 8) + b[3]) * (1u << 22);
+        t += (unsigned long long)((b[4] << 8) + b[5]) * 16u;
+        t += (unsigned long long)((b[2] << 8) + b[3]) * (1u << 20);
         const uint32_t p0 = (b[0] << 8) + b[1];
-        return (long long)(t + ((unsigned long long)(p0 << 6) << 32));
+        return (long long)(t + ((unsigned long long)(p0 << 4) << 32));
     };
     vr = total(br, lr);
     vi = total(bi, li);
@@ -281,7 +281,7 @@ __device__ __forceinline__ bool run_chunk_oz(uint32_t buf, uint32_t segs, uint32
     }
     // |X| <= 0.985 * 2^55: seven balanced digits reach 0.996 * 2^55
     const int E = max(top >> 20, 100) + ((top & 0xFFFFF) >= 0xF8000 ? 1 : 0);
-    int e = E - 1077;  // value = X 2^e
+    int e = E - 1077, scale = 0;  // value = X 2^e
     const int lane = ctid & 31, quarter = (threadIdx.x >> 5) & 3, sub = ctid >> 7;
     const uint32_t lane_off = (uint32_t)(quarter * 32) << 16;
     const uint32_t acol = tcol + 2 * kDCols;  // digits: [half of K][digit][8 columns]
@@ -294,7 +294,7 @@ __device__ __forceinline__ bool run_chunk_oz(uint32_t buf, uint32_t segs, uint32
         const uint32_t ld1 = lds_u32(tab + OZ_LD + 4 * 49), ld2 = lds_u32(tab + OZ_LD + 4 * 50);
         const uint32_t st_lane = lds_u32(tab + OZ_ST + 4 * lane) ^ lds_u32(tab + OZ_ST + 4 * (48 + 2 * sub));
         const uint32_t st1 = lds_u32(tab + OZ_ST + 4 * 49), st8 = lds_u32(tab + OZ_ST + 4 * 56);
-        // shift of the last group's sums back to 0.992 * 2^55, with its rounding and the digits' bias
+        // shift of the last group's sums (scale: its s) back to 0.992 * 2^55, with its rounding and the digits' bias
         int shift = 0;
         unsigned long long add = kOzBias;
         if (!first) {
@@ -302,8 +302,9 @@ __device__ __forceinline__ bool run_chunk_oz(uint32_t buf, uint32_t segs, uint32
             shift = max(0, 9 - __clz((int)high));
             shift += (high >> shift) >= 0x7EF000u;
             add = (kOzBias << shift) + ((1ull << shift) >> 1);
-            e += shift - 4;
+            e += shift - 2 - scale;
         }
+        scale = (int)lds_u32(tab + OZ_SCALE);
         int vmax = 0, vmin = 0;  // extreme high words of the group's sums
         // this thread's 4 amplitudes of tile t (group bits 3, 2 = sub) to digit buffer t & 1
         auto stage = [&](int t) {
@@ -351,7 +352,7 @@ __device__ __forceinline__ bool run_chunk_oz(uint32_t buf, uint32_t segs, uint32
                 oz_sum(dr, di, vr, vi);
                 const uint32_t at = buf + (q ? at0 ^ st1 : at0);
                 if (last) {
-                    SM<double>::st(at, oz_to_double(vr, e - 4), oz_to_double(vi, e - 4));
+                    SM<double>::st(at, oz_to_double(vr, e - 2 - scale), oz_to_double(vi, e - 2 - scale));
                 } else {
                     vmax = __vimax3_s32(vmax, (int)(vr >> 32), (int)(vi >> 32));
                     vmin = __vimin3_s32(vmin, (int)(vr >> 32), (int)(vi >> 32));

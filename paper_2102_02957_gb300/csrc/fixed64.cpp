@@ -135,8 +135,8 @@ bool encode_fx(const std::vector<DevGate<double>> &gates, const std::vector<int>
         }
         head.insert(head.end(), {op, (int32_t)off, g.b, g.code});
     }
-    // merged runs: {count, 0, 0, 0}, {payload offset, outside bits, code, 0} per gate, then each
-    // consumer group's 16 entries; the run's first header points here
+    // merged runs: {count, 0, 0, 0}, {payload offset, outside bits, code, 0} per gate, then the
+    // consumer groups' tables; the run's first header points here
     for (size_t i = 0; merge && i < gates.size();) {
         size_t j = i;
         while (j < gates.size() && gates[j].op == OP_DIAGX &&
@@ -151,7 +151,7 @@ bool encode_fx(const std::vector<DevGate<double>> &gates, const std::vector<int>
                 const int32_t row[4] = {head[4 * k + 1], head[4 * k + 2], head[4 * k + 3], 0};
                 put(row, sizeof(row));
             }
-            body.resize(body.size() + (size_t)kFxGroups * 256, 0);
+            body.resize(body.size() + (size_t)kFxRunBytes, 0);
             head[4 * i] = OP_DIAGRUN;
             head[4 * i + 1] = (int32_t)off;
             head[4 * i + 2] = (int32_t)(j - i);

@@ -137,7 +137,8 @@ __global__ void __launch_bounds__(256) k_compose_f64(const ComposeSeg *__restric
 
 // Fused unitary of a complex128 group (block_oz.cuh), in block fixed point with the fixed scale 2^59
 // (all entries of unitaries are at most 1), from the section's own gate area; then
-// M = round(U 2^54) in balanced base-256 digits as FP16 B operands.  One CTA per group, one thread
+// M = round(U 2^(54 + s)) in balanced base-256 digits as FP16 B operands, s the most (up to 2) that
+// keeps |M| within 0.99 * 2^55.  One CTA per group, one thread
 // per element (row r, column j); element products read and write two shared copies in turn.
 __global__ void __launch_bounds__(256) k_compose_fx(const OzCompose *__restrict__ groups, unsigned char *__restrict__ prog) {
     constexpr int NA = 16;
@@ -195,7 +196,18 @@ __global__ void __launch_bounds__(256) k_compose_fx(const OzCompose *__restrict_
     }
     // entries (k, n) = (2j, 2r), (2j + 1, 2r), (2j, 2r + 1), (2j + 1, 2r + 1) = re, -im, im, re
     constexpr long long kBias = 0x0080808080808080ll;
-    const long long re = (fx::value(Ur[cur][e]) + 16) >> 5, im = (fx::value(Ui[cur][e]) + 16) >> 5;
+    const long long ure = fx::value(Ur[cur][e]), uim = fx::value(Ui[cur][e]);
+    __shared__ int top;  // largest |entry| in units of 2^-27
+    if (e == 0) top = 0;
+    __syncthreads();
+    atomicMax(&top, (int)(llabs(ure) >> 32));
+    atomicMax(&top, (int)(llabs(uim) >> 32));
+    __syncthreads();
+    const double most = (double)(top + 1) * 0x1p-27;
+    const int s = most <= 0.495 ? 2 : most <= 0.99 ? 1 : 0;
+    if (e == 0) *reinterpret_cast<int *>(prog + sg.scale_off) = s;
+    const long long half = 16 >> s;
+    const long long re = (ure + half) >> (5 - s), im = (uim + half) >> (5 - s);
     unsigned char *b = prog + sg.b_off + (r >> 3) * (kOzBBytes / 2);
 #pragma unroll
     for (int part = 0; part < 2; ++part) {
@@ -206,8 +218,8 @@ __global__ void __launch_bounds__(256) k_compose_fx(const OzCompose *__restrict_
             const int row = 16 * d + n;  // N row of digit block d
             __half2 v = __floats2half2_rn(0.f, 0.f);
             if (d < 7) {
-                const int s = 8 * (6 - d);
-                v = __floats2half2_rn((float)((int)((lo >> s) & 255) - 128), (float)((int)((hi >> s) & 255) - 128));
+                const int at = 8 * (6 - d);
+                v = __floats2half2_rn((float)((int)((lo >> at) & 255) - 128), (float)((int)((hi >> at) & 255) - 128));
             }
             *reinterpret_cast<__half2 *>(b + (row >> 3) * 512 + (j >> 2) * 128 + (row & 7) * 16 + (j & 3) * 4) = v;
         }

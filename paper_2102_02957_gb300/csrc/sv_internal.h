@@ -172,11 +172,13 @@ constexpr int kOzBBytes = 16384;
 // between the groups' DevSegs and the gate area.
 struct OzSeg {
     uint32_t ld[64], st[64];
+    int32_t scale, unused[3];  // s of the group's operand (written by the composer)
 };
 OzSeg oz_addresses(const HostSeg &seg, int width, bool natural_ld, bool natural_st);
-// One group to compose: gates [g0, g1) of the gate area at gates_off of the program, B at b_off.
+// One group to compose: gates [g0, g1) of the gate area at gates_off of the program, B at b_off, its
+// scale's word at scale_off.
 struct OzCompose {
-    uint32_t gates_off, b_off;
+    uint32_t gates_off, b_off, scale_off;
     int32_t g0, g1;
 };
 void launch_compose_oz(const void *dev_groups, int ngroups, void *dev_prog, cudaStream_t st);
@@ -189,7 +191,9 @@ void gather_outside_diagonals(std::vector<DevGate<double>> &gates, size_t first)
 // are merged where `merge` is set.
 bool encode_fx(const std::vector<DevGate<double>> &gates, const std::vector<int> &group_starts, bool merge,
                std::vector<unsigned char> &out);
-constexpr int kFxGroups = 2;  // consumer groups of the integer-pipe kernel, each with its own merged diagonals
+constexpr int kFxGroups = 2;  // consumer groups of the integer-pipe kernel, each with its own merged diagonals:
+// 16 entries and a part of each for its four warps
+constexpr int kFxRunBytes = kFxGroups * 5 * 256;
 
 // Gate fusion inside a register group (fuse.cpp): replaces gates[first..] by fewer records, and a
 // record in single precision.
@@ -343,9 +347,12 @@ void launch_renorm(int dtype, void *state, int n, const double *partials, int nb
                    cudaStream_t st);
 void launch_partial_expval(int dtype, const void *state, int n, uint64_t x, uint64_t z,
                            double *partials, int nblocks, cudaStream_t st);
-// Result words of a readout: a value and the handle's device error word.
+// (re, im) partial sums of the word's terms in index order, nblocks pairs.
+void launch_partial_expval_direct(int dtype, const void *state, int n, uint64_t x, uint64_t z, double *partials,
+                                  int nblocks, cudaStream_t st);
+// Result words of a readout: a value, the sum of its partials' magnitudes, the handle's error word.
 struct Readout {
-    double value;
+    double value, weight;
     int err;
 };
 // out->value = sum of the partials.
