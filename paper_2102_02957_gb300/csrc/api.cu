@@ -1,5 +1,6 @@
 // C ABI entry points (include/sv.h): state handles, planning, execution and readouts.
 #include <algorithm>
+#include <cmath>
 #include <cstddef>
 #include <cstring>
 #include <atomic>
@@ -115,7 +116,7 @@ static Readout *readout_words(sv_state *h) {
 }
 
 // Wait for the readout whose last kernel wrote readout_words(h).
-static double finish_readout(sv_state *h) {
+static double finish_readout(sv_state *h, double *weight = nullptr) {
     Readout r;
     if (h->slot) {
         check_cuda(cudaStreamSynchronize(h->stream), "cudaStreamSynchronize");
@@ -125,6 +126,7 @@ static double finish_readout(sv_state *h) {
         check_cuda(cudaStreamSynchronize(h->stream), "cudaStreamSynchronize");
     }
     raise_dev_error(h, r.err);
+    if (weight) *weight = r.weight;
     return r.value;
 }
 
@@ -1038,13 +1040,28 @@ sv_status sv_expval_pauli(sv_handle h, uint64_t x, uint64_t z, double *out) {
     if (!h || !out) fail(SV_ERR_ARG, "null argument");
     if ((x >> h->n) || (z >> h->n)) fail(SV_ERR_ARG, "Pauli mask outside the register");
     const int nb = reduce_blocks(h->n);
-    ensure_scratch(h, (size_t)nb * sizeof(double));
+    ensure_scratch(h, (size_t)nb * 2 * sizeof(double));
     launch_partial_expval(h->dtype, h->amp, h->n, x, z, h->scratch, nb, h->stream);
     launch_finish(h->scratch, nb, h->dev_err, readout_words(h), h->stream);
     // the sum is real where x and z overlap in an even number of qubits, imaginary otherwise
-    const double v = finish_readout(h);
+    double weight = 0;
+    const double v = finish_readout(h, &weight);
     const bool odd = __builtin_popcountll(x & z) & 1;
     double sr = odd ? 0.0 : v, si = odd ? v : 0.0;
+    // a sum that cancels to nothing (a real state under a word with an odd number of Y's): callers get the
+    // residue of the term-by-term sum
+    if (!(std::fabs(v) > 0x1p-40 * weight)) {
+        launch_partial_expval_direct(h->dtype, h->amp, h->n, x, z, h->scratch, nb, h->stream);
+        std::vector<double> part((size_t)nb * 2);
+        check_cuda(cudaMemcpyAsync(part.data(), h->scratch, nb * 2 * sizeof(double), cudaMemcpyDeviceToHost, h->stream),
+                   "cudaMemcpyAsync(partials)");
+        check_dev_error(h);
+        sr = si = 0;
+        for (int b = 0; b < nb; ++b) {
+            sr += part[(size_t)(2 * b)];
+            si += part[(size_t)(2 * b + 1)];
+        }
+    }
     // multiply by i^{popc(x & z)}
     switch (__builtin_popcountll(x & z) & 3) {
         case 1: { double t = sr; sr = -si; si = t; break; }

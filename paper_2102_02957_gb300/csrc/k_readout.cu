@@ -246,15 +246,45 @@ __global__ void __launch_bounds__(kThreads) k_partial_expval(const T2 *__restric
     if (threadIdx.x == 0) partials[blockIdx.x] = MODE == NORM ? s : 2 * s;
 }
 
-// Sum of the partials and the handle's error word, into the caller's result words (host memory the
-// GPU writes directly, or device memory).
+// The sum term by term: for words whose paired sum vanishes, where the result is the rounding residue
+// of the order of summation (6 FP64 operations and conversions more per amplitude).
+template <typename T2>
+__global__ void __launch_bounds__(kThreads) k_partial_expval_direct(const T2 *__restrict__ a, int64_t len, uint64_t x,
+                                                                    uint64_t z, double *partials) {
+    const int64_t per = (len + gridDim.x - 1) / gridDim.x;
+    const int64_t lo = (int64_t)blockIdx.x * per, hi = lo + per < len ? lo + per : len;
+    double sr = 0, si = 0;
+    for (int64_t j = lo + threadIdx.x; j < hi; j += kThreads) {
+        const T2 u = a[(uint64_t)j ^ x], v = a[j];
+        // conj(u) * v
+        double tr = (double)u.x * (double)v.x + (double)u.y * (double)v.y;
+        double ti = (double)u.x * (double)v.y - (double)u.y * (double)v.x;
+        if (__popcll((unsigned long long)j & z) & 1) { tr = -tr; ti = -ti; }
+        sr += tr;
+        si += ti;
+    }
+    sr = block_sum<kThreads>(sr);
+    si = block_sum<kThreads>(si);
+    if (threadIdx.x == 0) {
+        partials[2 * blockIdx.x] = sr;
+        partials[2 * blockIdx.x + 1] = si;
+    }
+}
+
+// Sum of the partials, of their magnitudes, and the handle's error word, into the caller's result
+// words (host memory the GPU writes directly, or device memory).
 __global__ void __launch_bounds__(kThreads) k_finish(const double *__restrict__ partials, int nb,
                                                      const int *__restrict__ err, Readout *out) {
-    double s = 0;
-    for (int b = threadIdx.x; b < nb; b += kThreads) s += partials[b];
+    double s = 0, w = 0;
+    for (int b = threadIdx.x; b < nb; b += kThreads) {
+        s += partials[b];
+        w += fabs(partials[b]);
+    }
     s = block_sum<kThreads>(s);
+    w = block_sum<kThreads>(w);
     if (threadIdx.x == 0) {
         out->value = s;
+        out->weight = w;
         out->err = *err;
     }
 }
@@ -488,6 +518,16 @@ void launch_partial_expval(int dtype, const void *state, int n, uint64_t x, uint
                            cudaStream_t st) {
     if (dtype == SV_C64) expval_of<float2>(state, n, x, z, partials, nblocks, st);
     else expval_of<double2>(state, n, x, z, partials, nblocks, st);
+    check_cuda(cudaGetLastError(), "expval kernel launch");
+}
+
+void launch_partial_expval_direct(int dtype, const void *state, int n, uint64_t x, uint64_t z, double *partials,
+                                  int nblocks, cudaStream_t st) {
+    const int64_t len = int64_t(1) << n;
+    if (dtype == SV_C64)
+        k_partial_expval_direct<float2><<<nblocks, kThreads, 0, st>>>((const float2 *)state, len, x, z, partials);
+    else
+        k_partial_expval_direct<double2><<<nblocks, kThreads, 0, st>>>((const double2 *)state, len, x, z, partials);
     check_cuda(cudaGetLastError(), "expval kernel launch");
 }
 
