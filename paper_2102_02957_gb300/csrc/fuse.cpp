@@ -3,10 +3,12 @@
 // A gate costs a thread its products and, whatever it does, about 90 integer instructions for its 16
 // amplitudes (reading the record, branching to its bits, moving results back), nearly as many as the
 // products of a dense one-qubit gate.  So gates whose fused matrix costs no more than they do apart
-// become one record: a one-qubit gate joins the last dense gate on its bit,
-// a two-qubit gate takes up the dense one-qubit gates waiting on both of its bits, and two-qubit
-// gates on the same pair are multiplied.  Matrices are multiplied in FP64 and rounded to FP32 once.
-// n = 27, 10 random layers in sections of 13 bits: 34.3 -> 28.8 ms.
+// become one record: a one-qubit gate joins the last dense gate on its bit, a two-qubit gate takes up
+// the one-qubit gates waiting on its bits if they are dense on both or it is dense itself, and
+// two-qubit gates on the same pair, one of them dense, are multiplied.  So a record mixes only
+// amplitudes that the separate gates mix (a non-finite one spreads as far as before).  Matrices are
+// multiplied in FP64 and rounded to FP32 once.  n = 27, 10 random layers in sections of 13 bits: 34.4 ->
+// 28.9 ms.
 #include <cstring>
 #include <vector>
 
@@ -70,18 +72,6 @@ void make_dense(Gate &g, const double *m) {
     std::memcpy(g.m, m, (one ? 8 : 32) * sizeof(double));
 }
 
-// real multiply-adds per amplitude
-int products(const Gate &g) {
-    switch (g.op) {
-        case OP_DENSE1: return 8;
-        case OP_DENSE2: return 16;
-        case OP_DIAG1: case OP_DIAG2: case OP_DIAGX: return 4;
-        default: return 0;
-    }
-}
-
-constexpr int kRecord = 6;  // a record's own instructions per amplitude
-
 }  // namespace
 
 void fuse_gates(std::vector<DevGate<double>> &gates, size_t first) {
@@ -111,7 +101,13 @@ void fuse_gates(std::vector<DevGate<double>> &gates, size_t first) {
     for (size_t i = first; i < gates.size(); ++i) {
         const Gate &g = gates[i];
         if (one_bit(g)) {
-            if (waiting[g.a]) {
+            if (waiting[g.a] && wait[g.a].op == OP_DIAG1 && g.op == OP_DIAG1) {
+                for (int l = 0; l < 4; l += 2) {
+                    const double re = wait[g.a].m[l], im = wait[g.a].m[l + 1];
+                    wait[g.a].m[l] = g.m[l] * re - g.m[l + 1] * im;
+                    wait[g.a].m[l + 1] = g.m[l] * im + g.m[l + 1] * re;
+                }
+            } else if (waiting[g.a]) {
                 dense(g, x);
                 dense(wait[g.a], y);
                 multiply(2, x, y, z);
@@ -139,11 +135,9 @@ void fuse_gates(std::vector<DevGate<double>> &gates, size_t first) {
             make_dense(p, z);
             continue;
         }
-        int apart = products(g) + kRecord;
-        for (int b : {g.a, g.b})
-            if (waiting[b]) apart += products(wait[b]) + kRecord;
+        const bool both = waiting[g.a] && waiting[g.b] && wait[g.a].op == OP_DENSE1 && wait[g.b].op == OP_DENSE1;
         Gate f = g;
-        if (apart >= 16 + kRecord && (waiting[g.a] || waiting[g.b])) {
+        if (both || (g.op == OP_DENSE2 && (waiting[g.a] || waiting[g.b]))) {
             dense(g, x);
             for (int b : {g.a, g.b})
                 if (waiting[b]) {
