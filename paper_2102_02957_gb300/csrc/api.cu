@@ -210,7 +210,7 @@ static void build_programs_tc(const sv_plan *plan, const sv_gate *gates, int r_p
         int r, width;
         GatherLayout lay;
         std::vector<BlockGate> gates;
-        std::vector<HostSeg> segs;
+        Groups segs;
     };
     std::vector<Section> secs;
     for (size_t oi = 0; oi < plan->ops.size(); ++oi) {
@@ -233,11 +233,15 @@ static void build_programs_tc(const sv_plan *plan, const sv_gate *gates, int r_p
         if (sc.width - plan->reserve < sc.r + 7) fail(SV_ERR_PLAN, "a section's chunk is too small for its register-group width");
         secs.push_back(std::move(sc));
     }
-    // register groups of every section (independent searches, spread over host threads; each
-    // section's result is its own, so the program does not depend on the threading)
-    parallel_for((int)secs.size(), [&](int i) {
-        Section &sc = secs[(size_t)i];
-        sc.segs = segment_block(sc.gates, sc.width, sc.r, 8);
+    // register groups of every section: the plan's, or (its first execution) independent searches
+    // spread over host threads; each section's result is its own, so the program does not depend on
+    // the threading
+    std::vector<Section *> fresh;
+    for (Section &sc : secs)
+        if (!(sc.segs = plan_groups(*plan, (int)sc.oi, sc.r, 8))) fresh.push_back(&sc);
+    parallel_for((int)fresh.size(), [&](int i) {
+        Section &sc = *fresh[(size_t)i];
+        sc.segs = keep_groups(*plan, (int)sc.oi, sc.r, 8, segment_block(sc.gates, sc.width, sc.r, 8));
     });
     for (const Section &sc : secs) {
         const size_t oi = sc.oi;
@@ -246,7 +250,7 @@ static void build_programs_tc(const sv_plan *plan, const sv_gate *gates, int r_p
         const int kMaxTcSegs = max_tc_segs(r);
         const int b_bytes = tc_b_bytes(r);
         const GatherLayout &lay = sc.lay;
-        const std::vector<HostSeg> &segs = sc.segs;
+        const std::vector<HostSeg> &segs = *sc.segs;
         for (size_t p0 = 0; p0 < segs.size(); p0 += kMaxTcSegs) {
             const size_t p1 = std::min(segs.size(), p0 + (size_t)kMaxTcSegs);
             BlockProg bp{};
@@ -359,8 +363,16 @@ static void build_programs(const sv_plan *plan, const sv_gate *gates, int seg_bi
         const unsigned char *p = static_cast<const unsigned char *>(data);
         host.insert(host.end(), p, p + bytes);
     };
-    auto section = [&](BlockProg bp, const std::vector<BlockGate> &section_gates, int width) {
-        std::vector<HostSeg> segs = segment_block(section_gates, width, seg_bits, (int)(2 * sizeof(T)));
+    // whole: all gates of the plan's section, whose register groups the plan keeps
+    auto section = [&](BlockProg bp, const std::vector<BlockGate> &section_gates, int width, bool whole) {
+        const int elem = (int)(2 * sizeof(T));
+        Groups kept = whole ? plan_groups(*plan, bp.op_index, seg_bits, elem) : nullptr;
+        if (!kept) {
+            std::vector<HostSeg> found = segment_block(section_gates, width, seg_bits, elem);
+            kept = whole ? keep_groups(*plan, bp.op_index, seg_bits, elem, std::move(found))
+                         : std::make_shared<const std::vector<HostSeg>>(std::move(found));
+        }
+        const std::vector<HostSeg> &segs = *kept;
         std::vector<DevSeg> dsegs;
         std::vector<DevGate<T>> dgates;
         for (const HostSeg &s : segs) {
@@ -487,12 +499,12 @@ static void build_programs(const sv_plan *plan, const sv_gate *gates, int seg_bi
             const size_t nm = segment_block(main, width, seg_bits, (int)(2 * sizeof(T))).size();
             const size_t nt = segment_block(tail, width, seg_bits, (int)(2 * sizeof(T))).size();
             if (2 * nm > nt + 1) {
-                section(bp, main, width);
-                section(bp, tail, width);
+                section(bp, main, width, false);
+                section(bp, tail, width, false);
                 continue;
             }
         }
-        section(bp, local, width);
+        section(bp, local, width, true);
     }
     align(256);
 }

@@ -887,6 +887,18 @@ void encode_gate(const sv_gate &g, const BlockGate &bg, const HostSeg &seg, DevG
     }
 }
 
+Groups plan_groups(const sv_plan &plan, int op_index, int r, int elem_bytes) {
+    std::lock_guard<std::mutex> lk(plan.groups_mu);
+    const auto it = plan.groups.find({op_index, r, elem_bytes});
+    return it == plan.groups.end() ? nullptr : it->second;
+}
+
+Groups keep_groups(const sv_plan &plan, int op_index, int r, int elem_bytes, std::vector<HostSeg> segs) {
+    Groups g = std::make_shared<const std::vector<HostSeg>>(std::move(segs));
+    std::lock_guard<std::mutex> lk(plan.groups_mu);
+    return plan.groups.emplace(std::array<int, 3>{op_index, r, elem_bytes}, g).first->second;
+}
+
 // Register groups over all blocking sections of a plan (statistics; the same groups the section
 // programs get).
 int plan_segment_count(const sv_plan &plan) {
