@@ -385,18 +385,11 @@ static void build_programs(const sv_plan *plan, const sv_gate *gates, int seg_bi
             for (int k = 0; k < s.nrest; ++k) d.rest[k] = (int8_t)s.rest[k];
             d.flags = (int8_t)s.flags;
             d.g0 = (int16_t)dgates.size();
-            std::vector<DevGate<double>> group;
             for (int32_t gi : s.gates) {
-                DevGate<double> dg;
+                DevGate<T> dg;
                 const BlockGate &bg = section_gates[gi];
-                encode_gate<double>(gates[bg.gi], bg, s, dg);
-                group.push_back(dg);
-            }
-            if constexpr (sizeof(T) == 4) {
-                fuse_gates(group, 0);
-                for (const DevGate<double> &g : group) dgates.push_back(narrow(g));
-            } else {
-                dgates.insert(dgates.end(), group.begin(), group.end());
+                encode_gate<T>(gates[bg.gi], bg, s, dg);
+                dgates.push_back(dg);
             }
             if (dgates.size() > 32767) fail(SV_ERR_UNSUPPORTED, "too many gates in one blocking section");
             d.g1 = (int16_t)dgates.size();

@@ -229,14 +229,11 @@ sv_status sv_batch_create(int32_t count, const sv_handle *states, const sv_gate 
                     d.flags = (int8_t)((q == 0 ? 1 : 0) | (q + 1 == segs.size() ? 2 : 0));
                     d.g0 = (int16_t)dg.size();
                     if (!tc) {
-                        std::vector<DevGate<double>> group;
                         for (int32_t gi : hs.gates) {
-                            DevGate<double> g;
-                            encode_gate<double>(gates[s][loc[gi].gi], loc[gi], hs, g);
-                            group.push_back(g);
+                            DevGate<float> g;
+                            encode_gate<float>(gates[s][loc[gi].gi], loc[gi], hs, g);
+                            dg.push_back(g);
                         }
-                        fuse_gates(group, 0);
-                        for (const DevGate<double> &g : group) dg.push_back(narrow(g));
                     }
                     d.g1 = (int16_t)dg.size();
                     ds.push_back(d);

@@ -209,11 +209,6 @@ constexpr int kFxGroups = 2;  // consumer groups of the integer-pipe kernel, eac
 // 16 entries and a part of each for its four warps
 constexpr int kFxRunBytes = kFxGroups * 5 * 256;
 
-// Gate fusion inside a register group (fuse.cpp): replaces gates[first..] by fewer records, and a
-// record in single precision.
-void fuse_gates(std::vector<DevGate<double>> &gates, size_t first);
-DevGate<float> narrow(const DevGate<double> &g);
-
 // Gathered chunk: the state is viewed as a tensor of rank <= 5 whose dimension d covers the
 // index bits [s[d], s[d+1]); each dimension starts with a run of chunk bits (its box, at most
 // 8 bits), the bits above it up to the next dimension are addressed by coordinates.  Chunk bits
