@@ -207,6 +207,7 @@ __device__ __forceinline__ void oz_issue(int half, uint32_t bops, int nseg, int 
             }
             ptx::tc_fence_after();
             const bool skip = *(volatile const int *)&sh->skip != 0;  // only with a chunk's first tile
+            __syncwarp();  // every lane has read it before the commit below lets the consumers clear it for their next chunk
             if ((threadIdx.x & 31) == 0) {
                 const uint32_t a = tcol + 2 * kDCols + (uint32_t)((k % T & 1) * kACols);
                 const uint64_t bd = ptx::smem_desc_kmajor(bops + (uint32_t)(k / T) * kOzBBytes, 128, 512) +
