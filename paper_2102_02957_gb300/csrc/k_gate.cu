@@ -11,8 +11,11 @@
 // A sweep touches only the amplitudes that its gate can change: local basis states whose row and
 // column are those of the identity are left out, so a controlled gate moves half of the state and a
 // controlled phase a quarter, and an exchange (X, CNOT, SWAP) moves amplitudes without arithmetic.
-// Complex128 products run in block fixed point on the integer pipe (fixed64.cuh).  480 gates of
+// Complex128 products run in block fixed point on the integer pipe (fixed64.cuh) where that is as exact,
+// amplitude by amplitude (apply_fx).  480 gates of
 // random layers on 16 qubits, complex128: 3.94 ms with every gate dense in FP64, 1.97 ms so.
+#include <cmath>
+
 #include "fixed64.cuh"
 #include "sv_internal.h"
 
@@ -228,13 +231,15 @@ __global__ void __launch_bounds__(kThreads) k_gate_c64(float4 *a, const __grid_c
     }
 }
 
-// Dense on the NA touched local states, complex128: FP64 values, and the fixed-point factors of a
-// unitary gate (FX).
+// Dense on the NA touched local states, complex128: FP64 values, and the fixed-point factors and
+// moduli of a unitary gate (FX).
 template <int NA>
 struct MatC128 {
     double m[2 * NA * NA];
     int32_t e[4 * NA * NA];
+    float w[NA * NA];  // non-zero ones at least kLeast
 };
+constexpr float kLeast = 0x1p-60f;
 
 template <int NA>
 __device__ __forceinline__ void apply_fp64(const double *m, double2 (&U)[NA]) {
@@ -250,6 +255,18 @@ __device__ __forceinline__ void apply_fp64(const double *m, double2 (&U)[NA]) {
     for (int r = 0; r < NA; ++r) U[r] = y[r];
 }
 
+// An amplitude's larger component as a share of the group's largest (high word top), to 12 %; 0 for a zero, else at
+// least kLeast.
+__device__ __forceinline__ float share_of(const double2 &x, int top) {
+    const int hi = max(__double2hiint(x.x) & 0x7FFFFFFF, __double2hiint(x.y) & 0x7FFFFFFF);
+    const float f = __int_as_float(max(hi - top + (127 << 20), 67 << 20) << 3);
+    return (hi | __double2loint(x.x) | __double2loint(x.y)) ? f : 0.0f;
+}
+
+// Fixed point is off by at most 3 units of 2^-58 of the largest component per output, FP64 by about 3.5 units of
+// 2^-53 of w = sum |m| |x| over the output's products.  So a group takes fixed point where every output
+// that is not structurally zero has w >= 1/32 of the largest component, and FP64 elsewhere: an amplitude
+// far below its partners that no product of theirs reaches keeps its digits.
 template <int NA>
 __device__ __forceinline__ void apply_fx(const MatC128<NA> &M, double2 (&U)[NA]) {
     int top = 0, any = 0;
@@ -258,7 +275,20 @@ __device__ __forceinline__ void apply_fx(const MatC128<NA> &M, double2 (&U)[NA])
         fx::scan(U[j].x, top, any);
         fx::scan(U[j].y, top, any);
     }
-    if (fx::special(top, any)) {
+    bool near = !fx::special(top, any);
+    if (NA > 1) {
+        float f[NA];
+#pragma unroll
+        for (int j = 0; j < NA; ++j) f[j] = share_of(U[j], top);
+#pragma unroll
+        for (int r = 0; r < NA; ++r) {
+            float w = 0.0f;
+#pragma unroll
+            for (int c = 0; c < NA; ++c) w = fmaf(M.w[NA * r + c], f[c], w);
+            near = near && !(w > 0.0f && w < 1.0f / 32);
+        }
+    }
+    if (!near) {
         apply_fp64<NA>(M.m, U);
         return;
     }
@@ -428,6 +458,10 @@ void launch_c128(void *state, const Touched &t, int n, int nq, const int *q, cud
     const bool small = P.groups <= (int64_t)num_sms() * kThreads * kUnroll;  // at most one CTA per SM
     if (fx_unitary(t.m, NA)) {
         fx_pack(t.m, NA * NA, P.m.e);
+        for (int i = 0; i < NA * NA; ++i) {
+            const double a = std::hypot(t.m[2 * i], t.m[2 * i + 1]);
+            P.m.w[i] = a > 0 ? std::max((float)a, kLeast) : 0.0f;
+        }
         if (small) launch_after(k_gate_c128<NA, true, 1>, grid_for(P.groups, 1), kThreads, st, a, P);
         else launch_after(k_gate_c128<NA, true, kUnroll>, grid_for(P.groups), kThreads, st, a, P);
     } else {
