@@ -108,7 +108,9 @@ typedef struct sv_options {
                                on expiry the kernel stops and the next synchronising call returns
                                SV_ERR_TIMEOUT.  0: the default (4000 ms).  Taken by sv_apply_circuit
                                from the plan's options. */
-    int32_t reserved[4];
+    int32_t fp64_sections;  /* 1: blocking sections of complex128 states run in FP64 throughout (slower;
+                               sv_apply_circuit states what the default keeps).  default 0 */
+    int32_t reserved[3];
 } sv_options;
 
 void sv_options_default(sv_options *opts);
@@ -184,7 +186,14 @@ sv_status sv_plan_serialize(sv_plan_h plan, int64_t *buf, int64_t cap, int64_t *
  * paper's baseline of Sec. V.A).  Otherwise the cache-blocked path (Listing 4): each chunk_swap
  * round is one in-place permutation pass and each blocking section one pass in which every
  * chunk is staged in shared memory, all its gates applied, and written back.  The plan must
- * have been made from the same n and gate list (SV_ERR_PLAN otherwise). */
+ * have been made from the same n and gate list (SV_ERR_PLAN otherwise).
+ * Precision.  complex64: FP32 per gate (tensor cores: 3xTF32 per register group).  complex128, per-gate path:
+ * every amplitude as exact as FP64 gives it.  complex128 sections: FP64, or, where that takes at least twice
+ * as long, block fixed point with a unit of 2^-54 of the chunk's largest component per register group.  A
+ * chunk is given to fixed point only if its amplitudes are comparable in size (all within 2^4 of the largest
+ * component; where the section's gates mix at least 6 of the chunk's qubits, all but 1 in 32 within
+ * 2^8) or all results turn out to be; its errors are then no larger than FP64's would be.  Other chunks, and plans with
+ * fp64_sections, run in FP64. */
 sv_status sv_apply_circuit(sv_handle h, const sv_gate *gates, int64_t n_gates, sv_plan_h plan);
 
 /* ------------------------------------------------------------------ partitioned states */
@@ -196,7 +205,7 @@ sv_status sv_apply_circuit(sv_handle h, const sv_gate *gates, int64_t n_gates, s
  * amplitude (piece index << h->n) | k.
  *
  * Run plan ops [op_begin, op_end) of a plan made with gather_pinned = 0 (contiguous chunks) on
- * the piece: blocking sections with SIMT register groups (the chunk must fit the piece: c <= h->n),
+ * the piece: blocking sections (without complex64 tensor cores; the chunk must fit the piece: c <= h->n),
  * and the chunk_swap / reordering pairs whose two bits are both below h->n.  Pairs with a bit at
  * or above h->n are left to the caller, who exchanges data between pieces with sv_shard_pack /
  * sv_shard_unpack.  With h->n == plan n this is a part of sv_apply_circuit (without its
@@ -223,8 +232,8 @@ sv_status sv_shard_unpack(sv_handle h, int32_t bit, int32_t value, const void *d
  * of the plan's own schedule (circuits without SWAP relabels, plans that restore the layout; the
  * result is the same up to rounding).  dev_work: a DEVICE buffer of work_bytes
  * (the caller's), or NULL to let the library allocate work_bytes for the call; it must hold two
- * sub-states of 2^(c+2) amplitudes unless it holds the whole state twice.  Sections run on SIMT
- * register groups.  Synchronous: returns when the state in host memory is final.  passes (may be
+ * sub-states of 2^(c+2) amplitudes unless it holds the whole state twice.  Sections run as in
+ * sv_apply_plan_ops.  Synchronous: returns when the state in host memory is final.  passes (may be
  * NULL): the number of passes over the state.  SV_ERR_PLAN / SV_ERR_UNSUPPORTED as for
  * sv_apply_circuit and for gathered plans; SV_ERR_ARG for a work buffer that is too small. */
 sv_status sv_apply_circuit_host(int32_t n, int32_t dtype, void *host_amps, const sv_gate *gates,

@@ -301,7 +301,7 @@ class Batch:
 
 
 _OPT_KEYS = ("chunk_bits", "reserve", "restore_layout", "seg_bits", "use_tc", "use_model", "threads", "gather_pinned",
-             "diag_outside", "lookahead", "tc_no_renorm", "wait_limit_ms")
+             "diag_outside", "lookahead", "tc_no_renorm", "wait_limit_ms", "fp64_sections")
 
 
 def batch_tune(states, gate_lists, **base):

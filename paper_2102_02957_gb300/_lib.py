@@ -29,7 +29,7 @@ class sv_options(ctypes.Structure):
                 ("seg_bits", ctypes.c_int32), ("use_tc", ctypes.c_int32), ("use_model", ctypes.c_int32),
                 ("threads", ctypes.c_int32), ("gather_pinned", ctypes.c_int32), ("diag_outside", ctypes.c_int32),
                 ("lookahead", ctypes.c_int32), ("tc_no_renorm", ctypes.c_int32), ("wait_limit_ms", ctypes.c_int32),
-                ("reserved", ctypes.c_int32 * 4)]
+                ("fp64_sections", ctypes.c_int32), ("reserved", ctypes.c_int32 * 3)]
 
 
 class sv_plan_info(ctypes.Structure):

@@ -141,13 +141,11 @@ static void validate_gates(int n, const sv_gate *gates, int64_t n_gates) {
     }
 }
 
-// Device program of one blocking section: register groups, then gate records, laid out as
-// the kernel copies them into shared memory.
+// Device program of one tensor-core sweep of a complex64 section: register groups, then B operands, laid
+// out as the kernel copies them into shared memory.
 struct BlockProg {
     size_t off;
-    int nseg, gate_bytes;  // SIMT: bytes of the gate area
-    bool fixed = false;    // complex128: fixed-point gate area
-    bool oz = false;       // complex128: tensor-core sweep (block_oz.cuh)
+    int nseg;
     int r = 0;         // tensor-core register-group width of the sweep
     GatherLayout lay;  // gathered sections only
     int op_index = -1;
@@ -261,7 +259,6 @@ static void build_programs_tc(const sv_plan *plan, const sv_gate *gates, int r_p
             align(256);
             bp.off = host.size();
             bp.nseg = (int)(p1 - p0);
-            bp.gate_bytes = 0;
             for (size_t k = p0; k < p1; ++k) {
                 const HostSeg &s = segs[k];
                 DevSeg d;
@@ -320,6 +317,7 @@ static void build_programs_tc(const sv_plan *plan, const sv_gate *gates, int r_p
 // is not unitary.
 static bool split_outside(const std::vector<BlockGate> &all, const sv_gate *gates, std::vector<BlockGate> &main,
                           std::vector<BlockGate> &tail) {
+    if (std::none_of(all.begin(), all.end(), [](const BlockGate &g) { return g.ext[0] >= 0 || g.ext[1] >= 0; })) return false;
     uint64_t later = 0;  // chunk bits that a later gate does not leave diagonal
     bool fits = true;
     for (size_t i = all.size(); i-- > 0;) {
@@ -346,30 +344,172 @@ static bool split_outside(const std::vector<BlockGate> &all, const sv_gate *gate
     return fits && !main.empty() && !tail.empty();
 }
 
-// Section programs with SIMT register groups, and (complex128, `oz` non-null) tensor-core sweeps:
-// sections of unitary gates that do more than exchange amplitudes and flip signs, none of them outside
-// its chunk, on chunks that hold a 128-row tile.  There a group costs about as much whatever its
-// gates are, less than one dense gate costs on the integer pipe (block_fx.cuh).  A section with
-// more groups than fit beside the chunks takes several sweeps.  *oz receives the groups to compose.
+// Clocks per amplitude and SM below which FP64 register groups take a section, per group.  The digit
+// products take 2.3 a group and the integer pipe 1.5 and about 0.35 of what the gates take in FP64
+// (fp64_clocks), so at this line either is twice as fast.  Lighter sections (a gate or two per
+// group) keep FP64.
+constexpr double kFixedClocks = 4.7;
+
+// The Dense rule of register groups [s0, s1) on chunks of `width` bits.
+static Dense dense_rule(const std::vector<DevSeg> &segs, const std::vector<DevGate<double>> &gates, int s0, int s1, int width) {
+    unsigned touched = 0, mixed = 0;
+    double ratio = 1;
+    for (int k = s0; k < s1; ++k)
+        for (int g = segs[(size_t)k].g0; g < segs[(size_t)k].g1; ++g) {
+            const DevGate<double> &dg = gates[(size_t)g];
+            if (dg.op != OP_DENSE1 && dg.op != OP_DENSE2) continue;
+            const unsigned a = 1u << segs[(size_t)k].pos[dg.a], b = dg.op == OP_DENSE2 ? 1u << segs[(size_t)k].pos[dg.b] : 0u;
+            const int m = mixed_bits(dg);
+            touched |= a | b;
+            ratio *= entry_ratio(dg);
+            mixed |= ((m & 1) ? a : 0u) | ((m & 2) ? b : 0u);
+        }
+    const int nm = __builtin_popcount(mixed);
+    const int trial = ratio <= (double)(1 << (2 * kNearOrders));
+    if (nm < kMixedBits) return Dense{kNearOrders, 0, touched, trial};
+    return Dense{kFarOrders, std::min(1 << (nm - 1), (1 << width) / 32), touched, trial};
+}
+
+// Section programs with SIMT register groups.  complex128 sections of unitary gates run in fixed point or
+// on the tensor cores where that is twice as fast as FP64: on the tensor cores if none of their gates has a
+// qubit outside its chunk and the chunk holds a 128-row tile (a group costs about as much there whatever its
+// gates are, less than one dense gate on the integer pipe, block_fx.cuh), in as many sweeps as
+// their groups need.  Each such sweep has an FP64 program too, for the chunks it leaves (Redo).
 template <typename T>
-static void build_programs(const sv_plan *plan, const sv_gate *gates, int seg_bits, std::vector<unsigned char> &host,
-                           std::vector<BlockProg> &progs, std::vector<OzCompose> *oz = nullptr) {
-    host.clear();
-    progs.clear();
-    auto align = [&](size_t a) {
-        while (host.size() % a) host.push_back(0);
-    };
-    auto put = [&](const void *data, size_t bytes) {
+struct ProgramBuilder {
+    const sv_plan *plan;
+    const sv_gate *gates;
+    int seg_bits;
+    std::vector<unsigned char> &host;
+    std::vector<SimtPrograms::Prog> &progs;
+    std::vector<OzCompose> &oz;  // receives the groups to compose
+    static constexpr int kElem = (int)(2 * sizeof(T));
+
+    void align(size_t a) { host.resize((host.size() + a - 1) / a * a, 0); }
+    void put(const void *data, size_t bytes) {
         const unsigned char *p = static_cast<const unsigned char *>(data);
         host.insert(host.end(), p, p + bytes);
-    };
+    }
+    // Register groups [s0, s1) and their gate area as one program; returns its offset.
+    size_t put_program(const std::vector<DevSeg> &segs, int s0, int s1, bool raw_flags, const void *area, size_t bytes) {
+        align(256);
+        const size_t off = host.size();
+        const int g0 = segs[(size_t)s0].g0;
+        for (int k = s0; k < s1; ++k) {
+            DevSeg d = segs[(size_t)k];
+            d.flags = (int8_t)((k == s0 ? 1 : 0) | (k + 1 == s1 ? 2 : 0) | (raw_flags ? d.flags & kSegRaw : 0));
+            d.g0 = (int16_t)(d.g0 - g0);
+            d.g1 = (int16_t)(d.g1 - g0);
+            put(&d, sizeof(d));
+        }
+        align(16);
+        put(area, bytes);
+        align(16);
+        return off;
+    }
+
+    // A complex128 section off FP64; false: it stays there.
+    bool fixed_section(SimtPrograms::Prog pg, const std::vector<HostSeg> &segs, std::vector<DevSeg> &dsegs,
+                       const std::vector<DevGate<double>> &all, int width) {
+        const int nseg = (int)dsegs.size();
+        bool exact = true;  // only exchanges and signs
+        for (DevSeg &d : dsegs) {
+            if (std::all_of(all.begin() + d.g0, all.begin() + d.g1, exact_gate)) d.flags |= kSegRaw;
+            else exact = false;
+        }
+        if (nseg == 0) return false;
+        if (!exact) {
+            double fp64 = 0;
+            for (const DevGate<double> &g : all) fp64 += fp64_clocks(g);
+            if (plan->fp64 || !(fp64 > kFixedClocks * nseg)) return false;
+        }
+        const bool outside = std::any_of(all.begin(), all.end(), [](const DevGate<double> &g) { return g.op == OP_DIAGX; });
+        if (!exact && plan->n - width < 31 && (1 << (plan->n - width)) <= num_sms()) {
+            // With at most a chunk per SM a sweep in vain is felt: 15 us beside 45 to 60 in FP64.  Real circuits leave
+            // states too uneven for one exponent (a 14-qubit RY/CZ ansatz: every chunk of every section), and the
+            // integer pipe alone wins a third at most.
+            if (std::all_of(all.begin(), all.end(), real_gate) || (!outside && oz_max_segs(width) == 0)) return false;
+        }
+        std::vector<DevGate<double>> moved;
+        std::vector<int> starts;
+        for (const DevSeg &d : dsegs) {
+            starts.push_back(d.g0);
+            if (!outside) continue;
+            std::vector<DevGate<double>> group(all.begin() + d.g0, all.begin() + d.g1);
+            gather_outside_diagonals(group, 0);
+            moved.insert(moved.end(), group.begin(), group.end());
+        }
+        const std::vector<DevGate<double>> &dgates = outside ? moved : all;
+        std::vector<unsigned char> area, merged;
+        if (!encode_fx(dgates, starts, false, area)) return false;
+        const int per = exact || outside ? 0 : oz_max_segs(width);
+        auto bounds = [&](int w, int sweeps) { return (int)((int64_t)nseg * w / sweeps); };
+        int sweeps = per > 0 ? (nseg + per - 1) / per : 1;
+        // more of them where an FP64 program would not fit beside a chunk
+        auto fits = [&] {
+            for (int w = 0; w < sweeps; ++w) {
+                const int s0 = bounds(w, sweeps), s1 = bounds(w + 1, sweeps);
+                if (simt_buffers(width, s1 - s0, (size_t)(dsegs[(size_t)s1 - 1].g1 - dsegs[(size_t)s0].g0) * sizeof(DevGate<double>)) == 0)
+                    return false;
+            }
+            return true;
+        };
+        while (!exact && !fits())
+            if (++sweeps > nseg) return false;
+        for (int w = 0; w < sweeps; ++w) {
+            const int s0 = bounds(w, sweeps), s1 = bounds(w + 1, sweeps);
+            const int g0 = dsegs[(size_t)s0].g0, g1 = dsegs[(size_t)s1 - 1].g1;
+            const std::vector<DevGate<double>> mine(dgates.begin() + g0, dgates.begin() + g1);
+            if (sweeps > 1) {
+                starts.clear();
+                for (int k = s0; k < s1; ++k) starts.push_back(dsegs[(size_t)k].g0 - g0);
+                encode_fx(mine, starts, false, area);
+            }
+            pg.nseg = s1 - s0;
+            pg.fixed = true;
+            if (per > 0) {
+                align(256);
+                pg.oz = true;
+                pg.off = host.size();
+                pg.gate_bytes = 0;
+                for (int k = s0; k < s1; ++k) {
+                    const OzSeg a = oz_addresses(segs[(size_t)k], width, k == s0, k + 1 == s1);
+                    put(&a, sizeof(a));
+                }
+                pg.b_off = oz.size() * kOzBBytes;
+                const size_t gates_off = host.size();
+                host.insert(host.end(), area.begin(), area.end());
+                align(16);
+                pg.oz_first = (int)oz.size();
+                for (int k = s0; k < s1; ++k)
+                    oz.push_back(OzCompose{(uint32_t)gates_off, (uint32_t)(oz.size() * kOzBBytes),
+                                           (uint32_t)(pg.off + (size_t)(k - s0) * sizeof(OzSeg) + offsetof(OzSeg, scale)),
+                                           dsegs[(size_t)k].g0 - g0, dsegs[(size_t)k].g1 - g0});
+            } else {
+                // merged diagonals take some more room, and give way where a consumer group would lose its chunk
+                if (outside && encode_fx(mine, starts, true, merged) &&
+                    simt_buffers(width, pg.nseg, merged.size()) >= std::min(kFxGroups, simt_buffers(width, pg.nseg, area.size())))
+                    area.swap(merged);
+                pg.off = put_program(dsegs, s0, s1, true, area.data(), area.size());
+                pg.gate_bytes = (int)area.size();
+            }
+            pg.redo = !exact;
+            if (pg.redo) {
+                pg.dense = dense_rule(dsegs, dgates, s0, s1, width);
+                pg.redo_bytes = (int)(mine.size() * sizeof(mine[0]));
+                pg.redo_off = put_program(dsegs, s0, s1, false, mine.data(), mine.size() * sizeof(mine[0]));
+            }
+            progs.push_back(pg);
+        }
+        return true;
+    }
+
     // whole: all gates of the plan's section, whose register groups the plan keeps
-    auto section = [&](BlockProg bp, const std::vector<BlockGate> &section_gates, int width, bool whole) {
-        const int elem = (int)(2 * sizeof(T));
-        Groups kept = whole ? plan_groups(*plan, bp.op_index, seg_bits, elem) : nullptr;
+    void section(SimtPrograms::Prog pg, const std::vector<BlockGate> &section_gates, int width, bool whole) {
+        Groups kept = whole ? plan_groups(*plan, pg.op_index, seg_bits, kElem) : nullptr;
         if (!kept) {
-            std::vector<HostSeg> found = segment_block(section_gates, width, seg_bits, elem);
-            kept = whole ? keep_groups(*plan, bp.op_index, seg_bits, elem, std::move(found))
+            std::vector<HostSeg> found = segment_block(section_gates, width, seg_bits, kElem);
+            kept = whole ? keep_groups(*plan, pg.op_index, seg_bits, kElem, std::move(found))
                          : std::make_shared<const std::vector<HostSeg>>(std::move(found));
         }
         const std::vector<HostSeg> &segs = *kept;
@@ -393,143 +533,103 @@ static void build_programs(const sv_plan *plan, const sv_gate *gates, int seg_bi
             }
             if (dgates.size() > 32767) fail(SV_ERR_UNSUPPORTED, "too many gates in one blocking section");
             d.g1 = (int16_t)dgates.size();
-            if constexpr (sizeof(T) == 8) gather_outside_diagonals(dgates, (size_t)d.g0);
-            if constexpr (sizeof(T) == 8)
-                if (std::all_of(dgates.begin() + d.g0, dgates.end(), exact_gate)) d.flags |= kSegRaw;
             dsegs.push_back(d);
         }
-        // complex128: fixed-point gates where every gate is unitary (their area is never the larger);
-        // merged diagonals take some more room, and give way where a consumer group would lose its chunk
-        std::vector<unsigned char> area;
-        if constexpr (sizeof(T) == 8) {
-            std::vector<int> starts;
-            for (const DevSeg &d : dsegs) starts.push_back(d.g0);
-            bp.fixed = encode_fx(dgates, starts, false, area);
-            std::vector<unsigned char> merged;
-            if (bp.fixed && std::any_of(dgates.begin(), dgates.end(), [](const DevGate<T> &g) { return g.op == OP_DIAGX; }) &&
-                encode_fx(dgates, starts, true, merged) &&
-                fx_buffers(width, (int)dsegs.size(), merged.size()) >=
-                    std::min(kFxGroups, fx_buffers(width, (int)dsegs.size(), area.size())))
-                area.swap(merged);
-        }
-        if constexpr (sizeof(T) == 8) {
-            int per = 0;  // groups per sweep
-            if (oz && bp.fixed && std::any_of(dsegs.begin(), dsegs.end(), [](const DevSeg &d) { return !(d.flags & kSegRaw); }) &&
-                std::none_of(dgates.begin(), dgates.end(), [](const DevGate<T> &g) { return g.op == OP_DIAGX; }))
-                per = oz_max_segs(width, area.size());
-            if (per > 0) {
-                const int nseg = (int)dsegs.size(), sweeps = (nseg + per - 1) / per;
-                for (int w = 0; w < sweeps; ++w) {
-                    const int s0 = (int)((int64_t)nseg * w / sweeps), s1 = (int)((int64_t)nseg * (w + 1) / sweeps);
-                    const int g0 = dsegs[(size_t)s0].g0, g1 = dsegs[(size_t)s1 - 1].g1;
-                    encode_fx(std::vector<DevGate<T>>(dgates.begin() + g0, dgates.begin() + g1), {}, false, area);
-                    align(256);
-                    bp.oz = true;
-                    bp.off = host.size();
-                    bp.nseg = s1 - s0;
-                    bp.gate_bytes = (int)area.size();
-                    for (int k = s0; k < s1; ++k) {
-                        DevSeg d = dsegs[(size_t)k];
-                        d.flags = (int8_t)((k == s0 ? 1 : 0) | (k + 1 == s1 ? 2 : 0));
-                        d.g0 = (int16_t)(d.g0 - g0);
-                        d.g1 = (int16_t)(d.g1 - g0);
-                        put(&d, sizeof(d));
-                    }
-                    align(16);
-                    const size_t tab_off = host.size();
-                    for (int k = s0; k < s1; ++k) {
-                        const OzSeg a = oz_addresses(segs[(size_t)k], width, k == s0, k + 1 == s1);
-                        put(&a, sizeof(a));
-                    }
-                    const size_t gates_off = host.size();
-                    host.insert(host.end(), area.begin(), area.end());
-                    align(16);
-                    const size_t b_off = host.size();
-                    host.resize(b_off + (size_t)bp.nseg * kOzBBytes, 0);
-                    for (int k = s0; k < s1; ++k)
-                        oz->push_back(OzCompose{(uint32_t)gates_off, (uint32_t)(b_off + (size_t)(k - s0) * kOzBBytes),
-                                                (uint32_t)(tab_off + (size_t)(k - s0) * sizeof(OzSeg) + offsetof(OzSeg, scale)),
-                                                dsegs[(size_t)k].g0 - g0, dsegs[(size_t)k].g1 - g0});
-                    progs.push_back(bp);
-                }
-                return;
-            }
-        }
-        if (!bp.fixed) {
-            const unsigned char *p = reinterpret_cast<const unsigned char *>(dgates.data());
-            area.assign(p, p + dgates.size() * sizeof(DevGate<T>));
-        }
+        if constexpr (sizeof(T) == 8)
+            if (fixed_section(pg, segs, dsegs, dgates, width)) return;
         align(256);
-        bp.off = host.size();
-        bp.nseg = (int)dsegs.size();
+        pg.off = host.size();
+        pg.nseg = (int)dsegs.size();
         put(dsegs.data(), dsegs.size() * sizeof(DevSeg));
         align(16);
-        bp.gate_bytes = (int)area.size();
-        host.insert(host.end(), area.begin(), area.end());
+        pg.gate_bytes = (int)(dgates.size() * sizeof(DevGate<T>));
+        put(dgates.data(), dgates.size() * sizeof(DevGate<T>));
         align(16);
-        progs.push_back(bp);
-    };
-    for (const PlanOp &op0 : plan->ops) {
-        if (op0.kind != 2 && op0.kind != 4) continue;
-        int width = std::min(plan->c, plan->n);
-        BlockProg bp{};
-        bp.op_index = (int)(&op0 - plan->ops.data());
-        std::vector<BlockGate> local;
-        if (op0.kind == 4) {  // gate bits -> chunk-local bits of the gathered layout
-            bp.lay = gather_layout(op0.mask, plan->n, (int)(2 * sizeof(T)));
-            local = localize_gates(op0, plan->n, plan->c, &bp.lay);
-            width = bp.lay.ce;
-            bp.gathered = true;
-        } else {
-            local = localize_gates(op0, plan->n, plan->c, nullptr);
-        }
-        // diagonals from outside the chunk keep a section off the tensor cores.  Where all of them
-        // commute to its end (no later gate but diagonal ones on their chunk bits) they get a sweep of
-        // their own, one merged diagonal per 4 bits, and the rest runs there: a group costs 2.3 clocks
-        // per amplitude and SM instead of 8.6 (n = 28 QFT: 160 ms in one sweep per section, 100 so)
-        std::vector<BlockGate> main, tail;
-        if (oz && oz_max_segs(width, 0) > 0 && split_outside(local, gates, main, tail)) {
-            const size_t nm = segment_block(main, width, seg_bits, (int)(2 * sizeof(T))).size();
-            const size_t nt = segment_block(tail, width, seg_bits, (int)(2 * sizeof(T))).size();
-            if (2 * nm > nt + 1) {
-                section(bp, main, width, false);
-                section(bp, tail, width, false);
-                continue;
-            }
-        }
-        section(bp, local, width, true);
+        progs.push_back(pg);
     }
-    align(256);
-}
+
+    void build() {
+        for (const PlanOp &op0 : plan->ops) {
+            if (op0.kind != 2 && op0.kind != 4) continue;
+            int width = std::min(plan->c, plan->n);
+            SimtPrograms::Prog pg{};
+            pg.op_index = (int)(&op0 - plan->ops.data());
+            std::vector<BlockGate> local;
+            if (op0.kind == 4) {  // gate bits -> chunk-local bits of the gathered layout
+                pg.lay = gather_layout(op0.mask, plan->n, kElem);
+                local = localize_gates(op0, plan->n, plan->c, &pg.lay);
+                width = pg.lay.ce;
+                pg.gathered = true;
+            } else {
+                local = localize_gates(op0, plan->n, plan->c, nullptr);
+            }
+            // diagonals from outside the chunk keep a section off the tensor cores.  Where all of them
+            // commute to its end (no later gate but diagonal ones on their chunk bits) they get a sweep of
+            // their own, one merged diagonal per 4 bits, and the rest runs there: a group costs 2.3 clocks
+            // per amplitude and SM instead of 8.6 (n = 28 QFT: 160 ms in one sweep per section, 100 so)
+            std::vector<BlockGate> main, tail;
+            if (sizeof(T) == 8 && !plan->fp64 && oz_max_segs(width) > 0 && split_outside(local, gates, main, tail)) {
+                const size_t nm = segment_block(main, width, seg_bits, kElem).size();
+                const size_t nt = segment_block(tail, width, seg_bits, kElem).size();
+                if (2 * nm > nt + 1) {
+                    section(pg, main, width, false);
+                    section(pg, tail, width, false);
+                    continue;
+                }
+            }
+            section(pg, local, width, true);
+        }
+        align(256);
+    }
+};
 
 void build_simt_programs(const sv_plan *plan, const sv_gate *gates, int dtype, SimtPrograms &out) {
+    out = SimtPrograms{};
     out.seg_bits = (dtype == SV_C64 && plan->seg_bits == 5) ? 5 : 4;
-    std::vector<BlockProg> progs;
     std::vector<OzCompose> oz;
-    if (dtype == SV_C64) build_programs<float>(plan, gates, out.seg_bits, out.host, progs);
-    else build_programs<double>(plan, gates, out.seg_bits, out.host, progs, &oz);
+    if (dtype == SV_C64) ProgramBuilder<float>{plan, gates, out.seg_bits, out.host, out.progs, oz}.build();
+    else ProgramBuilder<double>{plan, gates, out.seg_bits, out.host, out.progs, oz}.build();
     out.oz_off = out.host.size();
     out.noz = (int)oz.size();
+    out.b_bytes = oz.size() * kOzBBytes;
     const unsigned char *p = reinterpret_cast<const unsigned char *>(oz.data());
     out.host.insert(out.host.end(), p, p + oz.size() * sizeof(OzCompose));
-    out.progs.clear();
-    for (const BlockProg &bp : progs)
-        out.progs.push_back(
-            SimtPrograms::Prog{bp.off, bp.nseg, bp.gate_bytes, bp.op_index, bp.fixed, bp.oz, bp.gathered, bp.lay});
 }
 
-void launch_section(int dtype, void *state, int n, int c, const unsigned char *base, const SimtPrograms::Prog &p,
-                    int seg_bits, int *dev_err, cudaStream_t st, uint64_t wait_ns) {
-    if (p.oz)
-        launch_block_oz(state, n, c, p.gathered ? &p.lay : nullptr, base + p.off, p.nseg, p.gate_bytes, dev_err, st, wait_ns);
-    else if (p.gathered)
-        launch_block_gather(dtype, state, n, p.lay, base + p.off, p.nseg, p.gate_bytes, p.fixed, dev_err, seg_bits, st, wait_ns);
-    else
-        launch_block(dtype, state, n, c, base + p.off, p.nseg, p.gate_bytes, p.fixed, dev_err, seg_bits, st, wait_ns);
+size_t redo_list_bytes(const SimtPrograms &sp, int n, int c) {
+    size_t most = 0;
+    for (const SimtPrograms::Prog &p : sp.progs)
+        if (p.redo) most = std::max(most, ((size_t(1) << (n - (p.gathered ? p.lay.ce : std::min(c, n)))) + LIST_FIRST) * sizeof(int));
+    return (most + 255) / 256 * 256;
 }
 
-static void upload_program(sv_state *h, const std::vector<unsigned char> &host) {
-    const size_t bytes = std::max<size_t>(host.size(), 256);
+int launch_section(int dtype, void *state, int n, int c, const unsigned char *base, const unsigned char *operands,
+                   const SimtPrograms::Prog &p, int seg_bits, int *list, int *dev_err, cudaStream_t st, uint64_t wait_ns) {
+    auto simt = [&](size_t off, int gate_bytes, bool fixed, const SweepArgs &sa) {
+        if (p.gathered)
+            launch_block_gather(dtype, state, n, p.lay, base + off, p.nseg, gate_bytes, fixed, dev_err, seg_bits, st, wait_ns, sa);
+        else
+            launch_block(dtype, state, n, c, base + off, p.nseg, gate_bytes, fixed, dev_err, seg_bits, st, wait_ns, sa);
+    };
+    SweepArgs pass, rest;
+    pass.operands = operands + p.b_off;
+    if (p.redo) {
+        pass.to = list;
+        pass.dense = p.dense;
+        rest.from = list;
+    }
+    if (p.oz) launch_block_oz(state, n, c, p.gathered ? &p.lay : nullptr, base + p.off, p.nseg, dev_err, st, wait_ns, pass);
+    else simt(p.off, p.gate_bytes, p.fixed, pass);
+    if (!p.redo) return 1;
+    simt(p.redo_off, p.redo_bytes, false, rest);
+    return 2;
+}
+
+// Copies a program to the device.  `more` bytes behind it (256-byte aligned, the first 16 zeroed) are the
+// kernels' own: the return value.
+static unsigned char *upload_program(sv_state *h, std::vector<unsigned char> &host, size_t more = 0) {
+    if (more) host.resize((host.size() + 255) / 256 * 256 + 16, 0);
+    const size_t at = host.size() / 256 * 256, bytes = std::max<size_t>(host.size(), 256);
     if (h->prog_event) check_cuda(cudaEventSynchronize(h->prog_event), "cudaEventSynchronize");
     if (h->prog_host_bytes < bytes) {
         if (h->prog_host) cudaFreeHost(h->prog_host);
@@ -537,14 +637,15 @@ static void upload_program(sv_state *h, const std::vector<unsigned char> &host) 
         check_cuda(cudaHostAlloc(&h->prog_host, bytes, cudaHostAllocDefault), "cudaHostAlloc(program)");
         h->prog_host_bytes = bytes;
     }
-    if (h->prog_bytes < bytes) {
+    if (h->prog_bytes < std::max(bytes, at + more)) {
         if (h->prog) {
             check_cuda(cudaStreamSynchronize(h->stream), "cudaStreamSynchronize");
             cudaFree(h->prog);
         }
         h->prog = nullptr;
-        check_cuda(cudaMalloc(&h->prog, bytes), "cudaMalloc(program)");
-        h->prog_bytes = bytes;
+        h->prog_bytes = 0;
+        check_cuda(cudaMalloc(&h->prog, std::max(bytes, at + more)), "cudaMalloc(program)");
+        h->prog_bytes = std::max(bytes, at + more);
     }
     if (!host.empty()) {
         std::memcpy(h->prog_host, host.data(), host.size());
@@ -553,6 +654,7 @@ static void upload_program(sv_state *h, const std::vector<unsigned char> &host) 
     }
     if (!h->prog_event) check_cuda(cudaEventCreateWithFlags(&h->prog_event, cudaEventDisableTiming), "cudaEventCreate");
     check_cuda(cudaEventRecord(h->prog_event, h->stream), "cudaEventRecord");
+    return static_cast<unsigned char *>(h->prog) + at;
 }
 
 }  // namespace sv
@@ -847,7 +949,8 @@ sv_status sv_apply_circuit(sv_handle h, const sv_gate *gates, int64_t n_gates, s
         SimtPrograms sp;
         if (tc) build_programs_tc(plan, gates, tc_bits, host, progs, cs_off, ncs, g_off, flag_off);
         else build_simt_programs(plan, gates, h->dtype, sp);
-        upload_program(h, tc ? host : sp.host);
+        const size_t list_bytes = tc ? 0 : redo_list_bytes(sp, h->n, plan->c);
+        unsigned char *const list = upload_program(h, tc ? host : sp.host, list_bytes + sp.b_bytes), *const operands = list + list_bytes;
         const unsigned char *base = static_cast<const unsigned char *>(h->prog);
         int *unitary_flag = tc ? reinterpret_cast<int *>(static_cast<unsigned char *>(h->prog) + flag_off) : nullptr;
         if (tc) {  // fuse every register group into its B operand, in FP64 on the GPU
@@ -858,7 +961,7 @@ sv_status sv_apply_circuit(sv_handle h, const sv_gate *gates, int64_t n_gates, s
                 }
         }
         if (sp.noz) {
-            launch_compose_oz(base + sp.oz_off, sp.noz, h->prog, h->stream);
+            launch_compose_oz(base + sp.oz_off, sp.noz, h->prog, operands, h->stream);
             ++st.kernel_launches;
         }
         const uint64_t wait_ns = plan->wait_limit_ms > 0 ? (uint64_t)plan->wait_limit_ms * 1000000ull : kDefaultWaitNs;
@@ -868,22 +971,22 @@ sv_status sv_apply_circuit(sv_handle h, const sv_gate *gates, int64_t n_gates, s
             if (op.kind == 2 || op.kind == 4) {
                 auto sweep = [&](auto launch) {
                     mark_begin(h, 1, (int)oi);
-                    launch();
+                    st.kernel_launches += launch();
                     mark_end(h);
                     ++st.sweeps_block;
-                    ++st.kernel_launches;
                 };
                 for (; tc && bi < progs.size() && progs[bi].op_index == (int)oi; ++bi) {
                     const BlockProg &bp = progs[bi];
                     sweep([&] {
                         launch_block_tc(h->amp, h->n, plan->c, bp.gathered ? &bp.lay : nullptr, base + bp.off, bp.nseg,
                                         h->dev_err, bp.r, h->stream, wait_ns);
+                        return 1;
                     });
                 }
                 for (; !tc && bi < sp.progs.size() && sp.progs[bi].op_index == (int)oi; ++bi)
                     sweep([&] {
-                        launch_section(h->dtype, h->amp, h->n, plan->c, base, sp.progs[bi], sp.seg_bits, h->dev_err,
-                                       h->stream, wait_ns);
+                        return launch_section(h->dtype, h->amp, h->n, plan->c, base, operands, sp.progs[bi], sp.seg_bits,
+                                              reinterpret_cast<int *>(list), h->dev_err, h->stream, wait_ns);
                     });
                 continue;
             } else {
@@ -922,9 +1025,10 @@ sv_status sv_apply_plan_ops(sv_handle h, const sv_gate *gates, int64_t n_gates, 
     }
     SimtPrograms sp;
     build_simt_programs(plan, gates, h->dtype, sp);
-    upload_program(h, sp.host);
+    const size_t list_bytes = redo_list_bytes(sp, h->n, plan->c);
+    unsigned char *const list = upload_program(h, sp.host, list_bytes + sp.b_bytes), *const operands = list + list_bytes;
     const unsigned char *base = static_cast<const unsigned char *>(h->prog);
-    if (sp.noz) launch_compose_oz(base + sp.oz_off, sp.noz, h->prog, h->stream);
+    if (sp.noz) launch_compose_oz(base + sp.oz_off, sp.noz, h->prog, operands, h->stream);
     const uint64_t wait_ns = plan->wait_limit_ms > 0 ? (uint64_t)plan->wait_limit_ms * 1000000ull : kDefaultWaitNs;
     size_t bi = 0;  // programs are in op order
     for (int32_t oi = op_begin; oi < op_end; ++oi) {
@@ -933,7 +1037,8 @@ sv_status sv_apply_plan_ops(sv_handle h, const sv_gate *gates, int64_t n_gates, 
             while (bi < sp.progs.size() && sp.progs[bi].op_index < oi) ++bi;
             if (bi == sp.progs.size() || sp.progs[bi].op_index != oi) fail(SV_ERR_PLAN, "no program for a blocking section");
             for (; bi < sp.progs.size() && sp.progs[bi].op_index == oi; ++bi)
-                launch_section(h->dtype, h->amp, h->n, plan->c, base, sp.progs[bi], sp.seg_bits, h->dev_err, h->stream, wait_ns);
+                launch_section(h->dtype, h->amp, h->n, plan->c, base, operands, sp.progs[bi], sp.seg_bits,
+                               reinterpret_cast<int *>(list), h->dev_err, h->stream, wait_ns);
         } else {
             // pairs inside the piece; the others move data between pieces and are the caller's
             std::vector<std::pair<int32_t, int32_t>> local;

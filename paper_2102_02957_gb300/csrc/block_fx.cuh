@@ -12,6 +12,7 @@
 //   27, 8 random layers (12 sections, 44 groups)       417 -> 169 ms
 //   28, QFT with diagonals outside the chunk           393 -> 239 ms, with merged runs 160 ms
 //   25, quantum volume of 10 layers, gathered chunks   108 -> 38.6 ms
+// (all of them before the chunks were looked over, ChunkRange: two passes over a chunk in shared memory)
 //
 // The section's gate area is a table of 16-byte headers {op, payload offset, outside bits, code},
 // then the payloads (encode_fx writes them):
@@ -343,74 +344,106 @@ __device__ __forceinline__ void fx_merge(uint32_t gates, int g0, int g1, int64_t
     }
 }
 
-__device__ __forceinline__ double fx_entry_value(uint32_t a) {
-    const int h = lds_s32(a), l = lds_s32(a + 4);
-    return ((double)h * 4294967296.0 + (double)l) * 0x1p-61;
+// What a chunk's amplitudes look like, for the engines that give a whole register group (here) or chunk
+// (block_oz.cuh) one exponent.  Their error is a unit of the chunk's largest component, so they may run a chunk
+//   DENSE  of which few enough amplitudes (Dense, sv_internal.h) are small beside that component; or
+//   TRIAL  whose results are all within kNearOrders binary orders of it (chunk_filled): states that gates
+//          fill from a few amplitudes.  Tried where at most one amplitude in 64 is small and not zero, and only
+//          with gates like Hadamards (Dense::trial).
+//   ZERO   chunks stay as they are, and so do OTHER ones (and failed trials), which FP64 register groups run
+//          next (Redo): components that are not finite or near the ends of the exponent range, states with
+//          most of their weight on few amplitudes.
+struct ChunkRange {
+    int top, zeros, small, near;  // largest high word, amplitudes that are zero, below Dense's line, and below kNearOrders
+    int least_out, filled;        // of the results: smallest non-zero, number of non-zero ones,
+    unsigned any_bits, all_bits;  // or and and of their indices
+    __device__ void clear() volatile {
+        top = zeros = small = near = filled = 0;
+        least_out = 0x7FFFFFFF;
+        any_bits = 0;
+        all_bits = ~0u;
+    }
+};
+enum : int { CHUNK_DENSE = 0, CHUNK_TRIAL = 1, CHUNK_ZERO = 2, CHUNK_OTHER = 3 };
+constexpr int kMinTop = 200 << 20, kMaxTop = 2030 << 20;
+
+// High word of an amplitude's larger component; some: the amplitude is not zero.
+__device__ __forceinline__ int amp_top(uint32_t a, bool &some) {
+    double x, y;
+    SM<double>::ld(a, x, y);
+    const int hi = max(__double2hiint(x) & 0x7FFFFFFF, __double2hiint(y) & 0x7FFFFFFF);
+    some = (hi | __double2loint(x) | __double2loint(y)) != 0;
+    return hi;
 }
 
-// The group in FP64, for components outside the fixed-point range (infinities, NaN, magnitudes
-// near the ends of the exponent range).  Not a hot path: one copy of the code, amplitudes in
-// local memory.
-__device__ __noinline__ void fx_group_fp64(double *re, double *im, uint32_t gates, int g0, int g1, int64_t origin, int cg) {
-    for (int gi = g0; gi < g1; ++gi) {
-        const FxGate g = fx_gate(gates, gi, origin, cg);
-        if (g.op == OP_DIAGRUN) {
-            gi += g.more;
-            for (int x = 0; x < 16; ++x) {
-                const double dr = fx_entry_value(g.m + 16 * x), di = fx_entry_value(g.m + 16 * x + 8);
-                if (dr == 1.0 && di == 0.0) continue;
-                const double a = re[x], b = im[x];
-                re[x] = dr * a - di * b;
-                im[x] = dr * b + di * a;
-            }
-            continue;
-        }
-        const bool one = g.op == OP_DENSE1 || g.op == OP_REAL1 || g.op == OP_DIAG1 || g.op == OP_X1;
-        const int dim = one ? 2 : 4;
-        const int ba = one ? 1 << g.code : 1 << (g.code >> 3), bb = one ? 0 : 1 << (g.code & 7);
-        for (int x = 0; x < 16; ++x) {
-            if (x & (ba | bb)) continue;
-            double xr[4], xi[4], yr[4], yi[4];
-            for (int k = 0; k < dim; ++k) {
-                const int i = x | ((k & 1) ? ba : 0) | ((k & 2) ? bb : 0);
-                xr[k] = re[i];
-                xi[k] = im[i];
-            }
-            for (int r = 0; r < dim; ++r) {
-                int from = -1;  // exchanges move the amplitude of row `from`
-                if (g.op == OP_X1) from = r ^ 1;
-                else if (g.op == OP_CXA) from = r == 1 ? 3 : r == 3 ? 1 : r;
-                else if (g.op == OP_CXB) from = r == 2 ? 3 : r == 3 ? 2 : r;
-                else if (g.op == OP_SWAP2) from = r == 1 ? 2 : r == 2 ? 1 : r;
-                else if (g.op == OP_PERM2) from = lds_s32(g.m + 4 * r);
-                if (from >= 0) {
-                    yr[r] = xr[from];
-                    yi[r] = xi[from];
-                    continue;
-                }
-                if (g.op == OP_DIAG1 || g.op == OP_DIAG2) {
-                    const double dr = fx_entry_value(g.m + 16 * r), di = fx_entry_value(g.m + 16 * r + 8);
-                    const bool unit = dr == 1.0 && di == 0.0;
-                    yr[r] = unit ? xr[r] : dr * xr[r] - di * xi[r];
-                    yi[r] = unit ? xi[r] : dr * xi[r] + di * xr[r];
-                    continue;
-                }
-                double sr = 0, si = 0;
-                for (int c = 0; c < dim; ++c) {
-                    const uint32_t e = g.m + (g.op == OP_REAL1 ? 8 : 16) * (dim * r + c);
-                    const double mr = fx_entry_value(e), mi = g.op == OP_REAL1 ? 0.0 : fx_entry_value(e + 8);
-                    cmul_acc(sr, si, mr, mi, xr[c], xi[c]);
-                }
-                yr[r] = sr;
-                yi[r] = si;
-            }
-            for (int k = 0; k < dim; ++k) {
-                const int i = x | ((k & 1) ? ba : 0) | ((k & 2) ? bb : 0);
-                re[i] = yr[k];
-                im[i] = yi[k];
-            }
-        }
+// NC threads; sh was cleared before a barrier of theirs.  top: the largest component's high word.
+template <int NC>
+__device__ __forceinline__ int chunk_range(uint32_t buf, int c, int ctid, int bar_id, volatile ChunkRange *sh, const Dense &d,
+                                           int &top) {
+    int most = 0, zeros = 0;
+    for (int i = ctid; i < (1 << c); i += NC) {
+        bool some;
+        most = max(most, amp_top(buf + 16u * (uint32_t)i, some));
+        zeros += some ? 0 : 1;
     }
+    most = __reduce_max_sync(0xFFFFFFFFu, most);
+    zeros = (int)__reduce_add_sync(0xFFFFFFFFu, (unsigned)zeros);
+    if ((ctid & 31) == 0) {
+        atomicMax(const_cast<int *>(&sh->top), most);
+        if (zeros) atomicAdd(const_cast<int *>(&sh->zeros), zeros);
+    }
+    ptx::named_bar_sync(bar_id, NC);
+    top = sh->top;
+    zeros = sh->zeros;
+    if (zeros == 1 << c) return CHUNK_ZERO;
+    if (top < kMinTop || top >= kMaxTop) return CHUNK_OTHER;
+    const int line = top - (d.orders << 20), near = top - (kNearOrders << 20);
+    int below = 0;  // in two halves: of `line`, of `near`
+    for (int i = ctid; i < (1 << c); i += NC) {
+        bool some;
+        const int hi = amp_top(buf + 16u * (uint32_t)i, some);
+        below += (hi < line ? 1 : 0) + (hi < near ? 0x10000 : 0);
+    }
+    below = (int)__reduce_add_sync(0xFFFFFFFFu, (unsigned)below);
+    if ((ctid & 31) == 0 && below) {
+        atomicAdd(const_cast<int *>(&sh->small), below & 0xFFFF);
+        atomicAdd(const_cast<int *>(&sh->near), below >> 16);
+    }
+    ptx::named_bar_sync(bar_id, NC);
+    if (sh->small <= d.most) return CHUNK_DENSE;
+    return d.trial && (sh->near - zeros) * 64 <= (1 << c) ? CHUNK_TRIAL : CHUNK_OTHER;
+}
+
+// Whether the results of a TRIAL (in the natural layout, behind a barrier of the group) are within the orders.
+// A zero among them is one whose inputs are zero, not a small result lost, where the non-zero ones fill a
+// cube of the index space in which every bit that a dense gate touched (dense_bits) runs free.
+template <int NC>
+__device__ __forceinline__ bool chunk_filled(uint32_t buf, int c, int ctid, int bar_id, volatile ChunkRange *sh, int top,
+                                             unsigned dense_bits) {
+    int least = 0x7FFFFFFF, filled = 0;
+    unsigned any_bits = 0, all_bits = ~0u;
+    for (int i = ctid; i < (1 << c); i += NC) {
+        bool some;
+        const int hi = amp_top(buf + 16u * (uint32_t)i, some);
+        if (!some) continue;
+        least = min(least, hi);
+        ++filled;
+        any_bits |= (unsigned)i;
+        all_bits &= (unsigned)i;
+    }
+    least = __reduce_min_sync(0xFFFFFFFFu, least);
+    filled = (int)__reduce_add_sync(0xFFFFFFFFu, (unsigned)filled);
+    any_bits = __reduce_or_sync(0xFFFFFFFFu, any_bits);
+    all_bits = __reduce_and_sync(0xFFFFFFFFu, all_bits);
+    if ((ctid & 31) == 0) {
+        atomicMin(const_cast<int *>(&sh->least_out), least);
+        atomicAdd(const_cast<int *>(&sh->filled), filled);
+        atomicOr(const_cast<unsigned *>(&sh->any_bits), any_bits);
+        atomicAnd(const_cast<unsigned *>(&sh->all_bits), all_bits);
+    }
+    ptx::named_bar_sync(bar_id, NC);
+    const unsigned free_bits = sh->any_bits & ~sh->all_bits;
+    return sh->least_out >= top - (kNearOrders << 20) && sh->filled == 1 << __popc(free_bits) && (dense_bits & ~free_bits) == 0;
 }
 
 // One register group of 4 bits over the chunk in shared memory (see run_segment for the addressing).
@@ -444,7 +477,7 @@ __device__ __forceinline__ void run_segment_fx(uint32_t buf, uint32_t seg, uint3
         ld_step[j] = (uint32_t)((flags & 1) ? po[j] : pf[j]) << 4;
         st_step[j] = (uint32_t)((flags & 2) ? po[j] : pf[j]) << 4;
     }
-    for (int gb = ctid; (gb & ~31) < G; gb += NC) {  // whole warps: the range test votes
+    for (int gb = ctid; gb < G; gb += NC) {
         int bs = lbase, fb = lfb;
         for (int j = 0; j < nrest; ++j)
             if ((gb >> (5 + j)) & 1) {
@@ -452,7 +485,6 @@ __device__ __forceinline__ void run_segment_fx(uint32_t buf, uint32_t seg, uint3
                 bs |= 1 << p;
                 fb ^= swz[p];
             }
-        const bool live = gb < G;
         const uint32_t ld0 = (uint32_t)((flags & 1) ? bs : bs ^ fb) << 4, st0 = (uint32_t)((flags & 2) ? bs : bs ^ fb) << 4;
         double dr[NA], di[NA];
         int top = 0, any = 0;
@@ -461,8 +493,7 @@ __device__ __forceinline__ void run_segment_fx(uint32_t buf, uint32_t seg, uint3
         for (int b = 0; b < NA; ++b) {
             if (b) off ^= ld_step[low_bit(b)];
             const int g = b ^ (b >> 1);
-            dr[g] = di[g] = 0.0;
-            if (live) SM<double>::ld(buf + off, dr[g], di[g]);
+            SM<double>::ld(buf + off, dr[g], di[g]);
         }
 #pragma unroll
         for (int b = 0; b < NA; ++b) {
@@ -470,40 +501,29 @@ __device__ __forceinline__ void run_segment_fx(uint32_t buf, uint32_t seg, uint3
             fx::scan(di[b], top, any);
         }
         const bool raw = (flags & kSegRaw) != 0;
-        if (!raw && __any_sync(0xFFFFFFFFu, fx::special(top, any))) {
-            double lr[NA], li[NA];
+        const int E = fx::exponent(top);
+        FxGroup<NA> v;
 #pragma unroll
-            for (int b = 0; b < NA; ++b) { lr[b] = dr[b]; li[b] = di[b]; }
-            fx_group_fp64(lr, li, gates, g0, g1, origin, cg);
-#pragma unroll
-            for (int b = 0; b < NA; ++b) { dr[b] = lr[b]; di[b] = li[b]; }
-        } else {
-            const int E = fx::exponent(top);
-            FxGroup<NA> v;
-#pragma unroll
-            for (int b = 0; b < NA; ++b) {
-                v.re[b] = raw ? fx::from_bits(dr[b]) : fx::from_double(dr[b], E);
-                v.im[b] = raw ? fx::from_bits(di[b]) : fx::from_double(di[b], E);
-            }
-            for (int gi = g0; gi < g1; ++gi) {
-                const FxGate g = fx_gate(gates, gi, origin, cg);
-                fx_apply(g.op, g.code, g.m, v, raw);
-                gi += g.more;
-            }
-#pragma unroll
-            for (int b = 0; b < NA; ++b) {
-                dr[b] = raw ? fx::to_bits(v.re[b]) : fx::to_double(v.re[b], E);
-                di[b] = raw ? fx::to_bits(v.im[b]) : fx::to_double(v.im[b], E);
-            }
+        for (int b = 0; b < NA; ++b) {
+            v.re[b] = raw ? fx::from_bits(dr[b]) : fx::from_double(dr[b], E);
+            v.im[b] = raw ? fx::from_bits(di[b]) : fx::from_double(di[b], E);
         }
-        if (live) {
-            off = st0;
+        for (int gi = g0; gi < g1; ++gi) {
+            const FxGate g = fx_gate(gates, gi, origin, cg);
+            fx_apply(g.op, g.code, g.m, v, raw);
+            gi += g.more;
+        }
 #pragma unroll
-            for (int b = 0; b < NA; ++b) {
-                if (b) off ^= st_step[low_bit(b)];
-                const int g = b ^ (b >> 1);
-                SM<double>::st(buf + off, dr[g], di[g]);
-            }
+        for (int b = 0; b < NA; ++b) {
+            dr[b] = raw ? fx::to_bits(v.re[b]) : fx::to_double(v.re[b], E);
+            di[b] = raw ? fx::to_bits(v.im[b]) : fx::to_double(v.im[b], E);
+        }
+        off = st0;
+#pragma unroll
+        for (int b = 0; b < NA; ++b) {
+            if (b) off ^= st_step[low_bit(b)];
+            const int g = b ^ (b >> 1);
+            SM<double>::st(buf + off, dr[g], di[g]);
         }
     }
 }

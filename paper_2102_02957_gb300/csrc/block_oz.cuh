@@ -22,15 +22,18 @@
 // one's MMAs run, and a half's MMAs for the next tile start as soon as it is read.
 //
 // Measured against the integer-pipe sections (block_fx.cuh) and the FP64 ones before them, 12-bit
-// chunks: n = 27, 8 random layers (44 groups) 169 and 417 ms, here 55 to 61; n = 25, quantum volume of
-// 10 layers (44 groups) 38.6 and 108 ms, here 12.8.  A group costs about 2.3 clocks per amplitude and
+// chunks: n = 27, 8 random layers (44 groups) on a dense state 169 and 417 ms, here 57 to 63; n = 25, quantum volume of
+// 10 layers (44 groups) from a basis state 108 ms in FP64, here 20 to 21 (12.8 with the first sections, of few
+// amplitudes, here too; they are FP64's).  A group costs about 2.3 clocks per amplitude and
 // SM whatever its gates are; a dense one-qubit gate on the integer pipe alone takes 1.4, and the
 // conversions of a group there 1.5.
 //
 // Precision: a unit of X is 2^-54 to 2^-55 of the chunk's largest component; each group rounds once to it,
-// and U is within 2^-(55 + s), where FP64 rounds four to eight times per gate.  Chunks with a non-finite
-// component or one whose largest is outside 2^-923 .. 2^1017 run their gates in FP64
-// (fx_group_fp64).
+// and U is within 2^-(55 + s), where FP64 rounds four to eight times per gate.  That holds for the chunk as
+// a whole, so chunks run here only where ChunkRange finds them dense; FP64 register groups run the others
+// from memory, where they were left.  Relative error of single amplitudes against extended precision, here and in
+// FP64, after 8 layers on 13 qubits from a dense state: median 3.2e-16 and 7.4e-16, one in 1000 above 1.2e-14 and
+// 4.0e-14, largest 1.1e-13 and 2.5e-13; quantum volume 3.5e-16 and 7.0e-16, 1.0e-14 and 2.5e-14, 3.1e-14 and 6.7e-14.
 #pragma once
 #include "block_fx.cuh"
 
@@ -38,12 +41,11 @@ namespace sv {
 namespace {
 
 constexpr int kOzMaxSegs = 16;  // register groups per sweep (shared memory allows about six)
-constexpr int kOzMinTop = 100 << 20;
 
 // Per consumer group, in shared memory.
 struct OzShared {
-    int top, any;                // exponent search over the chunk
-    int skip;                    // the chunk runs in FP64: no MMAs
+    ChunkRange range;
+    int skip;                    // the chunk does not run: no MMAs
     unsigned high[kOzMaxSegs];   // largest magnitude's high word after each group
 };
 
@@ -149,41 +151,6 @@ __device__ __forceinline__ void oz_sum(const uint32_t (&dr)[8], const uint32_t (
     vi = total(bi, li);
 }
 
-// The chunk's gates in FP64, row by row (chunks outside the fixed-point range).
-template <int NC>
-__device__ __noinline__ void oz_chunk_fp64(uint32_t buf, uint32_t segs, uint32_t gates, int nseg, int ctid, const int *swz,
-                                           int c, int64_t origin, int bar_id) {
-    for (int si = 0; si < nseg; ++si) {
-        const uint32_t seg = segs + (uint32_t)(si * sizeof(DevSeg));
-        const int nrest = lds_s8(seg + 13), flags = lds_s8(seg + 14);
-        const int g0 = lds_s16(seg + 32), g1 = lds_s16(seg + 34);
-        for (int g = ctid; g < (1 << (c - 4)); g += NC) {
-            int base = 0;
-            for (int j = 0; j < 5; ++j)
-                if ((g >> j) & 1) base |= 1 << lds_s8(seg + 8 + j);
-            for (int j = 0; j < nrest; ++j)
-                if ((g >> (5 + j)) & 1) base |= 1 << lds_s8(seg + 16 + j);
-            double re[16], im[16];
-            for (int pass = 0; pass < 2; ++pass) {
-                const bool natural = flags & (pass ? 2 : 1);
-                for (int x = 0; x < 16; ++x) {
-                    int i = base;
-                    for (int j = 0; j < 4; ++j)
-                        if ((x >> j) & 1) i |= 1 << lds_s8(seg + j);
-                    int slot = i;
-                    if (!natural)
-                        for (int k = 3; k < c; ++k)
-                            if ((i >> k) & 1) slot ^= swz[k];
-                    if (pass == 0) SM<double>::ld(buf + 16u * (uint32_t)slot, re[x], im[x]);
-                    else SM<double>::st(buf + 16u * (uint32_t)slot, re[x], im[x]);
-                }
-                if (pass == 0) fx_group_fp64(re, im, gates, g0, g1, origin, 0);
-            }
-        }
-        ptx::named_bar_sync(bar_id, NC);
-    }
-}
-
 // MMA issue of half rows `half`, one warp: an MMA holds its issuing thread for about 88 cycles (14
 // of them in a row 1210), so the halves have a warp each and the threads that stage and drain
 // have none of it (with one of those issuing, a section of n = 24 took 645 us instead of 545).
@@ -228,33 +195,17 @@ __device__ __forceinline__ void oz_issue(int half, uint32_t bops, int nseg, int 
     }
 }
 
-// All register groups of a section on one chunk.  Returns false (uniformly) when a wait expired.
+// All register groups of a section on one chunk; kind (uniform): CHUNK_DENSE where the results stand, else
+// how the chunk was left.  Returns false (uniformly) when a wait expired.
 template <int NC>
-__device__ __forceinline__ bool run_chunk_oz(uint32_t buf, uint32_t segs, uint32_t tabs, uint32_t gates, uint32_t bops, int nseg, int ctid,
-                                             const int *swz, int c, int64_t origin, uint32_t tcol, int bar_id, uint64_t *mbar,
-                                             uint32_t (&phase)[2], volatile int *abort_flag, const uint64_t *wait_ns,
-                                             OzShared *sh) {
+__device__ __forceinline__ bool run_chunk_oz(uint32_t buf, uint32_t tabs, int nseg, int ctid, int c, const Dense &dense,
+                                             uint32_t tcol, int bar_id, uint64_t *mbar, uint32_t (&phase)[2],
+                                             volatile int *abort_flag, const uint64_t *wait_ns, OzShared *sh, int &kind) {
     static_assert(NC == 512, "four threads per row of a 128-row tile");
     constexpr int kDCols = 128, kACols = 112;  // D half 0, D half 1, digits 0, digits 1
     // exponent search (sh was cleared before the barrier that opened this chunk)
-    {
-        int top = 0, any = 0;
-        for (int i = ctid; i < (1 << c); i += NC) {
-            double x, y;
-            SM<double>::ld(buf + 16u * (uint32_t)i, x, y);
-            fx::scan(x, top, any);
-            fx::scan(y, top, any);
-        }
-        top = __reduce_max_sync(0xFFFFFFFFu, top);
-        any = (int)__reduce_or_sync(0xFFFFFFFFu, (unsigned)any);
-        if ((ctid & 31) == 0) {
-            atomicMax(&sh->top, top);
-            atomicOr(&sh->any, any);
-        }
-    }
-    ptx::named_bar_sync(bar_id, NC);
-    const int top = *(volatile int *)&sh->top, any = *(volatile int *)&sh->any;
-    const bool skip = (any != 0 && top < kOzMinTop) || top >= (2040 << 20);
+    int top;
+    kind = chunk_range<NC>(buf, c, ctid, bar_id, &sh->range, dense, top);
     auto ready = [&](int half) {  // this warp's part of a tile's half: digits staged, last sums read
         ptx::tc_fence_before();
         __syncwarp();
@@ -269,19 +220,17 @@ __device__ __forceinline__ bool run_chunk_oz(uint32_t buf, uint32_t segs, uint32
         phase[half] ^= 1;
         ptx::tc_fence_after();
     };
-    if (skip) {
+    if (kind >= CHUNK_ZERO) {
         if (ctid == 0) sh->skip = 1;
         ptx::named_bar_sync(bar_id, NC);
         for (int half = 0; half < 2; ++half) {
             ready(half);
             wait_mma(half);
         }
-        if (ptx::named_bar_or(bar_id, NC, failed)) return false;
-        oz_chunk_fp64<NC>(buf, segs, gates, nseg, ctid, swz, c, origin, bar_id);
-        return true;
+        return !ptx::named_bar_or(bar_id, NC, failed);
     }
     // |X| <= 0.985 * 2^55: seven balanced digits reach 0.996 * 2^55
-    const int E = max(top >> 20, 100) + ((top & 0xFFFFF) >= 0xF8000 ? 1 : 0);
+    const int E = (top >> 20) + ((top & 0xFFFFF) >= 0xF8000 ? 1 : 0);
     int e = E - 1077, scale = 0;  // value = X 2^e
     const int lane = ctid & 31, quarter = (threadIdx.x >> 5) & 3, sub = ctid >> 7;
     const uint32_t lane_off = (uint32_t)(quarter * 32) << 16;
@@ -378,6 +327,7 @@ __device__ __forceinline__ bool run_chunk_oz(uint32_t buf, uint32_t segs, uint32
         }
         if (ptx::named_bar_or(bar_id, NC, failed)) return false;  // the group's sums are in the chunk
     }
+    if (kind == CHUNK_TRIAL) kind = chunk_filled<NC>(buf, c, ctid, bar_id, &sh->range, top, dense.bits) ? CHUNK_DENSE : CHUNK_OTHER;
     return true;
 }
 

@@ -10,7 +10,7 @@ namespace {
 
 // Gate entry as two signed 32-bit factors: m * 2^61 = h * 2^32 + l, |l| < 2^31.
 void split(double m, int32_t &h, int32_t &l) {
-    int64_t M = std::llrint(std::ldexp(m, 61));
+    int64_t M = std::llrint(m * 0x1p61);
     if ((int32_t)(uint32_t)(uint64_t)M == INT32_MIN) ++M;  // keep -l representable
     l = (int32_t)(uint32_t)(uint64_t)M;
     h = (int32_t)((M - l) / (int64_t(1) << 32));
@@ -48,6 +48,57 @@ bool exact_gate(const DevGate<double> &g) {
     for (int l = 0; l < entries; ++l)
         if (std::fabs(g.m[2 * l]) != 1.0 || g.m[2 * l + 1] != 0.0) return false;
     return true;
+}
+
+double fp64_clocks(const DevGate<double> &g) {
+    int entries = 0;
+    switch (g.op) {
+        case OP_DENSE1: return 4.0;  // 8 multiply-adds an amplitude
+        case OP_DENSE2: return 8.0;
+        case OP_DIAG1: entries = 2; break;
+        case OP_DIAG2: entries = 4; break;
+        case OP_DIAGX: entries = ((g.b >> 8) & 0xFF) == 0xFF ? 4 : 8; break;
+        default: return 0.0;
+    }
+    int used = 0;  // entries of exactly 1 are skipped, the others take 4 multiply-adds
+    for (int l = 0; l < entries; ++l) used += g.m[2 * l] != 1.0 || g.m[2 * l + 1] != 0.0;
+    return 2.0 * used / entries;
+}
+
+double entry_ratio(const DevGate<double> &g) {
+    const int entries = g.op == OP_DENSE1 ? 4 : g.op == OP_DENSE2 ? 16 : 0;
+    double least = 4.0, most = 0.0;
+    for (int l = 0; l < entries; ++l) {
+        const double a = g.m[2 * l] * g.m[2 * l] + g.m[2 * l + 1] * g.m[2 * l + 1];
+        if (a > 0.0) least = std::min(least, a);
+        most = std::max(most, a);
+    }
+    return entries ? most / least : 1.0;
+}
+
+bool real_gate(const DevGate<double> &g) {
+    const int entries = g.op == OP_DENSE1 ? 4 : g.op == OP_DENSE2 ? 16 : g.op == OP_DIAG1 ? 2 : g.op == OP_DIAG2 ? 4 : g.op == OP_DIAGX ? 8 : 0;
+    for (int l = 0; l < entries; ++l)
+        if (g.m[2 * l + 1] != 0.0) return false;
+    return true;
+}
+
+int mixed_bits(const DevGate<double> &g) {
+    const int nb = g.op == OP_DENSE1 ? 1 : g.op == OP_DENSE2 ? 2 : 0, d = 1 << nb;
+    int mixed = 0;
+    for (int b = 0; b < nb; ++b) {
+        bool all = true;
+        for (int r = 0; r < d; ++r) {
+            double part[2] = {0, 0};  // squared moduli on columns with either value of the bit
+            for (int c = 0; c < d; ++c) {
+                const double *e = g.m + 2 * (r * d + c);
+                part[(c >> b) & 1] += e[0] * e[0] + e[1] * e[1];
+            }
+            all = all && part[0] >= 1.0 / 256 && part[1] >= 1.0 / 256;
+        }
+        if (all) mixed |= 1 << b;
+    }
+    return mixed;
 }
 
 void gather_outside_diagonals(std::vector<DevGate<double>> &gates, size_t first) {
@@ -175,12 +226,12 @@ OzSeg oz_addresses(const HostSeg &seg, int width, bool natural_ld, bool natural_
     for (int side = 0; side < 2; ++side) {
         uint32_t *t = side ? out.st : out.ld;
         const bool natural = side ? natural_st : natural_ld;
+        // both layouts are linear: an entry is the exclusive or of its bits'
         auto fill = [&](int at, int count, const int32_t *bits) {
-            for (int v = 0; v < count; ++v) {
-                int index = 0;
-                for (int k = 0; (v >> k) != 0; ++k)
-                    if ((v >> k) & 1) index |= 1 << bits[k];
-                t[at + v] = slot(index, natural);
+            t[at] = 0;
+            for (int k = 0; (1 << k) < count; ++k) {
+                const uint32_t step = slot(1 << bits[k], natural);
+                for (int v = 1 << k; v < std::min(count, 2 << k); ++v) t[at + v] = t[at + v - (1 << k)] ^ step;
             }
         };
         fill(0, 32, seg.lane);

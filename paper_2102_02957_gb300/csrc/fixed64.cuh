@@ -2,8 +2,8 @@
 //
 // Measured on GB300, per clock and SM: 2.0 FP64 FMAs, 57 to 61 32-bit integer multiply-adds into a
 // 64-bit accumulator (mad.wide.s32), 63 shifts or logic operations, 125 32-bit adds.  So a
-// complex128 gate runs faster as integer arithmetic, and no less precisely: the amplitudes that a thread holds (one gate's pair or
-// quadruple, or a register group's 16) share one exponent E, the largest of their components',
+// complex128 gate runs faster as integer arithmetic where its amplitudes are comparable in size: those that a
+// thread holds (one gate's pair or quadruple, or a register group's 16) share one exponent E, the largest of their components',
 // and every component becomes a signed 64-bit integer
 //     X = x * 2^(1081 - E)          (E: biased exponent; |X| < 2^59 on entry, 6 bits below the
 //                                    last mantissa bit of the largest component)
@@ -21,10 +21,12 @@
 //
 // Precision: a gate's output component is off by about a unit, 2^-59 of 2^E, where FP64 rounds four
 // or eight times per gate, each time to 2^-53 of the partial sum; back in FP64 it is rounded once.
-// Components more than 2^6 below the group's largest keep fewer than 53 bits of their own, an
-// absolute error that FP64 makes too as soon as a gate mixes the two.  Zeros, ones and
-// permutations stay exact.  Groups with a non-finite component or with a largest component outside
-// 2^-959 .. 2^1017 are left to the caller's FP64 code (fx::special).
+// So amplitudes near the largest gain, and those more than 2^6 below it, which FP64 would keep to 53 bits as
+// long as no gate adds anything larger to them (a phase, a small angle, a product state), lose.  Callers
+// therefore take this form only where the results draw on comparable amplitudes, and FP64 elsewhere: the
+// per-gate sweeps decide group by group (k_gate.cu, apply_fx), sections chunk by chunk (block_fx.cuh,
+// ChunkRange).  Zeros, ones and permutations stay exact.  Not for components that are not finite or for a
+// largest one outside 2^-959 .. 2^1017 (fx::special).
 #pragma once
 #include <stdint.h>
 

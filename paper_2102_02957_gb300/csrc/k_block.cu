@@ -74,7 +74,13 @@ __device__ __forceinline__ void gather_coords(const GatherArgs &ga, int64_t x, i
     for (int d = ga.rank; d < 5; ++d) coord[d] = 0;
 }
 
-// Producer (one warp): stream this CTA's chunks j = blockIdx.x + it * gridDim.x into the ring
+// Chunk number of a CTA's it-th chunk: the numbers in turn, or (from non-null) those of a list behind its count.
+__device__ __forceinline__ int64_t chunk_number(const int *from, int64_t it) {
+    const int64_t k = blockIdx.x + it * gridDim.x;
+    return from ? from[LIST_FIRST + k] : k;
+}
+
+// Producer (one warp): stream this CTA's chunks (chunk_number) into the ring
 // of nbuf shared-memory buffers (bulk copies for contiguous chunks, tensor copies for gathered
 // ones), each completing on full[slot]; a slot is reused once the store warp released it on
 // empty[slot].  A gathered chunk with more runs of bits than a tensor map has dimensions takes
@@ -83,7 +89,7 @@ __device__ __forceinline__ void gather_coords(const GatherArgs &ga, int64_t x, i
 template <typename T2>
 __device__ __forceinline__ void produce_chunks(T2 *state, int c, int64_t count, int nbuf, T2 *bufs, uint64_t *full,
                                                uint64_t *empty, volatile int *abort_flag, int *err,
-                                               const GatherArgs &ga, const CUtensorMap *tmap, uint64_t wait_ns) {
+                                               const GatherArgs &ga, const CUtensorMap *tmap, uint64_t wait_ns, const int *from) {
     const int lane = threadIdx.x & 31;
     const int chunk_amps = 1 << c;
     const uint32_t chunk_bytes = (uint32_t)chunk_amps * (uint32_t)sizeof(T2);
@@ -99,7 +105,7 @@ __device__ __forceinline__ void produce_chunks(T2 *state, int c, int64_t count, 
             }
             break;
         }
-        const int64_t j = blockIdx.x + it * gridDim.x;
+        const int64_t j = chunk_number(from, it);
         unsigned char *dst = reinterpret_cast<unsigned char *>(bufs + (size_t)s * chunk_amps);
         if (lane == 0) ptx::mbar_arrive_expect_tx(&full[s], chunk_bytes);
         __syncwarp();
@@ -146,14 +152,15 @@ __device__ __forceinline__ void write_chunk(T2 *state, int c, int64_t j, const T
     }
 }
 
-// Store warp: write the CTA's chunks back in order as their consumers finish them (done[slot])
-// and release each slot to the producer (empty[slot]) as soon as the copies have read it.
+// Store warp: write the CTA's chunks back in order as their consumers finish them (done[slot]; a non-zero
+// hold[slot]: the chunk stays as it is in memory) and release each slot to the producer (empty[slot]) as soon as the copies have read it.
 // (Keeping two write-backs in flight, releasing chunk it - 1 after chunk it's copies are issued,
 // was measured slower: the slot is held longer and the prefetch depth shrinks.)
 template <typename T2>
 __device__ __forceinline__ void store_chunks(T2 *state, int c, int64_t count, int nbuf, const T2 *bufs, uint64_t *done,
                                              uint64_t *empty, volatile int *abort_flag, int *err,
-                                             const GatherArgs &ga, const CUtensorMap *tmap, uint64_t wait_ns) {
+                                             const GatherArgs &ga, const CUtensorMap *tmap, uint64_t wait_ns, const int *from,
+                                             const volatile int *hold) {
     const int lane = threadIdx.x & 31;
     const int chunk_amps = 1 << c;
     for (int64_t it = 0; it < count; ++it) {
@@ -167,7 +174,7 @@ __device__ __forceinline__ void store_chunks(T2 *state, int c, int64_t count, in
             }
             break;
         }
-        write_chunk<T2>(state, c, blockIdx.x + it * gridDim.x, bufs + (size_t)s * chunk_amps, ga, tmap, lane);
+        if (!hold || !hold[s]) write_chunk<T2>(state, c, chunk_number(from, it), bufs + (size_t)s * chunk_amps, ga, tmap, lane);
         ptx::bulk_commit();
         ptx::bulk_wait_read<0>();
         __syncwarp();
@@ -181,20 +188,39 @@ enum : int { ENG_NONE = 0, ENG_FX = 1, ENG_OZ = 2 };
 
 static_assert(kFxGroups == 2, "scratch for merged diagonals");
 constexpr int CG2 = 2;  // consumer groups per CTA (default)
+constexpr int kFixedBufs = 3;  // chunk buffers of the fixed-point engines (at most)
 
-// G consumer groups per CTA; tensor-core groups keep NB tile buffers each
-// (G * NB * TcGeom<R>::COLS <= 512 TMEM columns).
 // Service threads of a section kernel: producer and store warp, and for complex128 tensor-core
 // sections a warp per half row that issues its MMAs; mbarriers per consumer group beside the ring's.
 constexpr int svc_threads(int eng) { return eng == ENG_OZ ? 128 : kSvcThreads; }
 constexpr int mma_bars(int eng) { return eng == ENG_OZ ? 4 : 2; }
 
+// G consumer groups per CTA; tensor-core groups keep NB tile buffers each
+// (G * NB * TcGeom<R>::COLS <= 512 TMEM columns).
 template <typename T, int R, int NC, int KU, bool TC, int G, int NB, int ENG>
 __device__ __forceinline__ void block_body(typename V2<T>::type *__restrict__ state, int c, int64_t nchunks, int nbuf,
                                            const unsigned char *__restrict__ prog, int nseg, int gate_bytes, int *err,
-                                           const CUtensorMap &tmap, const GatherArgs &ga_in, uint64_t wait_ns) {
+                                           const CUtensorMap &tmap, const GatherArgs &ga_in, uint64_t wait_ns,
+                                           const SweepArgs &sa) {
     using T2 = typename V2<T>::type;
     constexpr int kSvc = svc_threads(ENG), kBars = mma_bars(ENG);
+    // complex128 in FP64: the chunks that a fixed-point pass left, if it was one's
+    const int *from = nullptr;
+    if constexpr (ENG == ENG_NONE && sizeof(T) == 8) {
+        from = sa.from;
+        if (from) {
+            __shared__ int listed;
+            if (threadIdx.x == 0) {
+                listed = *(volatile int *)&sa.from[LIST_COUNT];
+                __threadfence();
+                // the last CTA that has read the count empties the list for the next pass
+                if (atomicInc(reinterpret_cast<unsigned *>(sa.from + LIST_READERS), gridDim.x - 1) == gridDim.x - 1) sa.from[LIST_COUNT] = 0;
+            }
+            __syncthreads();
+            nchunks = listed;
+            if (blockIdx.x >= nchunks) return;
+        }
+    }
     __shared__ GatherArgs ga;  // gathered chunks (rank > 0); rank 0 = contiguous chunk j
     if (threadIdx.x == 0) ga = ga_in;
     extern __shared__ __align__(1024) unsigned char smem[];
@@ -202,16 +228,14 @@ __device__ __forceinline__ void block_body(typename V2<T>::type *__restrict__ st
     const uint32_t chunk_bytes = (uint32_t)chunk_amps * (uint32_t)sizeof(T2);
     T2 *bufs = reinterpret_cast<T2 *>(smem);
     // block program copied into shared memory: register groups, then gate records (SIMT) or the
-    // groups' B operands (tensor cores), 16-byte aligned
-    const int seg_bytes = (int)((nseg * sizeof(DevSeg) + 15) & ~size_t(15));
+    // groups' B operands (tensor cores), 16-byte aligned; complex128 on tensor cores: address tables, B operands
+    const int seg_bytes = ENG == ENG_OZ ? 0 : (int)((nseg * sizeof(DevSeg) + 15) & ~size_t(15));
     constexpr int kBBytes = TcGeom<(R < 3 ? 3 : R)>::B_BYTES;  // B operand of one tensor-core group
     const int tab_bytes = ENG == ENG_OZ ? nseg * (int)sizeof(OzSeg) : 0;
-    const int gate_pad = (gate_bytes + 15) & ~15;  // complex128 tensor-core programs: gate area, then B operands
-    const int prog_bytes =
-        seg_bytes + tab_bytes + (ENG == ENG_OZ ? gate_pad + nseg * kOzBBytes : TC ? nseg * kBBytes : gate_bytes);
+    const int prog_bytes = seg_bytes + tab_bytes + (ENG == ENG_OZ ? nseg * kOzBBytes : TC ? nseg * kBBytes : gate_bytes);
     unsigned char *sprog = smem + (size_t)nbuf * chunk_bytes;
     const DevSeg *segs = reinterpret_cast<const DevSeg *>(sprog);
-    const unsigned char *gates = sprog + seg_bytes + tab_bytes;
+    const unsigned char *gates = sprog + seg_bytes + tab_bytes;  // or B operands
     uint64_t *full = reinterpret_cast<uint64_t *>(sprog + ((prog_bytes + 15) & ~15));
     uint64_t *empty = full + nbuf;
     uint64_t *done = empty + nbuf;
@@ -220,12 +244,18 @@ __device__ __forceinline__ void block_body(typename V2<T>::type *__restrict__ st
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(mma_bar + kBars * G) + 1;
     __shared__ int swz[24];
     [[maybe_unused]] __shared__ OzShared oz[ENG == ENG_OZ ? G : 1];
+    [[maybe_unused]] __shared__ ChunkRange range[ENG == ENG_FX ? G : 1];
+    [[maybe_unused]] __shared__ int hold[ENG == ENG_NONE ? 1 : kFixedBufs];  // per buffer: not to be written back
     // the wait bound lives in shared memory: waits are rare, a register for it in every thread is not
     __shared__ uint64_t s_wait_ns;
     constexpr uint32_t kTmemCols = 512;  // G consumer groups x NB tile buffers x TcGeom<R>::COLS
 
-    for (int k = threadIdx.x * 16; k < prog_bytes; k += blockDim.x * 16)
+    const int own_bytes = ENG == ENG_OZ ? tab_bytes : prog_bytes;
+    for (int k = threadIdx.x * 16; k < own_bytes; k += blockDim.x * 16)
         *reinterpret_cast<uint4 *>(sprog + k) = *reinterpret_cast<const uint4 *>(prog + k);
+    if constexpr (ENG == ENG_OZ)
+        for (int k = threadIdx.x * 16; k < nseg * kOzBBytes; k += blockDim.x * 16)
+            *reinterpret_cast<uint4 *>(sprog + tab_bytes + k) = *reinterpret_cast<const uint4 *>(static_cast<const unsigned char *>(sa.operands) + k);
     if (threadIdx.x < 24) swz[threadIdx.x] = sizeof(T2) == 8 ? c_swz64[threadIdx.x] : c_swz128[threadIdx.x];
     if (threadIdx.x == 0) {
         s_wait_ns = wait_ns;
@@ -253,13 +283,14 @@ __device__ __forceinline__ void block_body(typename V2<T>::type *__restrict__ st
     if (threadIdx.x < kSvc) {
         // ------------------------------------------------- producer (warp 0), store (warp 1)
         if (threadIdx.x < 32)
-            produce_chunks<T2>(state, c, count, nbuf, bufs, full, empty, abort_flag, err, ga, &tmap, wait_ns);
+            produce_chunks<T2>(state, c, count, nbuf, bufs, full, empty, abort_flag, err, ga, &tmap, wait_ns, from);
         else if (threadIdx.x < 64)
-            store_chunks<T2>(state, c, count, nbuf, bufs, done, empty, abort_flag, err, ga, &tmap, wait_ns);
+            store_chunks<T2>(state, c, count, nbuf, bufs, done, empty, abort_flag, err, ga, &tmap, wait_ns, from,
+                             ENG != ENG_NONE ? hold : nullptr);
         if constexpr (ENG == ENG_OZ) {
             static_assert(ENG != ENG_OZ || G == 1, "one consumer group");
             if (threadIdx.x >= 64) {
-                oz_issue((int)(threadIdx.x >> 5) - 2, ptx::smem_addr(gates) + (uint32_t)gate_pad, nseg, c, count, tmem_base,
+                oz_issue((int)(threadIdx.x >> 5) - 2, ptx::smem_addr(gates), nseg, c, count, tmem_base,
                          mma_bar, abort_flag, err, &s_wait_ns, &oz[0]);
                 ptx::tc_fence_before();
                 ptx::named_bar_sync(1 + G, G * NC + 64);  // before tensor memory is freed
@@ -287,7 +318,7 @@ __device__ __forceinline__ void block_body(typename V2<T>::type *__restrict__ st
     for (int64_t it = cg; cg < geff && it < count; it += geff) {
         const int s = (int)(it % nbuf);
         const int64_t u = it / nbuf;
-        const int64_t j = blockIdx.x + it * gridDim.x;
+        const int64_t j = chunk_number(from, it);
         const uint64_t *wl = &s_wait_ns;
         const bool bad = (u > 0 && !ptx::mbar_wait(&empty[s], (uint32_t)((u - 1) & 1), *(volatile const uint64_t *)wl)) ||
                          !ptx::mbar_wait(&full[s], (uint32_t)(u & 1), *(volatile const uint64_t *)wl);
@@ -297,7 +328,10 @@ __device__ __forceinline__ void block_body(typename V2<T>::type *__restrict__ st
         }
         if constexpr (ENG == ENG_OZ) {  // the last chunk's values are read: cleared before the barrier
             if (ctid < kOzMaxSegs) oz[cg].high[ctid] = 0;
-            if (ctid == 0) oz[cg].top = oz[cg].any = oz[cg].skip = 0;
+            if (ctid == 0) oz[cg].range.clear();
+            if (ctid == 0) oz[cg].skip = 0;
+        } else if constexpr (ENG == ENG_FX) {
+            if (ctid == 0) range[cg].clear();
         }
         // every thread of the group leaves together (the flag is read before the barrier)
         if (ptx::named_bar_or(bar_id, NC, bad || *abort_flag)) break;
@@ -305,15 +339,16 @@ __device__ __forceinline__ void block_body(typename V2<T>::type *__restrict__ st
         // state index of the chunk's first amplitude (its bits outside the chunk are the chunk's)
         const int64_t origin = ga.rank > 0 ? gather_origin(ga, j, 0) : j << c;
         bool failed = false;
+        [[maybe_unused]] int kind = CHUNK_DENSE, top = 0;  // uniform over the group
         if constexpr (ENG == ENG_OZ) {
-            const uint32_t gates_s = ptx::smem_addr(gates);
-            failed = !run_chunk_oz<NC>(ptx::smem_addr(buf), ptx::smem_addr(segs), gates_s - (uint32_t)tab_bytes, gates_s, gates_s + (uint32_t)gate_pad, nseg,
-                                       ctid, swz, c, origin, tmem_base, bar_id, &mma_bar[kBars * cg],
-                                       mma_phase, abort_flag, &s_wait_ns, &oz[cg]);
+            failed = !run_chunk_oz<NC>(ptx::smem_addr(buf), ptx::smem_addr(sprog), nseg, ctid, c, sa.dense, tmem_base, bar_id, &mma_bar[kBars * cg], mma_phase, abort_flag, &s_wait_ns, &oz[cg],
+                                       kind);
             ptx::fence_proxy_async_smem();
             if (ptx::named_bar_or(bar_id, NC, failed)) failed = true;
+        } else if constexpr (ENG == ENG_FX) {
+            if (sa.to) kind = chunk_range<NC>(ptx::smem_addr(buf), c, ctid, bar_id, &range[cg], sa.dense, top);
         }
-        for (int si = 0; ENG != ENG_OZ && si < nseg; ++si) {
+        for (int si = 0; ENG != ENG_OZ && kind < CHUNK_ZERO && si < nseg; ++si) {
             const uint32_t seg_addr = ptx::smem_addr(segs) + (uint32_t)(si * sizeof(DevSeg));
             [[maybe_unused]] bool ok = true;
             if constexpr (TC && ENG == ENG_NONE) {
@@ -340,6 +375,17 @@ __device__ __forceinline__ void block_body(typename V2<T>::type *__restrict__ st
             atomicCAS(err, DEV_OK, DEV_ERR_TIMEOUT);
             break;
         }
+        if constexpr (ENG == ENG_FX) {
+            if (kind == CHUNK_TRIAL)
+                kind = chunk_filled<NC>(ptx::smem_addr(buf), c, ctid, bar_id, &range[cg], top, sa.dense.bits) ? CHUNK_DENSE : CHUNK_OTHER;
+            if (sa.to) ptx::named_bar_sync(bar_id, NC);  // all have read the range before it is cleared
+        }
+        if constexpr (ENG != ENG_NONE) {
+            if (ctid == 0) {
+                hold[s] = kind != CHUNK_DENSE;
+                if (kind == CHUNK_OTHER) sa.to[LIST_FIRST + atomicAdd(sa.to + LIST_COUNT, 1)] = (int)j;
+            }
+        }
         if (nseg == 0) ptx::fence_proxy_async_smem();
         // hand the chunk to the store thread (the group's last barrier ordered all its writes)
         if (ctid == 0) ptx::mbar_arrive(&done[s]);
@@ -360,8 +406,8 @@ template <typename T, int R, int NC, int KU, bool TC, int G = CG2, int NB = 2, i
 __global__ void __launch_bounds__(G * NC + kSvcThreads, 1)
     k_block(typename V2<T>::type *__restrict__ state, int c, int64_t nchunks, int nbuf,
             const unsigned char *__restrict__ prog, int nseg, int gate_bytes, int *err,
-            const __grid_constant__ CUtensorMap tmap, const GatherArgs ga_in, uint64_t wait_ns) {
-    block_body<T, R, NC, KU, TC, G, NB, ENG>(state, c, nchunks, nbuf, prog, nseg, gate_bytes, err, tmap, ga_in, wait_ns);
+            const __grid_constant__ CUtensorMap tmap, const GatherArgs ga_in, uint64_t wait_ns, const SweepArgs sa) {
+    block_body<T, R, NC, KU, TC, G, NB, ENG>(state, c, nchunks, nbuf, prog, nseg, gate_bytes, err, tmap, ga_in, wait_ns, sa);
 }
 
 // Tensor-core sections: one CTA per SM (it takes all of the SM's tensor memory).  The register
@@ -379,30 +425,29 @@ template <typename T, int R, int NC, int KU, bool TC, int G, int NB, int ENG>
 __global__ void __maxnreg__(tc_max_regs(G * NC + svc_threads(ENG)))
     k_block_tc(typename V2<T>::type *__restrict__ state, int c, int64_t nchunks, int nbuf,
                const unsigned char *__restrict__ prog, int nseg, int gate_bytes, int *err,
-               const __grid_constant__ CUtensorMap tmap, const GatherArgs ga_in, uint64_t wait_ns) {
+               const __grid_constant__ CUtensorMap tmap, const GatherArgs ga_in, uint64_t wait_ns, const SweepArgs sa) {
     block_body<T, R, NC, KU, TC, G, NB, ENG>(state, c, nchunks, nbuf, prog, nseg, gate_bytes, err, tmap, ga_in,
-                                               wait_ns);
+                                               wait_ns, sa);
 }
 
 constexpr size_t kMaxBlockSmem = 227 * 1024 - 1024;  // minus the static swizzle table (1 KiB aligned)
 
 template <typename T, int R, int NC, int KU, bool TC = false, int G = CG2, int NB = 2, int ENG = ENG_NONE>
 void launch_typed(void *state, int n, int ce, const void *prog, int nseg, int gate_bytes, int *err, cudaStream_t st,
-                  const CUtensorMap &tmap, const GatherArgs &ga, uint64_t wait_ns) {
+                  const CUtensorMap &tmap, const GatherArgs &ga, uint64_t wait_ns, const SweepArgs &sa = SweepArgs{}) {
     if (ce - R - 5 > kMaxRest) fail(SV_ERR_UNSUPPORTED, "chunk too wide for the register-group layout");
     using T2 = typename V2<T>::type;
     const size_t chunk_bytes = (size_t(1) << ce) * sizeof(T2);
     const int64_t nchunks = int64_t(1) << (n - ce);
-    const size_t seg_bytes = (nseg * sizeof(DevSeg) + 15) & ~size_t(15);
-    const size_t prog_bytes =
-        (seg_bytes +
-         (ENG == ENG_OZ ? (((size_t)gate_bytes + 15) & ~size_t(15)) + (size_t)nseg * (kOzBBytes + sizeof(OzSeg))
-          : TC          ? (size_t)nseg * TcGeom<(R < 3 ? 3 : R)>::B_BYTES
-                        : (size_t)gate_bytes) +
-         15) &
-        ~size_t(15);
+    const size_t seg_bytes = ENG == ENG_OZ ? 0 : (nseg * sizeof(DevSeg) + 15) & ~size_t(15);
+    const size_t prog_bytes = (seg_bytes +
+                               (ENG == ENG_OZ ? (size_t)nseg * (kOzBBytes + sizeof(OzSeg))
+                                : TC          ? (size_t)nseg * TcGeom<(R < 3 ? 3 : R)>::B_BYTES
+                                              : (size_t)gate_bytes) +
+                               15) &
+                              ~size_t(15);
     if (TC && ENG == ENG_NONE && G * NB * TcGeom<(R < 3 ? 3 : R)>::COLS > 512) fail(SV_ERR_UNSUPPORTED, "tile buffers exceed tensor memory");
-    int nbuf = TC && ENG == ENG_NONE ? G + 2 : 3;  // tensor cores: every consumer group holds a chunk, plus prefetch
+    int nbuf = TC && ENG == ENG_NONE ? G + 2 : kFixedBufs;  // tensor cores: every consumer group holds a chunk, plus prefetch
     // program + mbarriers (full, empty, done per buffer; two per consumer group), abort flag,
     // TMEM address
     const size_t extra = prog_bytes + (size_t)(3 * nbuf + mma_bars(ENG) * G) * 8 + 16;
@@ -426,11 +471,11 @@ void launch_typed(void *state, int n, int ce, const void *prog, int nseg, int ga
     if constexpr (TC) {
         auto kern = k_block_tc<T, R, NC, KU, TC, G, NB, ENG>;
         kern<<<grid_of(kern), G * NC + svc_threads(ENG), smem, st>>>((T2 *)state, ce, nchunks, nbuf, (const unsigned char *)prog, nseg,
-                                                     gate_bytes, err, tmap, ga, wait_ns);
+                                                     gate_bytes, err, tmap, ga, wait_ns, sa);
     } else {
         auto kern = k_block<T, R, NC, KU, TC, G, NB, ENG>;
         kern<<<grid_of(kern), G * NC + svc_threads(ENG), smem, st>>>((T2 *)state, ce, nchunks, nbuf, (const unsigned char *)prog, nseg,
-                                                     gate_bytes, err, tmap, ga, wait_ns);
+                                                     gate_bytes, err, tmap, ga, wait_ns, sa);
     }
     check_cuda(cudaGetLastError(), "block kernel launch");
 }
@@ -482,30 +527,33 @@ CUtensorMap make_gather_map(void *state, const GatherLayout &lay, int elem_bytes
 // consumers (17 warps, <= 96 registers a thread); 2^5-amplitude groups and complex128 run
 // 2 x 128 (9 warps, <= 168 registers).  Each thread holds one register group at a time.
 static void dispatch(int dtype, int r, void *state, int n, int ce, const void *prog, int nseg, int gate_bytes, bool fixed,
-                     int *err, cudaStream_t st, const CUtensorMap &m, const GatherArgs &ga, uint64_t wait_ns) {
+                     int *err, cudaStream_t st, const CUtensorMap &m, const GatherArgs &ga, uint64_t wait_ns,
+                     const SweepArgs &sa) {
     if (dtype == SV_C64) {
         if (r == 4) launch_typed<float, 4, 256, 1>(state, n, ce, prog, nseg, gate_bytes, err, st, m, ga, wait_ns);
         else launch_typed<float, 5, 128, 1>(state, n, ce, prog, nseg, gate_bytes, err, st, m, ga, wait_ns);
     } else if (fixed) {
-        launch_typed<double, 4, 128, 1, false, CG2, 2, ENG_FX>(state, n, ce, prog, nseg, gate_bytes, err, st, m, ga, wait_ns);
+        launch_typed<double, 4, 128, 1, false, CG2, 2, ENG_FX>(state, n, ce, prog, nseg, gate_bytes, err, st, m, ga, wait_ns,
+                                                                         sa);
     } else {
-        launch_typed<double, 4, 128, 1>(state, n, ce, prog, nseg, gate_bytes, err, st, m, ga, wait_ns);
+        launch_typed<double, 4, 128, 1>(state, n, ce, prog, nseg, gate_bytes, err, st, m, ga, wait_ns, sa);
     }
 }
 
 void launch_block(int dtype, void *state, int n, int c, const void *dev_prog, int nseg, int gate_bytes, bool fixed,
-                  int *dev_err, int seg_bits, cudaStream_t st, uint64_t wait_ns) {
+                  int *dev_err, int seg_bits, cudaStream_t st, uint64_t wait_ns, const SweepArgs &sa) {
     const int ce = c < n ? c : n;
     if (ce < 4) fail(SV_ERR_UNSUPPORTED, "blocked path needs a chunk of at least 4 bits");
     const int r = seg_bits < ce ? seg_bits : ce;  // the register groups were built with this width
     GatherArgs ga{};  // rank 0: contiguous chunk j
     CUtensorMap none;
     std::memset(&none, 0, sizeof(none));
-    dispatch(dtype, r, state, n, ce, dev_prog, nseg, gate_bytes, fixed, dev_err, st, none, ga, wait_ns);
+    dispatch(dtype, r, state, n, ce, dev_prog, nseg, gate_bytes, fixed, dev_err, st, none, ga, wait_ns, sa);
 }
 
 void launch_block_gather(int dtype, void *state, int n, const GatherLayout &lay, const void *dev_prog, int nseg,
-                         int gate_bytes, bool fixed, int *dev_err, int seg_bits, cudaStream_t st, uint64_t wait_ns) {
+                         int gate_bytes, bool fixed, int *dev_err, int seg_bits, cudaStream_t st, uint64_t wait_ns,
+                         const SweepArgs &sa) {
     const int ce = lay.ce;
     if (ce < 4) fail(SV_ERR_UNSUPPORTED, "blocked path needs a chunk of at least 4 bits");
     if (reinterpret_cast<uintptr_t>(state) % 16) fail(SV_ERR_ARG, "state buffer not 16-byte aligned");
@@ -515,7 +563,7 @@ void launch_block_gather(int dtype, void *state, int n, const GatherLayout &lay,
         fail(SV_ERR_UNSUPPORTED, "gathered chunk boxes smaller than 128 bytes (pin more low bits)");
     const CUtensorMap m = make_gather_map(state, lay, elem);
     const int r = seg_bits < ce ? seg_bits : ce;
-    dispatch(dtype, r, state, n, ce, dev_prog, nseg, gate_bytes, fixed, dev_err, st, m, lay.args, wait_ns);
+    dispatch(dtype, r, state, n, ce, dev_prog, nseg, gate_bytes, fixed, dev_err, st, m, lay.args, wait_ns, sa);
 }
 
 }  // namespace sv
@@ -549,7 +597,7 @@ void launch_block_tc(void *state, int n, int c, const GatherLayout *lay, const v
         launch_typed<float, 4, 128, 1, true, 2, 2>(state, n, ce, dev_prog, nseg, 0, dev_err, st, m, ga, wait_ns);
 }
 
-int fx_buffers(int ce, int nseg, size_t gate_bytes) {
+int simt_buffers(int ce, int nseg, size_t gate_bytes) {
     const size_t chunk = size_t(16) << ce, fixed = nseg * sizeof(DevSeg) + gate_bytes + 256;
     int n = 3;
     while (n > 0 && n * chunk + fixed > kMaxBlockSmem) --n;
@@ -558,22 +606,23 @@ int fx_buffers(int ce, int nseg, size_t gate_bytes) {
 
 // Shared memory beside the chunk buffers: barriers and flags (launch_typed's `extra`), the groups'
 // static words.
-int oz_max_segs(int ce, size_t gate_bytes) {
+int oz_max_segs(int ce) {
     if (ce < 11 || ce > 13) return 0;
     const size_t chunk = size_t(16) << ce;
     // two chunk buffers (one computed on, one in transfer) where that leaves room for two groups
     for (int bufs = 2; bufs >= 1; --bufs) {
-        const size_t fixed = bufs * chunk + kOzMaxSegs * sizeof(DevSeg) + ((gate_bytes + 15) & ~size_t(15)) + 1024;
+        const size_t fixed = bufs * chunk + 1024;
         const size_t room = fixed < kMaxBlockSmem ? (kMaxBlockSmem - fixed) / (kOzBBytes + sizeof(OzSeg)) : 0;
         if (room >= 2 || (bufs == 1 && room >= 1)) return (int)std::min<size_t>(room, kOzMaxSegs);
     }
     return 0;
 }
 
-void launch_block_oz(void *state, int n, int c, const GatherLayout *lay, const void *dev_prog, int nseg, int gate_bytes,
-                     int *dev_err, cudaStream_t st, uint64_t wait_ns) {
+void launch_block_oz(void *state, int n, int c, const GatherLayout *lay, const void *dev_prog, int nseg, int *dev_err,
+                     cudaStream_t st, uint64_t wait_ns, const SweepArgs &sa) {
     const int ce = lay ? lay->ce : (c < n ? c : n);
     if (ce < 11 || nseg < 1 || nseg > kOzMaxSegs) fail(SV_ERR_UNSUPPORTED, "complex128 tensor-core sections need chunks of at least 2^11 amplitudes");
+    if (reinterpret_cast<uintptr_t>(state) % 16) fail(SV_ERR_ARG, "state buffer not 16-byte aligned");
     GatherArgs ga{};
     CUtensorMap m;
     std::memset(&m, 0, sizeof(m));
@@ -583,7 +632,7 @@ void launch_block_oz(void *state, int n, int c, const GatherLayout *lay, const v
         m = make_gather_map(state, *lay, 16);
         ga = lay->args;
     }
-    launch_typed<double, 4, 512, 1, true, 1, 1, ENG_OZ>(state, n, ce, dev_prog, nseg, gate_bytes, dev_err, st, m, ga, wait_ns);
+    launch_typed<double, 4, 512, 1, true, 1, 1, ENG_OZ>(state, n, ce, dev_prog, nseg, 0, dev_err, st, m, ga, wait_ns, sa);
 }
 
 }  // namespace sv

@@ -140,7 +140,8 @@ __global__ void __launch_bounds__(256) k_compose_f64(const ComposeSeg *__restric
 // M = round(U 2^(54 + s)) in balanced base-256 digits as FP16 B operands, s the most (up to 2) that
 // keeps |M| within 0.99 * 2^55.  One CTA per group, one thread
 // per element (row r, column j); element products read and write two shared copies in turn.
-__global__ void __launch_bounds__(256) k_compose_fx(const OzCompose *__restrict__ groups, unsigned char *__restrict__ prog) {
+__global__ void __launch_bounds__(256) k_compose_fx(const OzCompose *__restrict__ groups, unsigned char *__restrict__ prog,
+                                                    unsigned char *__restrict__ operands) {
     constexpr int NA = 16;
     __shared__ fx::Real Ur[2][NA * NA], Ui[2][NA * NA];
     const OzCompose sg = groups[blockIdx.x];
@@ -208,7 +209,7 @@ __global__ void __launch_bounds__(256) k_compose_fx(const OzCompose *__restrict_
     if (e == 0) *reinterpret_cast<int *>(prog + sg.scale_off) = s;
     const long long half = 16 >> s;
     const long long re = (ure + half) >> (5 - s), im = (uim + half) >> (5 - s);
-    unsigned char *b = prog + sg.b_off + (r >> 3) * (kOzBBytes / 2);
+    unsigned char *b = operands + sg.b_off + (r >> 3) * (kOzBBytes / 2);
 #pragma unroll
     for (int part = 0; part < 2; ++part) {
         const int n = 2 * (r & 7) + part;  // output real within its half row
@@ -228,9 +229,9 @@ __global__ void __launch_bounds__(256) k_compose_fx(const OzCompose *__restrict_
 
 }  // namespace
 
-void launch_compose_oz(const void *dev_groups, int ngroups, void *dev_prog, cudaStream_t st) {
+void launch_compose_oz(const void *dev_groups, int ngroups, void *dev_prog, void *dev_operands, cudaStream_t st) {
     if (ngroups <= 0) return;
-    k_compose_fx<<<ngroups, 256, 0, st>>>((const OzCompose *)dev_groups, (unsigned char *)dev_prog);
+    k_compose_fx<<<ngroups, 256, 0, st>>>((const OzCompose *)dev_groups, (unsigned char *)dev_prog, (unsigned char *)dev_operands);
     check_cuda(cudaGetLastError(), "compose kernel launch");
 }
 

@@ -61,6 +61,7 @@ sv_plan *plan_blocking(int n, const sv_gate *gates, int64_t n_gates, const sv_op
     plan->tc_no_renorm = o.tc_no_renorm ? 1 : 0;
     if (o.wait_limit_ms < 0) { delete plan; fail(SV_ERR_ARG, "wait_limit_ms must be >= 0"); }
     plan->wait_limit_ms = o.wait_limit_ms;
+    plan->fp64 = o.fp64_sections ? 1 : 0;
     plan->keys.reserve((size_t)n_gates);
 
     std::vector<int32_t> lab(n);

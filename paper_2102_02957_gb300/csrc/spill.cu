@@ -135,7 +135,7 @@ std::vector<Pass> make_passes(const sv_plan &plan, int M) {
 struct PassRun {
     int m = 0;
     std::vector<int> high;
-    std::function<void(void *buf, int nsub, cudaStream_t st)> work;
+    std::function<void(void *buf, int nsub, int slot, cudaStream_t st)> work;  // slot: which half of the work buffer
 };
 
 int local_bit(const std::vector<int> &high, int m, int b) {
@@ -186,7 +186,7 @@ void run_pass(const PassRun &p, int n, size_t elem, unsigned char *host, unsigne
                                            st[k]),
                            "cudaMemcpyAsync(host slab in)");
         }
-        p.work(buf, nsub, st[k]);
+        p.work(buf, nsub, k, st[k]);
         if (by_kernel) {
             k_slab_copy<false><<<grid, 256, 0, st[k]>>>(reinterpret_cast<uint4 *>(buf), reinterpret_cast<uint4 *>(host_dev), sa);
             check_cuda(cudaGetLastError(), "slab scatter launch");
@@ -209,7 +209,7 @@ struct GatheredPass {
     std::vector<sv_gate> gates;  // on sub-state bits
     std::unique_ptr<sv_plan> plan;
     SimtPrograms sp;
-    size_t off = 0;  // of its programs in the upload
+    size_t off = 0, b_off = 0;  // of its programs in the upload, of their operands
 };
 
 // The sections of the circuit on M-bit chunks with the low bits pinned: the widest slabs among those
@@ -232,7 +232,7 @@ std::unique_ptr<sv_plan> outer_plan(int n, const sv_gate *gates, int64_t n_gates
     return best;
 }
 
-std::vector<GatheredPass> gathered_passes(const sv_plan &outer, const sv_gate *gates, int c, int seg_bits, int dtype) {
+std::vector<GatheredPass> gathered_passes(const sv_plan &outer, const sv_gate *gates, int c, int seg_bits, int fp64, int dtype) {
     std::vector<GatheredPass> out;
     for (const PlanOp &op : outer.ops) {
         if (op.gates.empty()) continue;
@@ -251,6 +251,7 @@ std::vector<GatheredPass> gathered_passes(const sv_plan &outer, const sv_gate *g
         sv_options_default(&o);
         o.chunk_bits = std::min(c, nsub);
         o.seg_bits = seg_bits;
+        o.fp64_sections = fp64;
         if (o.chunk_bits >= 9 && o.chunk_bits < nsub) {
             o.gather_pinned = 4;
             o.lookahead = g.gates.size() <= 4000;
@@ -315,7 +316,7 @@ extern "C" sv_status sv_apply_circuit_host(int32_t n, int32_t dtype, void *host_
         for (int64_t i = 0; i < n_gates; ++i) natural = natural && !(gates[i].flags & SV_GATE_SWAP);
         if (natural && passes.size() > 1) {
             const std::unique_ptr<sv_plan> outer = outer_plan(n, gates, n_gates, M, elem, host_dev != nullptr);
-            if (outer && outer->ops.size() < passes.size()) gathered = gathered_passes(*outer, gates, c, plan->seg_bits, dtype);
+            if (outer && outer->ops.size() < passes.size()) gathered = gathered_passes(*outer, gates, c, plan->seg_bits, plan->fp64, dtype);
         }
         SimtPrograms sp;
         std::vector<unsigned char> programs;
@@ -328,16 +329,30 @@ extern "C" sv_status sv_apply_circuit_host(int32_t n, int32_t dtype, void *host_
             g.off = programs.size();
             programs.insert(programs.end(), g.sp.host.begin(), g.sp.host.end());
         }
-        check_cuda(cudaMalloc(&progbuf, std::max<size_t>(programs.size(), 256)), "cudaMalloc(programs)");
+        // behind the programs: a list of chunks (launch_section) for each of the two streams, B operands
+        size_t list_bytes = gathered.empty() ? redo_list_bytes(sp, M, c) : 0;
+        for (const GatheredPass &g : gathered)
+            list_bytes = std::max(list_bytes, redo_list_bytes(g.sp, g.m + (int)g.high.size(), g.plan->c));
+        const size_t list_off = (programs.size() + 255) / 256 * 256, b_off = list_off + 2 * list_bytes;
+        size_t b_bytes = sp.b_bytes;
+        for (GatheredPass &g : gathered) {
+            g.b_off = b_off + b_bytes;
+            b_bytes += g.sp.b_bytes;
+        }
+        check_cuda(cudaMalloc(&progbuf, b_off + b_bytes + 256), "cudaMalloc(programs)");
         check_cuda(cudaMalloc(&dev_err, sizeof(int)), "cudaMalloc(error word)");
         const cudaStream_t caller = (cudaStream_t)cuda_stream;
         check_cuda(cudaMemsetAsync(dev_err, 0, sizeof(int), caller), "cudaMemsetAsync");
         unsigned char *const prog = static_cast<unsigned char *>(progbuf);
+        if (list_bytes)
+            for (int k = 0; k < 2; ++k)
+                check_cuda(cudaMemsetAsync(prog + list_off + (size_t)k * list_bytes, 0, LIST_FIRST * sizeof(int), caller), "cudaMemsetAsync(list)");
+        auto list_of = [=](int slot) { return reinterpret_cast<int *>(prog + list_off + (size_t)slot * list_bytes); };
         if (!programs.empty())
             check_cuda(cudaMemcpyAsync(prog, programs.data(), programs.size(), cudaMemcpyHostToDevice, caller),
                        "upload programs");
-        launch_compose_oz(prog + sp.oz_off, sp.noz, prog, caller);
-        for (const GatheredPass &g : gathered) launch_compose_oz(prog + g.off + g.sp.oz_off, g.sp.noz, prog + g.off, caller);
+        launch_compose_oz(prog + sp.oz_off, sp.noz, prog, prog + b_off, caller);
+        for (const GatheredPass &g : gathered) launch_compose_oz(prog + g.off + g.sp.oz_off, g.sp.noz, prog + g.off, prog + g.b_off, caller);
         for (auto &s : st) check_cuda(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking), "cudaStreamCreate");
         check_cuda(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming), "cudaEventCreate");
         auto join = [&](cudaStream_t from, cudaStream_t to) {
@@ -355,7 +370,7 @@ extern "C" sv_status sv_apply_circuit_host(int32_t n, int32_t dtype, void *host_
                 for (size_t i = 0; i < p.items.size(); ++i)
                     for (const auto &pq : p.items[i].pairs)
                         pairs[i].emplace_back(local_bit(p.high, p.m, pq.first), local_bit(p.high, p.m, pq.second));
-                runs.push_back(PassRun{p.m, p.high, [&, pairs](void *buf, int nsub, cudaStream_t s) {
+                runs.push_back(PassRun{p.m, p.high, [&, pairs](void *buf, int nsub, int slot, cudaStream_t s) {
                                            for (size_t i = 0; i < p.items.size(); ++i) {
                                                const int op = p.items[i].op;
                                                if (plan->ops[(size_t)op].kind != 2) {
@@ -366,8 +381,8 @@ extern "C" sv_status sv_apply_circuit_host(int32_t n, int32_t dtype, void *host_
                                                for (const auto &q : sp.progs)
                                                    if (q.op_index == op) {
                                                        found = true;
-                                                       launch_section(dtype, buf, nsub, plan->c, prog, q, sp.seg_bits, dev_err,
-                                                                      s, wait_ns);
+                                                       launch_section(dtype, buf, nsub, plan->c, prog, prog + b_off, q, sp.seg_bits,
+                                                                      list_of(slot), dev_err, s, wait_ns);
                                                    }
                                                if (!found) fail(SV_ERR_PLAN, "no program for a blocking section");
                                            }
@@ -375,14 +390,14 @@ extern "C" sv_status sv_apply_circuit_host(int32_t n, int32_t dtype, void *host_
             }
         } else {
             for (const GatheredPass &g : gathered)
-                runs.push_back(PassRun{g.m, g.high, [&](void *buf, int nsub, cudaStream_t s) {
+                runs.push_back(PassRun{g.m, g.high, [&](void *buf, int nsub, int slot, cudaStream_t s) {
                                            size_t k = 0;
                                            for (size_t op = 0; op < g.plan->ops.size(); ++op) {
                                                if (g.plan->ops[op].kind == 1 || g.plan->ops[op].kind == 3)
                                                    launch_permute(dtype, buf, nsub, g.plan->ops[op].pairs, s);
                                                for (; k < g.sp.progs.size() && g.sp.progs[k].op_index == (int)op; ++k)
-                                                   launch_section(dtype, buf, nsub, g.plan->c, prog + g.off, g.sp.progs[k],
-                                                                  g.sp.seg_bits, dev_err, s, wait_ns);
+                                                   launch_section(dtype, buf, nsub, g.plan->c, prog + g.off, prog + g.b_off, g.sp.progs[k],
+                                                                  g.sp.seg_bits, list_of(slot), dev_err, s, wait_ns);
                                            }
                                        }});
         }

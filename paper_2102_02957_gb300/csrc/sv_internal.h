@@ -59,7 +59,7 @@ struct HostSeg;
 
 struct sv_plan {
     int32_t n = 0, c = 0, reserve = 0, restore = 1, seg_bits = 4, use_tc = 0, pinned = 0;
-    int32_t tc_no_renorm = 0, wait_limit_ms = 0;  // executor options carried by the plan
+    int32_t tc_no_renorm = 0, wait_limit_ms = 0, fp64 = 0;  // executor options carried by the plan
     std::vector<sv::PlanOp> ops;
     std::vector<int32_t> final_map;
     std::vector<sv::GateKey> keys;  // structure of the gate list it was made from
@@ -172,30 +172,37 @@ void encode_gate(const sv_gate &g, const BlockGate &bg, const HostSeg &seg, DevG
 // Block fixed-point programs of complex128 sections (fixed64.cuh, block_fx.cuh).
 // Whether the dim x dim matrix is unitary to 1e-9, as the fixed-point ranges need.
 bool fx_unitary(const double *m, int dim);
+// Clocks per amplitude and SM that a gate takes in FP64 register groups, at 2 FP64 operations a clock.
+double fp64_clocks(const DevGate<double> &g);
+// Square of the ratio of the largest to the smallest non-zero entry of a gate that mixes amplitudes, else 1.
+double entry_ratio(const DevGate<double> &g);
+// Whether a gate's entries are all real.
+bool real_gate(const DevGate<double> &g);
+// Local bits of a gate that its matrix mixes (bit 0: a, bit 1: b), see Dense.
+int mixed_bits(const DevGate<double> &g);
 // Fixed-point factors of `count` complex entries (4 ints each).
 void fx_pack(const double *m, int count, int32_t *entries);
 // Whether a gate only exchanges amplitudes or multiplies them by 1 or -1.
 bool exact_gate(const DevGate<double> &g);
-// Tensor-core programs of complex128 sections (block_oz.cuh): after the gate area, per register
-// group the B operand of its unitary in base-256 digits, two halves of 16 output reals, each 8 digit
-// blocks side by side (the last zero), K-major FP16.
+// Tensor-core programs of complex128 sections (block_oz.cuh): address tables (OzSeg) of the register groups, and
+// in device memory of their own per group the B operand of its unitary in base-256 digits, two halves of 16
+// output reals, each 8 digit blocks side by side (the last zero), K-major FP16.
 constexpr int kOzBBytes = 16384;
 // Addresses of a register group's rows in the chunk, loading and storing side: byte offsets of the 32
 // lanes, of the 16 row blocks (quarter | tile << 2) and of the 16 amplitudes, to be combined by
-// exclusive or (both the natural and the swizzled layout are linear).  Programs hold one per group
-// between the groups' DevSegs and the gate area.
+// exclusive or (both the natural and the swizzled layout are linear).
 struct OzSeg {
     uint32_t ld[64], st[64];
     int32_t scale, unused[3];  // s of the group's operand (written by the composer)
 };
 OzSeg oz_addresses(const HostSeg &seg, int width, bool natural_ld, bool natural_st);
-// One group to compose: gates [g0, g1) of the gate area at gates_off of the program, B at b_off, its
-// scale's word at scale_off.
+// One group to compose: gates [g0, g1) of the gate area at gates_off of the program, its scale's word at
+// scale_off; B at b_off of the operands.
 struct OzCompose {
     uint32_t gates_off, b_off, scale_off;
     int32_t g0, g1;
 };
-void launch_compose_oz(const void *dev_groups, int ngroups, void *dev_prog, cudaStream_t st);
+void launch_compose_oz(const void *dev_groups, int ngroups, void *dev_prog, void *dev_operands, cudaStream_t st);
 // Moves the OP_DIAGX gates of a register group's list as far back as they commute (a diagonal on a
 // register bit passes every gate that is diagonal or acts on other bits, a phase every gate), so
 // that they meet in few runs.
@@ -295,25 +302,50 @@ struct Mat2 { float m[32]; };
 
 void launch_gate(int dtype, void *state, int n, const sv_gate &g, cudaStream_t st);
 void launch_init_basis(int dtype, void *state, int n, uint64_t basis, cudaStream_t st);
+// When a chunk is dense enough for one exponent: at most `most` of its amplitudes (zeros too) are more than
+// `orders` binary orders below its largest component.  A unit is 2^-54 of that component, and FP64 is as
+// inexact only for results that draw on amplitudes near it.  So it depends on what the sweep's gates mix:
+// a bit is mixed where every row of some gate has at least 1/16 of its norm on either value of the
+// bit.  With kMixedBits of them or more, up to half of the 2^bits amplitudes that every result draws on
+// may be small (and at most 1 in 32 of the chunk): a chunk of 2^12 of a state as random circuits leave it has 1 amplitude
+// below 8 orders where it is complex, 45 where it is real, so that practically none falls out.  Else
+// (phases, small angles) all have to be within kNearOrders.
+struct Dense {
+    int orders, most;
+    unsigned bits;  // chunk bits that dense gates act on
+    int trial;      // whether gates may fill a chunk within kNearOrders from one amplitude
+};
+constexpr int kNearOrders = 4, kFarOrders = 8, kMixedBits = 6;
 // Section programs of a plan with SIMT register groups (complex128: tensor-core sweeps where they
 // apply), laid out as one device upload (api.cu).
 struct SimtPrograms {
     struct Prog {
         size_t off;
         int nseg, gate_bytes, op_index;
-        bool fixed, oz, gathered;
+        bool fixed, oz, gathered;  // complex128 off FP64: on the integer pipe, or the tensor cores (block_oz.cuh)
+        bool redo;                 // ... with an FP64 program for the chunks it leaves
+        size_t redo_off;
+        int redo_bytes;
+        Dense dense;
+        int oz_first;      // of its nseg groups to compose
+        size_t b_off;      // their operands
         GatherLayout lay;  // gathered chunks
     };
     std::vector<unsigned char> host;
     std::vector<Prog> progs;
     size_t oz_off = 0;  // groups to compose once uploaded (launch_compose_oz)
     int noz = 0;
+    size_t b_bytes = 0;  // device memory for their operands
     int seg_bits = 4;
 };
 void build_simt_programs(const sv_plan *plan, const sv_gate *gates, int dtype, SimtPrograms &out);
-// Launch one section of 2^n amplitudes (chunks of c bits) from its program at base + p.off.
-void launch_section(int dtype, void *state, int n, int c, const unsigned char *base, const SimtPrograms::Prog &p,
-                    int seg_bits, int *dev_err, cudaStream_t st, uint64_t wait_ns);
+// Device memory that launch_section's `list` needs for a state of 2^n amplitudes in chunks of c bits (0: none),
+// its first LIST_FIRST ints zeroed.  One list serves one stream at a time.
+size_t redo_list_bytes(const SimtPrograms &sp, int n, int c);
+// Launch one section of 2^n amplitudes (chunks of c bits) from its program at base + p.off and operands
+// + p.b_off; returns the number of kernels.
+int launch_section(int dtype, void *state, int n, int c, const unsigned char *base, const unsigned char *operands,
+                   const SimtPrograms::Prog &p, int seg_bits, int *list, int *dev_err, cudaStream_t st, uint64_t wait_ns);
 // Amplitudes with bit `bit` == value, in index order, to / from a buffer of 2^(n-1) (k_shard.cu).
 void launch_shard_half(bool pack, int dtype, void *state, int n, int bit, int value, void *buf, cudaStream_t st);
 
@@ -323,23 +355,33 @@ void launch_permute(int dtype, void *state, int n, const std::vector<std::pair<i
 
 // Bounded device waits: wait_ns (kDefaultWaitNs unless the plan sets wait_limit_ms).
 constexpr uint64_t kDefaultWaitNs = 4000000000ull;
+// Chunks of a complex128 section that a fixed-point or tensor-core pass leaves to FP64 (block_fx.cuh,
+// ChunkRange): the pass appends their numbers to `to` (device memory), and an FP64 pass with `from` set runs
+// those alone and empties the list.  to null: all gates of the section are exact, every chunk runs.
+struct SweepArgs {
+    int *to = nullptr;
+    Dense dense;
+    int *from = nullptr;
+    const void *operands = nullptr;  // B operands of a tensor-core sweep
+};
+enum : int { LIST_COUNT = 0, LIST_READERS = 1, LIST_FIRST = 2 };  // both 0 in an empty list; then room for every chunk
 // SIMT sections: the program is nseg register groups and a gate area of gate_bytes bytes, gate
 // records (DevGate) or, `fixed` (complex128), a fixed-point area (encode_fx).
 void launch_block(int dtype, void *state, int n, int c, const void *dev_prog, int nseg, int gate_bytes, bool fixed,
-                  int *dev_err, int seg_bits, cudaStream_t st, uint64_t wait_ns = kDefaultWaitNs);
+                  int *dev_err, int seg_bits, cudaStream_t st, uint64_t wait_ns = kDefaultWaitNs, const SweepArgs &sa = SweepArgs{});
 // Blocking section over a gathered chunk (bits in `mask`), fetched and written back with
 // tensor copies.
 void launch_block_gather(int dtype, void *state, int n, const GatherLayout &lay, const void *dev_prog, int nseg,
                          int gate_bytes, bool fixed, int *dev_err, int seg_bits, cudaStream_t st,
-                         uint64_t wait_ns = kDefaultWaitNs);
-// Chunk buffers that an integer-pipe section of 2^ce amplitudes gets beside its program.
-int fx_buffers(int ce, int nseg, size_t gate_bytes);
-// Register groups (at most) that one tensor-core sweep of a complex128 chunk of ce bits takes beside
-// gate_bytes of gate area; 0: the chunk cannot run there.
-int oz_max_segs(int ce, size_t gate_bytes);
+                         uint64_t wait_ns = kDefaultWaitNs, const SweepArgs &sa = SweepArgs{});
+// Chunk buffers that a complex128 SIMT section of 2^ce amplitudes gets beside its program (0: it does not fit).
+int simt_buffers(int ce, int nseg, size_t gate_bytes);
+// Register groups (at most) that one tensor-core sweep of a complex128 chunk of ce bits takes; 0: the
+// chunk cannot run there.
+int oz_max_segs(int ce);
 // Tensor-core blocking section of a complex128 state; `lay` null for a contiguous chunk of c bits.
-void launch_block_oz(void *state, int n, int c, const GatherLayout *lay, const void *dev_prog, int nseg, int gate_bytes,
-                     int *dev_err, cudaStream_t st, uint64_t wait_ns = kDefaultWaitNs);
+void launch_block_oz(void *state, int n, int c, const GatherLayout *lay, const void *dev_prog, int nseg, int *dev_err,
+                     cudaStream_t st, uint64_t wait_ns, const SweepArgs &sa);
 // Tensor-core blocking section (complex64, register groups of seg_bits = 3, 4 or 5 bits, B
 // operands in the program, tc_b_bytes(seg_bits) each); `lay` null for a contiguous chunk of c bits.
 void launch_block_tc(void *state, int n, int c, const GatherLayout *lay, const void *dev_prog, int nseg, int *dev_err,
