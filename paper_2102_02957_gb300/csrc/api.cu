@@ -397,7 +397,7 @@ struct ProgramBuilder {
         const int g0 = segs[(size_t)s0].g0;
         for (int k = s0; k < s1; ++k) {
             DevSeg d = segs[(size_t)k];
-            d.flags = (int8_t)((k == s0 ? 1 : 0) | (k + 1 == s1 ? 2 : 0) | (raw_flags ? d.flags & kSegRaw : 0));
+            d.flags = (int8_t)((k == s0 ? 1 : 0) | (k + 1 == s1 ? 2 : 0) | (raw_flags ? d.flags & (kSegRaw | kSegDiag) : 0));
             d.g0 = (int16_t)(d.g0 - g0);
             d.g1 = (int16_t)(d.g1 - g0);
             put(&d, sizeof(d));
@@ -412,19 +412,25 @@ struct ProgramBuilder {
     bool fixed_section(SimtPrograms::Prog pg, const std::vector<HostSeg> &segs, std::vector<DevSeg> &dsegs,
                        const std::vector<DevGate<double>> &all, int width) {
         const int nseg = (int)dsegs.size();
-        bool exact = true;  // only exchanges and signs
+        bool exact = true, single = true;  // only exchanges and signs; amplitude by amplitude: these and diagonals
         for (DevSeg &d : dsegs) {
-            if (std::all_of(all.begin() + d.g0, all.begin() + d.g1, exact_gate)) d.flags |= kSegRaw;
-            else exact = false;
+            if (std::all_of(all.begin() + d.g0, all.begin() + d.g1, exact_gate)) {
+                d.flags |= kSegRaw;
+                continue;
+            }
+            exact = false;
+            if (std::all_of(all.begin() + d.g0, all.begin() + d.g1, diagonal_gate)) d.flags |= kSegDiag;
+            else single = false;
         }
         if (nseg == 0) return false;
-        if (!exact) {
+        const bool outside = std::any_of(all.begin(), all.end(), [](const DevGate<double> &g) { return g.op == OP_DIAGX; });
+        if (single && !exact && (plan->fp64 || !outside)) return false;  // diagonals from outside are merged, the others are not
+        if (!single) {
             double fp64 = 0;
             for (const DevGate<double> &g : all) fp64 += fp64_clocks(g);
             if (plan->fp64 || !(fp64 > kFixedClocks * nseg)) return false;
         }
-        const bool outside = std::any_of(all.begin(), all.end(), [](const DevGate<double> &g) { return g.op == OP_DIAGX; });
-        if (!exact && plan->n - width < 31 && (1 << (plan->n - width)) <= num_sms()) {
+        if (!single && plan->n - width < 31 && (1 << (plan->n - width)) <= num_sms()) {
             // With at most a chunk per SM a sweep in vain is felt: 15 us beside 45 to 60 in FP64.  Real circuits leave
             // states too uneven for one exponent (a 14-qubit RY/CZ ansatz: every chunk of every section), and the
             // integer pipe alone wins a third at most.
@@ -442,7 +448,7 @@ struct ProgramBuilder {
         const std::vector<DevGate<double>> &dgates = outside ? moved : all;
         std::vector<unsigned char> area, merged;
         if (!encode_fx(dgates, starts, false, area)) return false;
-        const int per = exact || outside ? 0 : oz_max_segs(width);
+        const int per = single || outside ? 0 : oz_max_segs(width);
         auto bounds = [&](int w, int sweeps) { return (int)((int64_t)nseg * w / sweeps); };
         int sweeps = per > 0 ? (nseg + per - 1) / per : 1;
         // more of them where an FP64 program would not fit beside a chunk
@@ -454,7 +460,7 @@ struct ProgramBuilder {
             }
             return true;
         };
-        while (!exact && !fits())
+        while (!single && !fits())
             if (++sweeps > nseg) return false;
         for (int w = 0; w < sweeps; ++w) {
             const int s0 = bounds(w, sweeps), s1 = bounds(w + 1, sweeps);
@@ -493,7 +499,8 @@ struct ProgramBuilder {
                 pg.off = put_program(dsegs, s0, s1, true, area.data(), area.size());
                 pg.gate_bytes = (int)area.size();
             }
-            pg.redo = !exact;
+            if (single && !exact) pg.dense = Dense{-1, 0, 0, 0};
+            pg.redo = !single;
             if (pg.redo) {
                 pg.dense = dense_rule(dsegs, dgates, s0, s1, width);
                 pg.redo_bytes = (int)(mine.size() * sizeof(mine[0]));
@@ -504,14 +511,13 @@ struct ProgramBuilder {
         return true;
     }
 
-    // whole: all gates of the plan's section, whose register groups the plan keeps
-    void section(SimtPrograms::Prog pg, const std::vector<BlockGate> &section_gates, int width, bool whole) {
-        Groups kept = whole ? plan_groups(*plan, pg.op_index, seg_bits, kElem) : nullptr;
-        if (!kept) {
-            std::vector<HostSeg> found = segment_block(section_gates, width, seg_bits, kElem);
-            kept = whole ? keep_groups(*plan, pg.op_index, seg_bits, kElem, std::move(found))
-                         : std::make_shared<const std::vector<HostSeg>>(std::move(found));
-        }
+    // Register groups of a section, or of the part of it that `which` says: kept with the plan.
+    Groups groups(int op_index, const std::vector<BlockGate> &section_gates, int width, int which) {
+        if (Groups kept = plan_groups(*plan, op_index, seg_bits, kElem, which)) return kept;
+        return keep_groups(*plan, op_index, seg_bits, kElem, segment_block(section_gates, width, seg_bits, kElem), which);
+    }
+
+    void section(SimtPrograms::Prog pg, const std::vector<BlockGate> &section_gates, int width, const Groups &kept) {
         const std::vector<HostSeg> &segs = *kept;
         std::vector<DevSeg> dsegs;
         std::vector<DevGate<T>> dgates;
@@ -563,21 +569,18 @@ struct ProgramBuilder {
             } else {
                 local = localize_gates(op0, plan->n, plan->c, nullptr);
             }
-            // diagonals from outside the chunk keep a section off the tensor cores.  Where all of them
+            // Diagonals from outside the chunk keep a section off the tensor cores.  Where all of them
             // commute to its end (no later gate but diagonal ones on their chunk bits) they get a sweep of
-            // their own, one merged diagonal per 4 bits, and the rest runs there: a group costs 2.3 clocks
-            // per amplitude and SM instead of 8.6 (n = 28 QFT: 160 ms in one sweep per section, 100 so)
+            // their own, one merged diagonal per 4 bits, and the rest runs there.  25 qubits, 12-bit chunks, dense
+            // state: 8 layers and 12 phases a qubit 16.1 ms in one sweep and 4.0 so, one layer and one phase 5.0 and
+            // 4.1, QFT 84 and 22.5
             std::vector<BlockGate> main, tail;
             if (sizeof(T) == 8 && !plan->fp64 && oz_max_segs(width) > 0 && split_outside(local, gates, main, tail)) {
-                const size_t nm = segment_block(main, width, seg_bits, kElem).size();
-                const size_t nt = segment_block(tail, width, seg_bits, kElem).size();
-                if (2 * nm > nt + 1) {
-                    section(pg, main, width, false);
-                    section(pg, tail, width, false);
-                    continue;
-                }
+                section(pg, main, width, groups(pg.op_index, main, width, INSIDE_GATES));
+                section(pg, tail, width, groups(pg.op_index, tail, width, OUTSIDE_GATES));
+                continue;
             }
-            section(pg, local, width, true);
+            section(pg, local, width, groups(pg.op_index, local, width, ALL_GATES));
         }
         align(256);
     }
@@ -613,9 +616,9 @@ int launch_section(int dtype, void *state, int n, int c, const unsigned char *ba
     };
     SweepArgs pass, rest;
     pass.operands = operands + p.b_off;
+    pass.dense = p.dense;
     if (p.redo) {
         pass.to = list;
-        pass.dense = p.dense;
         rest.from = list;
     }
     if (p.oz) launch_block_oz(state, n, c, p.gathered ? &p.lay : nullptr, base + p.off, p.nseg, dev_err, st, wait_ns, pass);

@@ -287,8 +287,10 @@ __device__ __forceinline__ void fx_product(fx::Real &ar, fx::Real &ai, const fx:
 // is cut into a part per half warp: lane x of a half multiplies entry x over every eighth gate,
 // the halves join by shuffle, and a half warp multiplies the warps' parts.  (One half warp alone took
 // a chain of up to 64 products per group, longer than the group's own work.)
+// as_double: the tables' entries are doubles, for a group of diagonals alone.
 template <int NC>
-__device__ __forceinline__ void fx_merge(uint32_t gates, int g0, int g1, int64_t origin, int cg, int ctid, int bar_id) {
+__device__ __forceinline__ void fx_merge(uint32_t gates, int g0, int g1, int64_t origin, int cg, int ctid, int bar_id,
+                                         bool as_double) {
     constexpr int W = NC / 32;
     const int lane = ctid & 31, warp = ctid >> 5, x = lane & 15;
     auto store = [](uint32_t a, const fx::Real &r, const fx::Real &i) {
@@ -334,10 +336,12 @@ __device__ __forceinline__ void fx_merge(uint32_t gates, int g0, int g1, int64_t
                                  : "r"(parts + 256u * (uint32_t)w + 16u * (uint32_t)x));
                     fx_product(pr, pi, qr, qi);
                 }
-                fx::Real er = fx::pack(fx::value(pr) * 4), ei = fx::pack(fx::value(pi) * 4);
+                const long long vr = fx::value(pr), vi = fx::value(pi);
+                fx::Real er = fx::pack(vr * 4), ei = fx::pack(vi * 4);
                 er.l += er.l == (int)0x80000000;
                 ei.l += ei.l == (int)0x80000000;
-                if (lane < 16) store(table + 16u * (uint32_t)x, er, ei);
+                if (lane < 16 && as_double) SM<double>::st(table + 16u * (uint32_t)x, (double)vr * 0x1p-59, (double)vi * 0x1p-59);
+                else if (lane < 16) store(table + 16u * (uint32_t)x, er, ei);
             }
         }
         ptx::named_bar_sync(bar_id, NC);
@@ -396,6 +400,7 @@ __device__ __forceinline__ int chunk_range(uint32_t buf, int c, int ctid, int ba
     top = sh->top;
     zeros = sh->zeros;
     if (zeros == 1 << c) return CHUNK_ZERO;
+    if (d.orders < 0) return CHUNK_DENSE;
     if (top < kMinTop || top >= kMaxTop) return CHUNK_OTHER;
     const int line = top - (d.orders << 20), near = top - (kNearOrders << 20);
     int below = 0;  // in two halves: of `line`, of `near`
@@ -446,6 +451,30 @@ __device__ __forceinline__ bool chunk_filled(uint32_t buf, int c, int ctid, int 
     return sh->least_out >= top - (kNearOrders << 20) && sh->filled == 1 << __popc(free_bits) && (dense_bits & ~free_bits) == 0;
 }
 
+// A group of diagonals in FP64: they mix nothing, so every amplitude keeps an exponent of its own, and a merged
+// run is one product of 4 FP64 operations an amplitude, fewer than the conversions to fixed point and back.
+__device__ __forceinline__ void fx_diagonals(double (&re)[16], double (&im)[16], uint32_t gates, int g0, int g1, int64_t origin, int cg) {
+    auto entry = [](uint32_t a) { return ((double)lds_s32(a) * 4294967296.0 + (double)lds_s32(a + 4)) * 0x1p-61; };
+    for (int gi = g0; gi < g1; ++gi) {
+        const FxGate g = fx_gate(gates, gi, origin, cg);
+        gi += g.more;
+        const int a = g.op == OP_DIAG2 ? g.code >> 3 : g.code, b = g.code & 7;
+#pragma unroll
+        for (int x = 0; x < 16; ++x) {
+            double tr, ti;
+            if (g.op == OP_DIAGRUN) {
+                SM<double>::ld(g.m + 16u * (uint32_t)x, tr, ti);
+            } else {
+                const uint32_t e = g.m + 16u * (uint32_t)(((x >> a) & 1) | (g.op == OP_DIAG2 ? ((x >> b) & 1) << 1 : 0));
+                tr = entry(e);
+                ti = entry(e + 8);
+            }
+            if (tr == 1.0 && ti == 0.0) continue;
+            scale_amp(re[x], im[x], tr, ti);
+        }
+    }
+}
+
 // One register group of 4 bits over the chunk in shared memory (see run_segment for the addressing).
 template <int NC>
 __device__ __forceinline__ void run_segment_fx(uint32_t buf, uint32_t seg, uint32_t gates, int ctid, const int *swz,
@@ -470,7 +499,8 @@ __device__ __forceinline__ void run_segment_fx(uint32_t buf, uint32_t seg, uint3
     const int G = 1 << (c - R);
     bool merged = false;  // uniform: whether the group has merged runs
     for (int gi = g0; gi < g1; ++gi) merged = merged || lds_s32(gates + 16u * (uint32_t)gi) == OP_DIAGRUN;
-    if (merged) fx_merge<NC>(gates, g0, g1, origin, cg, ctid, bar_id);
+    const bool diagonal = (flags & kSegDiag) != 0;
+    if (merged) fx_merge<NC>(gates, g0, g1, origin, cg, ctid, bar_id, diagonal);
     uint32_t ld_step[R], st_step[R];
 #pragma unroll
     for (int j = 0; j < R; ++j) {
@@ -500,23 +530,27 @@ __device__ __forceinline__ void run_segment_fx(uint32_t buf, uint32_t seg, uint3
             fx::scan(dr[b], top, any);
             fx::scan(di[b], top, any);
         }
-        const bool raw = (flags & kSegRaw) != 0;
-        const int E = fx::exponent(top);
-        FxGroup<NA> v;
+        if (diagonal) {
+            fx_diagonals(dr, di, gates, g0, g1, origin, cg);
+        } else {
+            const bool raw = (flags & kSegRaw) != 0;
+            const int E = fx::exponent(top);
+            FxGroup<NA> v;
 #pragma unroll
-        for (int b = 0; b < NA; ++b) {
-            v.re[b] = raw ? fx::from_bits(dr[b]) : fx::from_double(dr[b], E);
-            v.im[b] = raw ? fx::from_bits(di[b]) : fx::from_double(di[b], E);
-        }
-        for (int gi = g0; gi < g1; ++gi) {
-            const FxGate g = fx_gate(gates, gi, origin, cg);
-            fx_apply(g.op, g.code, g.m, v, raw);
-            gi += g.more;
-        }
+            for (int b = 0; b < NA; ++b) {
+                v.re[b] = raw ? fx::from_bits(dr[b]) : fx::from_double(dr[b], E);
+                v.im[b] = raw ? fx::from_bits(di[b]) : fx::from_double(di[b], E);
+            }
+            for (int gi = g0; gi < g1; ++gi) {
+                const FxGate g = fx_gate(gates, gi, origin, cg);
+                fx_apply(g.op, g.code, g.m, v, raw);
+                gi += g.more;
+            }
 #pragma unroll
-        for (int b = 0; b < NA; ++b) {
-            dr[b] = raw ? fx::to_bits(v.re[b]) : fx::to_double(v.re[b], E);
-            di[b] = raw ? fx::to_bits(v.im[b]) : fx::to_double(v.im[b], E);
+            for (int b = 0; b < NA; ++b) {
+                dr[b] = raw ? fx::to_bits(v.re[b]) : fx::to_double(v.re[b], E);
+                di[b] = raw ? fx::to_bits(v.im[b]) : fx::to_double(v.im[b], E);
+            }
         }
         off = st0;
 #pragma unroll

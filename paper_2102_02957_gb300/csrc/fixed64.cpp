@@ -50,6 +50,8 @@ bool exact_gate(const DevGate<double> &g) {
     return true;
 }
 
+bool diagonal_gate(const DevGate<double> &g) { return g.op == OP_DIAG1 || g.op == OP_DIAG2 || g.op == OP_DIAGX; }
+
 double fp64_clocks(const DevGate<double> &g) {
     int entries = 0;
     switch (g.op) {

@@ -346,7 +346,7 @@ __device__ __forceinline__ void block_body(typename V2<T>::type *__restrict__ st
             ptx::fence_proxy_async_smem();
             if (ptx::named_bar_or(bar_id, NC, failed)) failed = true;
         } else if constexpr (ENG == ENG_FX) {
-            if (sa.to) kind = chunk_range<NC>(ptx::smem_addr(buf), c, ctid, bar_id, &range[cg], sa.dense, top);
+            if (sa.to || sa.dense.orders < 0) kind = chunk_range<NC>(ptx::smem_addr(buf), c, ctid, bar_id, &range[cg], sa.dense, top);
         }
         for (int si = 0; ENG != ENG_OZ && kind < CHUNK_ZERO && si < nseg; ++si) {
             const uint32_t seg_addr = ptx::smem_addr(segs) + (uint32_t)(si * sizeof(DevSeg));
@@ -378,7 +378,7 @@ __device__ __forceinline__ void block_body(typename V2<T>::type *__restrict__ st
         if constexpr (ENG == ENG_FX) {
             if (kind == CHUNK_TRIAL)
                 kind = chunk_filled<NC>(ptx::smem_addr(buf), c, ctid, bar_id, &range[cg], top, sa.dense.bits) ? CHUNK_DENSE : CHUNK_OTHER;
-            if (sa.to) ptx::named_bar_sync(bar_id, NC);  // all have read the range before it is cleared
+            if (sa.to || sa.dense.orders < 0) ptx::named_bar_sync(bar_id, NC);  // all have read the range before it is cleared
         }
         if constexpr (ENG != ENG_NONE) {
             if (ctid == 0) {

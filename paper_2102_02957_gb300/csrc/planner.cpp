@@ -888,16 +888,16 @@ void encode_gate(const sv_gate &g, const BlockGate &bg, const HostSeg &seg, DevG
     }
 }
 
-Groups plan_groups(const sv_plan &plan, int op_index, int r, int elem_bytes) {
+Groups plan_groups(const sv_plan &plan, int op_index, int r, int elem_bytes, int gates) {
     std::lock_guard<std::mutex> lk(plan.groups_mu);
-    const auto it = plan.groups.find({op_index, r, elem_bytes});
+    const auto it = plan.groups.find({op_index, r, elem_bytes, gates});
     return it == plan.groups.end() ? nullptr : it->second;
 }
 
-Groups keep_groups(const sv_plan &plan, int op_index, int r, int elem_bytes, std::vector<HostSeg> segs) {
+Groups keep_groups(const sv_plan &plan, int op_index, int r, int elem_bytes, std::vector<HostSeg> segs, int gates) {
     Groups g = std::make_shared<const std::vector<HostSeg>>(std::move(segs));
     std::lock_guard<std::mutex> lk(plan.groups_mu);
-    return plan.groups.emplace(std::array<int, 3>{op_index, r, elem_bytes}, g).first->second;
+    return plan.groups.emplace(std::array<int, 4>{op_index, r, elem_bytes, gates}, g).first->second;
 }
 
 // Register groups over all blocking sections of a plan (statistics; the same groups the section

@@ -67,7 +67,7 @@ struct sv_plan {
     // from its structure alone, like the sections): plan_groups.  A plan may serve several threads.
     // (20-qubit ansatz, 69 groups: a repeated evaluation 1.09 ms with a search each time, 0.90 without.)
     mutable std::mutex groups_mu;
-    mutable std::map<std::array<int, 3>, std::shared_ptr<const std::vector<sv::HostSeg>>> groups;
+    mutable std::map<std::array<int, 4>, std::shared_ptr<const std::vector<sv::HostSeg>>> groups;
 };
 
 namespace sv {
@@ -135,7 +135,8 @@ struct DevSeg {
 };
 static_assert(sizeof(DevSeg) == 36, "DevSeg layout");
 
-constexpr int kSegRaw = 4;  // fixed-point programs: every gate of the group is exact_gate()
+constexpr int kSegRaw = 4;   // fixed-point programs: every gate of the group is exact_gate()
+constexpr int kSegDiag = 8;  // ... or diagonal_gate(): in FP64, amplitude by amplitude
 
 template <typename T>
 struct DevGate {
@@ -162,9 +163,11 @@ std::vector<HostSeg> segment_block(const std::vector<BlockGate> &gates, int widt
                                    bool search = true);
 int plan_segment_count(const sv_plan &plan);
 using Groups = std::shared_ptr<const std::vector<HostSeg>>;
-// The groups kept for a section (null before keep_groups): by plan op, group width and element size.
-Groups plan_groups(const sv_plan &plan, int op_index, int r, int elem_bytes);
-Groups keep_groups(const sv_plan &plan, int op_index, int r, int elem_bytes, std::vector<HostSeg> segs);
+// The groups kept for a section (null before keep_groups): by plan op, group width and element size, and
+// the gates they are of.
+enum : int { ALL_GATES = 0, INSIDE_GATES = 1, OUTSIDE_GATES = 2 };  // without / only the ones with qubits outside the chunk
+Groups plan_groups(const sv_plan &plan, int op_index, int r, int elem_bytes, int gates = ALL_GATES);
+Groups keep_groups(const sv_plan &plan, int op_index, int r, int elem_bytes, std::vector<HostSeg> segs, int gates = ALL_GATES);
 
 template <typename T>
 void encode_gate(const sv_gate &g, const BlockGate &bg, const HostSeg &seg, DevGate<T> &out);
@@ -203,6 +206,8 @@ struct OzCompose {
     int32_t g0, g1;
 };
 void launch_compose_oz(const void *dev_groups, int ngroups, void *dev_prog, void *dev_operands, cudaStream_t st);
+// Whether a gate is diagonal.
+bool diagonal_gate(const DevGate<double> &g);
 // Moves the OP_DIAGX gates of a register group's list as far back as they commute (a diagonal on a
 // register bit passes every gate that is diagonal or acts on other bits, a phase every gate), so
 // that they meet in few runs.
@@ -311,7 +316,7 @@ void launch_init_basis(int dtype, void *state, int n, uint64_t basis, cudaStream
 // below 8 orders where it is complex, 45 where it is real, so that practically none falls out.  Else
 // (phases, small angles) all have to be within kNearOrders.
 struct Dense {
-    int orders, most;
+    int orders, most;  // orders < 0: every chunk but one of zeros
     unsigned bits;  // chunk bits that dense gates act on
     int trial;      // whether gates may fill a chunk within kNearOrders from one amplitude
 };
@@ -357,7 +362,7 @@ void launch_permute(int dtype, void *state, int n, const std::vector<std::pair<i
 constexpr uint64_t kDefaultWaitNs = 4000000000ull;
 // Chunks of a complex128 section that a fixed-point or tensor-core pass leaves to FP64 (block_fx.cuh,
 // ChunkRange): the pass appends their numbers to `to` (device memory), and an FP64 pass with `from` set runs
-// those alone and empties the list.  to null: all gates of the section are exact, every chunk runs.
+// those alone and empties the list.  to null: the section's gates keep the amplitudes apart, every chunk runs.
 struct SweepArgs {
     int *to = nullptr;
     Dense dense;
