@@ -459,7 +459,8 @@ void launch_typed(void *state, int n, int ce, const void *prog, int nseg, int ga
     // so that the scheduler never places two on one SM
     if (TC && smem < 120 * 1024) smem = 120 * 1024;
     auto grid_of = [&](auto kern) -> unsigned {
-        check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
+        // the limit, not this launch's size: another thread may be about to launch the kernel with a larger one
+        check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxBlockSmem),
                    "cudaFuncSetAttribute(block)");
         int per_sm = 0;
         check_cuda(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, G * NC + svc_threads(ENG), smem),
