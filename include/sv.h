@@ -391,7 +391,7 @@ sv_status sv_expval_pauli(sv_handle h, uint64_t x_mask, uint64_t z_mask, double 
  * the call (a memory budget or pool they do not own, or loops where a cudaMalloc/cudaFree would
  * stall the device).  The paper has no counterpart; this is a service of this library.
  * It calls no cudaMalloc, cudaFree or other allocating routine: its partial sums go to a fixed
- * 64 KiB array compiled into the library (4096 (re, im) pairs plus the result), which every GPU
+ * 64 KiB array compiled into the library (two doubles for each of 4096 CTAs plus the result), which every GPU
  * that loads the library holds until the process exits.  The first call on a device looks up
  * that array's device address (cudaGetSymbolAddress) with the device current, so make that
  * first call before any stream capture.  The handle's device must be the current device

@@ -116,7 +116,7 @@ static Readout *readout_words(sv_state *h) {
 }
 
 // Wait for the readout whose last kernel wrote readout_words(h).
-static double finish_readout(sv_state *h, double *weight = nullptr) {
+static Readout finish_readout(sv_state *h) {
     Readout r;
     if (h->slot) {
         check_cuda(cudaStreamSynchronize(h->stream), "cudaStreamSynchronize");
@@ -126,8 +126,7 @@ static double finish_readout(sv_state *h, double *weight = nullptr) {
         check_cuda(cudaStreamSynchronize(h->stream), "cudaStreamSynchronize");
     }
     raise_dev_error(h, r.err);
-    if (weight) *weight = r.weight;
-    return r.value;
+    return r;
 }
 
 static void validate_gates(int n, const sv_gate *gates, int64_t n_gates) {
@@ -1143,8 +1142,8 @@ sv_status sv_norm2(sv_handle h, double *out) {
     const int nb = reduce_blocks(h->n);
     ensure_scratch(h, (size_t)nb * sizeof(double));
     launch_partial_norm(h->dtype, h->amp, h->n, h->scratch, nb, h->stream);
-    launch_finish(h->scratch, nb, h->dev_err, readout_words(h), h->stream);
-    *out = finish_readout(h);
+    launch_finish(h->scratch, nb, false, h->dev_err, readout_words(h), h->stream);
+    *out = finish_readout(h).value;
     SV_API_END
 }
 
@@ -1155,15 +1154,12 @@ sv_status sv_expval_pauli(sv_handle h, uint64_t x, uint64_t z, double *out) {
     const int nb = reduce_blocks(h->n);
     ensure_scratch(h, (size_t)nb * 2 * sizeof(double));
     launch_partial_expval(h->dtype, h->amp, h->n, x, z, h->scratch, nb, h->stream);
-    launch_finish(h->scratch, nb, h->dev_err, readout_words(h), h->stream);
+    launch_finish(h->scratch, nb, true, h->dev_err, readout_words(h), h->stream);
+    const Readout r = finish_readout(h);
     // the sum is real where x and z overlap in an even number of qubits, imaginary otherwise
-    double weight = 0;
-    const double v = finish_readout(h, &weight);
     const bool odd = __builtin_popcountll(x & z) & 1;
-    double sr = odd ? 0.0 : v, si = odd ? v : 0.0;
-    // a sum that cancels to nothing (a real state under a word with an odd number of Y's): callers get the
-    // residue of the term-by-term sum
-    if (!(std::fabs(v) > 0x1p-40 * weight)) {
+    double sr = odd ? 0.0 : r.value, si = odd ? r.value : 0.0;
+    if (expval_cancels(r)) {
         launch_partial_expval_direct(h->dtype, h->amp, h->n, x, z, h->scratch, nb, h->stream);
         std::vector<double> part((size_t)nb * 2);
         check_cuda(cudaMemcpyAsync(part.data(), h->scratch, nb * 2 * sizeof(double), cudaMemcpyDeviceToHost, h->stream),
@@ -1175,15 +1171,7 @@ sv_status sv_expval_pauli(sv_handle h, uint64_t x, uint64_t z, double *out) {
             si += part[(size_t)(2 * b + 1)];
         }
     }
-    // multiply by i^{popc(x & z)}
-    switch (__builtin_popcountll(x & z) & 3) {
-        case 1: { double t = sr; sr = -si; si = t; break; }
-        case 2: sr = -sr; si = -si; break;
-        case 3: { double t = sr; sr = si; si = -t; break; }
-        default: break;
-    }
-    out[0] = sr;
-    out[1] = si;
+    pauli_phase(x, z, sr, si, out);
     SV_API_END
 }
 
@@ -1200,7 +1188,7 @@ sv_status sv_sample(sv_handle h, int64_t shots, uint64_t seed, uint64_t *out) {
     double *sums = h->scratch, *totals = sums + nb;
     uint64_t *d_out = reinterpret_cast<uint64_t *>(totals + nt);
     launch_sample(h->dtype, h->amp, h->n, sb, sums, totals, seed, shots, d_out, h->dev_err, readout_words(h), h->stream);
-    const double total = finish_readout(h);
+    const double total = finish_readout(h).value;
     if (!(total > 0)) fail(SV_ERR_ARG, "state has zero norm");
     check_cuda(cudaMemcpyAsync(out, d_out, shots * sizeof(uint64_t), cudaMemcpyDeviceToHost, h->stream), "D2H");
     check_cuda(cudaStreamSynchronize(h->stream), "cudaStreamSynchronize");

@@ -20,12 +20,11 @@
 namespace sv {
 namespace {
 
-constexpr int kThreads = 256;
 constexpr int kMaxPartials = 4096;  // up to 4096 CTAs of partial sums (64 KiB of scratch)
 constexpr int kMaxDevices = 64;
 
-// (re, im) partial sums of up to kMaxPartials CTAs, then the final (re, im) pair.
-static __device__ __align__(256) double g_expval_scratch[2 * kMaxPartials + 2];
+// Two doubles for each of up to kMaxPartials CTAs, then the final (re, im) pair and the paired sum's words.
+static __device__ __align__(256) double g_expval_scratch[2 * kMaxPartials + 2 + (sizeof(Readout) + 7) / 8];
 
 std::mutex g_mu;
 std::array<double *, kMaxDevices> g_addr{};
@@ -40,49 +39,6 @@ double *scratch_address(int dev) {
         g_addr[dev] = p;
     }
     return g_addr[dev];
-}
-
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
-// CTA b sums conj(a_{j^x}) a_j (-1)^{popc(j&z)} over its contiguous range of j and writes
-// (re, im) to scratch[2b], scratch[2b+1]; every CTA overwrites its own slots, so nothing has
-// to start at zero.
-template <typename T2>
-__global__ void __launch_bounds__(kThreads) k_expval_partials_noalloc(const T2 *__restrict__ a, int64_t len,
-                                                                      uint64_t x, uint64_t z, double *scratch) {
-    __shared__ double red[2][kThreads / 32];
-    const int64_t per = (len + gridDim.x - 1) / gridDim.x;
-    const int64_t lo = (int64_t)blockIdx.x * per, hi = lo + per < len ? lo + per : len;
-    double sr = 0, si = 0;
-    for (int64_t j = lo + threadIdx.x; j < hi; j += kThreads) {
-        const T2 u = a[(uint64_t)j ^ x], v = a[j];
-        double tr = (double)u.x * (double)v.x + (double)u.y * (double)v.y;
-        double ti = (double)u.x * (double)v.y - (double)u.y * (double)v.x;
-        if (__popcll((unsigned long long)j & z) & 1) { tr = -tr; ti = -ti; }
-        sr += tr;
-        si += ti;
-    }
-    sr = warp_sum(sr);
-    si = warp_sum(si);
-    if ((threadIdx.x & 31) == 0) {
-        red[0][threadIdx.x >> 5] = sr;
-        red[1][threadIdx.x >> 5] = si;
-    }
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        double r = threadIdx.x < kThreads / 32 ? red[0][threadIdx.x] : 0.0;
-        double i = threadIdx.x < kThreads / 32 ? red[1][threadIdx.x] : 0.0;
-        r = warp_sum(r);
-        i = warp_sum(i);
-        if (threadIdx.x == 0) {
-            scratch[2 * blockIdx.x] = r;
-            scratch[2 * blockIdx.x + 1] = i;
-        }
-    }
 }
 
 // One thread adds the partials in CTA order into the final pair.
@@ -114,29 +70,24 @@ extern "C" sv_status sv_expval_pauli_noalloc(sv_handle h, uint64_t x, uint64_t z
             fail(SV_ERR_UNSUPPORTED, "sv_expval_pauli_noalloc: needs " + std::to_string(nb) +
                                          " partial sums, more than the fixed scratch holds (4096)");
         double *scratch = scratch_address(dev);
-        if (h->dtype == SV_C64)
-            k_expval_partials_noalloc<float2><<<(unsigned)nb, kThreads, 0, h->stream>>>((const float2 *)h->amp, len, x,
-                                                                                        z, scratch);
-        else
-            k_expval_partials_noalloc<double2><<<(unsigned)nb, kThreads, 0, h->stream>>>((const double2 *)h->amp, len,
-                                                                                         x, z, scratch);
-        check_cuda(cudaGetLastError(), "expval (no-alloc) kernel launch");
-        k_expval_final_noalloc<<<1, 1, 0, h->stream>>>(scratch, (int)nb);
-        check_cuda(cudaGetLastError(), "expval (no-alloc) final kernel launch");
-        double res[2] = {0, 0};
-        check_cuda(cudaMemcpyAsync(res, scratch + 2 * kMaxPartials, sizeof(res), cudaMemcpyDeviceToHost, h->stream),
-                   "cudaMemcpyAsync(expval result)");
+        // the same kernels and the same order of summation as sv_expval_pauli's
+        Readout *words = reinterpret_cast<Readout *>(scratch + 2 * kMaxPartials + 2), r;
+        launch_partial_expval(h->dtype, h->amp, h->n, x, z, scratch, (int)nb, h->stream);
+        launch_finish(scratch, (int)nb, true, h->dev_err, words, h->stream);
+        check_cuda(cudaMemcpyAsync(&r, words, sizeof(r), cudaMemcpyDeviceToHost, h->stream), "cudaMemcpyAsync(expval result)");
         // synchronise and report a failure an earlier kernel on this handle left in its error word
         check_dev_error(h);
-        double sr = res[0], si = res[1];
-        switch (__builtin_popcountll(x & z) & 3) {  // times i^{popc(x & z)}
-            case 1: { const double t = sr; sr = -si; si = t; break; }
-            case 2: sr = -sr; si = -si; break;
-            case 3: { const double t = sr; sr = si; si = -t; break; }
-            default: break;
+        const bool odd = __builtin_popcountll(x & z) & 1;
+        double res[2] = {odd ? 0.0 : r.value, odd ? r.value : 0.0};
+        if (expval_cancels(r)) {
+            launch_partial_expval_direct(h->dtype, h->amp, h->n, x, z, scratch, (int)nb, h->stream);
+            k_expval_final_noalloc<<<1, 1, 0, h->stream>>>(scratch, (int)nb);
+            check_cuda(cudaGetLastError(), "expval (no-alloc) final kernel launch");
+            check_cuda(cudaMemcpyAsync(res, scratch + 2 * kMaxPartials, sizeof(res), cudaMemcpyDeviceToHost, h->stream),
+                       "cudaMemcpyAsync(expval result)");
+            check_dev_error(h);
         }
-        out[0] = sr;
-        out[1] = si;
+        pauli_phase(x, z, res[0], res[1], out);
         return SV_OK;
     } catch (const sv::Error &e) {
         sv::set_error(e.msg);

@@ -203,6 +203,13 @@ __device__ __forceinline__ void add_term(double &s, T ux, T uy, T vx, T vy, unsi
     }
 }
 
+// |x| in FP32, for the sum of the terms' magnitudes (a double's to 12 %, out of FP32's range as 0 or huge).
+__device__ __forceinline__ float magnitude(float x) { return fabsf(x); }
+__device__ __forceinline__ float magnitude(double x) {
+    return __int_as_float(min(max((__double2hiint(x) & 0x7FFFFFFF) - (896 << 20), 0), 254 << 20) << 3);
+}
+
+// Per CTA its sum, and at partials[gridDim.x ..] the magnitudes of its products.
 template <typename T2, int MODE>
 __global__ void __launch_bounds__(kThreads) k_partial_expval(const T2 *__restrict__ a, int64_t terms, uint64_t x,
                                                              uint64_t zt, int hb, double *partials) {
@@ -212,6 +219,7 @@ __global__ void __launch_bounds__(kThreads) k_partial_expval(const T2 *__restric
     for (int k = 0; k < kSteps; ++k)
         step_sign[k] = (unsigned)((__popcll(((uint64_t)k * kThreads + threadIdx.x) & zt) & 1) << 31);
     double s = 0;
+    float w = 0;
     for (int64_t t0 = (int64_t)blockIdx.x * kTile; t0 < terms; t0 += (int64_t)gridDim.x * kTile) {
         const unsigned tile_sign = (unsigned)((__popcll((uint64_t)t0 & zt) & 1) << 31);
         T2 u[kSteps], v[kSteps];
@@ -241,9 +249,18 @@ __global__ void __launch_bounds__(kThreads) k_partial_expval(const T2 *__restric
             for (int k = 0; k < kSteps; ++k)
                 add_term<MODE, true>(s, u[k].x, u[k].y, v[k].x, v[k].y, tile_sign ^ step_sign[k]);
         }
+#pragma unroll
+        for (int k = 0; k < kSteps; ++k) {
+            w = fmaf(magnitude(u[k].x), magnitude(MODE == ODD ? v[k].y : v[k].x), w);
+            w = fmaf(magnitude(u[k].y), magnitude(MODE == ODD ? v[k].x : v[k].y), w);
+        }
     }
     s = block_sum<kThreads>(s);
-    if (threadIdx.x == 0) partials[blockIdx.x] = MODE == NORM ? s : 2 * s;
+    const double total = block_sum<kThreads>((double)w);
+    if (threadIdx.x == 0) {
+        partials[blockIdx.x] = MODE == NORM ? s : 2 * s;
+        partials[gridDim.x + blockIdx.x] = MODE == NORM ? total : 2 * total;
+    }
 }
 
 // The sum term by term: for words whose paired sum vanishes, where the result is the rounding residue
@@ -271,14 +288,14 @@ __global__ void __launch_bounds__(kThreads) k_partial_expval_direct(const T2 *__
     }
 }
 
-// Sum of the partials, of their magnitudes, and the handle's error word, into the caller's result
-// words (host memory the GPU writes directly, or device memory).
-__global__ void __launch_bounds__(kThreads) k_finish(const double *__restrict__ partials, int nb,
+// Sum of the partials, of the weights behind them if there are any, and the handle's error word, into the
+// caller's result words (host memory the GPU writes directly, or device memory).
+__global__ void __launch_bounds__(kThreads) k_finish(const double *__restrict__ partials, int nb, bool weights,
                                                      const int *__restrict__ err, Readout *out) {
     double s = 0, w = 0;
     for (int b = threadIdx.x; b < nb; b += kThreads) {
         s += partials[b];
-        w += fabs(partials[b]);
+        if (weights) w += partials[nb + b];
     }
     s = block_sum<kThreads>(s);
     w = block_sum<kThreads>(w);
@@ -521,6 +538,15 @@ void launch_partial_expval(int dtype, const void *state, int n, uint64_t x, uint
     check_cuda(cudaGetLastError(), "expval kernel launch");
 }
 
+void pauli_phase(uint64_t x, uint64_t z, double sr, double si, double *out) {
+    switch (__builtin_popcountll(x & z) & 3) {
+        case 1: out[0] = -si; out[1] = sr; break;
+        case 2: out[0] = -sr; out[1] = -si; break;
+        case 3: out[0] = si; out[1] = -sr; break;
+        default: out[0] = sr; out[1] = si; break;
+    }
+}
+
 void launch_partial_expval_direct(int dtype, const void *state, int n, uint64_t x, uint64_t z, double *partials,
                                   int nblocks, cudaStream_t st) {
     const int64_t len = int64_t(1) << n;
@@ -531,8 +557,8 @@ void launch_partial_expval_direct(int dtype, const void *state, int n, uint64_t 
     check_cuda(cudaGetLastError(), "expval kernel launch");
 }
 
-void launch_finish(const double *partials, int nblocks, const int *err, Readout *out, cudaStream_t st) {
-    k_finish<<<1, kThreads, 0, st>>>(partials, nblocks, err, out);
+void launch_finish(const double *partials, int nblocks, bool weights, const int *err, Readout *out, cudaStream_t st) {
+    k_finish<<<1, kThreads, 0, st>>>(partials, nblocks, weights, err, out);
     check_cuda(cudaGetLastError(), "readout kernel launch");
 }
 

@@ -6,6 +6,7 @@
 
 #include <algorithm>
 #include <array>
+#include <cmath>
 #include <map>
 #include <memory>
 #include <mutex>
@@ -401,18 +402,24 @@ void launch_partial_norm(int dtype, const void *state, int n, double *partials, 
 // partial sums, then n_out's; d: one float of device scratch.
 void launch_renorm(int dtype, void *state, int n, const double *partials, int nblocks, const int *flag, float *d,
                    cudaStream_t st);
+// nblocks partial sums of a Pauli word's paired terms, then as many of the magnitudes of their products.
 void launch_partial_expval(int dtype, const void *state, int n, uint64_t x, uint64_t z,
                            double *partials, int nblocks, cudaStream_t st);
 // (re, im) partial sums of the word's terms in index order, nblocks pairs.
 void launch_partial_expval_direct(int dtype, const void *state, int n, uint64_t x, uint64_t z, double *partials,
                                   int nblocks, cudaStream_t st);
-// Result words of a readout: a value, the sum of its partials' magnitudes, the handle's error word.
+// Result words of a readout: a value, the magnitude of what was summed to it, the handle's error word.
 struct Readout {
     double value, weight;
     int err;
 };
-// out->value = sum of the partials.
-void launch_finish(const double *partials, int nblocks, const int *err, Readout *out, cudaStream_t st);
+// out->value = sum of the partials, out->weight (weights) that of the nblocks behind them.
+void launch_finish(const double *partials, int nblocks, bool weights, const int *err, Readout *out, cudaStream_t st);
+// Whether a Pauli word's sum cancels to nothing beside its products (a real state under a word with an odd number of
+// Y's): callers then get the residue of the term-by-term sum, as they always have.
+inline bool expval_cancels(const Readout &r) { return !(std::fabs(r.value) > 0x1p-40 * r.weight); }
+// (sr + i si) i^{popcount(x & z)}
+void pauli_phase(uint64_t x, uint64_t z, double sr, double si, double *out);
 // Inverse-CDF sampling over ranges of 2^sb amplitudes: sums holds 2^(n-sb) doubles, totals
 // sample_totals(n, sb); total->value receives the squared norm.
 int64_t sample_totals(int n, int sb);
