@@ -274,7 +274,7 @@ def _traffic_for(kernel_src: str, workload: str):
     return e.get("dram_bytes_per_launch")
 
 
-def _per_gate(sv, st, desc, stream, args, sweep_bytes):
+def _per_gate(sv, st, desc, stream, args):
     import torch
     G = len(desc)
     gates = sv.make_gates(desc)
@@ -294,8 +294,8 @@ def _per_gate(sv, st, desc, stream, args, sweep_bytes):
     pg_ms = e0.elapsed_time(e1) / pg_steps
     s = st.stats()
     per_gate = {"gates_per_s": G / (pg_ms / 1000.0), "ms_per_step": pg_ms,
-                "effective_GBs": G * sweep_bytes / (pg_ms / 1000.0) / 1e9,
-                "kernel_GBs": G * sweep_bytes / (s.ms_gate / 1000.0) / 1e9 if s.ms_gate else None}
+                "effective_GBs": s.algorithmic_bytes / (pg_ms / 1000.0) / 1e9,
+                "kernel_GBs": s.algorithmic_bytes / (s.ms_gate / 1000.0) / 1e9 if s.ms_gate else None}
     return per_gate, pg_ms
 
 
@@ -587,7 +587,7 @@ def run_ours(args):
         ms_perm += s.ms_permute
         n_block += s.sweeps_block
         n_perm += s.sweeps_permute
-        launches += s.kernel_launches + 2  # + init (set-one kernel) + norm reduction
+        launches += s.kernel_launches + 3  # + init (set-one kernel) + norm (partial sums, their sum)
     t_end.record(stream)
     torch.cuda.synchronize()
     bar.barrier()
@@ -641,7 +641,7 @@ def run_ours(args):
     per_gate = None
     pg_ms = float("nan")
     if not args.no_per_gate:
-        per_gate, pg_ms = _per_gate(sv, st, desc, stream, args, sweep_bytes)
+        per_gate, pg_ms = _per_gate(sv, st, desc, stream, args)
 
     # end to end through the C ABI with host buffers: every step uploads its input state from
     # pinned host memory, builds its gate records and plan on the host, applies the circuit and

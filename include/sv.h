@@ -246,7 +246,8 @@ typedef struct sv_apply_stats {
     int64_t sweeps_block;       /* blocked-section passes                */
     int64_t sweeps_permute;     /* chunk_swap + reordering passes        */
     int64_t sweeps_gate;        /* per-gate passes                       */
-    double algorithmic_bytes;   /* (passes) x 2 x 2^n x bytes/amplitude  */
+    double algorithmic_bytes;   /* (passes) x 2 x 2^n x bytes/amplitude; per-gate passes count the
+                                   amplitudes that they read and write (an identity none)    */
     double ms_block;            /* device time of the blocked-section kernels (profiling on) */
     double ms_permute;          /* device time of the permutation kernels (profiling on)     */
     double ms_gate;             /* device time of the per-gate kernels (profiling on)        */

@@ -916,9 +916,10 @@ sv_status sv_apply_circuit(sv_handle h, const sv_gate *gates, int64_t n_gates, s
     if (!plan) {
         for (int64_t i = 0; i < n_gates; ++i) {
             mark_begin(h, 0);
-            launch_gate(h->dtype, h->amp, h->n, gates[i], h->stream);
+            const double bytes = launch_gate(h->dtype, h->amp, h->n, gates[i], h->stream);
             mark_end(h);
-            ++st.kernel_launches;
+            st.kernel_launches += bytes > 0;
+            st.algorithmic_bytes += bytes;
             ++st.sweeps_gate;
         }
     } else {
@@ -1006,7 +1007,7 @@ sv_status sv_apply_circuit(sv_handle h, const sv_gate *gates, int64_t n_gates, s
             st.kernel_launches += 3;
         }
     }
-    st.algorithmic_bytes = sweep * (double)(st.sweeps_block + st.sweeps_permute + st.sweeps_gate);
+    st.algorithmic_bytes += sweep * (double)(st.sweeps_block + st.sweeps_permute);
     h->stats = st;
     SV_API_END
 }

@@ -11,6 +11,7 @@
 // A sweep touches only the amplitudes that its gate can change: local basis states whose row and
 // column are those of the identity are left out, so a controlled gate moves half of the state and a
 // controlled phase a quarter, and an exchange (X, CNOT, SWAP) moves amplitudes without arithmetic.
+// (Complex64 gates on qubit 0 sweep the whole state: every unit holds both values of it.)
 // Complex128 products run in block fixed point on the integer pipe (fixed64.cuh) where that is as exact,
 // amplitude by amplitude (apply_fx).  480 gates of
 // random layers on 16 qubits, complex128: 3.94 ms with every gate dense in FP64, 1.97 ms so.
@@ -471,7 +472,8 @@ void launch_c128(void *state, const Touched &t, int n, int nq, const int *q, cud
 
 }  // namespace
 
-void launch_gate(int dtype, void *state, int n, const sv_gate &g, cudaStream_t st) {
+double launch_gate(int dtype, void *state, int n, const sv_gate &g, cudaStream_t st) {
+    const double full = 2.0 * (double)(int64_t(1) << n) * (dtype == SV_C64 ? 8.0 : 16.0);
     if (dtype == SV_C64 && (g.q[0] == 0 || (g.nq == 2 && g.q[1] == 0))) {
         float4 *a = (float4 *)state;
         if (g.nq == 1) {
@@ -490,10 +492,10 @@ void launch_gate(int dtype, void *state, int n, const sv_gate &g, cudaStream_t s
             const int64_t groups = int64_t(1) << (n - 2);
             launch_after(k_gate2_c64_lo, grid_for(groups), kThreads, st, a, groups, other - 1, g.q[0] == 0 ? 1 : 0, M);
         }
-        return;
+        return full;
     }
     const Touched t = touched_states(g);
-    if (t.n == 0) return;  // the identity
+    if (t.n == 0) return 0.0;  // the identity
     // complex64: units of two amplitudes, so unit bit q - 1 for qubit q >= 1
     const int shift = dtype == SV_C64 ? 1 : 0, units_log2 = n - shift;
     const int q[2] = {g.q[0] - shift, g.nq == 2 ? g.q[1] - shift : 0};
@@ -510,6 +512,7 @@ void launch_gate(int dtype, void *state, int n, const sv_gate &g, cudaStream_t s
         else if (t.n == 2) launch_c128<2>(state, t, n, g.nq, q, st);
         else launch_c128<4>(state, t, n, g.nq, q, st);
     }
+    return full * t.n / (1 << g.nq);
 }
 
 void launch_init_basis(int dtype, void *state, int n, uint64_t basis, cudaStream_t st) {

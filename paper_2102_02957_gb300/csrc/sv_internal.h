@@ -306,7 +306,8 @@ void launch_mlp_reduce(const float *part, int nblk, const double *lpart, double 
 struct Mat1 { float m[8]; };
 struct Mat2 { float m[32]; };
 
-void launch_gate(int dtype, void *state, int n, const sv_gate &g, cudaStream_t st);
+// Returns the bytes that the sweep reads and writes (0: the identity, nothing is launched).
+double launch_gate(int dtype, void *state, int n, const sv_gate &g, cudaStream_t st);
 void launch_init_basis(int dtype, void *state, int n, uint64_t basis, cudaStream_t st);
 // When a chunk is dense enough for one exponent: at most `most` of its amplitudes (zeros too) are more than
 // `orders` binary orders below its largest component.  A unit is 2^-54 of that component, and FP64 is as
