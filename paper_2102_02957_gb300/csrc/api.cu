@@ -1031,7 +1031,14 @@ sv_status sv_apply_plan_ops(sv_handle h, const sv_gate *gates, int64_t n_gates, 
     const size_t list_bytes = redo_list_bytes(sp, h->n, plan->c);
     unsigned char *const list = upload_program(h, sp.host, list_bytes + sp.b_bytes), *const operands = list + list_bytes;
     const unsigned char *base = static_cast<const unsigned char *>(h->prog);
-    if (sp.noz) launch_compose_oz(base + sp.oz_off, sp.noz, h->prog, operands, h->stream);
+    // the operands of the ops to run: a contiguous range of the list
+    int oz0 = sp.noz, oz1 = 0;
+    for (const SimtPrograms::Prog &p : sp.progs)
+        if (p.oz && p.op_index >= op_begin && p.op_index < op_end) {
+            oz0 = std::min(oz0, p.oz_first);
+            oz1 = std::max(oz1, p.oz_first + p.nseg);
+        }
+    launch_compose_oz(base + sp.oz_off + (size_t)oz0 * sizeof(OzCompose), oz1 - oz0, h->prog, operands, h->stream);
     const uint64_t wait_ns = plan->wait_limit_ms > 0 ? (uint64_t)plan->wait_limit_ms * 1000000ull : kDefaultWaitNs;
     size_t bi = 0;  // programs are in op order
     for (int32_t oi = op_begin; oi < op_end; ++oi) {
