@@ -373,7 +373,7 @@ static Dense dense_rule(const std::vector<DevSeg> &segs, const std::vector<DevGa
 // on the tensor cores where that is twice as fast as FP64: on the tensor cores if none of their gates has a
 // qubit outside its chunk and the chunk holds a 128-row tile (a group costs about as much there whatever its
 // gates are, less than one dense gate on the integer pipe, block_fx.cuh), in as many sweeps as
-// their groups need.  Each such sweep has an FP64 program too, for the chunks it leaves (Redo).
+// their groups need.  Each such sweep has an FP64 program too, for the chunks it leaves (SweepArgs).
 template <typename T>
 struct ProgramBuilder {
     const sv_plan *plan;

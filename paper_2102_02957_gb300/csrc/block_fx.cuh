@@ -3,7 +3,8 @@
 // Same shape as run_segment: a thread loads the 16 amplitudes spanned by the group's 4 chunk bits,
 // applies every gate of the group, stores them back.  In between the components are block
 // fixed-point integers with one exponent per thread, converted once each way per group -- or, in a
-// group that only exchanges amplitudes and flips signs (kSegRaw), the doubles' own words.
+// group that only exchanges amplitudes and flips signs (kSegRaw), the doubles' own words, and in one of
+// diagonals alone (kSegDiag) doubles.
 //
 // Bound by the multiply-add pipe (57 % busy on random-layer sections, where run_segment kept the
 // FP64 pipe full) and by the dependent chains that two warps per scheduler leave exposed: 168
@@ -355,7 +356,7 @@ __device__ __forceinline__ void fx_merge(uint32_t gates, int g0, int g1, int64_t
 //          fill from a few amplitudes.  Tried where at most one amplitude in 64 is small and not zero, and only
 //          with gates like Hadamards (Dense::trial).
 //   ZERO   chunks stay as they are, and so do OTHER ones (and failed trials), which FP64 register groups run
-//          next (Redo): components that are not finite or near the ends of the exponent range, states with
+//          next (SweepArgs): components that are not finite or near the ends of the exponent range, states with
 //          most of their weight on few amplitudes.
 struct ChunkRange {
     int top, zeros, small, near;  // largest high word, amplitudes that are zero, below Dense's line, and below kNearOrders

@@ -18,7 +18,10 @@
 //    register groups -- SIMT (run_segment: each thread loads the 2^R amplitudes spanned by the
 //    group's R chunk bits into registers, applies every gate of the group there, stores them
 //    back) or tensor cores (run_segment_tc: the group's fused unitary applied to 128-row tiles
-//    with tcgen05 MMAs) -- then hand it to the store warp through a "done" mbarrier;
+//    with tcgen05 MMAs; complex128 in fixed point: run_segment_fx on the integer pipe, or run_chunk_oz, which keeps
+//    a chunk in digits from group to group) -- then hand it to the store warp through a "done" mbarrier.
+//    The fixed-point engines look every chunk over first and leave those of uneven amplitudes, listed, to a second
+//    launch with FP64 register groups (block_fx.cuh, ChunkRange);
 //  * warp 1 is the store warp (store_chunks): it writes the chunks back in order, a box or piece
 //    per lane, and releases each buffer to the producer through an "empty" mbarrier once the
 //    copies have read it.
@@ -153,7 +156,8 @@ __device__ __forceinline__ void write_chunk(T2 *state, int c, int64_t j, const T
 }
 
 // Store warp: write the CTA's chunks back in order as their consumers finish them (done[slot]; a non-zero
-// hold[slot]: the chunk stays as it is in memory) and release each slot to the producer (empty[slot]) as soon as the copies have read it.
+// hold[slot]: the chunk stays as it is in memory) and release each slot to the producer (empty[slot]) as
+// soon as the copies have read it.
 // (Keeping two write-backs in flight, releasing chunk it - 1 after chunk it's copies are issued,
 // was measured slower: the slot is held longer and the prefetch depth shrinks.)
 template <typename T2>
@@ -214,7 +218,8 @@ __device__ __forceinline__ void block_body(typename V2<T>::type *__restrict__ st
                 listed = *(volatile int *)&sa.from[LIST_COUNT];
                 __threadfence();
                 // the last CTA that has read the count empties the list for the next pass
-                if (atomicInc(reinterpret_cast<unsigned *>(sa.from + LIST_READERS), gridDim.x - 1) == gridDim.x - 1) sa.from[LIST_COUNT] = 0;
+                if (atomicInc(reinterpret_cast<unsigned *>(sa.from + LIST_READERS), gridDim.x - 1) == gridDim.x - 1)
+                    sa.from[LIST_COUNT] = 0;
             }
             __syncthreads();
             nchunks = listed;
@@ -255,7 +260,8 @@ __device__ __forceinline__ void block_body(typename V2<T>::type *__restrict__ st
         *reinterpret_cast<uint4 *>(sprog + k) = *reinterpret_cast<const uint4 *>(prog + k);
     if constexpr (ENG == ENG_OZ)
         for (int k = threadIdx.x * 16; k < nseg * kOzBBytes; k += blockDim.x * 16)
-            *reinterpret_cast<uint4 *>(sprog + tab_bytes + k) = *reinterpret_cast<const uint4 *>(static_cast<const unsigned char *>(sa.operands) + k);
+            *reinterpret_cast<uint4 *>(sprog + tab_bytes + k) =
+                *reinterpret_cast<const uint4 *>(static_cast<const unsigned char *>(sa.operands) + k);
     if (threadIdx.x < 24) swz[threadIdx.x] = sizeof(T2) == 8 ? c_swz64[threadIdx.x] : c_swz128[threadIdx.x];
     if (threadIdx.x == 0) {
         s_wait_ns = wait_ns;
@@ -341,8 +347,8 @@ __device__ __forceinline__ void block_body(typename V2<T>::type *__restrict__ st
         bool failed = false;
         [[maybe_unused]] int kind = CHUNK_DENSE, top = 0;  // uniform over the group
         if constexpr (ENG == ENG_OZ) {
-            failed = !run_chunk_oz<NC>(ptx::smem_addr(buf), ptx::smem_addr(sprog), nseg, ctid, c, sa.dense, tmem_base, bar_id, &mma_bar[kBars * cg], mma_phase, abort_flag, &s_wait_ns, &oz[cg],
-                                       kind);
+            failed = !run_chunk_oz<NC>(ptx::smem_addr(buf), ptx::smem_addr(sprog), nseg, ctid, c, sa.dense, tmem_base, bar_id,
+                                       &mma_bar[kBars * cg], mma_phase, abort_flag, &s_wait_ns, &oz[cg], kind);
             ptx::fence_proxy_async_smem();
             if (ptx::named_bar_or(bar_id, NC, failed)) failed = true;
         } else if constexpr (ENG == ENG_FX) {
@@ -377,7 +383,8 @@ __device__ __forceinline__ void block_body(typename V2<T>::type *__restrict__ st
         }
         if constexpr (ENG == ENG_FX) {
             if (kind == CHUNK_TRIAL)
-                kind = chunk_filled<NC>(ptx::smem_addr(buf), c, ctid, bar_id, &range[cg], top, sa.dense.bits) ? CHUNK_DENSE : CHUNK_OTHER;
+                kind = chunk_filled<NC>(ptx::smem_addr(buf), c, ctid, bar_id, &range[cg], top, sa.dense.bits) ? CHUNK_DENSE
+                                                                                                              : CHUNK_OTHER;
             if (sa.to || sa.dense.orders < 0) ptx::named_bar_sync(bar_id, NC);  // all have read the range before it is cleared
         }
         if constexpr (ENG != ENG_NONE) {
